@@ -131,6 +131,17 @@ struct lrs_ctx {
       *tctr = nullptr;
   unsigned long long* ttasks = nullptr;
   unsigned long long* tprof = nullptr;  // kTaskProf counters (profile = 2)
+  // streaming engine (engine == 4): per sweep mode (INIT, LS, ITER)
+  StreamProblem sp[3]{};
+  StreamShape sshape[3]{};
+  StreamProblem* dsp = nullptr;      // device copies [3]
+  StreamAssign* sasg = nullptr;      // W assignments
+  int n_sasg = 0;
+  std::vector<StreamAssign> sasg_host;
+  int *s_cnt = nullptr, *s_list = nullptr, *s_supj = nullptr, *s_nsup = nullptr, *s_sweep = nullptr;
+  float *s_nmax = nullptr, *s_Wp = nullptr, *s_Wk = nullptr, *s_AG = nullptr, *s_u = nullptr,
+        *s_d = nullptr, *s_g = nullptr, *s_supv = nullptr;
+  double* s_Gi = nullptr;
   // graphs of one steady-state iteration: [0] plain, [1] with the refinement
   // of the measurements (low-precision forms)
   cudaGraph_t graph[2] = {nullptr, nullptr};
@@ -231,8 +242,11 @@ cudaError_t repack_a(lrs_ctx* h, const float* src, int64_t k0, int64_t kc) {
   if (h->engine == 3)
     return res_repack(src, static_cast<int>(h->n), static_cast<int>(h->m), static_cast<int>(k0),
                       static_cast<int>(kc), static_cast<float*>(h->A), h->stream);
-  return repack_gauss(h->L, src, static_cast<int>(k0), static_cast<int>(kc), h->A, nullptr,
-                      h->stream);
+  cudaError_t e = repack_gauss(h->L, src, static_cast<int>(k0), static_cast<int>(kc), h->A, nullptr,
+                               h->stream);
+  if (e == cudaSuccess && h->engine == 4)
+    e = stream_norms(h->L, h->A, nullptr, static_cast<int>(k0), static_cast<int>(kc), h->s_nmax, h->stream);
+  return e;
 }
 
 lrs_status check_device_error(lrs_ctx* h, const char* where) {
@@ -278,6 +292,18 @@ lrs_status launch_sweep(lrs_ctx* h, int mode, int tau) {
     a.wait_ns = wait_bound_ns(h);
     a.prof = (h->opt.profile == 2 && mode == kModeIter) ? h->tprof : nullptr;
     CUDA_TRY(res_launch(a, h->res_ncl, h->stream));
+    return LRS_OK;
+  }
+  if (h->engine == 4) {
+    StreamTable T{};
+    T.probs = h->dsp + mode;
+    T.nprob = 1;
+    T.ncols = static_cast<int>(h->q);
+    T.cnt = h->s_cnt;
+    T.list = h->s_list;
+    T.ncnt = h->sshape[mode].te + 1;
+    T.wait_ns = wait_bound_ns(h);
+    CUDA_TRY(stream_sweep(T, h->sshape[mode], mode, h->sasg, h->n_sasg, h->stream));
     return LRS_OK;
   }
   if (h->engine == 2) {
@@ -490,7 +516,9 @@ void free_all(lrs_ctx* h) {
     h->graph[g] = nullptr;
   }
   void* ps2[] = {h->dtp, h->dseed, h->tWk, h->tWp, h->tu, h->tg, h->tsupv, h->tGi, h->tsupj, h->tAs,
-                 h->tnsup, h->tcnt, h->tstop, h->tseq, h->tctr, h->ttasks, h->tprof};
+                 h->tnsup, h->tcnt, h->tstop, h->tseq, h->tctr, h->ttasks, h->tprof,
+                 h->dsp, h->sasg, h->s_cnt, h->s_list, h->s_supj, h->s_nsup, h->s_sweep, h->s_nmax,
+                 h->s_Wp, h->s_Wk, h->s_AG, h->s_u, h->s_d, h->s_g, h->s_supv, h->s_Gi};
   for (void* p : ps2)
     if (p) cudaFreeAsync(p, h->stream);
   void* ps[] = {h->gsplit, h->A, h->y, h->Aex, h->rscale, h->ycorr, h->U, h->Upad, h->Bk, h->S_idx, h->S_val, h->H, h->grad, h->Z,
@@ -685,6 +713,71 @@ lrs_status plan_tables(lrs_ctx* h, int task_kib, int F) {
   return LRS_OK;
 }
 
+// Streaming engine: problem descriptions (without buffers), launch shapes and
+// W assignments of the three sweep modes.  False when it cannot hold the shape.
+bool plan_stream(lrs_ctx* h, int nsm) {
+  const int R = sweep_rpad(h->r);
+  for (int mode = 0; mode < 3; ++mode) {
+    StreamProblem& P = h->sp[mode];
+    P = StreamProblem{};
+    P.L = h->L;
+    P.mode = mode;
+    P.te = h->rho == 0 ? 0 : (mode == kModeInit ? h->opt.tau0 : mode == kModeIter ? h->opt.tau : 0);
+    stream_plan(P, R);
+    if (!stream_shape(&P, 1, R, h->L.et, nsm, h->opt.grid, &h->sshape[mode], &h->sasg_host))
+      return false;
+  }
+  h->n_sasg = static_cast<int>(h->sasg_host.size());
+  return true;
+}
+
+lrs_status alloc_stream(lrs_ctx* h) {
+  const StreamProblem& P0 = h->sp[kModeIter];
+  const size_t q = static_cast<size_t>(h->q), rho1 = std::max(1, h->rho);
+  const size_t as = P0.astride, ws = P0.wstride, planes = h->L.et == 3 ? 2 : 1;
+  lrs_status st = LRS_OK;
+  if ((st = dalloc(&h->dsp, 3, h->stream)) || (st = dalloc(&h->sasg, h->n_sasg, h->stream)) ||
+      (st = dalloc(&h->s_cnt, kStreamMaxRounds + 2, h->stream)) || (st = dalloc(&h->s_list, 2 * q, h->stream)) ||
+      (st = dalloc(&h->s_supj, q * rho1, h->stream)) || (st = dalloc(&h->s_supv, q * rho1, h->stream)) ||
+      (st = dalloc(&h->s_nsup, q, h->stream)) || (st = dalloc(&h->s_sweep, q, h->stream)) ||
+      (st = dalloc(&h->s_nmax, q, h->stream)) || (st = dalloc(&h->s_Wp, q * P0.ncw * ws, h->stream)) ||
+      (st = dalloc(&h->s_Wk, q * ws, h->stream)) || (st = dalloc(&h->s_AG, q * rho1 * as, h->stream)) ||
+      (st = dalloc(&h->s_u, q * planes * as, h->stream)) || (st = dalloc(&h->s_d, q * as, h->stream)) ||
+      (st = dalloc(&h->s_g, q * h->L.ns, h->stream)) || (st = dalloc(&h->s_Gi, q * 256, h->stream)))
+    return st;
+  CUDA_TRY(cudaMemsetAsync(h->s_cnt, 0, (kStreamMaxRounds + 2) * sizeof(int), h->stream));
+  CUDA_TRY(cudaMemsetAsync(h->s_u, 0, q * planes * as * sizeof(float), h->stream));
+  for (int mode = 0; mode < 3; ++mode) {
+    StreamProblem& P = h->sp[mode];
+    P.A = h->A;
+    P.rscale = h->rscale;
+    P.y = (mode == kModeIter && h->L.et != 0) ? h->ycorr : h->y;
+    P.Upad = h->Upad;
+    P.nmax = h->s_nmax;
+    P.S_idx = h->S_idx;
+    P.S_val = h->S_val;
+    P.B = h->Bk;
+    P.H = h->H;
+    P.err = h->err;
+    P.Wp = h->s_Wp;
+    P.Wk = h->s_Wk;
+    P.Gi = h->s_Gi;
+    P.AG = h->s_AG;
+    P.uvec = h->s_u;
+    P.dvec = h->s_d;
+    P.g = h->s_g;
+    P.supj = h->s_supj;
+    P.supv = h->s_supv;
+    P.nsup = h->s_nsup;
+    P.sweep = h->s_sweep;
+  }
+  CUDA_TRY(cudaMemcpyAsync(h->dsp, h->sp, sizeof(h->sp), cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(cudaMemcpyAsync(h->sasg, h->sasg_host.data(), h->n_sasg * sizeof(StreamAssign),
+                           cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(cudaStreamSynchronize(h->stream));  // the host tables may go once this returns
+  return LRS_OK;
+}
+
 // Scratch, queue and seeds sized for every shape the autotuner may pick
 // (the smallest tasks and all q columns in flight), then the tables.
 lrs_status alloc_task_engine(lrs_ctx* h) {
@@ -727,6 +820,143 @@ lrs_status alloc_task_engine(lrs_ctx* h) {
   CUDA_TRY(cudaMemsetAsync(h->tnsup, 0, q * sizeof(int), h->stream));
   CUDA_TRY(cudaMemsetAsync(h->tstop, 0, q * sizeof(int), h->stream));
   return plan_tables(h, kib, h->tF);
+}
+
+// The shared sweep of a batch: its device tables (freed by release, stream-
+// ordered) and its launch.
+struct BatchLaunch {
+  int nh = 0, n_asg = 0;
+  // task engine
+  TaskQueue Q{};
+  TaskShape shape{};
+  TaskProblem* dP = nullptr;
+  unsigned long long *dtasks = nullptr, *dseed = nullptr;
+  int *dseq = nullptr, *dctr = nullptr, *dcnt = nullptr;
+  int64_t nseed = 0;
+  int R = 0, et = 0, m_max = 0, ns_max = 0, rho_max = 0;
+  // streaming engine
+  StreamTable T{};
+  StreamShape S{};
+  StreamProblem* dS = nullptr;
+  StreamAssign* dasg = nullptr;
+  int *s_cnt = nullptr, *s_list = nullptr;
+
+  cudaError_t sweep(cudaStream_t s) const {
+    if (dS) return stream_sweep(T, S, kModeIter, dasg, n_asg, s);
+    return task_launch_seeded(Q, dseed, static_cast<int>(nseed), dcnt, R, et, shape, m_max, ns_max,
+                              rho_max, s);
+  }
+  void release(cudaStream_t s) {
+    for (void* p : {static_cast<void*>(dP), static_cast<void*>(dtasks), static_cast<void*>(dseed),
+                    static_cast<void*>(dseq), static_cast<void*>(dctr), static_cast<void*>(dcnt),
+                    static_cast<void*>(dS), static_cast<void*>(dasg), static_cast<void*>(s_cnt),
+                    static_cast<void*>(s_list)})
+      if (p) cudaFreeAsync(p, s);
+  }
+};
+
+// Every handle's ITER-mode problem in one table, columns numbered across the
+// handles in order.
+lrs_status batch_stream(lrs_t* hs, int nh, int nsm, BatchLaunch* b) {
+  lrs_ctx* h0 = hs[0];
+  cudaStream_t s = h0->stream;
+  std::vector<StreamProblem> P(nh);
+  int64_t cols = 0;
+  for (int i = 0; i < nh; ++i) {
+    P[i] = hs[i]->sp[kModeIter];
+    P[i].col0 = static_cast<int>(cols);
+    cols += hs[i]->q;
+  }
+  if (cols >= (int64_t(1) << 30))
+    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: too many columns for one launch");
+  std::vector<StreamAssign> asg;
+  if (!stream_shape(P.data(), nh, sweep_rpad(h0->r), h0->L.et, nsm, h0->opt.grid, &b->S, &asg))
+    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: the problems' shared memory does not fit one CTA");
+  b->n_asg = static_cast<int>(asg.size());
+  lrs_status st = dalloc(&b->dS, nh, s);
+  if (!st) st = dalloc(&b->dasg, asg.size(), s);
+  if (!st) st = dalloc(&b->s_cnt, kStreamMaxRounds + 2, s);
+  if (!st) st = dalloc(&b->s_list, 2 * static_cast<size_t>(cols), s);
+  if (st) return st;
+  CUDA_TRY(cudaMemcpyAsync(b->dS, P.data(), nh * sizeof(StreamProblem), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaMemcpyAsync(b->dasg, asg.data(), asg.size() * sizeof(StreamAssign),
+                           cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaStreamSynchronize(s));  // the host tables may go once this returns
+  b->T.probs = b->dS;
+  b->T.nprob = nh;
+  b->T.ncols = static_cast<int>(cols);
+  b->T.cnt = b->s_cnt;
+  b->T.list = b->s_list;
+  b->T.ncnt = b->S.te + 1;
+  b->T.wait_ns = wait_bound_ns(h0);
+  return LRS_OK;
+}
+
+lrs_status batch_task(lrs_t* hs, int nh, int nsm, BatchLaunch* b) {
+  lrs_ctx* h0 = hs[0];
+  cudaStream_t s = h0->stream;
+  const int R = sweep_rpad(h0->r), et = h0->L.et;
+  // all columns in flight
+  std::vector<TaskProblem> P(nh);
+  int64_t cols = 0, total = 0, nseed = 0;
+  int pb_max = 0;
+  for (int i = 0; i < nh; ++i) {
+    const lrs_ctx* h = hs[i];
+    P[i] = h->tp[kModeIter];
+    P[i].col0 = static_cast<int>(cols);
+    cols += h->q;
+    total += static_cast<int64_t>(P[i].tasks_per_col) * h->q;
+    nseed += static_cast<int64_t>(phase_tasks(P[i], 0)) * h->q;
+    b->m_max = std::max<int>(b->m_max, static_cast<int>(h->m));
+    b->ns_max = std::max(b->ns_max, h->L.ns);
+    b->rho_max = std::max(b->rho_max, h->rho);
+    pb_max = std::max(pb_max, h->tshape.piece_bytes);
+  }
+  if (total >= (int64_t(1) << 31) || cols >= (int64_t(1) << 30))
+    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: too many tasks for one launch");
+  b->R = R;
+  b->et = et;
+  b->shape = h0->tshape;
+  b->shape.stages = kTaskStages;
+  b->shape.piece_bytes = pb_max;
+  b->shape.smem = task_smem_bytes(R, et, b->m_max, b->ns_max, b->rho_max, kTaskStages, pb_max);
+  if (b->shape.smem > static_cast<size_t>(max_smem_optin()))
+    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: the problems' shared memory does not fit one CTA");
+  const int cps = std::min(2, task_ctas_per_sm(R, et, b->shape.smem));
+  if (cps < 1) return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: no CTA fits an SM");
+  b->shape.grid = cps * nsm;
+  if (h0->opt.grid > 0) b->shape.grid = std::min(b->shape.grid, h0->opt.grid);
+  lrs_status st = dalloc(&b->dP, nh, s);
+  if (!st) st = dalloc(&b->dtasks, total, s);
+  if (!st) st = dalloc(&b->dseq, total, s);
+  if (!st) st = dalloc(&b->dctr, 4, s);
+  if (!st) st = dalloc(&b->dcnt, cols, s);
+  if (!st) st = dalloc(&b->dseed, nseed, s);
+  if (st) return st;
+  std::vector<unsigned long long> seed;
+  seed.reserve(nseed);
+  for (int i = 0; i < nh; ++i) {
+    P[i].cnt = b->dcnt + P[i].col0;
+    const int n0 = phase_tasks(P[i], 0);
+    for (int64_t k = 0; k < hs[i]->q; ++k)
+      for (int t = 0; t < n0; ++t)
+        seed.push_back(tdesc(static_cast<int>(k), i, phase_type(P[i], 0), 0, t));
+  }
+  CUDA_TRY(cudaMemcpyAsync(b->dP, P.data(), nh * sizeof(TaskProblem), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaMemcpyAsync(b->dseed, seed.data(), nseed * 8, cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaStreamSynchronize(s));  // the host tables may go once this returns
+  b->nseed = nseed;
+  b->Q.tasks = b->dtasks;
+  b->Q.seq = b->dseq;
+  b->Q.ctr = b->dctr;
+  b->Q.total = static_cast<int>(total);
+  b->Q.ncols = static_cast<int>(cols);
+  b->Q.F = static_cast<int>(cols);
+  b->Q.nprob = nh;
+  b->Q.probs = b->dP;
+  b->Q.prof = nullptr;
+  b->Q.wait_ns = wait_bound_ns(h0);
+  return LRS_OK;
 }
 
 }  // namespace
@@ -849,6 +1079,13 @@ lrs_status lrs_create(int64_t n, int64_t m, int64_t q, int32_t r, int32_t rho, l
   }
   if (h->engine == 2) {
     h->L = gauss_shape(h, 1, 0);
+    // The library's own choice is the streaming engine (a third of the task
+    // engine's time at n = q = 1000 near convergence); options that only the
+    // task engine has ask for that one.
+    const bool task_only = o.inflight || o.task_kib || o.ctas_per_sm || o.test_withhold || o.profile == 2;
+    if (o.engine == 0 && !task_only && plan_stream(h, nsm)) h->engine = 4;
+  }
+  if (h->engine == 2) {
     if (!plan_task_engine(h, nsm)) {
       if (o.engine == 2 || m > 512) {
         delete h;
@@ -889,7 +1126,7 @@ lrs_status lrs_create(int64_t n, int64_t m, int64_t q, int32_t r, int32_t rho, l
       (st = dalloc(&h->P, size_t(q) * r, h->stream)) || (st = dalloc(&h->part, size_t(h->nblk) * r * r, h->stream)) ||
       (st = dalloc(&h->small, 4 * 16 * 16 + 64, h->stream)) || (st = dalloc(&h->eta, 1, h->stream)) ||
       (st = dalloc(&h->err, 2, h->stream)) || (st = dalloc(&h->errpart, 2 * size_t(q), h->stream)) ||
-      (h->engine == 2 && (st = alloc_task_engine(h))) || (st = alloc_split(h, nsm))) {
+      (h->engine == 2 && (st = alloc_task_engine(h))) || (h->engine == 4 && (st = alloc_stream(h))) || (st = alloc_split(h, nsm))) {
     std::string msg = g_last_error;
     free_all(h);
     delete h;
@@ -907,6 +1144,7 @@ lrs_status lrs_create(int64_t n, int64_t m, int64_t q, int32_t r, int32_t rho, l
   }
   cudaError_t e = h->engine == 1   ? sweep_prepare(h->L, kThreads)
                   : h->engine == 3 ? res_prepare(res_rpad(r), static_cast<int>((m + 31) / 32))
+                  : h->engine == 4 ? stream_prepare(sweep_rpad(r), h->L.et)
                                    : task_prepare(sweep_rpad(r), h->L.et, h->tshape.smem);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 2 * sizeof(int), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->Upad, 0, sizeof(float) * upad_n, h->stream);
@@ -976,6 +1214,9 @@ lrs_status lrs_set_measurements(lrs_t h, const void* y, const void* A_or_mask, i
       const int64_t kc = std::min(chunk, h->q - k0);
       CUDA_TRY(repack_gauss(h->L, h->Aex + k0 * col_elems, static_cast<int>(k0),
                             static_cast<int>(kc), h->A, h->rscale, h->stream));
+      if (h->engine == 4)
+        CUDA_TRY(stream_norms(h->L, h->A, h->rscale, static_cast<int>(k0), static_cast<int>(kc),
+                              h->s_nmax, h->stream));
     }
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->state = kMeasured;
@@ -1317,72 +1558,29 @@ lrs_status lrs_iterate_batch(lrs_t* hs, int32_t nh, int32_t iters) {
   const int R = sweep_rpad(h0->r), et = h0->L.et;
   for (int i = 0; i < nh; ++i) {
     const lrs_ctx* h = hs[i];
-    if (h->F || h->engine != 2 || h->opt.reduce || sweep_rpad(h->r) != R || h->L.et != et)
+    if (h->F || (h->engine != 2 && h->engine != 4) || h->opt.reduce || sweep_rpad(h->r) != R || h->L.et != et)
       return fail(LRS_ERR_UNSUPPORTED,
-                  "lrs_iterate_batch: Gaussian task-engine handles of one rank width and A_k form");
+                  "lrs_iterate_batch: Gaussian task- or streaming-engine handles of one rank width and A_k form");
   }
   if (nh == 1) return lrs_iterate(h0, iters, nullptr);
-  // the launch's work table: every handle's ITER-mode problem, columns
-  // numbered across the handles in order; all columns in flight
-  std::vector<TaskProblem> P(nh);
-  int64_t cols = 0, total = 0, nseed = 0;
-  int m_max = 0, ns_max = 0, rho_max = 0, pb_max = 0;
-  for (int i = 0; i < nh; ++i) {
-    const lrs_ctx* h = hs[i];
-    P[i] = h->tp[kModeIter];
-    P[i].col0 = static_cast<int>(cols);
-    cols += h->q;
-    total += static_cast<int64_t>(P[i].tasks_per_col) * h->q;
-    nseed += static_cast<int64_t>(phase_tasks(P[i], 0)) * h->q;
-    m_max = std::max<int>(m_max, static_cast<int>(h->m));
-    ns_max = std::max(ns_max, h->L.ns);
-    rho_max = std::max(rho_max, h->rho);
-    pb_max = std::max(pb_max, h->tshape.piece_bytes);
+  int n4 = 0;
+  for (int i = 0; i < nh; ++i) n4 += hs[i]->engine == 4;
+  if (n4 != 0 && n4 != nh) {  // different engines share no launch: one after another, same results
+    for (int i = 0; i < nh; ++i) {
+      const lrs_status st = lrs_iterate(hs[i], iters, nullptr);
+      if (st) return st;
+    }
+    return LRS_OK;
   }
-  if (total >= (int64_t(1) << 31) || cols >= (int64_t(1) << 30))
-    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: too many tasks for one launch");
   int dev = 0, nsm = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  TaskShape shape = h0->tshape;
-  shape.stages = kTaskStages;
-  shape.piece_bytes = pb_max;
-  shape.smem = task_smem_bytes(R, et, m_max, ns_max, rho_max, kTaskStages, pb_max);
-  if (shape.smem > static_cast<size_t>(max_smem_optin()))
-    return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: the problems' shared memory does not fit one CTA");
-  const int cps = std::min(2, task_ctas_per_sm(R, et, shape.smem));
-  if (cps < 1) return fail(LRS_ERR_UNSUPPORTED, "lrs_iterate_batch: no CTA fits an SM");
-  int grid = cps * nsm;
-  if (h0->opt.grid > 0) grid = std::min(grid, h0->opt.grid);
-  shape.grid = grid;
-  // device tables (freed at the end of the call, stream-ordered)
   cudaStream_t s = h0->stream;
-  TaskProblem* dP = nullptr;
-  unsigned long long *dtasks = nullptr, *dseed = nullptr;
-  int *dseq = nullptr, *dctr = nullptr, *dcnt = nullptr;
-  lrs_status st = dalloc(&dP, nh, s);
-  if (!st) st = dalloc(&dtasks, total, s);
-  if (!st) st = dalloc(&dseq, total, s);
-  if (!st) st = dalloc(&dctr, 4, s);
-  if (!st) st = dalloc(&dcnt, cols, s);
-  if (!st) st = dalloc(&dseed, nseed, s);
-  auto release = [&]() {
-    for (void* p : {static_cast<void*>(dP), static_cast<void*>(dtasks), static_cast<void*>(dseed),
-                    static_cast<void*>(dseq), static_cast<void*>(dctr), static_cast<void*>(dcnt)})
-      if (p) cudaFreeAsync(p, s);
-  };
+  BatchLaunch bl;
+  lrs_status st = n4 ? batch_stream(hs, nh, nsm, &bl) : batch_task(hs, nh, nsm, &bl);
   if (st) {
-    release();
+    bl.release(s);
     return st;
-  }
-  std::vector<unsigned long long> seed;
-  seed.reserve(nseed);
-  for (int i = 0; i < nh; ++i) {
-    P[i].cnt = dcnt + P[i].col0;
-    const int n0 = phase_tasks(P[i], 0);
-    for (int64_t k = 0; k < hs[i]->q; ++k)
-      for (int t = 0; t < n0; ++t)
-        seed.push_back(tdesc(static_cast<int>(k), i, phase_type(P[i], 0), 0, t));
   }
   // every handle's stream waits for what was queued on it before; the
   // shared sweep runs on the first handle's stream, each handle's gradient,
@@ -1391,8 +1589,6 @@ lrs_status lrs_iterate_batch(lrs_t* hs, int32_t nh, int32_t iters) {
   cudaError_t e = cudaSuccess;
   for (auto& ev : evs)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dP, P.data(), nh * sizeof(TaskProblem), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dseed, seed.data(), nseed * 8, cudaMemcpyHostToDevice, s);
   lrs_status rs = LRS_OK;
   for (int it = 0; it < iters && e == cudaSuccess && rs == LRS_OK; ++it) {
     for (int i = 1; i < nh && e == cudaSuccess; ++i) {
@@ -1410,19 +1606,7 @@ lrs_status lrs_iterate_batch(lrs_t* hs, int32_t nh, int32_t iters) {
       }
     }
     if (e != cudaSuccess) break;
-    TaskQueue Q{};
-    Q.tasks = dtasks;
-    Q.seq = dseq;
-    Q.ctr = dctr;
-    Q.total = static_cast<int>(total);
-    Q.ncols = static_cast<int>(cols);
-    Q.F = static_cast<int>(cols);
-    Q.nprob = nh;
-    Q.probs = dP;
-    Q.prof = nullptr;
-    Q.wait_ns = wait_bound_ns(h0);
-    e = task_launch_seeded(Q, dseed, static_cast<int>(nseed), dcnt, R, et, shape, m_max, ns_max,
-                           rho_max, s);
+    e = bl.sweep(s);
     if (e == cudaSuccess) e = cudaEventRecord(evs[0], s);
     for (int i = 0; i < nh && e == cudaSuccess && rs == LRS_OK; ++i) {
       lrs_ctx* h = hs[i];
@@ -1442,7 +1626,7 @@ lrs_status lrs_iterate_batch(lrs_t* hs, int32_t nh, int32_t iters) {
     }
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  release();
+  bl.release(s);
   for (int i = 0; i < nh; ++i) cudaStreamSynchronize(hs[i]->stream);
   for (auto ev : evs)
     if (ev) cudaEventDestroy(ev);
@@ -1628,7 +1812,7 @@ lrs_status lrs_sweep_trace(lrs_t h, uint64_t* out, int64_t len) {
 // one kernel), Cholesky-QR2 (Gram partials, two factorisations, two
 // applications).
 static int launches_per_iteration(const lrs_ctx* h) {
-  const int sweep = h->engine == 2 ? 2 : 1;
+  const int sweep = h->engine == 4 ? stream_launches(h->sshape[kModeIter].te) : h->engine == 2 ? 2 : 1;
   const int grad = (h->ks > 1 || h->qc > 0) ? 2 : 1;
   return sweep + grad + 5;
 }
@@ -1651,6 +1835,18 @@ lrs_status lrs_describe(lrs_t h, char* buf, int32_t len) {
              h->res_CS, h->res_ncl, MR, R,
              res_smem_bytes(R, MR, static_cast<int>(h->m), h->rho, h->res_CS),
              launches_per_iteration(h));
+    return LRS_OK;
+  }
+  if (h->engine == 4) {
+    const StreamProblem& P = h->sp[kModeIter];
+    const StreamShape& S = h->sshape[kModeIter];
+    snprintf(buf, static_cast<size_t>(len),
+             "{\"op\": \"gaussian\", \"engine\": \"stream\", \"grid\": %d, \"w_chunks\": %d, "
+             "\"w_row_blocks\": %d, \"w_stages\": %d, \"rows_per_piece\": %d, \"g_stages\": %d, "
+             "\"step_grid\": %d, \"step_smem\": %zu, \"a_dtype\": %d, \"refine_every\": %d, "
+             "\"launches_per_iteration\": %d}",
+             S.grid, P.ncw, P.nrb, S.wS, S.grp, S.gS, S.fgrid, S.fsmem, h->L.et,
+             h->opt.refine_every, launches_per_iteration(h));
     return LRS_OK;
   }
   if (h->engine == 2) {
@@ -1679,7 +1875,8 @@ lrs_status lrs_describe(lrs_t h, char* buf, int32_t len) {
 lrs_status lrs_autotune(lrs_t h, int32_t trial_iters, char* report, int32_t len) {
   if (!h) return fail(LRS_ERR_ARG, "lrs_autotune: NULL handle");
   if (trial_iters < 1) return fail(LRS_ERR_ARG, "lrs_autotune: trial_iters < 1");
-  if (h->F || h->engine != 2) return fail(LRS_ERR_UNSUPPORTED, "lrs_autotune: task engine only");
+  if (h->F || (h->engine != 2 && h->engine != 4))
+    return fail(LRS_ERR_UNSUPPORTED, "lrs_autotune: task engine only");
   if (h->opt.reduce)
     return fail(LRS_ERR_UNSUPPORTED, "lrs_autotune: not on a column-sharded handle");
   if (h->state < kInitialised) return fail(LRS_ERR_STATE, "lrs_autotune: call lrs_init first");
@@ -1731,18 +1928,20 @@ lrs_status lrs_autotune(lrs_t h, int32_t trial_iters, char* report, int32_t len)
   };
   cudaError_t e = copy_state(true);
   const int q = static_cast<int>(h->q);
+  const bool task = h->engine == 2;  // the streaming engine has one shape: it is timed, nothing is chosen
   std::vector<std::pair<int, int>> cands;
+  if (!task) cands.push_back({0, q});
   for (int kib : kTuneKib)
     for (int F : {q, std::max(1, q / 2), std::min(q, 2 * h->tshape.grid)}) {
       std::pair<int, int> c{kib, F};
-      if (std::find(cands.begin(), cands.end(), c) == cands.end()) cands.push_back(c);
+      if (task && std::find(cands.begin(), cands.end(), c) == cands.end()) cands.push_back(c);
     }
   const int kib0 = h->t_kib, F0 = h->tF;
   std::pair<int, int> best{kib0, F0};
   float best_ms = 1e30f;
   std::string rep = "{\"trials\": [";
   for (size_t ci = 0; ci < cands.size() && e == cudaSuccess; ++ci) {
-    lrs_status st = plan_tables(h, cands[ci].first, cands[ci].second);
+    lrs_status st = task ? plan_tables(h, cands[ci].first, cands[ci].second) : LRS_OK;
     if (st) {
       cleanup();
       return st;
@@ -1775,7 +1974,7 @@ lrs_status lrs_autotune(lrs_t h, int32_t trial_iters, char* report, int32_t len)
     rep += buf;
   }
   lrs_status st = LRS_OK;
-  if (e == cudaSuccess) st = plan_tables(h, best.first, best.second);
+  if (e == cudaSuccess && task) st = plan_tables(h, best.first, best.second);
   if (e == cudaSuccess && st == LRS_OK) e = copy_state(false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   cleanup();
@@ -1787,7 +1986,7 @@ lrs_status lrs_autotune(lrs_t h, int32_t trial_iters, char* report, int32_t len)
     h->gexec[g] = nullptr;
     h->graph[g] = nullptr;
   }
-  {
+  if (task) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[tune_key(h)] = best;
   }

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace lrs {
 
 // Error codes written to the device error word {code, column} (first writer wins).
@@ -211,6 +213,75 @@ int task_ctas_per_sm(int R, int et, size_t smem);
 cudaError_t task_launch_seeded(const TaskQueue& Q, const unsigned long long* seed, int n_seed,
                                int* cnt_all, int R, int et, const TaskShape& S, int m_max,
                                int ns_max, int rho_max, cudaStream_t s);
+
+// ---- streaming engine (stream.cu; kernels in stream_impl.cuh) -----------------
+// The phases of a sweep over all columns of a launch, one kernel each; see
+// stream_impl.cuh.  One slab per column (cs == 1 layout, as the task engine).
+struct StreamProblem {
+  GaussLayout L;
+  int mode, te;         // sweep mode; IHT sweeps (0 when rho == 0)
+  const void* A;        // slab layout, element type L.et
+  const float* rscale;  // FP8 forms: q x m x (1 or 2) row scales
+  const float* y;       // q x m measurements seen by the sweep
+  const float* Upad;    // ns x R zero-padded U
+  const float* nmax;    // q: max_j ||a_j|| of the stored A_k
+  int* S_idx;           // q x rho in/out (ascending)
+  float* S_val;
+  float* B;             // q x r
+  float* H;             // q x n
+  int* err;
+  // per-column scratch
+  float* Wp;            // q x ncw x wstride: partial W per column chunk
+  float* Wk;            // q x wstride: W of the columns that wait for a pass
+  double* Gi;           // q x 16 x 16: their G^{-1}
+  float* AG;            // q x rho x astride: columns of A_k on the support
+  float* uvec;          // q x planes x astride: vector of the next pass (FP8: x row scales)
+  float* dvec;          // q x astride: A_k s - y_k of the columns that wait
+  float* g;             // q x ns result of an IHT pass
+  int* supj;            // q x rho support of the columns that wait
+  float* supv;
+  int* nsup;            // q
+  int* sweep;           // q: IHT sweep the awaited pass belongs to
+  int col0;             // index of this problem's first column in the launch
+  int wstride, astride; // m R and m rounded up to 4
+  int tbw, ncw, nrb;    // W units: tiles per column chunk, chunks, row blocks
+};
+// one CTA's share of the W units of column chunk cc of a problem: units
+// (warp idx * 8 + w) + i * 8 cnt
+struct StreamAssign {
+  int prob, cc, idx, cnt;
+};
+struct StreamTable {
+  const StreamProblem* probs;  // device
+  int nprob, ncols;
+  int* cnt;                    // [ncnt] columns in the list of each round
+  int* list;                   // [2][ncols] columns waiting for a pass (round & 1)
+  int ncnt;
+  unsigned long long wait_ns;
+};
+constexpr int kStreamMaxRounds = 126;  // IHT sweeps of a problem (counters: one per round)
+struct StreamShape {  // launch configuration of a table of problems
+  int R, et, te, maxtile, grid;
+  int wS, wtpp, gS, grp;
+  unsigned us_bytes;
+  size_t wsmem, gsmem, fsmem, nsmem;
+  int f_ag, n_ag, fgrid, ngrid;
+};
+// Fill the shape fields of P (strides, W units) for compiled rank width R.
+void stream_plan(StreamProblem& P, int R);
+// Launch shape and the W assignments of `nprob` problems (host copies); false
+// when a column's step does not fit shared memory.  grid_limit: CTAs of the
+// streaming kernels (0: all that fit).
+bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int grid_limit,
+                  StreamShape* S, std::vector<StreamAssign>* asg);
+cudaError_t stream_prepare(int R, int et);
+// One sweep of every problem of the table (all in the same mode) on stream s.
+cudaError_t stream_sweep(const StreamTable& T, const StreamShape& S, int mode,
+                         const StreamAssign* asg, int nasg, cudaStream_t s);
+int stream_launches(int te);  // kernels of one ITER sweep
+// nmax[k] = max_j ||a_j|| of columns [k0, k0 + kc) of the stored operator
+cudaError_t stream_norms(const GaussLayout& L, const void* A, const float* rscale, int k0, int kc,
+                         float* nmax, cudaStream_t s);
 
 // ---- register-resident cluster engine (resident.cu) ---------------------------
 // One thread-block cluster of CS CTAs per column at a time (persistent: the

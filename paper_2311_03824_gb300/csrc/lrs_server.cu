@@ -112,7 +112,6 @@ void run_group(const std::vector<std::shared_ptr<Job>>& g, int grid, cudaStream_
     lrs_options o = rq.opt;
     o.stream = stream;
     if (o.grid == 0) o.grid = grid;
-    if (o.engine == 0) o.engine = 2;
     lrs_status e = lrs_create(rq.n, rq.m, rq.q, rq.r, rq.rho, rq.kind, &o, &hs[i]);
     if (e == LRS_OK) e = lrs_set_measurements(hs[i], rq.y, rq.A_or_mask, rq.mem_kind);
     if (e == LRS_OK) e = lrs_init(hs[i]);

@@ -1,0 +1,20 @@
+// Instantiation of the streaming engine for rank width 16 (all stored forms
+// of A_k).
+#include "stream_impl.cuh"
+
+namespace lrs {
+void* stream_w_kernel_r16(int et) {
+  using namespace stream;
+  switch (et) {
+    case 1: return reinterpret_cast<void*>(&w_kernel<16, 1>);
+    case 2: return reinterpret_cast<void*>(&w_kernel<16, 2>);
+    case 3: return reinterpret_cast<void*>(&w_kernel<16, 3>);
+    default: return reinterpret_cast<void*>(&w_kernel<16, 0>);
+  }
+}
+void* stream_step_kernel_r16(int next) {
+  using namespace stream;
+  return next ? reinterpret_cast<void*>(&step_next_kernel<16>)
+              : reinterpret_cast<void*>(&step_first_kernel<16>);
+}
+}  // namespace lrs

@@ -1,0 +1,20 @@
+// Instantiation of the streaming engine for rank width 5 (all stored forms
+// of A_k).
+#include "stream_impl.cuh"
+
+namespace lrs {
+void* stream_w_kernel_r5(int et) {
+  using namespace stream;
+  switch (et) {
+    case 1: return reinterpret_cast<void*>(&w_kernel<5, 1>);
+    case 2: return reinterpret_cast<void*>(&w_kernel<5, 2>);
+    case 3: return reinterpret_cast<void*>(&w_kernel<5, 3>);
+    default: return reinterpret_cast<void*>(&w_kernel<5, 0>);
+  }
+}
+void* stream_step_kernel_r5(int next) {
+  using namespace stream;
+  return next ? reinterpret_cast<void*>(&step_next_kernel<5>)
+              : reinterpret_cast<void*>(&step_first_kernel<5>);
+}
+}  // namespace lrs

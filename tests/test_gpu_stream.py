@@ -1,0 +1,135 @@
+"""The streaming engine (the library's choice for Gaussian operators) against
+the FP64 oracle, step by step, at the edges of its shapes: rank widths and
+their padding, rows that end inside a 16- or 32-row block, one to several
+tiles and column chunks, no IHT, supports that fill the column, stored forms;
+and bit for bit against itself under another grid, in a batch, as a replayed
+graph and column-sharded.  Bars and exclusions as in tests/gpu_helpers.py."""
+import numpy as np
+import pytest
+
+from lrsgen import GaussianInstance
+from tests.gpu_helpers import gpu_available, new_solver
+from tests.test_gpu_parity import run_one_step, run_trajectory
+from tests.test_gpu_precision import form_one_step
+from tests.test_gpu_sharded import run_shards
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    if not gpu_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_03824_gb300 import build
+    build.build()
+
+
+def run(inst, T, **opts):
+    from paper_2311_03824_gb300 import lrs as L
+    s = new_solver(inst, **opts)
+    try:
+        assert L.lrs_describe(s.h)["engine"] == "stream"
+        s.init()
+        s.iterate(T)
+        return s.get()
+    finally:
+        s.close()
+
+
+@pytest.mark.parametrize("n,q,r,m,rho", [
+    (40, 30, 1, 20, 1),        # one row block, two tiles, padded rank
+    (64, 30, 3, 32, 0),        # no IHT
+    (140, 24, 4, 300, 5),      # m > n, several row blocks and pieces
+    (257, 30, 7, 97, 4),       # ragged tile, m = 96 + 1, rank 7 in width 8
+    (330, 30, 9, 145, 5),      # rank 9 in width 10, 16-row blocks + 1
+    (200, 30, 11, 130, 3),
+    (300, 24, 16, 160, 3),
+    (1100, 16, 5, 150, 40),    # more than 32 support entries, several chunks
+], ids=str)
+def test_one_step_shapes(n, q, r, m, rho):
+    inst = GaussianInstance(n=n, q=q, r=r, m=m, rho=rho, seed=300 + n)
+    run_one_step(inst, 10, min_whole=5, max_excluded=0.03)
+
+
+def test_support_fills_the_column():
+    inst = GaussianInstance(n=24, q=1, r=1, m=20, rho=24, seed=300)
+    run_one_step(inst, 5, min_whole=5)
+
+
+def test_trajectory():
+    inst = GaussianInstance(n=200, q=200, r=3, m=80, rho=4, seed=1)
+    run_trajectory(inst, 120, min_whole=115)
+
+
+def test_kept_entries_exceed_the_true_support():
+    """rho_max > rho: the extra entries are near zero, so their supports keep
+    changing and every sweep needs its pass."""
+    inst = GaussianInstance(n=200, q=60, r=3, m=90, rho=3, seed=14)
+    run_one_step(inst, 16, min_whole=10, rho=8, rho_max=8, max_excluded=0.03)
+
+
+@pytest.mark.parametrize("a_dtype", [1, 2, 3])
+@pytest.mark.parametrize("n,q,r,m,rho", [(200, 48, 3, 80, 4), (230, 32, 8, 150, 6),
+                                         (200, 24, 12, 130, 3)], ids=str)
+def test_stored_forms(a_dtype, n, q, r, m, rho):
+    inst = GaussianInstance(n=n, q=q, r=r, m=m, rho=rho, seed=90 + r)
+    form_one_step(inst, a_dtype, 6, min_whole=4)
+
+
+@pytest.mark.parametrize("a_dtype", [0, 1, 3])
+def test_results_do_not_depend_on_the_launch(a_dtype):
+    """Another grid, a replayed graph, a batch of uneven problems."""
+    import torch
+    from paper_2311_03824_gb300 import lrs as L
+    insts = [GaussianInstance(n=200, q=60, r=3, m=80, rho=4, seed=61),
+             GaussianInstance(n=430, q=32, r=3, m=150, rho=6, seed=62),
+             GaussianInstance(n=150, q=50, r=3, m=61, rho=0, seed=63)]
+    T = 9
+    alone = [run(i, T, a_dtype=a_dtype) for i in insts]
+    for i, a in zip(insts, alone):
+        for opts in (dict(grid=16), dict(use_graph=1, stream=torch.cuda.Stream())):
+            for x, y in zip(a, run(i, T, a_dtype=a_dtype, **opts)):
+                assert np.array_equal(x, y)
+    ss = [new_solver(i, a_dtype=a_dtype) for i in insts]
+    try:
+        for s in ss:
+            s.init()
+        L.lrs_iterate_batch([s.h for s in ss], T)
+        for s, a in zip(ss, alone):
+            for x, y in zip(a, s.get()):
+                assert np.array_equal(x, y)
+    finally:
+        for s in ss:
+            s.close()
+
+
+def test_two_shards_equal_one_handle_bit_for_bit():
+    inst = GaussianInstance(n=200, q=120, r=3, m=80, rho=4, seed=1)
+    gb, T = 16, 6
+    ranges, shards = run_shards(inst, 2, gb, T)
+    s = new_solver(inst, grad_block=gb)
+    try:
+        s.init()
+        s.iterate(T)
+        U, B, Si, Sv = s.get()
+    finally:
+        s.close()
+    for (k0, k1), states in zip(ranges, shards):
+        Us, Bs, Sis, Svs = states[T]
+        assert np.array_equal(Us, U) and np.array_equal(Bs, B[:, k0:k1])
+        assert np.array_equal(Sis, Si[k0:k1]) and np.array_equal(Svs, Sv[k0:k1])
+
+
+def test_autotune_call_keeps_the_iterate():
+    from paper_2311_03824_gb300 import lrs as L
+    inst = GaussianInstance(n=200, q=40, r=3, m=80, rho=4, seed=15)
+    s = new_solver(inst)
+    try:
+        s.init()
+        before = s.get()
+        rep = L.lrs_autotune(s.h, 2)
+        assert rep["chosen"]["ms"] > 0
+        for a, b in zip(before, s.get()):
+            assert np.array_equal(a, b)
+    finally:
+        s.close()
