@@ -161,9 +161,15 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     const unsigned char* A = static_cast<const unsigned char*>(pr.A);
     P.err = pr.err;
     __syncthreads();
-    for (int t = threadIdx.x; t < (b1 - b0) * kTW * R / 4; t += kStreamNT)
-      reinterpret_cast<float4*>(Us)[t] =
+    // U of a tile as [z][q]: the 4 R floats of the four columns of lane group q
+    // are R 16-byte chunks z, chunk z of the eight groups side by side, so that
+    // a warp's read is one conflict-free wavefront for every R (row-major, the
+    // groups lie 16 R bytes apart: 8-way conflicts at R = 8 and 16)
+    for (int t = threadIdx.x; t < (b1 - b0) * kTW * R / 4; t += kStreamNT) {
+      const int b = t / (8 * R), w = t - b * 8 * R, g = w / R, z = w - g * R;
+      reinterpret_cast<float4*>(Us)[b * 8 * R + z * 8 + g] =
           reinterpret_cast<const float4*>(pr.Upad + static_cast<size_t>(b0) * kTW * R)[t];
+    }
     __syncthreads();
     const int u0 = as.idx * kSW + wid, ustep = as.cnt * kSW;
     int pu = u0, pbt = b0;  // next piece to issue: unit, first tile
@@ -215,14 +221,14 @@ __global__ void __launch_bounds__(kStreamNT, 2)
         if (P.dead) break;
         const int nt = min(tpp, b1 - b);
         for (int tt = 0; tt < nt; ++tt, st += sub) {
-          const float* Ut = Us + static_cast<size_t>(b + tt - b0) * kTW * R + 4 * q * R;
+          const float4* Ut = reinterpret_cast<const float4*>(Us) + (b + tt - b0) * 8 * R + q;
           float4 av[RT];
 #pragma unroll
           for (int c0 = 0; c0 < 4; c0 += CP) {
             float uu[CP * R];
 #pragma unroll
             for (int z = 0; z < CP * R / 4; ++z) {
-              const float4 w = reinterpret_cast<const float4*>(Ut + c0 * R)[z];
+              const float4 w = Ut[(c0 * R / 4 + z) * 8];
               uu[4 * z] = w.x; uu[4 * z + 1] = w.y; uu[4 * z + 2] = w.z; uu[4 * z + 3] = w.w;
             }
 #pragma unroll
