@@ -395,6 +395,8 @@ cudaError_t eta_from_grad(const GlobalWork& g, double c_eta, double* eta_dev, cu
 }
 
 cudaError_t cholqr2(const GlobalWork& g, const float* Zin, float* Uout, int* err, cudaStream_t s) {
+  if (qr_cluster_fits(g.n, g.r))
+    return qr_cluster(g.n, g.r, Zin, nullptr, 0, nullptr, Uout, g.Upad, g.rpad, err, s);
   const int rr = g.r * g.r;
   double* R1 = g.small;
   double* R2 = g.small + rr;
@@ -417,6 +419,7 @@ int qr_blocks(int64_t n) {
 
 cudaError_t cholqr2_into(int n, int r, const float* Z, float* Q, float* tmp, double* part,
                          double* rfac, int* err, int nblk, cudaStream_t s) {
+  if (qr_cluster_fits(n, r)) return qr_cluster(n, r, Z, nullptr, 0, nullptr, Q, nullptr, 0, err, s);
   double* R1 = rfac;
   double* R2 = rfac + r * r;
   gram_part_kernel<<<nblk, 256, 0, s>>>(n, r, Z, nullptr, nullptr, nullptr, part);
@@ -427,8 +430,10 @@ cudaError_t cholqr2_into(int n, int r, const float* Z, float* Q, float* tmp, dou
   return cudaGetLastError();
 }
 
-cudaError_t qr_step(const GlobalWork& g, float* U, const double* eta_dev, int* err,
-                    cudaStream_t s) {
+cudaError_t qr_step(const GlobalWork& g, float* U, const float* parts, int nparts,
+                    const double* eta_dev, int* err, cudaStream_t s) {
+  if (qr_cluster_fits(g.n, g.r))
+    return qr_cluster(g.n, g.r, U, parts, nparts, eta_dev, U, g.Upad, g.rpad, err, s);
   const int rr = g.r * g.r;
   double* R1 = g.small;
   double* R2 = g.small + rr;

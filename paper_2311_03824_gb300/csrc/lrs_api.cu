@@ -348,6 +348,27 @@ lrs_status launch_sweep(lrs_ctx* h, int mode, int tau) {
 
 lrs_status column_reduce(lrs_ctx* h, const GlobalWork& g, const float* H, const float* Bk);
 
+// The gradient from H and B, eta at t = 1, and U <- Q(U - eta grad).  The QR
+// launch adds the gradient's partial blocks itself unless eta, a reducer or
+// its size needs the sum before it.  mid: event between gradient and QR.
+lrs_status gradient_and_qr(lrs_ctx* h, bool first, cudaEvent_t mid) {
+  GlobalWork g = gw(h);
+  const float* parts = g.grad;
+  int nparts = 1;
+  if (!first && !h->opt.reduce && g.gsplit && qr_cluster_fits(g.n, g.r)) {
+    CUDA_TRY(grad_partials(g, h->H, h->Bk, h->stream));
+    parts = g.gsplit;
+    nparts = g.ks;
+  } else {
+    const lrs_status st = column_reduce(h, g, h->H, h->Bk);
+    if (st != LRS_OK) return st;
+  }
+  if (mid) CUDA_TRY(cudaEventRecord(mid, h->stream));
+  if (first) CUDA_TRY(eta_from_grad(g, h->opt.c_eta, h->eta, h->stream));
+  CUDA_TRY(qr_step(g, h->U, parts, nparts, h->eta, h->err, h->stream));
+  return LRS_OK;
+}
+
 // One GDmin iteration (Algorithm 1): sweep, gradient, eta at t = 1, QR.
 // With `evs` (4 events) the phase boundaries are recorded on the stream.
 // Low-precision forms of A_k first refresh the defect-corrected measurements
@@ -361,12 +382,8 @@ lrs_status enqueue_iteration(lrs_ctx* h, bool first, cudaEvent_t* evs = nullptr,
   lrs_status st = launch_sweep(h, kModeIter, h->opt.tau);
   if (st != LRS_OK) return st;
   if (evs) CUDA_TRY(cudaEventRecord(evs[1], h->stream));
-  GlobalWork g = gw(h);
-  st = column_reduce(h, g, h->H, h->Bk);
+  st = gradient_and_qr(h, first, evs ? evs[2] : nullptr);
   if (st != LRS_OK) return st;
-  if (evs) CUDA_TRY(cudaEventRecord(evs[2], h->stream));
-  if (first) CUDA_TRY(eta_from_grad(g, h->opt.c_eta, h->eta, h->stream));
-  CUDA_TRY(qr_step(g, h->U, h->eta, h->err, h->stream));
   if (evs) CUDA_TRY(cudaEventRecord(evs[3], h->stream));
   return LRS_OK;
 }
@@ -1612,10 +1629,7 @@ lrs_status lrs_iterate_batch(lrs_t* hs, int32_t nh, int32_t iters) {
       lrs_ctx* h = hs[i];
       if (i > 0) e = cudaStreamWaitEvent(h->stream, evs[0], 0);
       if (e != cudaSuccess) break;
-      GlobalWork g = gw(h);
-      rs = column_reduce(h, g, h->H, h->Bk);
-      if (rs == LRS_OK && h->t == 0) e = eta_from_grad(g, h->opt.c_eta, h->eta, h->stream);
-      if (rs == LRS_OK && e == cudaSuccess) e = qr_step(g, h->U, h->eta, h->err, h->stream);
+      rs = gradient_and_qr(h, h->t == 0, nullptr);
       h->t += 1;
       h->state = kIterating;
     }
@@ -1808,13 +1822,15 @@ lrs_status lrs_sweep_trace(lrs_t h, uint64_t* out, int64_t len) {
 
 // Kernels one steady GDmin iteration launches (no refinement of the
 // measurements, step size already frozen): the sweep (task engine: queue
-// reset + persistent kernel), the gradient (k-split partials + their sum, or
-// one kernel), Cholesky-QR2 (Gram partials, two factorisations, two
-// applications).
+// reset + persistent kernel), the gradient (k-split partials, or one kernel),
+// and the QR, which adds the partials (one cluster launch; beyond its size the
+// partials' sum, then Gram partials, two factorisations, two applications).
 static int launches_per_iteration(const lrs_ctx* h) {
   const int sweep = h->engine == 4 ? stream_launches(h->sshape[kModeIter].te) : h->engine == 2 ? 2 : 1;
-  const int grad = (h->ks > 1 || h->qc > 0) ? 2 : 1;
-  return sweep + grad + 5;
+  const bool split = h->ks > 1 || h->qc > 0;
+  if (qr_cluster_fits(static_cast<int>(h->n), h->r))
+    return sweep + (split && h->opt.reduce ? 2 : 1) + 1;
+  return sweep + (split ? 2 : 1) + 5;
 }
 
 lrs_status lrs_describe(lrs_t h, char* buf, int32_t len) {

@@ -366,8 +366,18 @@ cudaError_t grad_reduce(const GlobalWork& g, const float* H, const float* Bk, cu
 cudaError_t grad_partials(const GlobalWork& g, const float* H, const float* Bk, cudaStream_t s);
 cudaError_t sum_blocks(int n, int r, int nb, const float* parts, float* out, cudaStream_t s);
 cudaError_t eta_from_grad(const GlobalWork& g, double c_eta, double* eta_dev, cudaStream_t s);
-cudaError_t qr_step(const GlobalWork& g, float* U, const double* eta_dev, int* err,
-                    cudaStream_t s);
+// U <- Q(U - eta grad); grad is the sum of nparts n x r blocks at parts (one
+// launch on a cluster when the matrix fits its shared memory, which also adds
+// the blocks; otherwise the blocks must already be summed: nparts == 1 and
+// parts == g.grad).
+cudaError_t qr_step(const GlobalWork& g, float* U, const float* parts, int nparts,
+                    const double* eta_dev, int* err, cudaStream_t s);
+// Cholesky-QR2 of X - eta sum of the blocks on one cluster (qr_cluster.cu).
+constexpr int kQrSmem = 200 * 1024;  // shared memory of the matrix rows of a CTA
+bool qr_cluster_fits(int n, int r);
+cudaError_t qr_cluster(int n, int r, const float* X, const float* Gparts, int nparts,
+                       const double* eta, float* Q, float* Qpad, int rpad, int* err,
+                       cudaStream_t s);
 cudaError_t cholqr2(const GlobalWork& g, const float* Zin, float* Uout, int* err,
                     cudaStream_t s);
 cudaError_t project_cols(const GlobalWork& g, const float* H, const float* U, float* P,
