@@ -140,8 +140,8 @@ struct lrs_ctx {
   std::vector<StreamAssign> sasg_host;
   int *s_cnt = nullptr, *s_list = nullptr, *s_supj = nullptr, *s_nsup = nullptr, *s_sweep = nullptr;
   float *s_nmax = nullptr, *s_Wp = nullptr, *s_Wk = nullptr, *s_AG = nullptr, *s_u = nullptr,
-        *s_d = nullptr, *s_g = nullptr, *s_supv = nullptr;
-  double* s_Gi = nullptr;
+        *s_g = nullptr, *s_supv = nullptr;
+  double* s_Li = nullptr;
   // graphs of one steady-state iteration: [0] plain, [1] with the refinement
   // of the measurements (low-precision forms)
   cudaGraph_t graph[2] = {nullptr, nullptr};
@@ -535,7 +535,7 @@ void free_all(lrs_ctx* h) {
   void* ps2[] = {h->dtp, h->dseed, h->tWk, h->tWp, h->tu, h->tg, h->tsupv, h->tGi, h->tsupj, h->tAs,
                  h->tnsup, h->tcnt, h->tstop, h->tseq, h->tctr, h->ttasks, h->tprof,
                  h->dsp, h->sasg, h->s_cnt, h->s_list, h->s_supj, h->s_nsup, h->s_sweep, h->s_nmax,
-                 h->s_Wp, h->s_Wk, h->s_AG, h->s_u, h->s_d, h->s_g, h->s_supv, h->s_Gi};
+                 h->s_Wp, h->s_Wk, h->s_AG, h->s_u, h->s_g, h->s_supv, h->s_Li};
   for (void* p : ps2)
     if (p) cudaFreeAsync(p, h->stream);
   void* ps[] = {h->gsplit, h->A, h->y, h->Aex, h->rscale, h->ycorr, h->U, h->Upad, h->Bk, h->S_idx, h->S_val, h->H, h->grad, h->Z,
@@ -759,8 +759,8 @@ lrs_status alloc_stream(lrs_ctx* h) {
       (st = dalloc(&h->s_nsup, q, h->stream)) || (st = dalloc(&h->s_sweep, q, h->stream)) ||
       (st = dalloc(&h->s_nmax, q, h->stream)) || (st = dalloc(&h->s_Wp, q * P0.ncw * ws, h->stream)) ||
       (st = dalloc(&h->s_Wk, q * ws, h->stream)) || (st = dalloc(&h->s_AG, q * rho1 * as, h->stream)) ||
-      (st = dalloc(&h->s_u, q * planes * as, h->stream)) || (st = dalloc(&h->s_d, q * as, h->stream)) ||
-      (st = dalloc(&h->s_g, q * h->L.ns, h->stream)) || (st = dalloc(&h->s_Gi, q * 256, h->stream)))
+      (st = dalloc(&h->s_u, q * planes * as, h->stream)) || 
+      (st = dalloc(&h->s_g, q * h->L.ns, h->stream)) || (st = dalloc(&h->s_Li, q * 256, h->stream)))
     return st;
   CUDA_TRY(cudaMemsetAsync(h->s_cnt, 0, (kStreamMaxRounds + 2) * sizeof(int), h->stream));
   CUDA_TRY(cudaMemsetAsync(h->s_u, 0, q * planes * as * sizeof(float), h->stream));
@@ -778,10 +778,9 @@ lrs_status alloc_stream(lrs_ctx* h) {
     P.err = h->err;
     P.Wp = h->s_Wp;
     P.Wk = h->s_Wk;
-    P.Gi = h->s_Gi;
+    P.Li = h->s_Li;
     P.AG = h->s_AG;
     P.uvec = h->s_u;
-    P.dvec = h->s_d;
     P.g = h->s_g;
     P.supj = h->s_supj;
     P.supv = h->s_supv;
@@ -1861,7 +1860,7 @@ lrs_status lrs_describe(lrs_t h, char* buf, int32_t len) {
              "\"w_row_blocks\": %d, \"w_stages\": %d, \"rows_per_piece\": %d, \"g_stages\": %d, "
              "\"step_grid\": %d, \"step_smem\": %zu, \"a_dtype\": %d, \"refine_every\": %d, "
              "\"launches_per_iteration\": %d}",
-             S.grid, P.ncw, P.nrb, S.wS, S.grp, S.gS, S.fgrid, S.fsmem, h->L.et,
+             S.grid, P.ncw, P.nrb, S.wS, S.grp, S.gS, S.fgrid[P.variant], S.fsmem[P.variant], h->L.et,
              h->opt.refine_every, launches_per_iteration(h));
     return LRS_OK;
   }

@@ -232,11 +232,10 @@ struct StreamProblem {
   int* err;
   // per-column scratch
   float* Wp;            // q x ncw x wstride: partial W per column chunk
-  float* Wk;            // q x wstride: W of the columns that wait for a pass
-  double* Gi;           // q x 16 x 16: their G^{-1}
+  float* Wk;            // q x wstride: Q = W L^{-T} (R x m) of the columns that wait for a pass
+  double* Li;           // q x 16 x 16: their L^{-1}, W^T W = L L^T
   float* AG;            // q x rho x astride: columns of A_k on the support
   float* uvec;          // q x planes x astride: vector of the next pass (FP8: x row scales)
-  float* dvec;          // q x astride: A_k s - y_k of the columns that wait
   float* g;             // q x ns result of an IHT pass
   int* supj;            // q x rho support of the columns that wait
   float* supv;
@@ -245,6 +244,7 @@ struct StreamProblem {
   int col0;             // index of this problem's first column in the launch
   int wstride, astride; // m R and m rounded up to 4
   int tbw, ncw, nrb;    // W units: tiles per column chunk, chunks, row blocks
+  int variant;          // kernel of the column steps (stream_impl.cuh)
 };
 // one CTA's share of the W units of column chunk cc of a problem: units
 // (warp idx * 8 + w) + i * 8 cnt
@@ -264,8 +264,9 @@ struct StreamShape {  // launch configuration of a table of problems
   int R, et, te, maxtile, grid;
   int wS, wtpp, gS, grp;
   unsigned us_bytes;
-  size_t wsmem, gsmem, fsmem, nsmem;
-  int f_ag, n_ag, fgrid, ngrid;
+  size_t wsmem, gsmem;
+  size_t fsmem[3], nsmem[3];  // column steps by variant (0: none of it)
+  int fgrid[3], ngrid[3];
 };
 // Fill the shape fields of P (strides, W units) for compiled rank width R.
 void stream_plan(StreamProblem& P, int R);

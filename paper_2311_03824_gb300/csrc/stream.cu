@@ -8,7 +8,7 @@
 
 namespace lrs {
 #define LRS_STREAM_R(X) X(2) X(3) X(4) X(5) X(6) X(8) X(10) X(12) X(16)
-#define LRS_DECL(R) void* stream_w_kernel_r##R(int et); void* stream_step_kernel_r##R(int next);
+#define LRS_DECL(R) void* stream_w_kernel_r##R(int et); void* stream_step_kernel_r##R(int next, int variant);
 LRS_STREAM_R(LRS_DECL)
 #undef LRS_DECL
 
@@ -21,8 +21,8 @@ void* pick_w(int R, int et) {
 #undef LRS_CASE
   return nullptr;
 }
-void* pick_step(int R, int next) {
-#define LRS_CASE(X) case X: return stream_step_kernel_r##X(next);
+void* pick_step(int R, int next, int variant) {
+#define LRS_CASE(X) case X: return stream_step_kernel_r##X(next, variant);
   switch (R) { LRS_STREAM_R(LRS_CASE) }
 #undef LRS_CASE
   return nullptr;
@@ -278,6 +278,12 @@ void stream_plan(StreamProblem& P, int R) {
   P.tbw = std::max(1, std::min(cap, want));
   P.ncw = (ntile + P.tbw - 1) / P.tbw;
   P.nrb = (m + w_rows(R) - 1) / w_rows(R);
+  // Column steps: 128 threads while four columns fit an SM with their support
+  // staged, 256 threads for larger columns, the support's columns read from
+  // memory when two staged columns do not fit.  By the problem's own sizes, so
+  // that a batch runs the same arithmetic.
+  auto smem = [&](int v) { return step_carve(R, m, P.L.n, P.L.rho, P.astride, v, true).total; };
+  P.variant = smem(0) <= 54 * 1024 ? 0 : smem(1) <= 112 * 1024 ? 1 : 2;
 }
 
 bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int grid_limit,
@@ -290,7 +296,6 @@ bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int
   int m_max = 0, ncols = 0;
   unsigned us = 0;
   double work = 0;
-  size_t f0 = 0, f1 = 0, n0 = 0, n1 = 0;
   for (int i = 0; i < nprob; ++i) {
     const StreamProblem& p = P[i];
     m_max = std::max(m_max, p.L.m);
@@ -299,18 +304,12 @@ bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int
     us = std::max(us, static_cast<unsigned>(p.tbw * kTW * R * 4));
     ncols += p.L.q;
     work += static_cast<double>(p.L.q) * p.nrb * p.ncw * p.tbw;
-    f0 = std::max<size_t>(f0, step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, false, false).total);
-    f1 = std::max<size_t>(f1, step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, true, false).total);
-    n0 = std::max<size_t>(n0, step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, false, true).total);
-    n1 = std::max<size_t>(n1, step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, true, true).total);
+    const int v = p.variant;
+    S->fsmem[v] = std::max<size_t>(S->fsmem[v], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, v, false).total);
+    S->nsmem[v] = std::max<size_t>(S->nsmem[v], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, v, true).total);
+    if (S->nsmem[v] > one) return false;
   }
   if (S->te > kStreamMaxRounds) return false;
-  // column steps: the support's columns staged when two CTAs still fit an SM
-  S->f_ag = f1 <= two;
-  S->n_ag = n1 <= two;
-  S->fsmem = S->f_ag ? f1 : f0;
-  S->nsmem = S->n_ag ? n1 : n0;
-  if (S->fsmem > one || S->nsmem > one) return false;
   // W: pieces of about 4 KB, as many stages as two CTAs per SM allow
   S->us_bytes = (us + 127u) & ~127u;
   const unsigned sub = static_cast<unsigned>(w_rows(R) * kTW * eb);
@@ -331,11 +330,13 @@ bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int
   if (grid_limit > 0) S->grid = std::min(S->grid, grid_limit);
   // columns at once in the steps: what fits, scaled like the streaming grid
   auto step_grid = [&](size_t smem, int cap) {
-    const int fit = static_cast<int>(std::max<size_t>(1, std::min<size_t>(cap, 227 * 1024 / (smem + 1024))));
+    const int fit = static_cast<int>(std::max<size_t>(1, std::min<size_t>(cap, 227 * 1024 / (smem + 2048))));
     return std::max(1, std::min(ncols, static_cast<int>(static_cast<long>(fit) * S->grid / 2)));
   };
-  S->fgrid = step_grid(S->fsmem, 8);
-  S->ngrid = step_grid(S->nsmem, 6);
+  for (int v = 0; v < 3; ++v) {
+    S->fgrid[v] = S->fsmem[v] ? step_grid(S->fsmem[v], v == 0 ? 8 : 3) : 0;
+    S->ngrid[v] = S->nsmem[v] ? step_grid(S->nsmem[v], v == 0 ? 6 : 3) : 0;
+  }
   // W assignments: every (problem, chunk) gets CTAs by its share of the work
   // (at least one; CTAs take several assignments when there are more)
   asg->clear();
@@ -351,7 +352,8 @@ bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int
 }
 
 cudaError_t stream_prepare(int R, int et) {
-  void* fs[] = {pick_w(R, et), pick_g(et), pick_step(R, 0), pick_step(R, 1)};
+  void* fs[] = {pick_w(R, et),        pick_g(et),           pick_step(R, 0, 0), pick_step(R, 0, 1),
+                pick_step(R, 0, 2), pick_step(R, 1, 0), pick_step(R, 1, 1), pick_step(R, 1, 2)};
   for (void* f : fs) {
     // what a CTA may request beside the kernel's static shared memory
     cudaFuncAttributes at{};
@@ -371,14 +373,15 @@ cudaError_t stream_sweep(const StreamTable& T, const StreamShape& S, int mode,
   StreamTable t = T;
   cudaError_t e = cudaSuccess;
   auto first = [&]() {
-    int a_n = nasg, wS = S.wS, tpp = S.wtpp, ag = S.f_ag;
+    int a_n = nasg, wS = S.wS, tpp = S.wtpp;
     unsigned us = S.us_bytes;
     void* wa[] = {&t, &asg, &a_n, &wS, &tpp, &us};
     cudaError_t x = cudaLaunchKernel(pick_w(S.R, S.et), dim3(std::min(S.grid, nasg)), dim3(kStreamNT),
                                      wa, S.wsmem, s);
-    void* sa[] = {&t, &ag};
-    if (x == cudaSuccess)
-      x = cudaLaunchKernel(pick_step(S.R, 0), dim3(S.fgrid), dim3(kStepNT), sa, S.fsmem, s);
+    void* sa[] = {&t};
+    for (int v = 0; v < 3; ++v)
+      if (x == cudaSuccess && S.fgrid[v])
+        x = cudaLaunchKernel(pick_step(S.R, 0, v), dim3(S.fgrid[v]), dim3(step_threads(v)), sa, S.fsmem[v], s);
     return x;
   };
   auto pass = [&](const int* list, const int* count, int final) {
@@ -387,9 +390,12 @@ cudaError_t stream_sweep(const StreamTable& T, const StreamShape& S, int mode,
     return cudaLaunchKernel(pick_g(S.et), dim3(S.grid), dim3(kStreamNT), ga, S.gsmem, s);
   };
   auto next = [&](int round, int zero) {
-    int ag = S.n_ag;
-    void* na[] = {&t, &round, &zero, &ag};
-    return cudaLaunchKernel(pick_step(S.R, 1), dim3(S.ngrid), dim3(kStepNT), na, S.nsmem, s);
+    void* na[] = {&t, &round, &zero};
+    cudaError_t x = cudaSuccess;
+    for (int v = 0; v < 3; ++v)
+      if (x == cudaSuccess && S.ngrid[v])
+        x = cudaLaunchKernel(pick_step(S.R, 1, v), dim3(S.ngrid[v]), dim3(step_threads(v)), na, S.nsmem[v], s);
+    return x;
   };
   if (mode == kModeInit) {
     init_vec_kernel<<<std::min(T.ncols, 1216), 128, 0, s>>>(t);

@@ -52,8 +52,6 @@ using sweep::kTW;
 
 constexpr int kSW = 8;            // warps per streaming CTA
 constexpr int kStreamNT = 32 * kSW;
-constexpr int kStepNT = 128;      // threads per column step
-constexpr int kStepNW = kStepNT / 32;
 constexpr int kMaxStage = 4;
 
 __device__ __forceinline__ unsigned long long gtimer() {
@@ -328,38 +326,95 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   const float z = s - a;
   e = (a - (s - z)) + (b - z);
 }
+struct df {
+  float h, l;
+};
+__device__ __forceinline__ df df_norm(float s, float e) {
+  df r;
+  r.h = s + e;
+  r.l = e - (r.h - s);
+  return r;
+}
+__device__ __forceinline__ df df_make(double x) {
+  df r;
+  r.h = static_cast<float>(x);
+  r.l = static_cast<float>(x - static_cast<double>(r.h));
+  return r;
+}
+__device__ __forceinline__ df df_mul(df a, df b) {
+  const float p = a.h * b.h;
+  return df_norm(p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h));
+}
+__device__ __forceinline__ df df_sub(df a, df b) {
+  float s, e;
+  two_sum(a.h, -b.h, s, e);
+  return df_norm(s, e + (a.l - b.l));
+}
+__device__ __forceinline__ df df_shfl(df a, int src) {
+  return df{__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src)};
+}
+// 1 / sqrt(a): float estimate and one Newton step y + y (1 - a y^2) / 2
+__device__ __forceinline__ df df_rsqrt(df a) {
+  const float y = rsqrtf(a.h);
+  const float y2 = y * y, y2l = fmaf(y, y, -y2);
+  const df t = df_mul(a, df_norm(y2, y2l));
+  const float d = (1.f - t.h) - t.l;  // exact difference near 1
+  return df_norm(y, 0.5f * y * d);
+}
+
+// Sums over the warp of N values at once (N a power of two <= 16): after
+// the halving exchanges lane i holds the total of value i / (32 / N).
+template <int N>
+__device__ __forceinline__ float reduce_multi(float (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int off = 16;
+#pragma unroll
+  for (int n = N; n > 1; n >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int k = 0; k < n / 2; ++k) {
+      const float send = up ? v[k] : v[k + n / 2], keep = up ? v[k + n / 2] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+  return v[0];
+}
+
+// Column steps come in three variants by the column's size (stream_plan):
+// 128 threads with the support's columns in shared memory, 256 threads with
+// them, 256 threads reading them from AG_k.
+__host__ __device__ constexpr int step_threads(int variant) { return variant == 0 ? 128 : 256; }
+__host__ __device__ constexpr bool step_staged(int variant) { return variant < 2; }
 
 struct StepCarve {
-  unsigned W, d, u, v, p, uref, gG, sv, sj, src, red, gi, dbl, ag, vv, tie, hist, lists, total;
-  int ms;
+  unsigned dbl, Lf, Q, u, p, uref, gG, sv, sj, red, ag, vv, tie, hist, lists, total;
+  int ms, rp;
 };
-// Shared memory of a column step; ag: the support's columns are staged too;
-// next: the arrays of the full HardThreshold.
-__host__ __device__ inline StepCarve step_carve(int R, int m, int n, int rho, int astride, bool ag,
-                                                bool next) {
+// Shared memory of a column step; next: the arrays of the full HardThreshold.
+__host__ __device__ inline StepCarve step_carve(int R, int m, int n, int rho, int astride,
+                                                int variant, bool next) {
   StepCarve c;
   size_t o = 0;
-  const size_t rp = rho > 0 ? rho : 1;
+  c.rp = ((rho > 0 ? rho : 1) + 3) & ~3;
+  const size_t rp = c.rp;
   auto put = [&](size_t bytes) {
     const unsigned at = static_cast<unsigned>(o);
     o += a16(bytes);
     return at;
   };
   c.ms = m | 1;
-  c.dbl = put(static_cast<size_t>(3) * 16 * 16 * 8);
-  c.W = put(static_cast<size_t>(R) * c.ms * 4);
-  c.d = put(static_cast<size_t>(m) * 4);
+  c.dbl = put(static_cast<size_t>(3) * 256 * 8);
+  c.Lf = put(256 * 4);
+  c.ag = put(step_staged(variant) ? rp * static_cast<size_t>(astride) * 4 : 0);
+  c.Q = put(static_cast<size_t>(R) * c.ms * 4);
   c.u = put(static_cast<size_t>(m) * 4);
-  c.v = put(static_cast<size_t>(m) * 4);
   c.p = put(static_cast<size_t>(m) * 4);
   c.uref = put(next ? static_cast<size_t>(m) * 4 : 0);
   c.gG = put(rp * 4);
   c.sv = put(2 * rp * 4);
   c.sj = put(rp * 4);
-  c.src = put(rp * 4);
-  c.red = put((kStepNW * 16 + 4 * kStepNW + 16) * 4);
-  c.gi = put(static_cast<size_t>(2) * 16 * 16 * 4);
-  c.ag = put(ag ? rp * static_cast<size_t>(astride) * 4 : 0);
+  c.red = put((8 * 16 + 5 * 8) * 4);
   c.vv = put(next ? static_cast<size_t>(n) * 4 : 0);
   c.tie = put(next ? (static_cast<size_t>(n) + 2 * rp + 8) * 4 : 0);
   c.hist = put(next ? (256 + 16) * 4 : 0);
@@ -368,65 +423,103 @@ __host__ __device__ inline StepCarve step_carve(int R, int m, int n, int rho, in
   return c;
 }
 
-template <int R>
+// One column on one CTA.  P_perp is applied through an orthonormal basis Q of
+// range(W_k): Q = W L^{-T} with G = W^T W = L L^T, so P v = v - Q (Q^T v), the
+// residual of the LS step is e = Q Q^T r - r and b = L^{-T} (Q^T r): one matrix
+// in shared memory and no r x r solve inside the sweeps.
+// Slots of scal: 0 ||g_G||^2, 1 / 2 ||u||^2 (by sweep parity), 3 ||u - uref||^2,
+// 4 ||P A_G g_G||^2.
+template <int R, int V>
 struct Step {
+  static constexpr int NT = step_threads(V), NW = NT / 32;
+  static constexpr int RN = R <= 2 ? 2 : R <= 4 ? 4 : R <= 8 ? 8 : 16;
   const StreamTable& T;
-  const StreamProblem& pr;
-  int k, c, m, n, r, rho, te, ms, nl, par;
-  float *Wt, *d, *u, *v, *p, *uref, *gG, *svb, *red, *gi;
-  int *sj, *src;
-  double* G;
-  float* agsm;       // staged support columns, or nullptr (read from AG_k)
+  const StreamProblem& pr;  // shared-memory copy
+  int k, c, m, n, r, rho, te, ms, rp, nl, par, as;
+  float *Q, *u, *p, *uref, *gG, *svb, *red, *Lf;
+  int* sj;
+  double* G;     // Gram, then L (fallback), L^{-1} at G + 512 (16 x 16 each)
+  float* ag;     // support columns: slot e at ag + e as
   bool project;
 
   __device__ Step(const StreamTable& t, const StreamProblem& prob, unsigned char* smem,
-                  const StepCarve& cv, bool ag)
+                  const StepCarve& cv)
       : T(t), pr(prob) {
     m = pr.L.m;
     n = pr.L.n;
     r = pr.L.r;
     rho = pr.L.rho;
     te = pr.te;
+    as = pr.astride;
     ms = cv.ms;
+    rp = cv.rp;
     par = 0;
     nl = 0;
     auto f = [&](unsigned o) { return reinterpret_cast<float*>(smem + o); };
-    Wt = f(cv.W); d = f(cv.d); u = f(cv.u); v = f(cv.v); p = f(cv.p); uref = f(cv.uref); gG = f(cv.gG);
-    svb = f(cv.sv); red = f(cv.red); gi = f(cv.gi);
+    Q = f(cv.Q); u = f(cv.u); p = f(cv.p); uref = f(cv.uref); gG = f(cv.gG);
+    svb = f(cv.sv); red = f(cv.red); Lf = f(cv.Lf);
     sj = reinterpret_cast<int*>(smem + cv.sj);
-    src = reinterpret_cast<int*>(smem + cv.src);
     G = reinterpret_cast<double*>(smem + cv.dbl);
-    agsm = ag ? f(cv.ag) : nullptr;
     project = pr.mode != kModeInit;
   }
-  __device__ float* sv(int p) const { return svb + p * max(rho, 1); }
-  // column of A_k of support slot e
-  __device__ const float* ag(int e) const {
-    return agsm ? agsm + static_cast<size_t>(e) * pr.astride
-                : pr.AG + (static_cast<size_t>(k) * rho + src[e]) * pr.astride;
+  __device__ void at_column(int col, unsigned char* smem, const StepCarve& cv) {
+    c = col;
+    k = col - pr.col0;
+    if constexpr (step_staged(V)) ag = reinterpret_cast<float*>(smem + cv.ag);
+    else ag = pr.AG + static_cast<size_t>(k) * rho * as;
   }
-  // AG_k into shared memory (rows beyond m are never used)
-  __device__ void stage_support() const {
-    if (!agsm) return;
-    const int a4 = pr.astride / 4;
-#pragma unroll 4
-    for (int t = threadIdx.x; t < nl * a4; t += kStepNT) {
-      const int e = t / a4, i4 = t - e * a4;
-      reinterpret_cast<float4*>(agsm)[t] = __ldcg(
-          reinterpret_cast<const float4*>(pr.AG + (static_cast<size_t>(k) * rho + src[e]) * pr.astride) + i4);
+  __device__ float* sv(int q) const { return svb + q * rp; }
+  __device__ float* ag_global() const { return pr.AG + static_cast<size_t>(k) * rho * as; }
+
+  // ---- staging of AG_k by one bulk copy ----
+  __device__ void stage_begin(uint64_t* bar) const {
+    if constexpr (step_staged(V)) {
+      if (threadIdx.x == 0 && rho > 0) {
+        asm volatile("fence.proxy.async;" ::: "memory");  // earlier reads of the buffer first
+        const unsigned bytes = static_cast<unsigned>(rho * as * 4);
+        mbar_arrive_expect_tx(bar, bytes);
+        bulk_copy_g2s(ag, ag_global(), bytes, bar);
+      }
     }
   }
-  __device__ float* coefs() const { return red; }
-  __device__ float* scal(int s) const { return red + kStepNW * 16 + s * kStepNW; }
+  __device__ void stage_end(uint64_t* bar, unsigned& phase) const {
+    if constexpr (step_staged(V)) {
+      if (rho > 0) {
+        if (!mbar_try_wait(bar, phase)) {
+          const unsigned long long t0 = gtimer();
+          while (!mbar_try_wait(bar, phase))
+            if (gtimer() - t0 > T.wait_ns) {
+              report_error(pr.err, kErrTimeout, -1);
+              break;
+            }
+        }
+        phase ^= 1u;
+      }
+    }
+  }
 
+  // ---- reductions ----
   __device__ void put_coefs(const float (&acc)[R]) const {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float v[RN];
 #pragma unroll
-    for (int l = 0; l < R; ++l) {
-      const float t = warp_sum(acc[l]);
-      if (lane == 0) coefs()[w * 16 + l] = t;
-    }
+    for (int l = 0; l < RN; ++l) v[l] = l < R ? acc[l < R ? l : 0] : 0.f;
+    const float t = reduce_multi<RN>(v);
+    constexpr int step = 32 / RN;
+    if (lane % step == 0) red[w * 16 + lane / step] = t;
   }
+  // (after a barrier) the coefficients in every thread; returns this lane's own
+  __device__ float get_coefs(float (&cf)[R]) const {
+    const int lane = threadIdx.x & 31;
+    float own = 0.f;
+    if (lane < R)
+#pragma unroll
+      for (int w = 0; w < NW; ++w) own += red[w * 16 + lane];
+#pragma unroll
+    for (int l = 0; l < R; ++l) cf[l] = __shfl_sync(0xffffffffu, own, l);
+    return own;
+  }
+  __device__ float* scal(int s) const { return red + 8 * 16 + s * 8; }
   __device__ void put_scal(int s, float x) const {
     x = warp_sum(x);
     if ((threadIdx.x & 31) == 0) scal(s)[threadIdx.x >> 5] = x;
@@ -434,293 +527,286 @@ struct Step {
   __device__ float get_scal(int s) const {
     float x = 0.f;
 #pragma unroll
-    for (int w = 0; w < kStepNW; ++w) x += scal(s)[w];
+    for (int w = 0; w < NW; ++w) x += scal(s)[w];
     return x;
   }
-  // x = G^{-1} c from the warps' partial sums of c (after a barrier), in
-  // double-float; every warp computes it.  Returns this lane's own x_lane.
-  __device__ float solve(float (&x)[R]) const {
-    const int lane = threadIdx.x & 31;
-    float cl = 0.f;
-    if (lane < r)
-#pragma unroll
-      for (int w = 0; w < kStepNW; ++w) cl += coefs()[w * 16 + lane];
-    float xh = 0.f, xl = 0.f;
-    for (int b = 0; b < r; ++b) {
-      const float cb = __shfl_sync(0xffffffffu, cl, b);
-      if (lane < r) {
-        const float gh = gi[lane * 16 + b], gl = gi[256 + lane * 16 + b];
-        const float p = gh * cb;
-        const float e = fmaf(gl, cb, fmaf(gh, cb, -p));
-        float s, t;
-        two_sum(xh, p, s, t);
-        xh = s;
-        xl += t + e;
-      }
+  // sum_e AG(i, e) x_e over the support
+  __device__ float support_row(int i, const float* x) const {
+    float t = 0.f;
+    const float* a = ag + i;
+    int e = 0;
+    for (; e + 4 <= nl; e += 4, a += 4 * as) {
+      const float4 xe = *reinterpret_cast<const float4*>(x + e);
+      t = fmaf(a[0], xe.x, t);
+      t = fmaf(a[as], xe.y, t);
+      t = fmaf(a[2 * as], xe.z, t);
+      t = fmaf(a[3 * as], xe.w, t);
     }
-    const float own = lane < r ? xh + xl : 0.f;
-#pragma unroll
-    for (int l = 0; l < R; ++l) x[l] = __shfl_sync(0xffffffffu, own, l);
-    return own;
-  }
-  __device__ void load_inverse(const double* Gi) const {
-    for (int t = threadIdx.x; t < 256; t += kStepNT) {
-      const double g = (t >> 4) < r && (t & 15) < r ? Gi[t] : 0.0;
-      const float h = static_cast<float>(g);
-      gi[t] = h;
-      gi[256 + t] = static_cast<float>(g - static_cast<double>(h));
-    }
+    for (; e < nl; ++e, a += as) t = fmaf(a[0], x[e], t);
+    return t;
   }
 
-  // Gram W^T W summed in double-float from exact products (two floats hold a
-  // product exactly), then its inverse into G + 512 (16 x 16): Cholesky in
-  // FP32 and one Newton-Schulz step in FP64, or all in FP64 when a pivot is
-  // too small for FP32 (which also reports a Gram that is not positive).
-  __device__ void gram_inverse() const {
+  // ---- Gram of W (in Q's buffer), its inverse factor, Q = W L^{-T} in place ----
+  // The Gram is summed in double-float from exact products; the factor and
+  // its inverse are double-float in one warp's registers (lane = row, then
+  // lane = column).  A pivot below 1e-9 of its diagonal goes to the FP64
+  // routine, which also reports a Gram that is not positive.
+  __device__ void factor() const {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int t = w; t < r * (r + 1) / 2; t += kStepNW) {
-      int p = 0;
-      while ((p + 1) * (p + 2) / 2 <= t) ++p;
-      const int q2 = t - p * (p + 1) / 2;
-      const float *wp = Wt + p * ms, *wq = Wt + q2 * ms;
-      float hi = 0.f, lo = 0.f;
-      for (int i = lane; i < m; i += 32) {
-        const float a = wp[i], b = wq[i], pdt = a * b;
-        float s, e;
-        two_sum(hi, pdt, s, e);
-        hi = s;
-        lo += e + fmaf(a, b, -pdt);
+    const int ne = r * (r + 1) / 2;
+    for (int t0 = 4 * w; t0 < ne; t0 += 4 * NW) {
+      const float *pa[4], *pb[4];
+      float hi[4], lo[4];
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int t = min(t0 + z, ne - 1);
+        int a = 0;
+        while ((a + 1) * (a + 2) / 2 <= t) ++a;
+        pa[z] = Q + a * ms;
+        pb[z] = Q + (t - a * (a + 1) / 2) * ms;
+        hi[z] = lo[z] = 0.f;
+      }
+      for (int i = lane; i < m; i += 32)
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const float x = pa[z][i], y = pb[z][i], q = x * y;
+          float s, e;
+          two_sum(hi[z], q, s, e);
+          hi[z] = s;
+          lo[z] += e + fmaf(x, y, -q);
+        }
+      // two halvings leave one entry per lane group of eight, then its sum
+#pragma unroll
+      for (int h = 2, off = 16; h >= 1; h >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int z = 0; z < h; ++z) {
+          const float sh = up ? hi[z] : hi[z + h], sl = up ? lo[z] : lo[z + h];
+          const float kh = up ? hi[z + h] : hi[z], kl = up ? lo[z + h] : lo[z];
+          float s, e;
+          two_sum(kh, __shfl_xor_sync(0xffffffffu, sh, off), s, e);
+          hi[z] = s;
+          lo[z] = kl + __shfl_xor_sync(0xffffffffu, sl, off) + e;
+        }
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+      for (int off = 4; off > 0; off >>= 1) {
         float s, e;
-        two_sum(hi, bh, s, e);
-        hi = s;
-        lo += bl + e;
+        two_sum(hi[0], __shfl_xor_sync(0xffffffffu, hi[0], off), s, e);
+        hi[0] = s;
+        lo[0] += __shfl_xor_sync(0xffffffffu, lo[0], off) + e;
       }
-      if (lane == 0) {
-        const double s = static_cast<double>(hi) + static_cast<double>(lo);
-        G[p * 16 + q2] = s;
-        G[q2 * 16 + p] = s;
+      const int t = t0 + (lane >> 3);
+      if ((lane & 7) == 0 && t < ne) {
+        int a = 0;
+        while ((a + 1) * (a + 2) / 2 <= t) ++a;
+        const int b = t - a * (a + 1) / 2;
+        const double g = static_cast<double>(hi[0]) + static_cast<double>(lo[0]);
+        G[a * 16 + b] = g;
+        G[b * 16 + a] = g;
       }
     }
     __syncthreads();
-    float* Lf = reinterpret_cast<float*>(G + 256);
-    float* Lif = Lf + 256;
-    double* X = G + 512;
-    int ok = 1;
-    if (threadIdx.x < 32) {
-      float ij_own = 0.f;
-      for (int j = 0; j < r; ++j) {  // column j of L, a row per lane
-        float t = 0.f;
-        if (lane >= j && lane < r) {
-          t = static_cast<float>(G[lane * 16 + j]);
-          for (int p = 0; p < j; ++p) t = fmaf(-Lf[lane * 16 + p], Lf[j * 16 + p], t);
-        }
-        const float s = __shfl_sync(0xffffffffu, t, j);
-        if (!(s > 1e-5f * static_cast<float>(G[j * 16 + j])) || !(s < 1e30f)) { ok = 0; break; }
-        const float ij = rsqrtf(s);
-        if (lane == j) ij_own = ij;
-        if (lane >= j && lane < r) Lf[lane * 16 + j] = lane == j ? s * ij : t * ij;
-        __syncwarp();
+    double* Li = G + 512;
+    if (w == 0) {
+      bool ok = true;
+      df a[R], inv[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) a[q] = lane < r && q < r ? df_make(G[lane * 16 + q]) : df{0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        inv[j] = df{1.f, 0.f};
+        if (j >= r || !ok) continue;
+        const df pv = df_shfl(a[j], j);
+        ok = pv.h > 1e-9f * static_cast<float>(G[j * 16 + j]) && pv.h > 1e-30f && pv.h < 1e30f;
+        inv[j] = df_rsqrt(pv);
+        a[j] = df_mul(a[j], inv[j]);
+#pragma unroll
+        for (int q = j + 1; q < R; ++q) a[q] = df_sub(a[q], df_mul(a[j], df_shfl(a[j], q)));
       }
       if (ok) {
-        for (int i = 0; i < r; ++i) {  // L^{-1}, a column per lane
-          const float ii = __shfl_sync(0xffffffffu, ij_own, i);
-          if (lane < r) {
-            float t = i == lane ? 1.f : 0.f;
-            for (int p = lane; p < i; ++p) t = fmaf(-Lf[i * 16 + p], Lif[p * 16 + lane], t);
-            Lif[i * 16 + lane] = i < lane ? 0.f : t * ii;
+        df x[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {  // column `lane` of L^{-1}
+          df t = df{0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < i; ++q) t = df_sub(t, df_mul(df_shfl(a[q], i), x[q]));
+          t = df_mul(t, inv[i]);
+          x[i] = i < lane ? df{0.f, 0.f} : i == lane ? inv[i] : t;
+          if (lane < 16) {
+            const bool in = i < r && lane < r;
+            Li[i * 16 + lane] = in ? static_cast<double>(x[i].h) + static_cast<double>(x[i].l) : 0.0;
+            Lf[i * 16 + lane] = in ? x[i].h : 0.f;
           }
-          __syncwarp();
         }
-      }
-    }
-    ok = __syncthreads_and(ok);
-    if (!ok) {
-      if (threadIdx.x < 32) {
+      } else {
         double* L = G + 256;
         __shared__ double iL[16];
-        if (!chol_inverse_warp(G, L, X, iL, r, 16) && lane == 0) report_error(pr.err, kErrNotSPD, k);
+        if (!chol_inverse_warp(G, L, Li, iL, r, 16) && lane == 0) report_error(pr.err, kErrNotSPD, k);
         __syncwarp();
-        for (int t = lane; t < r * r; t += 32) {  // G^{-1} = L^{-T} L^{-1} into G
-          const int a = t / r, b = t - a * r;
-          double s = 0.0;
-          for (int p = max(a, b); p < r; ++p) s = __fma_rn(X[p * 16 + a], X[p * 16 + b], s);
-          G[a * 16 + b] = s;
+        for (int t = lane; t < 256; t += 32) {
+          const int i = t >> 4, q = t & 15;
+          if (q > i || i >= r) Li[t] = 0.0;
+          Lf[t] = static_cast<float>(Li[t]);
         }
-        __syncwarp();
-        for (int t = lane; t < r * r; t += 32) X[(t / r) * 16 + t % r] = G[(t / r) * 16 + t % r];
       }
-      __syncthreads();
-      return;
-    }
-    for (int t = threadIdx.x; t < r * r; t += kStepNT) {
-      const int a = t / r, b = t - a * r;
-      float x = 0.f;
-      for (int p = max(a, b); p < r; ++p) x = fmaf(Lif[p * 16 + a], Lif[p * 16 + b], x);
-      X[a * 16 + b] = x;
     }
     __syncthreads();
-    double* Tm = G + 256;
-    double t1[2];
-    for (int t = threadIdx.x, z = 0; t < r * r; t += kStepNT, ++z) {  // T = G X0
-      const int a = t / r, b = t - a * r;
-      double x = 0.0;
-      for (int p = 0; p < r; ++p) x = __fma_rn(G[a * 16 + p], X[p * 16 + b], x);
-      t1[z & 1] = x;
+    for (int i = threadIdx.x; i < m; i += NT) {
+      float x[R];
+#pragma unroll
+      for (int l = 0; l < R; ++l) x[l] = Q[l * ms + i];
+#pragma unroll
+      for (int l = 0; l < R; ++l) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q <= l; ++q) s = fmaf(x[q], Lf[l * 16 + q], s);
+        Q[l * ms + i] = s;
+      }
     }
-    for (int t = threadIdx.x, z = 0; t < r * r; t += kStepNT, ++z) Tm[(t / r) * 16 + t % r] = t1[z & 1];
-    __syncthreads();
-    for (int t = threadIdx.x, z = 0; t < r * r; t += kStepNT, ++z) {  // X1 = 2 X0 - X0 T
-      const int a = t / r, b = t - a * r;
-      double x = 2.0 * X[a * 16 + b];
-      for (int p = 0; p < r; ++p) x = __fma_rn(-X[a * 16 + p], Tm[p * 16 + b], x);
-      t1[z & 1] = x;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x, z = 0; t < r * r; t += kStepNT, ++z) X[(t / r) * 16 + t % r] = t1[z & 1];
-    __syncthreads();
+    // (every thread goes on with its own rows; other rows after the next barrier)
   }
 
-  // u = P_perp d (or d); ||u||^2 partial sums into scalar slot `slot`.
-  // Barriers inside; callers read the slot after their next barrier.
+  // u = P_perp (A_G s - y) for the values sv(par); ||u||^2 into slot `slot`
+  // (ready after the caller's next barrier).
   __device__ void residual(int slot) const {
-    float x[R];
-    if (project) {
-      float acc[R];
+    const float* y = pr.y + static_cast<size_t>(k) * m;
+    const float* s = sv(par);
+    float acc[R], nn = 0.f;
 #pragma unroll
-      for (int l = 0; l < R; ++l) acc[l] = 0.f;
-      for (int i = threadIdx.x; i < m; i += kStepNT) {
-        const float di = d[i];
+    for (int l = 0; l < R; ++l) acc[l] = 0.f;
+    for (int i = threadIdx.x; i < m; i += NT) {
+      const float t = support_row(i, s) - y[i];
+      u[i] = t;
+      if (project) {
 #pragma unroll
-        for (int l = 0; l < R; ++l) acc[l] = fmaf(Wt[l * ms + i], di, acc[l]);
+        for (int l = 0; l < R; ++l) acc[l] = fmaf(Q[l * ms + i], t, acc[l]);
+      } else {
+        nn = fmaf(t, t, nn);
       }
+    }
+    if (project) {
+      float cf[R];
       put_coefs(acc);
       __syncthreads();
-      solve(x);
-    }
-    float nn = 0.f;
-    for (int i = threadIdx.x; i < m; i += kStepNT) {
-      float s = d[i];
-      if (project)
+      get_coefs(cf);
+      for (int i = threadIdx.x; i < m; i += NT) {
+        float t = u[i];
 #pragma unroll
-        for (int l = 0; l < R; ++l) s = fmaf(-Wt[l * ms + i], x[l], s);
-      u[i] = s;
-      nn = fmaf(s, s, nn);
+        for (int l = 0; l < R; ++l) t = fmaf(-Q[l * ms + i], cf[l], t);
+        u[i] = t;
+        nn = fmaf(t, t, nn);
+      }
     }
     put_scal(slot, nn);
   }
 
-  // d = A_G s - y from the support's columns (own rows; no barrier inside)
-  __device__ void fresh_d() const {
-    const float* y = pr.y + static_cast<size_t>(k) * m;
-    const float* s = sv(par);
-    for (int i = threadIdx.x; i < m; i += kStepNT) {
-      float t = 0.f;
-      for (int e = 0; e < nl; ++e) t = fmaf(ag(e)[i], s[e], t);
-      d[i] = t - y[i];
-    }
-  }
-
-  // gG_e = (column e)^T u, a warp per entry, four entries at a time
+  // gG_e = (column e)^T u, a warp per four entries; ||g_G||^2 into slot 0
   __device__ void support_gradient() const {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int e0 = 4 * w; e0 < nl; e0 += 4 * kStepNW) {
-      const float* c0 = ag(e0);
-      const float* c1 = ag(min(e0 + 1, nl - 1));
-      const float* c2 = ag(min(e0 + 2, nl - 1));
-      const float* c3 = ag(min(e0 + 3, nl - 1));
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    float sq = 0.f;
+    for (int e0 = 4 * w; e0 < nl; e0 += 4 * NW) {
+      const float* a0 = ag + e0 * as;
+      const float* a1 = ag + min(e0 + 1, nl - 1) * as;
+      const float* a2 = ag + min(e0 + 2, nl - 1) * as;
+      const float* a3 = ag + min(e0 + 3, nl - 1) * as;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
       for (int i = lane; i < m; i += 32) {
         const float ui = u[i];
-        a0 = fmaf(c0[i], ui, a0);
-        a1 = fmaf(c1[i], ui, a1);
-        a2 = fmaf(c2[i], ui, a2);
-        a3 = fmaf(c3[i], ui, a3);
+        v[0] = fmaf(a0[i], ui, v[0]);
+        v[1] = fmaf(a1[i], ui, v[1]);
+        v[2] = fmaf(a2[i], ui, v[2]);
+        v[3] = fmaf(a3[i], ui, v[3]);
       }
-      a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3);
-      if (lane < 4 && e0 + lane < nl) gG[e0 + lane] = lane == 0 ? a0 : lane == 1 ? a1 : lane == 2 ? a2 : a3;
+      const float t = reduce_multi<4>(v);
+      const int e = e0 + (lane >> 3);
+      if ((lane & 7) == 0 && e < nl) {
+        gG[e] = t;
+        sq = fmaf(t, t, sq);
+      }
     }
+    put_scal(0, sq);
   }
 
-  // With gG ready (after a barrier): v = A_G g_G, p = P_perp v (own
-  // rows), num = ||g_G||^2, den = ||p||^2.  Two barriers.
-  __device__ void curvature(float& num, float& den) const {
-    const int lane = threadIdx.x & 31;
-    float acc[R], x[R];
+  // With gG and slot 0 ready (after a barrier): p = P_perp A_G g_G, num =
+  // ||g_G||^2, den = ||p||^2.  Two barriers.
+  __device__ void curvature(float& num, float& den, bool have_ref) const {
+    num = get_scal(0);
+    float acc[R], nd = 0.f;
 #pragma unroll
     for (int l = 0; l < R; ++l) acc[l] = 0.f;
-    for (int i = threadIdx.x; i < m; i += kStepNT) {
-      float t = 0.f;
-      for (int e = 0; e < nl; ++e) t = fmaf(ag(e)[i], gG[e], t);
-      v[i] = t;
-      if (project)
+    for (int i = threadIdx.x; i < m; i += NT) {
+      const float t = support_row(i, gG);
+      p[i] = t;
+      if (project) {
 #pragma unroll
-        for (int l = 0; l < R; ++l) acc[l] = fmaf(Wt[l * ms + i], t, acc[l]);
+        for (int l = 0; l < R; ++l) acc[l] = fmaf(Q[l * ms + i], t, acc[l]);
+      }
+      if (have_ref) {
+        const float x = u[i] - uref[i];
+        nd = fmaf(x, x, nd);
+      }
     }
     if (project) put_coefs(acc);
-    float t = 0.f;
-    for (int e = lane; e < nl; e += 32) t = fmaf(gG[e], gG[e], t);
-    num = warp_sum(t);
+    if (have_ref) put_scal(3, nd);
     __syncthreads();
-    if (project) solve(x);
+    float cf[R];
+    if (project) get_coefs(cf);
     float nn = 0.f;
-    for (int i = threadIdx.x; i < m; i += kStepNT) {
-      float s = v[i];
-      if (project)
+    for (int i = threadIdx.x; i < m; i += NT) {
+      float t = p[i];
+      if (project) {
 #pragma unroll
-        for (int l = 0; l < R; ++l) s = fmaf(-Wt[l * ms + i], x[l], s);
-      p[i] = s;
-      nn = fmaf(s, s, nn);
+        for (int l = 0; l < R; ++l) t = fmaf(-Q[l * ms + i], cf[l], t);
+        p[i] = t;
+      }
+      nn = fmaf(t, t, nn);
     }
-    put_scal(0, nn);
+    put_scal(4, nn);
     __syncthreads();
-    den = get_scal(0);
+    den = get_scal(4);
   }
 
   // The IHT sweeps sw .. te-1 that need no pass over A_k (see the head of
-  // the file); ||u||^2 lies in scalar slot 1 + (sw & 1).  have_ref: gmax and
-  // uref of an earlier pass.  Returns the first sweep that needs a pass, or te.
+  // the file), from u and ||u||^2 in slot 1 + (sw & 1).  have_ref: gmax and
+  // uref of an earlier pass.  Returns the first sweep that needs a pass (u is
+  // then that of sv(par)), or te.  The last barrier of a sweep is the first
+  // of the next one.
   __device__ int sweeps(int sw, bool have_ref, float gmax) {
-    const int lane = threadIdx.x & 31;
     const float N = pr.nmax[k];
+    __syncthreads();
     for (; sw < te; ++sw) {
-      __syncthreads();
       const float nu = sqrtf(get_scal(1 + (sw & 1)));
       support_gradient();
       __syncthreads();
       float num, den;
-      float nd = 0.f;
-      if (have_ref) {
-        for (int i = threadIdx.x; i < m; i += kStepNT) nd = fmaf(u[i] - uref[i], u[i] - uref[i], nd);
-        put_scal(3, nd);
-      }
-      curvature(num, den);
+      curvature(num, den, have_ref);
       if (!(den > 0.f)) return te;  // s is stationary: the remaining sweeps keep it
       const float mu = num / den;
-      const float* s = sv(par);
-      float vmin = INFINITY;
-      for (int e = lane; e < nl; e += 32) vmin = fminf(vmin, fabsf(fmaf(-mu, gG[e], s[e])));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
       float bound = N * nu;
       if (have_ref) bound = fminf(bound, fmaf(N, sqrtf(get_scal(3)), gmax));
       bound = bound * mu * 1.001f;
       // all comparisons are false for NaN: such a column takes the full path
-      if (!(nl == rho && isfinite(mu) && (bound < vmin || rho >= n))) return sw;
+      bool ok = nl == rho && isfinite(mu) && (bound >= 0.f || rho >= n);
+      const float* s = sv(par);
       float* s2 = sv(par ^ 1);
-      for (int e = threadIdx.x; e < nl; e += kStepNT) s2[e] = fmaf(-mu, gG[e], s[e]);
-      par ^= 1;
+      for (int e = threadIdx.x; e < nl; e += NT) {
+        const float v = fmaf(-mu, gG[e], s[e]);
+        s2[e] = v;
+        ok = ok && (bound < fabsf(v) || rho >= n);
+      }
       float nn = 0.f;
-      for (int i = threadIdx.x; i < m; i += kStepNT) {
-        d[i] = fmaf(-mu, v[i], d[i]);
+      for (int i = threadIdx.x; i < m; i += NT) {
         const float t = fmaf(-mu, p[i], u[i]);
         u[i] = t;
         nn = fmaf(t, t, nn);
       }
       put_scal(1 + ((sw + 1) & 1), nn);
+      if (!__syncthreads_and(ok)) {
+        residual(1 + (sw & 1));  // back to the u of sv(par), as the next step forms it
+        return sw;
+      }
+      par ^= 1;
     }
     return te;
   }
@@ -728,44 +814,30 @@ struct Step {
   // vector of the column's next pass: x_i, times the row scales of the FP8 forms
   __device__ void store_vec(int i, float x) const {
     const int planes = pr.L.et == 3 ? 2 : 1;
-    float* out = pr.uvec + static_cast<size_t>(k) * planes * pr.astride;
+    float* out = pr.uvec + static_cast<size_t>(k) * planes * as;
     if (pr.L.et < 2) {
       out[i] = x;
     } else {
       const size_t o = (static_cast<size_t>(k) * m + i) * planes;
       out[i] = x * pr.rscale[o];
-      if (planes == 2) out[pr.astride + i] = x * pr.rscale[o + 1];
+      if (planes == 2) out[as + i] = x * pr.rscale[o + 1];
     }
   }
 
   // the column waits for g: its state, and its entry in the next list
   __device__ void need_pass(int sw, int list, bool first) const {
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += kStepNT) {
-      store_vec(i, u[i]);
-      pr.dvec[static_cast<size_t>(k) * pr.astride + i] = d[i];
-    }
+    for (int i = threadIdx.x; i < m; i += NT) store_vec(i, u[i]);
     const float* s = sv(par);
-    for (int e = threadIdx.x; e < nl; e += kStepNT) {
+    for (int e = threadIdx.x; e < nl; e += NT) {
       pr.supj[static_cast<size_t>(k) * rho + e] = sj[e];
       pr.supv[static_cast<size_t>(k) * rho + e] = s[e];
     }
     if (first) {
-      for (int t = threadIdx.x; t < m * R; t += kStepNT) {
-        const int i = t / R, l = t - i * R;
-        pr.Wk[static_cast<size_t>(k) * pr.wstride + t] = Wt[l * ms + i];
-      }
-      for (int t = threadIdx.x; t < 256; t += kStepNT)
-        pr.Gi[static_cast<size_t>(k) * 256 + t] =
-            (t >> 4) < r && (t & 15) < r ? G[512 + t] : 0.0;
-      // AG_k keyed by support slot from here on (slots move only when entries
-      // of the given support were dropped)
-      for (int e = 0; e < nl; ++e) {
-        if (src[e] == e) continue;
-        const float* from = pr.AG + (static_cast<size_t>(k) * rho + src[e]) * pr.astride;
-        float* to = pr.AG + (static_cast<size_t>(k) * rho + e) * pr.astride;
-        for (int i = threadIdx.x; i < m; i += kStepNT) to[i] = from[i];
-      }
+      float* out = pr.Wk + static_cast<size_t>(k) * pr.wstride;
+      for (int i = threadIdx.x; i < m; i += NT)
+#pragma unroll
+        for (int l = 0; l < R; ++l) out[static_cast<size_t>(l) * m + i] = Q[l * ms + i];
+      for (int t = threadIdx.x; t < 256; t += NT) pr.Li[static_cast<size_t>(k) * 256 + t] = G[512 + t];
     }
     if (threadIdx.x == 0) {
       pr.nsup[k] = nl;
@@ -776,33 +848,42 @@ struct Step {
 
   // b_k, the vector of the final pass and S_k (ascending by index)
   __device__ void finish(bool store_s) const {
-    __syncthreads();
-    if (pr.mode == kModeInit) {
-      for (int i = threadIdx.x; i < m; i += kStepNT) store_vec(i, -d[i]);
-    } else {
-      float acc[R], x[R];
+    const float* y = pr.y + static_cast<size_t>(k) * m;
+    const float* s = sv(par);
+    float acc[R];
 #pragma unroll
-      for (int l = 0; l < R; ++l) acc[l] = 0.f;
-      for (int i = threadIdx.x; i < m; i += kStepNT) {
-        const float di = -d[i];
+    for (int l = 0; l < R; ++l) acc[l] = 0.f;
+    for (int i = threadIdx.x; i < m; i += NT) {
+      const float t = y[i] - support_row(i, s);
+      if (project) {
+        p[i] = t;
 #pragma unroll
-        for (int l = 0; l < R; ++l) acc[l] = fmaf(Wt[l * ms + i], di, acc[l]);
+        for (int l = 0; l < R; ++l) acc[l] = fmaf(Q[l * ms + i], t, acc[l]);
+      } else {
+        store_vec(i, t);
       }
+    }
+    if (project) {
+      float cf[R];
       put_coefs(acc);
       __syncthreads();
-      const float own = solve(x);
-      if (threadIdx.x < r) pr.B[static_cast<size_t>(k) * r + threadIdx.x] = own;
-      if (pr.mode == kModeIter)
-        for (int i = threadIdx.x; i < m; i += kStepNT) {
-          float s = d[i];
+      get_coefs(cf);
+      if (threadIdx.x < 32 && threadIdx.x < r) {  // b = L^{-T} (Q^T (y - A s))
+        double b = 0.0;
 #pragma unroll
-          for (int l = 0; l < R; ++l) s = fmaf(Wt[l * ms + i], x[l], s);
-          store_vec(i, s);
+        for (int l = 0; l < R; ++l) b = __fma_rn(G[512 + l * 16 + threadIdx.x], static_cast<double>(cf[l]), b);
+        pr.B[static_cast<size_t>(k) * r + threadIdx.x] = static_cast<float>(b);
+      }
+      if (pr.mode == kModeIter)
+        for (int i = threadIdx.x; i < m; i += NT) {  // e = W b + A s - y
+          float t = -p[i];
+#pragma unroll
+          for (int l = 0; l < R; ++l) t = fmaf(Q[l * ms + i], cf[l], t);
+          store_vec(i, t);
         }
     }
     if (store_s) {
-      const float* s = sv(par);
-      for (int e = threadIdx.x; e < nl; e += kStepNT) {
+      for (int e = threadIdx.x; e < nl; e += NT) {
         const int je = sj[e];
         int pos = 0;
         for (int f = 0; f < nl; ++f) pos += sj[f] < je;
@@ -813,68 +894,101 @@ struct Step {
   }
 };
 
+// The problem of column c into shared memory (every thread; ends with a
+// barrier, which also separates the previous column's use of the buffers).
+__device__ __forceinline__ void load_problem(const StreamTable& T, int c, StreamProblem* spr, int& cur) {
+  const int p = T.nprob == 1 ? 0 : prob_of(T, c);
+  __syncthreads();
+  if (p != cur) {
+    const int* from = reinterpret_cast<const int*>(T.probs + p);
+    int* to = reinterpret_cast<int*>(spr);
+    for (int t = threadIdx.x; t < static_cast<int>(sizeof(StreamProblem) / 4); t += blockDim.x) to[t] = from[t];
+    cur = p;
+    __syncthreads();
+  }
+}
+
 // The first step of a column (modes ITER and LS): W_k from the column chunks'
-// partial sums, Gram and inverse, u, and the sweeps.  Latency-bound (about a
-// dozen barriers and r x r chains per column), so the column gets 128 threads
-// and as many columns as fit run at once.
-template <int R>
-__global__ void __launch_bounds__(kStepNT, 8)
-    step_first_kernel(const StreamTable T, int use_ag) {
+// partial sums, its Gram, Q, u, and the sweeps.  Instruction- and barrier-
+// bound (four barriers a sweep), so as many columns as fit run at once: at
+// n = q = 1000, r = 5, m = 150, rho = 10 all of them.
+template <int R, int V>
+__global__ void __launch_bounds__(step_threads(V), V == 0 ? 8 : 3)
+    step_first_kernel(const StreamTable T) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ StreamProblem spr;
+  __shared__ int snl;
+  __shared__ uint64_t abar;
+  constexpr int NT = step_threads(V);
   const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) mbar_init(&abar, 1);
+  unsigned phase = 0;
+  int cur = -1;
   for (int c = blockIdx.x; c < T.ncols; c += gridDim.x) {
-    const StreamProblem& pr = T.probs[prob_of(T, c)];
-    const StepCarve cv = step_carve(R, pr.L.m, pr.L.n, pr.L.rho, pr.astride, use_ag, false);
-    Step<R> s(T, pr, smem, cv, use_ag);
-    s.c = c;
-    s.k = c - pr.col0;
+    load_problem(T, c, &spr, cur);
+    if (spr.variant != V) continue;
+    const StepCarve cv = step_carve(R, spr.L.m, spr.L.n, spr.L.rho, spr.astride, V, false);
+    Step<R, V> s(T, spr, smem, cv);
+    s.at_column(c, smem, cv);
+    s.stage_begin(&abar);
     const int m = s.m, rho = s.rho, k = s.k;
-    __syncthreads();  // the previous column is done with the buffers
     // the given support, entries outside the column dropped
-    __shared__ int snl;
     if (threadIdx.x < 32) {
       int cnt = 0;
       for (int e0 = 0; e0 < rho; e0 += 32) {
         const int e = e0 + lane;
-        const int j = e < rho ? pr.S_idx[static_cast<size_t>(k) * rho + e] : -1;
-        const float x = e < rho ? pr.S_val[static_cast<size_t>(k) * rho + e] : 0.f;
+        const int j = e < rho ? spr.S_idx[static_cast<size_t>(k) * rho + e] : -1;
+        const float x = e < rho ? spr.S_val[static_cast<size_t>(k) * rho + e] : 0.f;
         const bool in = j >= 0 && j < s.n;
         const unsigned b = __ballot_sync(0xffffffffu, in);
         if (in) {
           const int at = cnt + __popc(b & ((1u << lane) - 1));
           s.sj[at] = j;
           s.svb[at] = x;
-          s.src[at] = e;
         }
         cnt += __popc(b);
       }
       if (lane == 0) snl = cnt;
     }
-    const float* wp = pr.Wp + static_cast<size_t>(k) * pr.ncw * pr.wstride;
-    for (int t4 = threadIdx.x; t4 < pr.wstride / 4; t4 += kStepNT) {
+    const float* wp = spr.Wp + static_cast<size_t>(k) * spr.ncw * spr.wstride;
+    for (int t4 = threadIdx.x; t4 < spr.wstride / 4; t4 += NT) {
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int cc = 0; cc < pr.ncw; ++cc) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(wp + static_cast<size_t>(cc) * pr.wstride) + t4);
+#pragma unroll 8
+      for (int cc = 0; cc < spr.ncw; ++cc) {
+        const float4 a = __ldcg(reinterpret_cast<const float4*>(wp + static_cast<size_t>(cc) * spr.wstride) + t4);
         x.x += a.x; x.y += a.y; x.z += a.z; x.w += a.w;
       }
 #pragma unroll
       for (int z = 0; z < 4; ++z) {
         const int t = 4 * t4 + z, i = t / R, l = t - i * R;
-        if (i < m) s.Wt[l * s.ms + i] = z == 0 ? x.x : z == 1 ? x.y : z == 2 ? x.z : x.w;
+        if (i < m) s.Q[l * s.ms + i] = z == 0 ? x.x : z == 1 ? x.y : z == 2 ? x.z : x.w;
       }
     }
     __syncthreads();
     s.nl = snl;
-    s.stage_support();
-    s.gram_inverse();
-    s.load_inverse(s.G + 512);
-    s.fresh_d();
-    if (pr.mode == kModeLS || s.te == 0) {
-      s.finish(pr.mode == kModeIter);
-      continue;
+    s.factor();
+    s.stage_end(&abar, phase);
+    if (s.nl != rho) {
+      // entries of the given support were dropped: the columns of the others
+      // move down to their slots (in AG_k too, where the next step finds them)
+      __syncthreads();
+      for (int i = threadIdx.x; i < m; i += NT) {
+        int at = 0;
+        for (int e = 0; e < rho; ++e) {
+          const int j = spr.S_idx[static_cast<size_t>(k) * rho + e];
+          if (j < 0 || j >= s.n) continue;
+          const float a = s.ag_global()[static_cast<size_t>(e) * s.as + i];
+          s.ag_global()[static_cast<size_t>(at) * s.as + i] = a;
+          s.ag[static_cast<size_t>(at) * s.as + i] = a;
+          ++at;
+        }
+      }
     }
     __syncthreads();
+    if (spr.mode == kModeLS || s.te == 0) {
+      s.finish(spr.mode == kModeIter);
+      continue;
+    }
     s.residual(1);
     const int sw = s.sweeps(0, false, 0.f);
     if (sw < s.te) s.need_pass(sw, 0, true);
@@ -885,6 +999,7 @@ __global__ void __launch_bounds__(kStepNT, 8)
 // ---- HardThreshold of v (n entries) on one CTA --------------------------------
 // The rho largest keys (|v|, then the lower index) of vv into sel[0..K),
 // K = min(rho, n): 8-bit radix select on the float bits, ties by index.
+template <int NT>
 __device__ __forceinline__ int topk_radix(const float* vv, int n, int rho, int* hist, int* ties,
                                           int* sel) {
   const int K = min(rho, n), lane = threadIdx.x & 31;
@@ -892,9 +1007,9 @@ __device__ __forceinline__ int topk_radix(const float* vv, int n, int rho, int* 
   unsigned prefix = 0, mask = 0;
   if (threadIdx.x == 0) info[1] = K;
   for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int t = threadIdx.x; t < 256; t += kStepNT) hist[t] = 0;
+    for (int t = threadIdx.x; t < 256; t += NT) hist[t] = 0;
     __syncthreads();
-    for (int j0 = threadIdx.x - lane; j0 < n; j0 += kStepNT) {
+    for (int j0 = threadIdx.x - lane; j0 < n; j0 += NT) {
       const int j = j0 + lane;
       const unsigned key = j < n ? __float_as_uint(fabsf(vv[j])) : 0u;
       const bool in = j < n && (key & mask) == prefix;
@@ -936,28 +1051,28 @@ __device__ __forceinline__ int topk_radix(const float* vv, int n, int rho, int* 
   __syncthreads();
   if (threadIdx.x == 0) { info[2] = 0; info[3] = 0; }
   __syncthreads();
-  for (int j = threadIdx.x; j < n; j += kStepNT) {
+  for (int j = threadIdx.x; j < n; j += NT) {
     const unsigned key = __float_as_uint(fabsf(vv[j]));
     if (key > prefix) sel[atomicAdd(&info[3], 1)] = j;
     else if (key == prefix) ties[atomicAdd(&info[2], 1)] = j;
   }
   __syncthreads();
   const int nt = info[2];
-  for (int t = threadIdx.x; t < nt; t += kStepNT) {
+  for (int t = threadIdx.x; t < nt; t += NT) {
     int rank = 0;
     for (int z = 0; z < nt; ++z) rank += ties[z] < ties[t];
     if (rank < need) sel[info[3] + rank] = ties[t];
   }
   __syncthreads();
   // in key order: the order in which the threads found them is arbitrary
-  for (int t = threadIdx.x; t < K; t += kStepNT) {
+  for (int t = threadIdx.x; t < K; t += NT) {
     const uint64_t kj = ht_key(vv[sel[t]], sel[t]);
     int rank = 0;
     for (int z = 0; z < K; ++z) rank += ht_key(vv[sel[z]], sel[z]) > kj;
     ties[rank] = sel[t];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < K; t += kStepNT) sel[t] = ties[t];
+  for (int t = threadIdx.x; t < K; t += NT) sel[t] = ties[t];
   __syncthreads();
   return K;
 }
@@ -965,19 +1080,27 @@ __device__ __forceinline__ int topk_radix(const float* vv, int n, int rho, int* 
 // One listed column after its pass: HardThreshold with g, then the sweeps
 // that need no further pass.  zero: the first sweep of the initialisation
 // (s = 0: the support is the rho largest |g_j|, its values still 0).
-template <int R>
-__global__ void __launch_bounds__(kStepNT, 6)
-    step_next_kernel(const StreamTable T, int round, int zero, int use_ag) {
+template <int R, int V>
+__global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
+    step_next_kernel(const StreamTable T, int round, int zero) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ StreamProblem spr;
+  __shared__ uint64_t abar;
+  constexpr int NT = step_threads(V);
   const int lane = threadIdx.x & 31;
   const int count = zero ? T.ncols : T.cnt[round];
+  if (count == 0) return;
+  if (threadIdx.x == 0) mbar_init(&abar, 1);
+  unsigned phase = 0;
+  int cur = -1;
   for (int at = blockIdx.x; at < count; at += gridDim.x) {
     const int c = zero ? at : T.list[static_cast<size_t>(round & 1) * T.ncols + at];
-    const StreamProblem& pr = T.probs[prob_of(T, c)];
-    const StepCarve cv = step_carve(R, pr.L.m, pr.L.n, pr.L.rho, pr.astride, use_ag, true);
-    Step<R> s(T, pr, smem, cv, use_ag);
-    s.c = c;
-    s.k = c - pr.col0;
+    load_problem(T, c, &spr, cur);
+    if (spr.variant != V || spr.te == 0) continue;
+    const StepCarve cv = step_carve(R, spr.L.m, spr.L.n, spr.L.rho, spr.astride, V, true);
+    Step<R, V> s(T, spr, smem, cv);
+    s.at_column(c, smem, cv);
+    if (!zero) s.stage_begin(&abar);
     const int m = s.m, n = s.n, rho = s.rho, k = s.k;
     float* vv = reinterpret_cast<float*>(smem + cv.vv);
     int* ties = reinterpret_cast<int*>(smem + cv.tie);
@@ -985,179 +1108,178 @@ __global__ void __launch_bounds__(kStepNT, 6)
     int* hist = reinterpret_cast<int*>(smem + cv.hist);
     int* info = hist + 256;
     int* removed = reinterpret_cast<int*>(smem + cv.lists);
-    int* added = removed + max(rho, 1);
-    const float* g = pr.g + static_cast<size_t>(k) * pr.L.ns;
-    if (s.te == 0) continue;  // (a problem of the batch without IHT)
-    __syncthreads();
-    const int sw = zero ? 0 : pr.sweep[k];
-    s.nl = zero ? 0 : pr.nsup[k];
-    for (int e = threadIdx.x; e < rho; e += kStepNT) {
-      s.src[e] = e;
-      if (e < s.nl) {
-        s.sj[e] = pr.supj[static_cast<size_t>(k) * rho + e];
-        s.svb[e] = pr.supv[static_cast<size_t>(k) * rho + e];
-      }
+    int* added = removed + cv.rp;
+    const float* g = spr.g + static_cast<size_t>(k) * spr.L.ns;
+    const int sw = zero ? 0 : spr.sweep[k];
+    s.nl = zero ? 0 : spr.nsup[k];
+    for (int e = threadIdx.x; e < s.nl; e += NT) {
+      s.sj[e] = spr.supj[static_cast<size_t>(k) * rho + e];
+      s.svb[e] = spr.supv[static_cast<size_t>(k) * rho + e];
     }
-    for (int i = threadIdx.x; i < m; i += kStepNT)
-      s.d[i] = zero ? -pr.y[static_cast<size_t>(k) * m + i]
-                    : pr.dvec[static_cast<size_t>(k) * pr.astride + i];
     if (s.project) {
-      for (int t = threadIdx.x; t < m * R; t += kStepNT) {
-        const int i = t / R, l = t - i * R;
-        s.Wt[l * s.ms + i] = pr.Wk[static_cast<size_t>(k) * pr.wstride + t];
-      }
-      s.load_inverse(pr.Gi + static_cast<size_t>(k) * 256);
+      const float* w = spr.Wk + static_cast<size_t>(k) * spr.wstride;
+      for (int i = threadIdx.x; i < m; i += NT)
+#pragma unroll
+        for (int l = 0; l < R; ++l) s.Q[l * s.ms + i] = __ldcg(w + static_cast<size_t>(l) * m + i);
+      for (int t = threadIdx.x; t < 256; t += NT) s.G[512 + t] = spr.Li[static_cast<size_t>(k) * 256 + t];
     }
-    for (int j = threadIdx.x; j < n; j += kStepNT) vv[j] = __ldcg(g + j);
+    for (int j = threadIdx.x; j < n; j += NT) vv[j] = __ldcg(g + j);
+    if (!zero) s.stage_end(&abar, phase);
     __syncthreads();
-    s.stage_support();
-    bool stopped = false;
-    float mu = 0.f;
     if (zero) {
       // support of the zero start
-      const int K = topk_radix(vv, n, rho, hist, ties, sel);
-      for (int e = threadIdx.x; e < K; e += kStepNT) {
+      const int K = topk_radix<NT>(vv, n, rho, hist, ties, sel);
+      for (int e = threadIdx.x; e < K; e += NT) {
         s.sj[e] = sel[e];
         s.svb[e] = 0.f;
       }
       s.nl = K;
       __syncthreads();
-      for (int t = threadIdx.x; t < K * m; t += kStepNT) {
+      for (int t = threadIdx.x; t < K * m; t += NT) {
         const int e = t / m, i = t - e * m;
-        const float a = stream_elem(pr, k, i, s.sj[e]);
-        if (s.agsm) s.agsm[static_cast<size_t>(e) * pr.astride + i] = a;
-        pr.AG[(static_cast<size_t>(k) * rho + e) * pr.astride + i] = a;
+        const float a = stream_elem(spr, k, i, s.sj[e]);
+        s.ag[static_cast<size_t>(e) * s.as + i] = a;
+        if (step_staged(V)) s.ag_global()[static_cast<size_t>(e) * s.as + i] = a;
       }
+      __syncthreads();
     }
-    s.residual(1);  // u (the vector of the pass), ||u||^2 not needed here
-    for (int e = threadIdx.x; e < s.nl; e += kStepNT) s.gG[e] = vv[s.sj[e]];
+    s.residual(1);  // u, the vector of the pass
+    float sq = 0.f;
+    for (int e = threadIdx.x; e < s.nl; e += NT) {
+      const float x = vv[s.sj[e]];
+      s.gG[e] = x;
+      sq = fmaf(x, x, sq);
+    }
+    s.put_scal(0, sq);
     __syncthreads();
-    for (int i = threadIdx.x; i < m; i += kStepNT) s.uref[i] = s.u[i];
+    for (int i = threadIdx.x; i < m; i += NT) s.uref[i] = s.u[i];
     float num, den, gmax = 0.f;
-    s.curvature(num, den);
+    s.curvature(num, den, false);
+    if (!(den > 0.f)) {  // stationary: the remaining sweeps keep s
+      s.finish(true);
+      continue;
+    }
+    float mu = num / den;
+    if (!isfinite(mu)) {
+      if (threadIdx.x == 0) report_error(spr.err, kErrNaN, k);
+      mu = 0.f;
+    }
+    for (int j = threadIdx.x; j < n; j += NT) vv[j] = -mu * vv[j];
+    if (threadIdx.x == 0) info[3] = 0;
+    __syncthreads();
+    float* snew = s.sv(1);
+    const int nl = s.nl;
+    for (int e = threadIdx.x; e < nl; e += NT) {
+      const float x = fmaf(-mu, s.gG[e], s.svb[e]);
+      snew[e] = x;
+      vv[s.sj[e]] = x;
+    }
+    __syncthreads();
+    s.par = 1;
     bool kept = true;
-    if (!(den > 0.f)) {
-      stopped = true;
-    } else {
-      mu = num / den;
-      if (!isfinite(mu)) {
-        if (threadIdx.x == 0) report_error(pr.err, kErrNaN, k);
-        mu = 0.f;
-      }
-      for (int j = threadIdx.x; j < n; j += kStepNT) vv[j] = -mu * vv[j];
-      if (threadIdx.x == 0) info[3] = 0;
-      __syncthreads();
-      float* snew = s.sv(1);
-      const int nl = s.nl;
-      for (int e = threadIdx.x; e < nl; e += kStepNT) {
-        const float x = fmaf(-mu, s.gG[e], s.svb[e]);
-        snew[e] = x;
-        vv[s.sj[e]] = x;
-      }
-      __syncthreads();
-      s.par = 1;
-      // candidates: when the support holds rho entries, nothing below the
-      // smallest of them can enter
-      int K = -1;
-      if (nl == rho) {
-        float t0 = INFINITY;
-        for (int e = lane; e < nl; e += 32) t0 = fminf(t0, fabsf(snew[e]));
+    // candidates: when the support holds rho entries, nothing below the
+    // smallest of them can enter
+    int K = -1;
+    if (nl == rho) {
+      float t0 = INFINITY;
+      for (int e = lane; e < nl; e += 32) t0 = fminf(t0, fabsf(snew[e]));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t0 = fminf(t0, __shfl_xor_sync(0xffffffffu, t0, o));
-        const int cap = 2 * rho + 8;
-        for (int j = threadIdx.x; j < n; j += kStepNT)
-          if (fabsf(vv[j]) >= t0) {
-            const int slot = atomicAdd(&info[3], 1);
-            if (slot < cap) sel[slot] = j;
-          }
-        __syncthreads();
-        const int cn = info[3];
-        if (cn == rho) {
-          K = 0;  // the support itself: kept
-        } else if (cn <= cap && cn > rho) {
-          for (int t = threadIdx.x; t < cn; t += kStepNT) {
-            const uint64_t kj = ht_key(vv[sel[t]], sel[t]);
-            int rank = 0;
-            for (int z = 0; z < cn; ++z) rank += ht_key(vv[sel[z]], sel[z]) > kj;
-            if (rank < rho) ties[rank] = sel[t];
-          }
-          __syncthreads();
-          for (int t = threadIdx.x; t < rho; t += kStepNT) sel[t] = ties[t];
-          __syncthreads();
-          K = rho;
+      for (int o = 16; o > 0; o >>= 1) t0 = fminf(t0, __shfl_xor_sync(0xffffffffu, t0, o));
+      const int cap = 2 * rho + 8;
+      for (int j = threadIdx.x; j < n; j += NT)
+        if (fabsf(vv[j]) >= t0) {
+          const int slot = atomicAdd(&info[3], 1);
+          if (slot < cap) sel[slot] = j;
         }
-      }
-      if (K < 0) K = topk_radix(vv, n, rho, hist, ties, sel);
-      if (K > 0) {
-        // slots of the entries that left take the ones that entered (both in
-        // slot / selection order)
-        int nrem = 0, nadd = 0;
-        if (threadIdx.x < 32) {
-          for (int e0 = 0; e0 < rho; e0 += 32) {
-            const int e = e0 + lane;
-            bool gone = e < K && e >= nl;  // an unused slot
-            if (e < nl) {
-              gone = true;
-              for (int f = 0; f < K; ++f) gone = gone && sel[f] != s.sj[e];
-            }
-            const unsigned b = __ballot_sync(0xffffffffu, gone);
-            if (gone) removed[nrem + __popc(b & ((1u << lane) - 1))] = e;
-            nrem += __popc(b);
-          }
-          for (int f0 = 0; f0 < K; f0 += 32) {
-            const int f = f0 + lane;
-            bool in = f < K;
-            if (in)
-              for (int e = 0; e < nl; ++e) in = in && s.sj[e] != sel[f];
-            const unsigned b = __ballot_sync(0xffffffffu, in);
-            if (in) added[nadd + __popc(b & ((1u << lane) - 1))] = sel[f];
-            nadd += __popc(b);
-          }
-          if (lane == 0) { info[4] = nrem; info[5] = nadd; }
+      __syncthreads();
+      const int cn = info[3];
+      if (cn == rho) {
+        K = 0;  // the support itself: kept
+      } else if (cn <= cap && cn > rho) {
+        for (int t = threadIdx.x; t < cn; t += NT) {
+          const uint64_t kj = ht_key(vv[sel[t]], sel[t]);
+          int rank = 0;
+          for (int z = 0; z < cn; ++z) rank += ht_key(vv[sel[z]], sel[z]) > kj;
+          if (rank < rho) ties[rank] = sel[t];
         }
         __syncthreads();
-        nadd = min(info[5], info[4]);
-        s.nl = K;
-        kept = nadd == 0 && K == nl;
-        for (int t = threadIdx.x; t < nadd; t += kStepNT) {
-          s.sj[removed[t]] = added[t];
-          snew[removed[t]] = vv[added[t]];
-        }
-        for (int t = threadIdx.x; t < nadd * m; t += kStepNT) {
-          const int z = t / m, i = t - z * m;
-          const float a = stream_elem(pr, k, i, added[z]);
-          if (s.agsm) s.agsm[static_cast<size_t>(removed[z]) * pr.astride + i] = a;
-          pr.AG[(static_cast<size_t>(k) * rho + removed[z]) * pr.astride + i] = a;
-        }
-      }
-      __syncthreads();
-      // largest |g| outside the new support
-      for (int e = threadIdx.x; e < s.nl; e += kStepNT) vv[s.sj[e]] = INFINITY;
-      __syncthreads();
-      for (int j = threadIdx.x; j < n; j += kStepNT)
-        if (!isinf(vv[j])) gmax = fmaxf(gmax, fabsf(__ldcg(g + j)));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
-      if (lane == 0) s.scal(0)[threadIdx.x >> 5] = gmax;
-      __syncthreads();
-#pragma unroll
-      for (int w = 0; w < kStepNW; ++w) gmax = fmaxf(gmax, s.scal(0)[w]);
-      if (kept) {
-        float nn = 0.f;
-        for (int i = threadIdx.x; i < m; i += kStepNT) {
-          s.d[i] = fmaf(-mu, s.v[i], s.d[i]);
-          const float t = fmaf(-mu, s.p[i], s.u[i]);
-          s.u[i] = t;
-          nn = fmaf(t, t, nn);
-        }
-        s.put_scal(1 + ((sw + 1) & 1), nn);
-      } else {
-        s.fresh_d();
+        for (int t = threadIdx.x; t < rho; t += NT) sel[t] = ties[t];
         __syncthreads();
-        s.residual(1 + ((sw + 1) & 1));
+        K = rho;
       }
     }
-    const int nx = stopped ? s.te : s.sweeps(sw + 1, true, gmax);
+    if (K < 0) K = topk_radix<NT>(vv, n, rho, hist, ties, sel);
+    if (K > 0) {
+      // slots of the entries that left take the ones that entered (both in
+      // slot / key order)
+      if (threadIdx.x < 32) {
+        int nrem = 0, nadd = 0;
+        for (int e0 = 0; e0 < rho; e0 += 32) {
+          const int e = e0 + lane;
+          bool gone = e < K && e >= nl;  // an unused slot
+          if (e < nl) {
+            gone = true;
+            for (int f = 0; f < K; ++f) gone = gone && sel[f] != s.sj[e];
+          }
+          const unsigned b = __ballot_sync(0xffffffffu, gone);
+          if (gone) removed[nrem + __popc(b & ((1u << lane) - 1))] = e;
+          nrem += __popc(b);
+        }
+        for (int f0 = 0; f0 < K; f0 += 32) {
+          const int f = f0 + lane;
+          bool in = f < K;
+          if (in)
+            for (int e = 0; e < nl; ++e) in = in && s.sj[e] != sel[f];
+          const unsigned b = __ballot_sync(0xffffffffu, in);
+          if (in) added[nadd + __popc(b & ((1u << lane) - 1))] = sel[f];
+          nadd += __popc(b);
+        }
+        if (lane == 0) info[4] = min(nrem, nadd);
+      }
+      __syncthreads();
+      const int nadd = info[4];
+      s.nl = K;
+      kept = nadd == 0 && K == nl;
+      for (int t = threadIdx.x; t < nadd; t += NT) {
+        s.sj[removed[t]] = added[t];
+        snew[removed[t]] = vv[added[t]];
+      }
+      for (int t = threadIdx.x; t < nadd * m; t += NT) {
+        const int z = t / m, i = t - z * m;
+        const float a = stream_elem(spr, k, i, added[z]);
+        s.ag[static_cast<size_t>(removed[z]) * s.as + i] = a;
+        if (step_staged(V)) s.ag_global()[static_cast<size_t>(removed[z]) * s.as + i] = a;
+      }
+    }
+    __syncthreads();
+    if (sw + 1 >= s.te) {
+      s.finish(true);
+      continue;
+    }
+    // largest |g| outside the new support
+    for (int e = threadIdx.x; e < s.nl; e += NT) vv[s.sj[e]] = INFINITY;
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += NT)
+      if (!isinf(vv[j])) gmax = fmaxf(gmax, fabsf(__ldcg(g + j)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    if (lane == 0) s.scal(0)[threadIdx.x >> 5] = gmax;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) gmax = fmaxf(gmax, s.scal(0)[w]);
+    const int slot = 1 + ((sw + 1) & 1);
+    if (kept) {
+      float nn = 0.f;
+      for (int i = threadIdx.x; i < m; i += NT) {
+        const float t = fmaf(-mu, s.p[i], s.u[i]);
+        s.u[i] = t;
+        nn = fmaf(t, t, nn);
+      }
+      s.put_scal(slot, nn);
+    } else {
+      s.residual(slot);
+    }
+    const int nx = s.sweeps(sw + 1, true, gmax);
     if (nx < s.te) s.need_pass(nx, round + 1, false);
     else s.finish(true);
   }

@@ -12,9 +12,15 @@ void* stream_w_kernel_r10(int et) {
     default: return reinterpret_cast<void*>(&w_kernel<10, 0>);
   }
 }
-void* stream_step_kernel_r10(int next) {
+void* stream_step_kernel_r10(int next, int variant) {
   using namespace stream;
-  return next ? reinterpret_cast<void*>(&step_next_kernel<10>)
-              : reinterpret_cast<void*>(&step_first_kernel<10>);
+  switch (variant) {
+    case 0: return next ? reinterpret_cast<void*>(&step_next_kernel<10, 0>)
+                        : reinterpret_cast<void*>(&step_first_kernel<10, 0>);
+    case 1: return next ? reinterpret_cast<void*>(&step_next_kernel<10, 1>)
+                        : reinterpret_cast<void*>(&step_first_kernel<10, 1>);
+    default: return next ? reinterpret_cast<void*>(&step_next_kernel<10, 2>)
+                         : reinterpret_cast<void*>(&step_first_kernel<10, 2>);
+  }
 }
 }  // namespace lrs

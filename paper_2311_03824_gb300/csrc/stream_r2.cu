@@ -12,9 +12,15 @@ void* stream_w_kernel_r2(int et) {
     default: return reinterpret_cast<void*>(&w_kernel<2, 0>);
   }
 }
-void* stream_step_kernel_r2(int next) {
+void* stream_step_kernel_r2(int next, int variant) {
   using namespace stream;
-  return next ? reinterpret_cast<void*>(&step_next_kernel<2>)
-              : reinterpret_cast<void*>(&step_first_kernel<2>);
+  switch (variant) {
+    case 0: return next ? reinterpret_cast<void*>(&step_next_kernel<2, 0>)
+                        : reinterpret_cast<void*>(&step_first_kernel<2, 0>);
+    case 1: return next ? reinterpret_cast<void*>(&step_next_kernel<2, 1>)
+                        : reinterpret_cast<void*>(&step_first_kernel<2, 1>);
+    default: return next ? reinterpret_cast<void*>(&step_next_kernel<2, 2>)
+                         : reinterpret_cast<void*>(&step_first_kernel<2, 2>);
+  }
 }
 }  // namespace lrs

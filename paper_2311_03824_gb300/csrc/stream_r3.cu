@@ -12,9 +12,15 @@ void* stream_w_kernel_r3(int et) {
     default: return reinterpret_cast<void*>(&w_kernel<3, 0>);
   }
 }
-void* stream_step_kernel_r3(int next) {
+void* stream_step_kernel_r3(int next, int variant) {
   using namespace stream;
-  return next ? reinterpret_cast<void*>(&step_next_kernel<3>)
-              : reinterpret_cast<void*>(&step_first_kernel<3>);
+  switch (variant) {
+    case 0: return next ? reinterpret_cast<void*>(&step_next_kernel<3, 0>)
+                        : reinterpret_cast<void*>(&step_first_kernel<3, 0>);
+    case 1: return next ? reinterpret_cast<void*>(&step_next_kernel<3, 1>)
+                        : reinterpret_cast<void*>(&step_first_kernel<3, 1>);
+    default: return next ? reinterpret_cast<void*>(&step_next_kernel<3, 2>)
+                         : reinterpret_cast<void*>(&step_first_kernel<3, 2>);
+  }
 }
 }  // namespace lrs

@@ -12,9 +12,15 @@ void* stream_w_kernel_r4(int et) {
     default: return reinterpret_cast<void*>(&w_kernel<4, 0>);
   }
 }
-void* stream_step_kernel_r4(int next) {
+void* stream_step_kernel_r4(int next, int variant) {
   using namespace stream;
-  return next ? reinterpret_cast<void*>(&step_next_kernel<4>)
-              : reinterpret_cast<void*>(&step_first_kernel<4>);
+  switch (variant) {
+    case 0: return next ? reinterpret_cast<void*>(&step_next_kernel<4, 0>)
+                        : reinterpret_cast<void*>(&step_first_kernel<4, 0>);
+    case 1: return next ? reinterpret_cast<void*>(&step_next_kernel<4, 1>)
+                        : reinterpret_cast<void*>(&step_first_kernel<4, 1>);
+    default: return next ? reinterpret_cast<void*>(&step_next_kernel<4, 2>)
+                         : reinterpret_cast<void*>(&step_first_kernel<4, 2>);
+  }
 }
 }  // namespace lrs
