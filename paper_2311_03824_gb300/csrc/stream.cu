@@ -44,6 +44,10 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   constexpr int planes = ET == 3 ? 2 : 1;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int q = lane & 7, ro = lane >> 3;
+  // element offsets of this lane's chunk in rows 4 ro + s of a 16-row group
+  int off4[4];
+#pragma unroll
+  for (int z = 0; z < 4; ++z) off4[z] = (4 * ro + z) * kTW + ((q ^ ((4 * ro + z) & 7)) << 2);
   const int ncol = count ? *count : T.ncols;
   if (ncol == 0) return;
   const unsigned abytes = static_cast<unsigned>(rp * kTW * pb * planes);
@@ -53,59 +57,66 @@ __global__ void __launch_bounds__(kStreamNT, 2)
          reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(kSW) * S * stage) + wid * kMaxStage,
          stage, S, T.wait_ns);
   P.err = T.probs[0].err;
-  const long nunits = static_cast<long>(ncol) * maxtile;
-  const long ustep = static_cast<long>(gridDim.x) * kSW;
+  const int wk = blockIdx.x * kSW + wid, nw = gridDim.x * kSW;
   auto column = [&](int i) { return list ? list[i] : (final ? ncol - 1 - i : i); };
+  // units (entry i of the list, tile b) in steps of all warps
+  const int di = nw / maxtile, db = nw - di * maxtile;
+  const int i_first = wk / maxtile, b_first = wk - i_first * maxtile;
+  auto step = [&](int& i, int& b) {
+    i += di;
+    b += db;
+    if (b >= maxtile) {
+      b -= maxtile;
+      ++i;
+    }
+  };
   // producer cursor: unit, its problem data, next row
-  long pu = static_cast<long>(blockIdx.x) * kSW + wid;
-  int pi = 0, pm = 0, pk = 0, pas = 0;
+  int pu = i_first, pb_ = b_first, pi = 0, pm = 0, pas = 0;
   const unsigned char* ptile = nullptr;
   const float* pvec = nullptr;
-  auto open = [&]() {  // the next unit at or after pu that exists
-    for (; pu < nunits; pu += ustep) {
-      const int i = static_cast<int>(pu / maxtile), b = static_cast<int>(pu - static_cast<long>(i) * maxtile);
-      const int c = column(i);
+  auto open = [&]() {  // the next unit from the cursor on that exists
+    for (; pu < ncol; step(pu, pb_)) {
+      const int c = column(pu);
       const StreamProblem& pr = T.probs[prob_of(T, c)];
       const int ntile = pr.L.ns / kTW;
-      if (b >= ntile) continue;
-      pk = c - pr.col0;
+      if (pb_ >= ntile) continue;
+      const int k = c - pr.col0;
       pm = pr.L.m;
       pas = pr.astride;
       ptile = static_cast<const unsigned char*>(pr.A) +
-              (static_cast<size_t>(pk) * ntile + b) * (static_cast<size_t>(pm) * kTW * elem_bytes(ET));
-      pvec = pr.uvec + static_cast<size_t>(pk) * planes * pas;
+              (static_cast<size_t>(k) * ntile + pb_) * (static_cast<size_t>(pm) * kTW * elem_bytes(ET));
+      pvec = pr.uvec + static_cast<size_t>(k) * planes * pas;
       pi = 0;
       return;
     }
   };
   auto issue = [&]() {
-    if (pu >= nunits) return;
+    if (pu >= ncol) return;
     const int nr = min(rp, pm - pi);
-    const unsigned s = P.issued % S;
     const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
     const unsigned ub = static_cast<unsigned>(((nr + 3) & ~3) * 4);
-    unsigned char* dst = P.base + static_cast<size_t>(s) * stage;
+    unsigned char* dst = P.issue_at();
     if (lane == 0) {
-      mbar_arrive_expect_tx(&P.full[s], (hb + ub) * planes);
+      uint64_t* bar = P.issue_bar();
+      mbar_arrive_expect_tx(bar, (hb + ub) * planes);
 #pragma unroll
       for (int pl = 0; pl < planes; ++pl) {
         bulk_copy_g2s(dst + pl * hb, ptile + static_cast<size_t>(pl) * pm * kTW + static_cast<size_t>(pi) * kTW * pb,
-                      hb, &P.full[s]);
-        bulk_copy_g2s(dst + abytes + pl * rp * 4, pvec + pl * pas + pi, ub, &P.full[s]);
+                      hb, bar);
+        bulk_copy_g2s(dst + abytes + pl * rp * 4, pvec + pl * pas + pi, ub, bar);
       }
     }
-    ++P.issued;
+    P.issued();
     pi += nr;
     if (pi >= pm) {
-      pu += ustep;
+      step(pu, pb_);
       open();
     }
   };
   open();
   for (int i = 0; i < S; ++i) issue();
-  for (long u = static_cast<long>(blockIdx.x) * kSW + wid; u < nunits && !P.dead; u += ustep) {
-    const int i = static_cast<int>(u / maxtile), b = static_cast<int>(u - static_cast<long>(i) * maxtile);
-    const int c = column(i);
+  for (int u = i_first, b = b_first; u < ncol && !P.dead; step(u, b)) {
+    const int c = column(u);
     const StreamProblem& pr = T.probs[prob_of(T, c)];
     if (b >= pr.L.ns / kTW) continue;
     const int k = c - pr.col0, m = pr.L.m;
@@ -116,13 +127,18 @@ __global__ void __launch_bounds__(kStreamNT, 2)
       const int nr = min(rp, m - i0);
       const float* w1 = reinterpret_cast<const float*>(st + abytes);
       const float* w2 = w1 + rp;
-      auto row = [&](int r, float a1, float a2) {
-        const int off = r * kTW + ((q ^ (r & 7)) << 2);
+      auto row = [&](int off, float a1, float a2) {  // off: element offset of the chunk
         float4 a;
         if constexpr (ET >= 2) {
           a = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
         } else {
-          a = sweep::load4<ET>(st, nr, r, q, nullptr, nullptr);
+          if constexpr (ET == 0) {
+            a = *reinterpret_cast<const float4*>(st + static_cast<size_t>(off) * 4);
+          } else {
+            const uint2 raw = *reinterpret_cast<const uint2*>(st + static_cast<size_t>(off) * 2);
+            a = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                            __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+          }
         }
         acc.x = fmaf(a.x, a1, acc.x);
         acc.y = fmaf(a.y, a1, acc.y);
@@ -144,13 +160,14 @@ __global__ void __launch_bounds__(kStreamNT, 2)
         const float4 a1 = *reinterpret_cast<const float4*>(w1 + r);
         float4 a2 = make_float4(0.f, 0.f, 0.f, 0.f);
         if constexpr (ET == 3) a2 = *reinterpret_cast<const float4*>(w2 + r);
-        row(r, a1.x, a2.x);
-        row(r + 1, a1.y, a2.y);
-        row(r + 2, a1.z, a2.z);
-        row(r + 3, a1.w, a2.w);
+        row(t * kTW + off4[0], a1.x, a2.x);
+        row(t * kTW + off4[1], a1.y, a2.y);
+        row(t * kTW + off4[2], a1.z, a2.z);
+        row(t * kTW + off4[3], a1.w, a2.w);
       }
-      for (int r = t + ro; r < nr; r += 4) row(r, w1[r], ET == 3 ? w2[r] : 0.f);
-      ++P.taken;
+      for (int r = t + ro; r < nr; r += 4)
+        row(r * kTW + ((q ^ (r & 7)) << 2), w1[r], ET == 3 ? w2[r] : 0.f);
+      P.taken();
       __syncwarp();
       issue();
     }

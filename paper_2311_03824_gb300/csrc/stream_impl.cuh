@@ -68,7 +68,9 @@ struct Pipe {
   uint64_t* full;
   unsigned stage;        // bytes
   int S;
-  unsigned issued, taken;
+  int si, st;            // stage of the next piece to issue, to take
+  unsigned ph;           // phase bit of the next piece to take
+  int flying;            // pieces issued and not taken
   bool dead;
   int* err;
   unsigned long long wait_ns;
@@ -78,7 +80,9 @@ struct Pipe {
     full = f;
     stage = stg;
     S = s;
-    issued = taken = 0;
+    si = st = 0;
+    ph = 0;
+    flying = 0;
     dead = false;
     err = nullptr;
     wait_ns = w;
@@ -86,28 +90,39 @@ struct Pipe {
       for (int i = 0; i < S; ++i) mbar_init(&full[i], 1);
     __syncwarp();
   }
-  __device__ bool wait(uint64_t* bar, unsigned parity) const {
-    if (mbar_try_wait(bar, parity)) return true;
+  __device__ uint64_t* issue_bar() const { return full + si; }
+  __device__ unsigned char* issue_at() const { return base + static_cast<unsigned>(si) * stage; }
+  __device__ void issued() {
+    ++flying;
+    si = si + 1 == S ? 0 : si + 1;
+  }
+  __device__ bool wait() const {
+    uint64_t* bar = full + st;
+    if (mbar_try_wait(bar, ph)) return true;
     const unsigned long long t0 = gtimer();
-    while (!mbar_try_wait(bar, parity))
+    while (!mbar_try_wait(bar, ph))
       if (gtimer() - t0 > wait_ns) return false;
     return true;
   }
-  // the oldest piece in flight (every lane waits)
+  // the oldest piece in flight (every lane waits); taken() when it has been read
   __device__ const unsigned char* take() {
-    const unsigned s = taken % S;
-    bool ok = wait(&full[s], (taken / S) & 1u);
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok) {
+    if (!__all_sync(0xffffffffu, wait())) {
       dead = true;
       if ((threadIdx.x & 31) == 0) report_error(err, kErrTimeout, -1);
     }
-    return base + static_cast<size_t>(s) * stage;
+    return base + static_cast<unsigned>(st) * stage;
+  }
+  __device__ void taken() {
+    --flying;
+    if (++st == S) {
+      st = 0;
+      ph ^= 1u;
+    }
   }
   // before leaving after an expired wait: no copy may land in this CTA's
   // shared memory once it is gone
   __device__ void drain() {
-    for (; taken < issued; ++taken) wait(&full[taken % S], (taken / S) & 1u);
+    for (; flying > 0; taken()) wait();
   }
 };
 
@@ -120,7 +135,7 @@ __device__ __forceinline__ int prob_of(const StreamTable& T, int c) {
 // ------------------------------------------------------------------ W = A U --
 // Rows of a unit (a multiple of 8): accumulators rows/4 x R per lane and
 // 4 R registers of U at a time leave 128 registers, two CTAs per SM.
-__host__ __device__ constexpr int w_rows(int R) { return R <= 6 ? 32 : 16; }
+__host__ __device__ constexpr int w_rows(int R) { return R <= 6 ? 32 : R <= 12 ? 16 : 8; }
 
 // Unit: RB rows x one chunk of `tbw` tiles of one column.  A CTA keeps its
 // chunk of U in shared memory for all its units (a lane reads U of its four
@@ -137,10 +152,12 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   constexpr int RB = w_rows(R), RT = RB / 4;
   constexpr int pb = ET == 0 ? 4 : ET == 1 ? 2 : 1;
   constexpr int planes = ET == 3 ? 2 : 1;
-  constexpr int CP = R > 12 ? 2 : 4;  // columns of U held in registers at a time
+  constexpr int CP = 4;  // columns of U held in registers at a time
   constexpr unsigned sub = RB * kTW * pb * planes;  // bytes of one tile of a piece
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int q = lane & 7, ro = lane >> 3;
+  // element offsets of this lane's chunk in rows 8 z + ro and 8 z + 4 + ro
+  const int off0 = ro * kTW + ((q ^ ro) << 2), off1 = (4 + ro) * kTW + ((q ^ (4 + ro)) << 2);
   float* Us = reinterpret_cast<float*>(smem);
   const unsigned stage = sub * tpp;
   Pipe P;
@@ -170,33 +187,48 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     }
     __syncthreads();
     const int u0 = as.idx * kSW + wid, ustep = as.cnt * kSW;
-    int pu = u0, pbt = b0;  // next piece to issue: unit, first tile
+    const int dk = ustep / nrb, db = ustep - dk * nrb;  // a unit step in (column, row block)
+    int pu = u0, pk = u0 / nrb, prb = u0 - pk * nrb, pbt = b0;  // next piece to issue
     auto issue = [&]() {
       if (pu >= nunits) return;
-      const int k = pu / nrb, i0 = (pu - k * nrb) * RB, nr = min(RB, m - i0);
+      const int i0 = prb * RB, nr = min(RB, m - i0);
       const int nt = min(tpp, b1 - pbt);
-      const unsigned s = P.issued % S;
       const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
-      unsigned char* dst = P.base + static_cast<size_t>(s) * stage;
-      if (lane == 0) mbar_arrive_expect_tx(&P.full[s], hb * planes * nt);
+      unsigned char* dst = P.issue_at();
+      if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt);
       __syncwarp();
       if (lane < nt * planes) {
         const int t = lane / planes, pl = lane - t * planes;
-        const unsigned char* src = A + (static_cast<size_t>(k) * ntile + pbt + t) * tb +
+        const unsigned char* src = A + (static_cast<size_t>(pk) * ntile + pbt + t) * tb +
                                    static_cast<size_t>(pl) * m * kTW +
                                    static_cast<size_t>(i0) * kTW * pb;
-        bulk_copy_g2s(dst + t * sub + pl * hb, src, hb, &P.full[s]);
+        bulk_copy_g2s(dst + t * sub + pl * hb, src, hb, P.issue_bar());
       }
-      ++P.issued;
+      P.issued();
       pbt += nt;
       if (pbt >= b1) {
         pbt = b0;
         pu += ustep;
+        pk += dk;
+        prb += db;
+        if (prb >= nrb) {
+          prb -= nrb;
+          ++pk;
+        }
       }
     };
     for (int i = 0; i < S; ++i) issue();
-    for (int u = u0; u < nunits && !P.dead; u += ustep) {
-      const int k = u / nrb, i0 = (u - k * nrb) * RB, nr = min(RB, m - i0);
+    int k = u0 / nrb, rb = u0 - k * nrb;
+    auto next_unit = [&]() {
+      k += dk;
+      rb += db;
+      if (rb >= nrb) {
+        rb -= nrb;
+        ++k;
+      }
+    };
+    for (int u = u0; u < nunits; u += ustep, next_unit()) {
+      const int i0 = rb * RB, nr = min(RB, m - i0);
       float s1[RT], s2[RT];
 #pragma unroll
       for (int t = 0; t < RT; ++t) {
@@ -207,8 +239,10 @@ __global__ void __launch_bounds__(kStreamNT, 2)
           if (ET == 3) s2[t] = pr.rscale[o + 1];
         }
       }
+      // the column's support: entries 0..63 in registers, their tiles beside them
       const int* sidx = pr.S_idx + static_cast<size_t>(k) * rho;
-      const int j0 = lane < rho ? sidx[lane] : -1;
+      const int j0 = lane < rho ? sidx[lane] : -1, j1 = 32 + lane < rho ? sidx[32 + lane] : -1;
+      const int jt0 = j0 < n ? j0 >> 5 : -1, jt1 = j1 < n ? j1 >> 5 : -1;  // (-1 >> 5 = -1)
       float acc[RT][R];
 #pragma unroll
       for (int t = 0; t < RT; ++t)
@@ -231,23 +265,23 @@ __global__ void __launch_bounds__(kStreamNT, 2)
             }
 #pragma unroll
             for (int t = 0; t < RT; ++t) {
-              const int i = 4 * t + ro;
               if (c0 == 0) {
-                if (i < nr) {
-                  const int off = i * kTW + ((q ^ (i & 7)) << 2);
-                  if constexpr (ET == 2) {  // raw values; the row's scale multiplies the sum
-                    av[t] = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
-                  } else if constexpr (ET == 3) {
-                    const float4 fh = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
-                    const float4 fl = static_cast<float4>(
-                        *reinterpret_cast<const __nv_fp8x4_e4m3*>(st + nr * kTW + off));
-                    av[t] = make_float4(fmaf(fl.x, s2[t], fh.x * s1[t]), fmaf(fl.y, s2[t], fh.y * s1[t]),
-                                        fmaf(fl.z, s2[t], fh.z * s1[t]), fmaf(fl.w, s2[t], fh.w * s1[t]));
-                  } else {
-                    av[t] = sweep::load4<ET>(st, nr, i, q, nullptr, nullptr);
-                  }
+                // rows at or beyond nr hold stale data: their sums are not stored
+                const int off = (t & 1 ? off1 : off0) + (t >> 1) * 8 * kTW;
+                if constexpr (ET == 0) {
+                  av[t] = *reinterpret_cast<const float4*>(st + static_cast<size_t>(off) * 4);
+                } else if constexpr (ET == 1) {
+                  const uint2 raw = *reinterpret_cast<const uint2*>(st + static_cast<size_t>(off) * 2);
+                  av[t] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                                      __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+                } else if constexpr (ET == 2) {  // raw values; the row's scale multiplies the sum
+                  av[t] = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
                 } else {
-                  av[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                  const float4 fh = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
+                  const float4 fl = static_cast<float4>(
+                      *reinterpret_cast<const __nv_fp8x4_e4m3*>(st + nr * kTW + off));
+                  av[t] = make_float4(fmaf(fl.x, s2[t], fh.x * s1[t]), fmaf(fl.y, s2[t], fh.y * s1[t]),
+                                      fmaf(fl.z, s2[t], fh.z * s1[t]), fmaf(fl.w, s2[t], fh.w * s1[t]));
                 }
               }
 #pragma unroll
@@ -260,9 +294,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
             }
           }
           // support columns that lie in this tile -> AG_k (entry e of the input support)
-          for (int e0 = 0; e0 < rho; e0 += 32) {
-            const int j = e0 == 0 ? j0 : (e0 + lane < rho ? sidx[e0 + lane] : -1);
-            unsigned in = __ballot_sync(0xffffffffu, j >= 0 && j < n && (j >> 5) == b + tt);
+          auto extract = [&](unsigned in, int j, int e0) {
             while (in) {
               const int src = __ffs(in) - 1;
               in &= in - 1;
@@ -278,9 +310,17 @@ __global__ void __launch_bounds__(kStreamNT, 2)
                 ag[lane] = elem1s<ET>(st, nr, lane, jj, r1, r2);
               }
             }
+          };
+          if (const unsigned in = __ballot_sync(0xffffffffu, jt0 == b + tt)) extract(in, j0, 0);
+          if (rho > 32) {
+            if (const unsigned in = __ballot_sync(0xffffffffu, jt1 == b + tt)) extract(in, j1, 32);
+            for (int e0 = 64; e0 < rho; e0 += 32) {
+              const int j = e0 + lane < rho ? sidx[e0 + lane] : -1;
+              extract(__ballot_sync(0xffffffffu, j < n && j >> 5 == b + tt), j, e0);
+            }
           }
         }
-        ++P.taken;
+        P.taken();
         __syncwarp();
         issue();
       }
