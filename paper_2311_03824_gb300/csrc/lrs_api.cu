@@ -1860,7 +1860,7 @@ lrs_status lrs_describe(lrs_t h, char* buf, int32_t len) {
              "\"w_row_blocks\": %d, \"w_stages\": %d, \"rows_per_piece\": %d, \"g_stages\": %d, "
              "\"step_grid\": %d, \"step_smem\": %zu, \"a_dtype\": %d, \"refine_every\": %d, "
              "\"launches_per_iteration\": %d}",
-             S.grid, P.ncw, P.nrb, S.wS, S.grp, S.gS, S.fgrid[P.variant], S.fsmem[P.variant], h->L.et,
+             S.grid, P.ncw, P.nrb, S.wS, S.grp, S.gS, S.fgrid[P.fvar], S.fsmem[P.fvar], h->L.et,
              h->opt.refine_every, launches_per_iteration(h));
     return LRS_OK;
   }

@@ -244,7 +244,7 @@ struct StreamProblem {
   int col0;             // index of this problem's first column in the launch
   int wstride, astride; // m R and m rounded up to 4
   int tbw, ncw, nrb;    // W units: tiles per column chunk, chunks, row blocks
-  int variant;          // kernel of the column steps (stream_impl.cuh)
+  int fvar, nvar;       // kernels of the first and the next column steps (stream_impl.cuh)
 };
 // one CTA's share of the W units of column chunk cc of a problem: units
 // (warp idx * 8 + w) + i * 8 cnt

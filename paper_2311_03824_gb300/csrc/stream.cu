@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   const unsigned abytes = static_cast<unsigned>(rp * kTW * pb * planes);
   const unsigned stage = abytes + static_cast<unsigned>(planes * rp * 4);
   Pipe P;
-  P.init(smem + static_cast<size_t>(wid) * S * stage,
+  P.init(static_cast<unsigned>(wid * S) * stage,
          reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(kSW) * S * stage) + wid * kMaxStage,
          stage, S, T.wait_ns);
   P.err = T.probs[0].err;
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     const int nr = min(rp, pm - pi);
     const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
     const unsigned ub = static_cast<unsigned>(((nr + 3) & ~3) * 4);
-    unsigned char* dst = P.issue_at();
+    unsigned char* dst = smem + P.issue_at();
     if (lane == 0) {
       uint64_t* bar = P.issue_bar();
       mbar_arrive_expect_tx(bar, (hb + ub) * planes);
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     const int k = c - pr.col0, m = pr.L.m;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i0 = 0; i0 < m; i0 += rp) {
-      const unsigned char* st = P.take();
+      const unsigned char* st = smem + P.take();
       if (P.dead) break;
       const int nr = min(rp, m - i0);
       const float* w1 = reinterpret_cast<const float*>(st + abytes);
@@ -290,17 +290,23 @@ void stream_plan(StreamProblem& P, int R) {
   // grid: n = 1000, q = 1000 gives 16.4 units per warp), four from 96 tiles on
   // (the chunks' partial W are then 2 R / tbw / 32 of A_k's bytes), and U of a
   // chunk within 40 KB of shared memory.
-  const int cap = std::max(1, 40 * 1024 / (kTW * R * 4));
+  const int cap = std::max(1, 40 * 1024 / (kTW * w_chunks4(R) * 16));
   const int want = (ntile + (ntile >= 96 ? 4 : 8) - 1) / (ntile >= 96 ? 4 : 8);
   P.tbw = std::max(1, std::min(cap, want));
   P.ncw = (ntile + P.tbw - 1) / P.tbw;
   P.nrb = (m + w_rows(R) - 1) / w_rows(R);
   // Column steps: 128 threads while four columns fit an SM with their support
   // staged, 256 threads for larger columns, the support's columns read from
-  // memory when two staged columns do not fit.  By the problem's own sizes, so
-  // that a batch runs the same arithmetic.
-  auto smem = [&](int v) { return step_carve(R, m, P.L.n, P.L.rho, P.astride, v, true).total; };
-  P.variant = smem(0) <= 54 * 1024 ? 0 : smem(1) <= 112 * 1024 ? 1 : 2;
+  // memory when two staged columns do not fit.  The thread count (which fixes
+  // the order of the sums) by the problem's own sizes, so that a batch runs
+  // the same arithmetic.
+  auto smem = [&](int v, bool next) {
+    return step_carve(R, m, P.L.n, P.L.rho, P.astride, v, next).total;
+  };
+  const size_t two = 112 * 1024;
+  const bool small = smem(0, true) <= 54 * 1024;
+  P.fvar = small ? 0 : smem(1, false) <= two ? 1 : 2;
+  P.nvar = small ? 0 : smem(1, true) <= two ? 1 : 2;
 }
 
 bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int grid_limit,
@@ -318,13 +324,14 @@ bool stream_shape(const StreamProblem* P, int nprob, int R, int et, int nsm, int
     m_max = std::max(m_max, p.L.m);
     S->maxtile = std::max(S->maxtile, p.L.ns / kTW);
     S->te = std::max(S->te, p.te);
-    us = std::max(us, static_cast<unsigned>(p.tbw * kTW * R * 4));
+    us = std::max(us, static_cast<unsigned>(p.tbw * kTW * w_chunks4(R) * 16));
     ncols += p.L.q;
     work += static_cast<double>(p.L.q) * p.nrb * p.ncw * p.tbw;
-    const int v = p.variant;
-    S->fsmem[v] = std::max<size_t>(S->fsmem[v], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, v, false).total);
-    S->nsmem[v] = std::max<size_t>(S->nsmem[v], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, v, true).total);
-    if (S->nsmem[v] > one) return false;
+    S->fsmem[p.fvar] = std::max<size_t>(
+        S->fsmem[p.fvar], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, p.fvar, false).total);
+    S->nsmem[p.nvar] = std::max<size_t>(
+        S->nsmem[p.nvar], step_carve(R, p.L.m, p.L.n, p.L.rho, p.astride, p.nvar, true).total);
+    if (S->fsmem[p.fvar] > one || S->nsmem[p.nvar] > one) return false;
   }
   if (S->te > kStreamMaxRounds) return false;
   // W: pieces of about 4 KB, as many stages as two CTAs per SM allow

@@ -63,8 +63,11 @@ __device__ __forceinline__ unsigned long long gtimer() {
 // ------------------------------------------------------------- warp pipeline --
 // One warp's ring: `S` stages, full barriers only (the warp that refills a
 // stage is the one that has read it).
+// Places are byte offsets in the CTA's dynamic shared memory: an access through
+// the array itself stays a shared-memory load (a pointer kept in the ring is a
+// generic one, with 64-bit addresses).
 struct Pipe {
-  unsigned char* base;
+  unsigned base;
   uint64_t* full;
   unsigned stage;        // bytes
   int S;
@@ -75,7 +78,7 @@ struct Pipe {
   int* err;
   unsigned long long wait_ns;
 
-  __device__ void init(unsigned char* b, uint64_t* f, unsigned stg, int s, unsigned long long w) {
+  __device__ void init(unsigned b, uint64_t* f, unsigned stg, int s, unsigned long long w) {
     base = b;
     full = f;
     stage = stg;
@@ -91,7 +94,7 @@ struct Pipe {
     __syncwarp();
   }
   __device__ uint64_t* issue_bar() const { return full + si; }
-  __device__ unsigned char* issue_at() const { return base + static_cast<unsigned>(si) * stage; }
+  __device__ unsigned issue_at() const { return base + static_cast<unsigned>(si) * stage; }
   __device__ void issued() {
     ++flying;
     si = si + 1 == S ? 0 : si + 1;
@@ -105,7 +108,7 @@ struct Pipe {
     return true;
   }
   // the oldest piece in flight (every lane waits); taken() when it has been read
-  __device__ const unsigned char* take() {
+  __device__ unsigned take() {
     if (!__all_sync(0xffffffffu, wait())) {
       dead = true;
       if ((threadIdx.x & 31) == 0) report_error(err, kErrTimeout, -1);
@@ -133,9 +136,27 @@ __device__ __forceinline__ int prob_of(const StreamTable& T, int c) {
 }
 
 // ------------------------------------------------------------------ W = A U --
-// Rows of a unit (a multiple of 8): accumulators rows/4 x R per lane and
-// 4 R registers of U at a time leave 128 registers, two CTAs per SM.
-__host__ __device__ constexpr int w_rows(int R) { return R <= 6 ? 32 : R <= 12 ? 16 : 8; }
+// Rows of a unit (a multiple of 8), rows / 4 x R accumulators per lane.
+__host__ __device__ constexpr int w_rows(int R) { return R <= 6 ? 32 : 16; }
+// 16-byte chunks of one column's R ranks in the shared copy of U
+__host__ __device__ constexpr int w_chunks4(int R) { return (R + 3) / 4; }
+
+// Two multiply-adds in one instruction: (a.x b.x + c.x, a.y b.y + c.y).  The
+// pass is bound by instruction issue (R multiply-adds per element), so a pair
+// of ranks shares one; rounding is that of two fmaf.
+__device__ __forceinline__ void ffma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
 
 // Unit: RB rows x one chunk of `tbw` tiles of one column.  A CTA keeps its
 // chunk of U in shared memory for all its units (a lane reads U of its four
@@ -149,10 +170,9 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     w_kernel(const StreamTable T, const StreamAssign* __restrict__ asg, int nasg, int S, int tpp,
              unsigned us_bytes) {
   extern __shared__ __align__(128) unsigned char smem[];
-  constexpr int RB = w_rows(R), RT = RB / 4;
+  constexpr int RB = w_rows(R), RT = RB / 4, R2 = (R + 1) / 2, R4 = w_chunks4(R);
   constexpr int pb = ET == 0 ? 4 : ET == 1 ? 2 : 1;
   constexpr int planes = ET == 3 ? 2 : 1;
-  constexpr int CP = 4;  // columns of U held in registers at a time
   constexpr unsigned sub = RB * kTW * pb * planes;  // bytes of one tile of a piece
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int q = lane & 7, ro = lane >> 3;
@@ -161,7 +181,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   float* Us = reinterpret_cast<float*>(smem);
   const unsigned stage = sub * tpp;
   Pipe P;
-  P.init(smem + us_bytes + static_cast<size_t>(wid) * S * stage,
+  P.init(us_bytes + static_cast<unsigned>(wid * S) * stage,
          reinterpret_cast<uint64_t*>(smem + us_bytes + static_cast<size_t>(kSW) * S * stage) +
              wid * kMaxStage,
          stage, S, T.wait_ns);
@@ -176,14 +196,18 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     const unsigned char* A = static_cast<const unsigned char*>(pr.A);
     P.err = pr.err;
     __syncthreads();
-    // U of a tile as [z][q]: the 4 R floats of the four columns of lane group q
-    // are R 16-byte chunks z, chunk z of the eight groups side by side, so that
-    // a warp's read is one conflict-free wavefront for every R (row-major, the
+    // U of a tile as [c][z][q]: ranks 4 z .. 4 z + 3 of column 4 q + c in one
+    // 16-byte chunk (zero beyond R), the eight lane groups side by side: a
+    // warp's read is one conflict-free wavefront for every R (row-major, the
     // groups lie 16 R bytes apart: 8-way conflicts at R = 8 and 16)
-    for (int t = threadIdx.x; t < (b1 - b0) * kTW * R / 4; t += kStreamNT) {
-      const int b = t / (8 * R), w = t - b * 8 * R, g = w / R, z = w - g * R;
-      reinterpret_cast<float4*>(Us)[b * 8 * R + z * 8 + g] =
-          reinterpret_cast<const float4*>(pr.Upad + static_cast<size_t>(b0) * kTW * R)[t];
+    for (int t = threadIdx.x; t < (b1 - b0) * 32 * R4; t += kStreamNT) {
+      const int g = t & 7, z = (t >> 3) % R4, cb = (t >> 3) / R4, c = cb & 3, b = cb >> 2;
+      const float* from = pr.Upad + (static_cast<size_t>(b0 + b) * kTW + 4 * g + c) * R + 4 * z;
+      float4 x = make_float4(from[0], 0.f, 0.f, 0.f);
+      if (4 * z + 1 < R) x.y = from[1];
+      if (4 * z + 2 < R) x.z = from[2];
+      if (4 * z + 3 < R) x.w = from[3];
+      reinterpret_cast<float4*>(Us)[t] = x;
     }
     __syncthreads();
     const int u0 = as.idx * kSW + wid, ustep = as.cnt * kSW;
@@ -194,7 +218,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
       const int i0 = prb * RB, nr = min(RB, m - i0);
       const int nt = min(tpp, b1 - pbt);
       const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
-      unsigned char* dst = P.issue_at();
+      unsigned char* dst = smem + P.issue_at();
       if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt);
       __syncwarp();
       if (lane < nt * planes) {
@@ -243,54 +267,54 @@ __global__ void __launch_bounds__(kStreamNT, 2)
       const int* sidx = pr.S_idx + static_cast<size_t>(k) * rho;
       const int j0 = lane < rho ? sidx[lane] : -1, j1 = 32 + lane < rho ? sidx[32 + lane] : -1;
       const int jt0 = j0 < n ? j0 >> 5 : -1, jt1 = j1 < n ? j1 >> 5 : -1;  // (-1 >> 5 = -1)
-      float acc[RT][R];
+      unsigned long long acc[RT][R2];  // pairs of ranks
 #pragma unroll
       for (int t = 0; t < RT; ++t)
 #pragma unroll
-        for (int l = 0; l < R; ++l) acc[t][l] = 0.f;
+        for (int p = 0; p < R2; ++p) acc[t][p] = 0ull;
       for (int b = b0; b < b1; b += tpp) {
-        const unsigned char* st = P.take();
+        unsigned so = P.take();
         if (P.dead) break;
         const int nt = min(tpp, b1 - b);
-        for (int tt = 0; tt < nt; ++tt, st += sub) {
-          const float4* Ut = reinterpret_cast<const float4*>(Us) + (b + tt - b0) * 8 * R + q;
+        for (int tt = 0; tt < nt; ++tt, so += sub) {
+          const unsigned char* st = smem + so;
+          const float4* Ut = reinterpret_cast<const float4*>(smem) + (b + tt - b0) * 32 * R4 + q;
           float4 av[RT];
 #pragma unroll
-          for (int c0 = 0; c0 < 4; c0 += CP) {
-            float uu[CP * R];
+          for (int t = 0; t < RT; ++t) {
+            // rows at or beyond nr hold stale data: their sums are not stored
+            const int off = (t & 1 ? off1 : off0) + (t >> 1) * 8 * kTW;
+            if constexpr (ET == 0) {
+              av[t] = *reinterpret_cast<const float4*>(st + static_cast<size_t>(off) * 4);
+            } else if constexpr (ET == 1) {
+              const uint2 raw = *reinterpret_cast<const uint2*>(st + static_cast<size_t>(off) * 2);
+              av[t] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                                  __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+            } else if constexpr (ET == 2) {  // raw values; the row's scale multiplies the sum
+              av[t] = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
+            } else {
+              const float4 fh = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
+              const float4 fl = static_cast<float4>(
+                  *reinterpret_cast<const __nv_fp8x4_e4m3*>(st + nr * kTW + off));
+              av[t] = make_float4(fmaf(fl.x, s2[t], fh.x * s1[t]), fmaf(fl.y, s2[t], fh.y * s1[t]),
+                                  fmaf(fl.z, s2[t], fh.z * s1[t]), fmaf(fl.w, s2[t], fh.w * s1[t]));
+            }
+          }
 #pragma unroll
-            for (int z = 0; z < CP * R / 4; ++z) {
-              const float4 w = Ut[(c0 * R / 4 + z) * 8];
-              uu[4 * z] = w.x; uu[4 * z + 1] = w.y; uu[4 * z + 2] = w.z; uu[4 * z + 3] = w.w;
+          for (int c = 0; c < 4; ++c) {
+            unsigned long long uu[2 * R4];
+#pragma unroll
+            for (int z = 0; z < R4; ++z) {
+              const float4 w = Ut[(c * R4 + z) * 8];
+              uu[2 * z] = pack2(w.x, w.y);
+              uu[2 * z + 1] = pack2(w.z, w.w);
             }
 #pragma unroll
             for (int t = 0; t < RT; ++t) {
-              if (c0 == 0) {
-                // rows at or beyond nr hold stale data: their sums are not stored
-                const int off = (t & 1 ? off1 : off0) + (t >> 1) * 8 * kTW;
-                if constexpr (ET == 0) {
-                  av[t] = *reinterpret_cast<const float4*>(st + static_cast<size_t>(off) * 4);
-                } else if constexpr (ET == 1) {
-                  const uint2 raw = *reinterpret_cast<const uint2*>(st + static_cast<size_t>(off) * 2);
-                  av[t] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
-                                      __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
-                } else if constexpr (ET == 2) {  // raw values; the row's scale multiplies the sum
-                  av[t] = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
-                } else {
-                  const float4 fh = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(st + off));
-                  const float4 fl = static_cast<float4>(
-                      *reinterpret_cast<const __nv_fp8x4_e4m3*>(st + nr * kTW + off));
-                  av[t] = make_float4(fmaf(fl.x, s2[t], fh.x * s1[t]), fmaf(fl.y, s2[t], fh.y * s1[t]),
-                                      fmaf(fl.z, s2[t], fh.z * s1[t]), fmaf(fl.w, s2[t], fh.w * s1[t]));
-                }
-              }
+              const float x = c == 0 ? av[t].x : c == 1 ? av[t].y : c == 2 ? av[t].z : av[t].w;
+              const unsigned long long xx = pack2(x, x);
 #pragma unroll
-              for (int c = 0; c < CP; ++c) {
-                const int cc = c0 + c;
-                const float x = cc == 0 ? av[t].x : cc == 1 ? av[t].y : cc == 2 ? av[t].z : av[t].w;
-#pragma unroll
-                for (int l = 0; l < R; ++l) acc[t][l] = fmaf(x, uu[c * R + l], acc[t][l]);
-              }
+              for (int p = 0; p < R2; ++p) ffma2(acc[t][p], xx, uu[p]);
             }
           }
           // support columns that lie in this tile -> AG_k (entry e of the input support)
@@ -332,7 +356,8 @@ __global__ void __launch_bounds__(kStreamNT, 2)
         const int i = 4 * t + ro;
 #pragma unroll
         for (int l = 0; l < R; ++l) {
-          float v = acc[t][l];
+          const float2 pr2 = unpack2(acc[t][l >> 1]);
+          float v = l & 1 ? pr2.y : pr2.x;
           v += __shfl_xor_sync(0xffffffffu, v, 1);
           v += __shfl_xor_sync(0xffffffffu, v, 2);
           v += __shfl_xor_sync(0xffffffffu, v, 4);
@@ -966,7 +991,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 8 : 3)
   int cur = -1;
   for (int c = blockIdx.x; c < T.ncols; c += gridDim.x) {
     load_problem(T, c, &spr, cur);
-    if (spr.variant != V) continue;
+    if (spr.fvar != V) continue;
     const StepCarve cv = step_carve(R, spr.L.m, spr.L.n, spr.L.rho, spr.astride, V, false);
     Step<R, V> s(T, spr, smem, cv);
     s.at_column(c, smem, cv);
@@ -1136,7 +1161,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
   for (int at = blockIdx.x; at < count; at += gridDim.x) {
     const int c = zero ? at : T.list[static_cast<size_t>(round & 1) * T.ncols + at];
     load_problem(T, c, &spr, cur);
-    if (spr.variant != V || spr.te == 0) continue;
+    if (spr.nvar != V || spr.te == 0) continue;
     const StepCarve cv = step_carve(R, spr.L.m, spr.L.n, spr.L.rho, spr.astride, V, true);
     Step<R, V> s(T, spr, smem, cv);
     s.at_column(c, smem, cv);
