@@ -2,6 +2,8 @@
 // sweep_gauss_impl.cuh, one translation unit per compiled rank width so the
 // build runs in parallel): shared-memory sizing, cluster launch, and the
 // repacking of row-major A_k into the tiled slab layout.
+#include <algorithm>
+
 #include "sweep_gauss_impl.cuh"
 
 namespace lrs {
@@ -119,20 +121,27 @@ __global__ void repack_kernel(GaussLayout L, const float* __restrict__ Ain, int 
   }
 }
 
-// Defect correction of the low-precision forms: for column k (one block),
-// x_k = U b_k + s_k (kept in xbuf row k), then
+// Defect correction of the low-precision forms: for column k (gridDim.y blocks
+// share its rows), x_k = U b_k + s_k in shared memory (in xbuf, one block per
+// column, when n floats do not fit), then
 // ycorr_k(i) = y_k(i) - sum_j (A_k(i, j) - Atilde_k(i, j)) x_k(j)
-// with A the exact FP32 operator (row-major) and Atilde the stored form.
-template <int ET>
-__global__ void refine_kernel(GaussLayout L, const float* __restrict__ Aex,
-                              const unsigned char* __restrict__ Aq, const float* __restrict__ rscale,
-                              const float* __restrict__ U, const float* __restrict__ Bk,
-                              const int* __restrict__ S_idx, const float* __restrict__ S_val,
-                              const float* __restrict__ y, float* __restrict__ ycorr,
-                              float* __restrict__ xbuf) {
+// with A the exact FP32 operator (row-major) and Atilde the stored form, a warp
+// per row.  Bound by the reads of A: the BF16 value is rounded again from A
+// (the same rounding as the stored one) instead of being read, the FP8 codes
+// are read four at a time (a division per element would cost more).
+// V4: n is a multiple of four, rows are read by 16-byte loads.
+template <int ET, bool V4>
+__global__ void __launch_bounds__(256)
+    refine_kernel(GaussLayout L, const float* __restrict__ Aex,
+                  const unsigned char* __restrict__ Aq, const float* __restrict__ rscale,
+                  const float* __restrict__ U, const float* __restrict__ Bk,
+                  const int* __restrict__ S_idx, const float* __restrict__ S_val,
+                  const float* __restrict__ y, float* __restrict__ ycorr,
+                  float* __restrict__ xbuf) {
+  extern __shared__ __align__(16) float xs[];
   const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   const int n = L.n, m = L.m, r = L.r;
-  float* x = xbuf + static_cast<size_t>(k) * n;
+  float* x = xbuf ? xbuf + static_cast<size_t>(k) * n : xs;
   for (int j = tid; j < n; j += blockDim.x) {
     float v = 0.f;
     for (int l = 0; l < r; ++l)
@@ -146,20 +155,75 @@ __global__ void refine_kernel(GaussLayout L, const float* __restrict__ Aex,
   }
   __syncthreads();
   const size_t slab = static_cast<size_t>(L.ns / kTW) * m * kTW * elem_bytes(ET);
+  const size_t tb = static_cast<size_t>(m) * kTW * elem_bytes(ET);
   const int per = ET == 3 ? 2 : 1;
-  for (int i = tid >> 5; i < m; i += blockDim.x >> 5) {
+  const int nwy = (blockDim.x >> 5) * gridDim.y;
+  for (int i = (tid >> 5) + (blockDim.x >> 5) * blockIdx.y; i < m; i += nwy) {
     const float* arow = Aex + (static_cast<size_t>(k) * m + i) * n;
     const size_t ro = (static_cast<size_t>(k) * m + i) * per;
     const float s1 = ET >= 2 ? rscale[ro] : 0.f, s2 = ET == 3 ? rscale[ro + 1] : 0.f;
     float d = 0.f;
-    for (int j = lane; j < n; j += 32) {
-      const int c = j / L.ns, jl = j - c * L.ns;
-      const float at = elem1s<ET>(Aq + (static_cast<size_t>(k) * L.cs + c) * slab, m, i, jl, s1, s2);
-      d = fmaf(arow[j] - at, x[j], d);
+    if constexpr (V4) {
+#pragma unroll 8
+      for (int j = 4 * lane; j < n; j += 128) {
+        const float4 a = __ldcs(reinterpret_cast<const float4*>(arow + j));
+        float4 t;
+        if constexpr (ET == 1) {
+          t = make_float4(__bfloat162float(__float2bfloat16_rn(a.x)), __bfloat162float(__float2bfloat16_rn(a.y)),
+                          __bfloat162float(__float2bfloat16_rn(a.z)), __bfloat162float(__float2bfloat16_rn(a.w)));
+        } else {
+          const int c = j / L.ns, jl = j - c * L.ns;
+          const unsigned char* tile = Aq + (static_cast<size_t>(k) * L.cs + c) * slab + (jl >> 5) * tb;
+          const int off = i * kTW + ((((jl & 31) >> 2) ^ (i & 7)) << 2);
+          t = static_cast<float4>(*reinterpret_cast<const __nv_fp8x4_e4m3*>(tile + off));
+          t = make_float4(t.x * s1, t.y * s1, t.z * s1, t.w * s1);
+          if constexpr (ET == 3) {
+            const float4 lo = static_cast<float4>(
+                *reinterpret_cast<const __nv_fp8x4_e4m3*>(tile + static_cast<size_t>(m) * kTW + off));
+            t = make_float4(fmaf(lo.x, s2, t.x), fmaf(lo.y, s2, t.y), fmaf(lo.z, s2, t.z), fmaf(lo.w, s2, t.w));
+          }
+        }
+        const float4 xv = *reinterpret_cast<const float4*>(x + j);
+        d = fmaf(a.x - t.x, xv.x, d);
+        d = fmaf(a.y - t.y, xv.y, d);
+        d = fmaf(a.z - t.z, xv.z, d);
+        d = fmaf(a.w - t.w, xv.w, d);
+      }
+    } else {
+#pragma unroll 8
+      for (int j = lane; j < n; j += 32) {
+        const float a = __ldcs(arow + j);
+        float t;
+        if constexpr (ET == 1) {
+          t = __bfloat162float(__float2bfloat16_rn(a));
+        } else {
+          const int c = j / L.ns, jl = j - c * L.ns;
+          t = elem1s<ET>(Aq + (static_cast<size_t>(k) * L.cs + c) * slab, m, i, jl, s1, s2);
+        }
+        d = fmaf(a - t, x[j], d);
+      }
     }
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
     if (lane == 0) ycorr[static_cast<size_t>(k) * m + i] = y[static_cast<size_t>(k) * m + i] - d;
   }
+}
+
+template <int ET>
+void refine_launch(const GaussLayout& L, const float* A_exact, const unsigned char* aq,
+                   const float* rscale, const float* U, const float* Bk, const int* S_idx,
+                   const float* S_val, const float* y, float* ycorr, float* xbuf, cudaStream_t s) {
+  const size_t smem = static_cast<size_t>(L.n) * 4;
+  const bool fits = smem <= 48 * 1024;  // n <= 12288: x_k in shared memory
+  // rows of a column over enough blocks for about four per SM
+  const int ys = fits ? std::max(1, std::min((608 + L.q - 1) / L.q, (L.m + 15) / 16)) : 1;
+  const dim3 grid(static_cast<unsigned>(L.q), static_cast<unsigned>(ys));
+  // V4 also needs A_exact and xbuf aligned: both are this library's allocations
+  if (L.n % 4 == 0)
+    refine_kernel<ET, true><<<grid, 256, fits ? smem : 0, s>>>(L, A_exact, aq, rscale, U, Bk, S_idx,
+                                                               S_val, y, ycorr, fits ? nullptr : xbuf);
+  else
+    refine_kernel<ET, false><<<grid, 256, fits ? smem : 0, s>>>(L, A_exact, aq, rscale, U, Bk, S_idx,
+                                                                S_val, y, ycorr, fits ? nullptr : xbuf);
 }
 
 }  // namespace
@@ -240,11 +304,10 @@ cudaError_t refine_residual(const GaussLayout& L, const float* A_exact, const vo
                             const int* S_idx, const float* S_val, const float* y, float* ycorr,
                             float* xbuf, cudaStream_t s) {
   const unsigned char* aq = static_cast<const unsigned char*>(A_int);
-  const dim3 grid(static_cast<unsigned>(L.q)), block(256);
   switch (L.et) {
-    case 1: refine_kernel<1><<<grid, block, 0, s>>>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf); break;
-    case 2: refine_kernel<2><<<grid, block, 0, s>>>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf); break;
-    case 3: refine_kernel<3><<<grid, block, 0, s>>>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf); break;
+    case 1: refine_launch<1>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf, s); break;
+    case 2: refine_launch<2>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf, s); break;
+    case 3: refine_launch<3>(L, A_exact, aq, rscale, U, Bk, S_idx, S_val, y, ycorr, xbuf, s); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
