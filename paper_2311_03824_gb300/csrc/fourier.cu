@@ -7,11 +7,9 @@
 // Per GDmin iteration (Algorithm 1):
 //   FU = F2 U                      r forward 2D FFTs (shared by all frames),
 //                                  so W_k = A_k U = FU[Omega_k, :]
-//   sweep (one CTA per frame k)    G_k = W_k^H W_k and its inverse (FP64),
-//                                  IHT: A s and A g_G as sparse DFTs, g = A^H u
-//                                  as one inverse 2D FFT of the frame held in
-//                                  shared memory, HardThreshold by radix select,
-//                                  then b_k and res_k = W_k b_k + A_k s_k - y_k
+//   sweep (one CTA per frame k)    fourier_sweep.cuh: W_k's orthonormal basis,
+//                                  the IHT sweeps, then b_k and res_k = W_k b_k
+//                                  + A_k s_k - y_k
 //   K = sum_k zero-fill_k(res_k) b_k^H   k-space accumulation through the
 //                                  inverse index of the masks (fixed order)
 //   grad = F2^H K                  r inverse 2D FFTs (linearity of F2)
@@ -26,269 +24,14 @@
 #include <string>
 #include <vector>
 
-#include "lrs_dev.cuh"
-#include "lrs_internal.h"
+#include "fourier_sweep.cuh"
 
 namespace lrs {
+#define LRS_FSWEEP_R(X) X(2) X(4) X(6) X(8) X(12) X(16)
+#define LRS_DECL(R) void* fsweep_kernel_r##R(bool pow2);  // fsweep_r*.cu
+LRS_FSWEEP_R(LRS_DECL)
+#undef LRS_DECL
 namespace fourier {
-
-constexpr int kFT = 512;   // threads of the frame kernels
-constexpr int kFW = kFT / 32;
-// sweep profile slots: set-up and Gram, sparse DFTs, norms and vector
-// updates, 2D FFTs with the frame's fills and scalings, HardThreshold, final
-// stage, projections' W^H v and G^-1 solve, projections' v - W x
-constexpr int kFProf = 8;
-// static shared memory of the sweep (its profile counters), an upper bound
-constexpr size_t kFStaticSmem = 256;
-constexpr int kMaxR = 16;
-
-// ------------------------------------------------------------ complex --
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-// acc += a * b
-__device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 acc) {
-  acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
-  acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
-  return acc;
-}
-// acc += conj(a) * b
-__device__ __forceinline__ float2 ccfma(float2 a, float2 b, float2 acc) {
-  acc.x = fmaf(a.x, b.x, fmaf(a.y, b.y, acc.x));
-  acc.y = fmaf(a.x, b.y, fmaf(-a.y, b.x, acc.y));
-  return acc;
-}
-__device__ __forceinline__ double2 dcmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 dccmul(double2 a, double2 b) {  // conj(a) * b
-  return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
-__device__ __forceinline__ float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
-
-// Double-float accumulation (a value carried as hi + lo, two float32 words:
-// about 48 bits of significand on the FP32 units, whose dependent operations
-// are far cheaper than FP64's on this part).  df_fma: (hi, lo) += a * b with
-// the product's rounding error from an fma and the sum's from Knuth's
-// two-sum.  df_add: (hi, lo) += (bh, bl).
-__device__ __forceinline__ void df_fma(float& hi, float& lo, float a, float b) {
-  const float p = a * b;
-  const float pe = fmaf(a, b, -p);
-  const float s = hi + p;
-  const float bb = s - hi;
-  const float se = (hi - (s - bb)) + (p - bb);
-  hi = s;
-  lo += se + pe;
-}
-__device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl) {
-  const float s = hi + bh;
-  const float bb = s - hi;
-  const float se = (hi - (s - bb)) + (bh - bb);
-  hi = s;
-  lo += se + bl;
-}
-// warp sum of double-float values (xor butterfly: every lane ends with the
-// same value, the pairs added in a fixed order)
-__device__ __forceinline__ double warp_sum_df(float hi, float lo) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-    df_add(hi, lo, oh, ol);
-  }
-  return static_cast<double>(hi) + static_cast<double>(lo);
-}
-
-__device__ __forceinline__ float warp_sumf(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// ------------------------------------------------------------ 2D FFT --
-// Sides that are not powers of two take a direct DFT (frames of at most
-// kDirectPer * blockDim.x pixels): each thread keeps its outputs in
-// registers until every thread has read the frame.
-constexpr int kDirectPer = 8;
-
-__device__ void dft_direct_smem(float2* X, int nx, int ny, bool rows, const float2* tw,
-                                bool inverse) {
-  const int ld = ny + 1, n = nx * ny, len = rows ? ny : nx;
-  float2 acc[kDirectPer];
-#pragma unroll
-  for (int u = 0; u < kDirectPer; ++u) {
-    const int e = threadIdx.x + u * blockDim.x;
-    float2 s = make_float2(0.f, 0.f);
-    if (e < n) {
-      const int row = e / ny, col = e - row * ny;
-      const int j = rows ? col : row;  // output frequency along the transformed side
-      int idx = 0;                     // j * k mod len
-      for (int k = 0; k < len; ++k) {
-        float2 w = tw[idx];
-        if (inverse) w.y = -w.y;
-        s = cfma(rows ? X[row * ld + k] : X[k * ld + col], w, s);
-        idx += j;
-        if (idx >= len) idx -= len;
-      }
-    }
-    acc[u] = s;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < kDirectPer; ++u) {
-    const int e = threadIdx.x + u * blockDim.x;
-    if (e < n) {
-      const int row = e / ny, col = e - row * ny;
-      X[row * ld + col] = acc[u];
-    }
-  }
-  __syncthreads();
-}
-
-// Two radix-2 decimation-in-time stages s and s + 1 on the quad x0, x1, x2,
-// x3 at offsets 0, h, 2h, 3h (h = 2^s) of a block of 4h: stage s pairs
-// (x0, x1) and (x2, x3) with twiddle w1, stage s + 1 pairs (x0, x2) with w2a
-// and (x1, x3) with w2b.  Every element gets the operations of the two
-// stages run one after the other, in the same order, so the result is that
-// of two single-stage passes, with one shared-memory round trip instead of two.
-__device__ __forceinline__ void stage_pair(float2& x0, float2& x1, float2& x2, float2& x3,
-                                           float2 w1, float2 w2a, float2 w2b, bool inverse) {
-  if (inverse) {
-    w1.y = -w1.y;
-    w2a.y = -w2a.y;
-    w2b.y = -w2b.y;
-  }
-  const float2 a0 = x0, a2 = x2;
-  const float2 c1 = cmul(x1, w1), c3 = cmul(x3, w1);
-  const float2 b0 = cadd(a0, c1), b1 = csub(a0, c1), b2 = cadd(a2, c3), b3 = csub(a2, c3);
-  const float2 d2 = cmul(b2, w2a), d3 = cmul(b3, w2b);
-  x0 = cadd(b0, d2);
-  x2 = csub(b0, d2);
-  x1 = cadd(b1, d3);
-  x3 = csub(b1, d3);
-}
-
-// In-place unitary 2D FFT of the frame X (nx rows x ny columns, row stride
-// ny + 1 complex) in shared memory: along the rows, then along the columns,
-// each by radix-2 decimation in time (a power-of-two side, lny / lnx its
-// log2) or a direct DFT (lny / lnx = -1).  tx[k] = exp(-2 pi i k / nx),
-// k < nx (same for ty); inverse uses the conjugate twiddles.  All threads of
-// the CTA call it.
-__device__ void fft2_smem(float2* X, int nx, int ny, int lnx, int lny, const float2* tx,
-                          const float2* ty, bool inverse) {
-  const int ld = ny + 1, n = nx * ny;
-  if (lny < 0) {
-    dft_direct_smem(X, nx, ny, true, ty, inverse);
-  } else {
-    // rows: bit reversal, then lny stages.  Consecutive threads take the
-    // same position in consecutive rows: the row stride ny + 1 puts them in
-    // distinct banks, and they share the twiddle (a broadcast)
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int j = lnx >= 0 ? e >> lnx : e / nx, row = e - j * nx;
-      const int p = static_cast<int>(__brev(static_cast<unsigned>(j)) >> (32 - lny));
-      if (lny > 0 && p > j) {
-        const float2 t = X[row * ld + j];
-        X[row * ld + j] = X[row * ld + p];
-        X[row * ld + p] = t;
-      }
-    }
-    __syncthreads();
-    int s = 0;
-    for (; s + 1 < lny; s += 2) {  // stages s and s + 1 in one pass
-      const int h = 1 << s;
-      for (int b = threadIdx.x; b < n / 4; b += blockDim.x) {
-        const int t = lnx >= 0 ? b >> lnx : b / nx, row = b - t * nx;
-        const int j = t & (h - 1), i0 = ((t >> s) << (s + 2)) + j;
-        float2* x = X + row * ld;
-        stage_pair(x[i0], x[i0 + h], x[i0 + 2 * h], x[i0 + 3 * h], ty[j * (ny >> (s + 1))],
-                   ty[j * (ny >> (s + 2))], ty[(j + h) * (ny >> (s + 2))], inverse);
-      }
-      __syncthreads();
-    }
-    if (s < lny) {  // a last single stage
-      const int half = 1 << s, step = ny >> (s + 1);
-      for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
-        const int t = lnx >= 0 ? b >> lnx : b / nx, row = b - t * nx;
-        const int j = t & (half - 1), i1 = ((t >> s) << (s + 1)) + j, i2 = i1 + half;
-        float2 w = ty[j * step];
-        if (inverse) w.y = -w.y;
-        const float2 a = X[row * ld + i1], c = cmul(X[row * ld + i2], w);
-        X[row * ld + i1] = cadd(a, c);
-        X[row * ld + i2] = csub(a, c);
-      }
-      __syncthreads();
-    }
-  }
-  // the unitary scale 1/sqrt(n) is applied by the last column pass as it
-  // stores (the same multiply as a separate pass), else by a pass of its own
-  const float sc = rsqrtf(static_cast<float>(n));
-  bool scaled = false;
-  if (lnx < 0) {
-    dft_direct_smem(X, nx, ny, false, tx, inverse);
-  } else {
-    // columns: bit reversal, then lnx stages
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int i = lny >= 0 ? e >> lny : e / ny, col = e - i * ny;
-      const int p = static_cast<int>(__brev(static_cast<unsigned>(i)) >> (32 - lnx));
-      if (lnx > 0 && p > i) {
-        const float2 t = X[i * ld + col];
-        X[i * ld + col] = X[p * ld + col];
-        X[p * ld + col] = t;
-      }
-    }
-    __syncthreads();
-    int s = 0;
-    for (; s + 1 < lnx; s += 2) {  // stages s and s + 1 in one pass
-      const int h = 1 << s;
-      const float f = (s + 2 == lnx) ? sc : 1.f;  // the last pass scales
-      for (int b = threadIdx.x; b < n / 4; b += blockDim.x) {
-        const int t = lny >= 0 ? b >> lny : b / ny, col = b - t * ny;
-        const int j = t & (h - 1), i0 = ((t >> s) << (s + 2)) + j;
-        float2* p0 = X + i0 * ld + col;
-        float2 x0 = p0[0], x1 = p0[h * ld], x2 = p0[2 * h * ld], x3 = p0[3 * h * ld];
-        stage_pair(x0, x1, x2, x3, tx[j * (nx >> (s + 1))], tx[j * (nx >> (s + 2))],
-                   tx[(j + h) * (nx >> (s + 2))], inverse);
-        if (s + 2 == lnx) {
-          x0 = make_float2(x0.x * f, x0.y * f);
-          x1 = make_float2(x1.x * f, x1.y * f);
-          x2 = make_float2(x2.x * f, x2.y * f);
-          x3 = make_float2(x3.x * f, x3.y * f);
-        }
-        p0[0] = x0;
-        p0[h * ld] = x1;
-        p0[2 * h * ld] = x2;
-        p0[3 * h * ld] = x3;
-      }
-      __syncthreads();
-    }
-    if (s < lnx) {  // a last single stage
-      const int half = 1 << s, step = nx >> (s + 1);
-      for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
-        const int t = lny >= 0 ? b >> lny : b / ny, col = b - t * ny;
-        const int j = t & (half - 1), i1 = ((t >> s) << (s + 1)) + j, i2 = i1 + half;
-        float2 w = tx[j * step];
-        if (inverse) w.y = -w.y;
-        const float2 a = X[i1 * ld + col], c = cmul(X[i2 * ld + col], w);
-        const float2 o1 = cadd(a, c), o2 = csub(a, c);
-        X[i1 * ld + col] = make_float2(o1.x * sc, o1.y * sc);
-        X[i2 * ld + col] = make_float2(o2.x * sc, o2.y * sc);
-      }
-      __syncthreads();
-    }
-    scaled = lnx > 0;
-  }
-  if (!scaled) {
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int row = e / ny, j = e - row * ny;
-      X[row * ld + j].x *= sc;
-      X[row * ld + j].y *= sc;
-    }
-    __syncthreads();
-  }
-}
 
 // g = log2 G consecutive radix-2 decimation-in-time stages s .. s + g - 1 on
 // the G elements x[t] at positions i0 + t h (h = 2^s, i0 = j mod h) of a block
@@ -429,25 +172,13 @@ __device__ void fft2_dit(float2* X, int nx, int ny, int lnx, int lny, const floa
     __syncthreads();
   }
 }
-
-struct Geo {
-  int nx, ny, lnx, lny, n;  // lnx / lny: log2 of a power-of-two side, else -1
-  int L, sxL, syL, lL;      // L = lcm(nx, ny), L / nx, L / ny, log2 L (or -1)
-};
-
-// row, column of pixel e = row * ny + column, and an index modulo nx (ny)
-__device__ __forceinline__ int frow(const Geo& g, int e) { return g.lny >= 0 ? e >> g.lny : e / g.ny; }
-__device__ __forceinline__ int fcol(const Geo& g, int e) {
-  return g.lny >= 0 ? e & (g.ny - 1) : e - (e / g.ny) * g.ny;
-}
-__device__ __forceinline__ int fwrapx(const Geo& g, int v) { return g.lnx >= 0 ? v & (g.nx - 1) : v % g.nx; }
-__device__ __forceinline__ int fwrapy(const Geo& g, int v) { return g.lny >= 0 ? v & (g.ny - 1) : v % g.ny; }
-__device__ __forceinline__ int fwrapL(const Geo& g, int v) { return g.lL >= 0 ? v & (g.L - 1) : v % g.L; }
-
 // out[f] = F2(in[f]) (or F2^H) for frames f; frames are n-vectors in natural
-// row-major order (pixel kx*ny + ky), frame f at in + f*n.
+// row-major order (pixel kx*ny + ky), frame f at in + f*n; its pixel e goes to
+// out[e * es + f * fs] (F2 U is stored sample by sample, so that the sweep reads
+// the r values of a sampled frequency from one or two sectors, not from r).
 __global__ void __launch_bounds__(kFT) fft_frames_kernel(Geo g, const float2* __restrict__ in,
-                                                         float2* __restrict__ out, int inverse,
+                                                         float2* __restrict__ out, size_t es, size_t fs,
+                                                         int inverse,
                                                          const float2* __restrict__ twx,
                                                          const float2* __restrict__ twy) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -465,830 +196,8 @@ __global__ void __launch_bounds__(kFT) fft_frames_kernel(Geo g, const float2* __
   fft2_dit(X, g.nx, g.ny, g.lnx, g.lny, tx, ty, inverse != 0);
   for (int e = threadIdx.x; e < g.n; e += blockDim.x) {
     const int row = e / g.ny, j = e - row * g.ny;
-    out[f * g.n + e] = X[row * (g.ny + 1) + j];
+    out[e * es + f * fs] = X[row * (g.ny + 1) + j];
   }
-}
-
-// ----------------------------------------------------------- the sweep --
-struct FArgs {
-  Geo g;
-  int m, q, r, rho, tau, mode;
-  const float2* y;      // q x m
-  const int* mask;      // q x m
-  const float2* FU;     // r x n (column l = F2 u_l)
-  int* S_idx;           // q x rho
-  float2* S_val;        // q x rho
-  float2* B;            // q x r
-  float2* RES;          // q x m: W b + A s - y (iteration)
-  float2* H;            // q x n: L0 columns A^H (y - A s) (initialisation)
-  const float2* twx;
-  const float2* twy;
-  const float2* twl;    // exp(-2 pi i j / L), j < L = lcm(nx, ny)
-  int* err;
-  float2* vecs;         // q x 3m: y, and the two m-vectors of the sweep, when
-                        // they do not fit shared memory beside the frame
-  float2* Wk;           // q x r x m: W_k = (F2 U)[Omega_k], gathered once per
-                        // frame and sweep (row l of frame k contiguous)
-  float2* AS;           // q x m: A_k s_k of the last sweep's final stage
-  int* asv;             // q: 1 while AS[k] is A_k s_k of the current s_k
-  unsigned long long* prof;  // optional kFProf cycle counters (thread 0 of each CTA)
-};
-
-struct FCarve {
-  size_t X, tx, ty, tl, yv, dv, ev, msk, sp, pq, spo, sv, gv, G, Gi, vec, red, hist, cand, cl, ck, total;
-};
-
-// HardThreshold candidates of the threshold filter (indices and keys; the
-// sort needs one thread per candidate)
-constexpr int kCandCap = 512;
-static_assert(kCandCap <= kFT, "one thread per threshold-filter candidate");
-
-__host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
-
-// Shared-memory carve of the sweep; with vglob the three m-vectors (y, and
-// the sweep's two) live in global memory (FArgs::vecs) and take no space.
-__host__ __device__ inline FCarve fcarve(const Geo& g, int m, int rho, bool vglob = false) {
-  FCarve c;
-  size_t o = 0;
-  const int rh = rho > 0 ? rho : 1;
-  const size_t mv = vglob ? 0 : al16(static_cast<size_t>(m) * 8);
-  c.X = o;    o += al16(static_cast<size_t>(g.nx) * (g.ny + 1) * 8);
-  c.tx = o;   o += al16(static_cast<size_t>(g.nx) * 8);
-  c.ty = o;   o += al16(static_cast<size_t>(g.ny) * 8);
-  c.tl = o;   o += al16(static_cast<size_t>(g.L) * 8);
-  c.yv = o;   o += mv;
-  c.dv = o;   o += mv;
-  c.ev = o;   o += mv;
-  c.msk = o;  o += al16(static_cast<size_t>(m) * 4);
-  c.sp = o;   o += al16(static_cast<size_t>(rh) * 4 + 16);
-  c.pq = o;   o += al16(static_cast<size_t>(rh) * 8);
-  c.spo = o;  o += al16(static_cast<size_t>(rh) * 4);
-  c.sv = o;   o += al16(static_cast<size_t>(rh) * 8);
-  c.gv = o;   o += al16(static_cast<size_t>(rh) * 8);
-  c.G = o;    o += al16(4 * kMaxR * kMaxR * 16);     // G, L, Linv, Ginv (complex FP64)
-  c.vec = o;  o += al16((64 + kMaxR * kMaxR) * 16);   // c, x, scalars, iL; r x r products
-  c.red = o;  o += al16(static_cast<size_t>(kFW) * 2 * kMaxR * 4 + 64);
-  c.hist = o; o += al16(256 * 4 + 64);
-  c.cand = o; o += al16(static_cast<size_t>(2 * rh + 64) * 4);
-  c.cl = o;   o += al16(static_cast<size_t>(kCandCap) * 4);
-  c.ck = o;   o += al16(static_cast<size_t>(kCandCap) * 4);
-  c.total = o;
-  return c;
-}
-
-struct FCtx {
-  Geo g;
-  int m, r, rho, k;
-  float2* X;
-  float2* tx;      // full-period twiddles exp(-2 pi i k / nx), k < nx
-  float2* ty;
-  float2* tl;      // exp(-2 pi i j / L), j < L = lcm(nx, ny)
-  int2* pq;        // sparse DFT: a support pixel's row and column scaled to L
-  int* spo;        // the support before the last HardThreshold
-  float2* yv;
-  float2* dv;
-  float2* ev;
-  int* msk;
-  int* sp;         // support pixels
-  float2* sv;      // support values
-  float2* gv;      // g on the support
-  double2* G;      // r x r (ld kMaxR): G, then scratch
-  double2* Lc;
-  double2* Li;
-  double2* Gi;
-  double2* vec;    // [0,16) c, [16,32) x
-  float* red;
-  int* hist;
-  int* cand;
-  int* cl;         // threshold-filter candidates: pixels
-  unsigned* ck;    // and their keys
-  const float2* FU;
-  float2* Wk;      // this frame's W_k (r x m, row l contiguous)
-  int* err;
-};
-
-__device__ __forceinline__ float2 W_at(const FCtx& C, int i, int l) {
-  return C.Wk[static_cast<size_t>(l) * C.m + i];
-}
-
-// out[i] = (A x)[i] for the sparse frame x with pixels p[e], values v[e]
-// (direct DFT of the nonzeros at the sampled frequencies).  With L =
-// lcm(nx, ny), exp(-2 pi i (kx px / nx + ky py / ny)) is the one table entry
-// j = (kx px L/nx + ky py L/ny) mod L: one look-up (or, along a run of
-// pixels in a row, one complex multiply) and one complex multiply-add per
-// term.
-constexpr int kSdPer = 4;
-__device__ void sparse_dft(const FCtx& C, const int* p, const float2* v, int nnz, float2* out) {
-  const float sc = rsqrtf(static_cast<float>(C.g.n));
-  for (int e = threadIdx.x; e < nnz; e += blockDim.x) {
-    const int pe = p[e];
-    C.pq[e] = make_int2(frow(C.g, pe) * C.g.sxL, fcol(C.g, pe) * C.g.syL);
-  }
-  __syncthreads();
-  // each thread takes kSdPer frequencies at once, so that a term's index and
-  // value (shared-memory broadcasts) serve all of them
-  const int bd = blockDim.x;
-  for (int i0 = threadIdx.x; i0 < C.m; i0 += kSdPer * bd) {
-    int kx[kSdPer], ky[kSdPer];
-    float2 wy[kSdPer], acc[kSdPer];
-#pragma unroll
-    for (int u = 0; u < kSdPer; ++u) {
-      const int i = i0 + u * bd;
-      const int om = i < C.m ? C.msk[i] : 0;
-      kx[u] = frow(C.g, om);
-      ky[u] = fcol(C.g, om);
-      wy[u] = C.tl[fwrapL(C.g, ky[u] * C.g.syL)];  // exp(-2 pi i ky / ny)
-      acc[u] = make_float2(0.f, 0.f);
-    }
-    // a pixel right after the previous one in its row (blob supports; the
-    // pixels are ascending) takes the previous twiddle times exp(-2 pi i ky / ny)
-    float2 w[kSdPer];
-    int2 qp = make_int2(-1, -1);
-    for (int e = 0; e < nnz; ++e) {
-      const int2 q = C.pq[e];
-      const float2 ve = v[e];
-      if (q.x == qp.x && q.y == qp.y + C.g.syL) {  // the same for every lane
-#pragma unroll
-        for (int u = 0; u < kSdPer; ++u) w[u] = cmul(w[u], wy[u]);
-      } else {
-#pragma unroll
-        for (int u = 0; u < kSdPer; ++u) w[u] = C.tl[fwrapL(C.g, kx[u] * q.x + ky[u] * q.y)];
-      }
-      qp = q;
-#pragma unroll
-      for (int u = 0; u < kSdPer; ++u) acc[u] = cfma(w[u], ve, acc[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < kSdPer; ++u) {
-      const int i = i0 + u * bd;
-      if (i < C.m) out[i] = make_float2(acc[u].x * sc, acc[u].y * sc);
-    }
-  }
-}
-
-// rows of W a thread takes at once in the solves and projections
-constexpr int kApPer = 4;
-
-// x = G^{-1} W^H v (W^H v in FP32, block-summed in fixed order; solve FP64);
-// x in C.vec[16 + l] (double2)
-__device__ void fls_solve(const FCtx& C, const float2* v) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = C.r;
-  float2 acc[kMaxR];
-#pragma unroll
-  for (int l = 0; l < kMaxR; ++l) acc[l] = make_float2(0.f, 0.f);
-  // kApPer rows per thread at once (their W loads independent), each sum
-  // still over the thread's rows in increasing order
-  const int bd = blockDim.x;
-  for (int i0 = threadIdx.x; i0 < C.m; i0 += kApPer * bd) {
-    float2 vi[kApPer];
-#pragma unroll
-    for (int u = 0; u < kApPer; ++u) {
-      const int i = i0 + u * bd;
-      vi[u] = i < C.m ? v[i] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int l = 0; l < kMaxR; ++l) {
-      if (l < r) {
-        float2 wv[kApPer];
-#pragma unroll
-        for (int u = 0; u < kApPer; ++u) {
-          const int i = i0 + u * bd;
-          wv[u] = i < C.m ? W_at(C, i, l) : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < kApPer; ++u)
-          if (i0 + u * bd < C.m) acc[l] = ccfma(wv[u], vi[u], acc[l]);
-      }
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < kMaxR; ++l) {
-    if (l >= r) break;
-    const float sx = warp_sumf(acc[l].x), sy = warp_sumf(acc[l].y);
-    if (lane == 0) {
-      C.red[(w * kMaxR + l) * 2] = sx;
-      C.red[(w * kMaxR + l) * 2 + 1] = sy;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < r) {  // the warps' partials in warp order (float32, like the sums)
-    float sx = 0.f, sy = 0.f;
-    for (int ww = 0; ww < kFW; ++ww) {
-      sx += C.red[(ww * kMaxR + threadIdx.x) * 2];
-      sy += C.red[(ww * kMaxR + threadIdx.x) * 2 + 1];
-    }
-    C.vec[threadIdx.x] = make_double2(sx, sy);
-  }
-  __syncthreads();
-  // x = G^{-1} c (FP64): the r x r products in parallel, then each row's sum
-  double2* prod = C.vec + 64;
-  if (threadIdx.x < r * r) {
-    const int a = threadIdx.x / r, b = threadIdx.x - a * r;
-    prod[threadIdx.x] = dcmul(C.Gi[a * kMaxR + b], C.vec[b]);
-  }
-  __syncthreads();
-  if (threadIdx.x < r) {
-    double2 x = make_double2(0, 0);
-    for (int b = 0; b < r; ++b) {
-      x.x += prod[threadIdx.x * r + b].x;
-      x.y += prod[threadIdx.x * r + b].y;
-    }
-    C.vec[16 + threadIdx.x] = x;
-  }
-  __syncthreads();
-}
-
-// v <- v - W x with x from fls_solve (float arithmetic).  A thread takes
-// kApPer rows at once, so that the loads of W for one l are independent.
-__device__ void fapply_Wx(const FCtx& C, float2* v, float sign) {
-  const int bd = blockDim.x;
-  for (int i0 = threadIdx.x; i0 < C.m; i0 += kApPer * bd) {
-    float2 s[kApPer];
-#pragma unroll
-    for (int u = 0; u < kApPer; ++u) {
-      const int i = i0 + u * bd;
-      s[u] = i < C.m ? v[i] : make_float2(0.f, 0.f);
-    }
-    for (int l = 0; l < C.r; ++l) {
-      const double2 xd = C.vec[16 + l];
-      const float2 x = make_float2(sign * static_cast<float>(xd.x), sign * static_cast<float>(xd.y));
-      float2 wv[kApPer];
-#pragma unroll
-      for (int u = 0; u < kApPer; ++u) {
-        const int i = i0 + u * bd;
-        wv[u] = i < C.m ? W_at(C, i, l) : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-      for (int u = 0; u < kApPer; ++u) s[u] = cfma(wv[u], x, s[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < kApPer; ++u) {
-      const int i = i0 + u * bd;
-      if (i < C.m) v[i] = s[u];
-    }
-  }
-  __syncthreads();
-}
-
-__device__ double fnorm2(const FCtx& C, const float2* v) {
-  float acc = 0.f;
-  for (int i = threadIdx.x; i < C.m; i += blockDim.x) acc += cabs2(v[i]);
-  acc = warp_sumf(acc);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) C.red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  float s = 0.f;  // the warps' partials in warp order
-  for (int i = 0; i < kFW; ++i) s += C.red[i];
-  __syncthreads();
-  return s;
-}
-
-// Hermitian Gram G = W^H W (products exact, sums in double-float, stored as
-// FP64), complex Cholesky G = L L^H in FP64 (lane 0, inverse pivots by
-// Newton rsqrt), L^{-1} per lane, G^{-1} = L^{-H} L^{-1}.
-__device__ void fgram_factor(const FCtx& C) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = C.r;
-  // entry t of the lower triangle: (a, b), b <= a; a lane's rows i are
-  // spread over four independent double-float chains
-  for (int t = w; t < r * (r + 1) / 2; t += kFW) {
-    int a = 0, b = t;
-    while (b > a) b -= ++a;
-    // conj(W_ib) W_ia summed in double-float: exact products, ~48-bit sums
-    constexpr int kCh = 4;
-    float xh[kCh], xl[kCh], yh[kCh], yl[kCh];
-#pragma unroll
-    for (int hh = 0; hh < kCh; ++hh) xh[hh] = xl[hh] = yh[hh] = yl[hh] = 0.f;
-    for (int i0 = lane; i0 < C.m; i0 += 32 * kCh) {
-      float2 wa[kCh], wb[kCh];
-#pragma unroll
-      for (int hh = 0; hh < kCh; ++hh) {
-        const int i = i0 + 32 * hh;
-        wa[hh] = i < C.m ? W_at(C, i, a) : make_float2(0.f, 0.f);
-        wb[hh] = i < C.m ? W_at(C, i, b) : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-      for (int hh = 0; hh < kCh; ++hh) {
-        df_fma(xh[hh], xl[hh], wb[hh].x, wa[hh].x);
-        df_fma(xh[hh], xl[hh], wb[hh].y, wa[hh].y);
-        df_fma(yh[hh], yl[hh], wb[hh].x, wa[hh].y);
-        df_fma(yh[hh], yl[hh], -wb[hh].y, wa[hh].x);
-      }
-    }
-#pragma unroll
-    for (int hh = 1; hh < kCh; ++hh) {
-      df_add(xh[0], xl[0], xh[hh], xl[hh]);
-      df_add(yh[0], yl[0], yh[hh], yl[hh]);
-    }
-    const double sx = warp_sum_df(xh[0], xl[0]);
-    const double sy = warp_sum_df(yh[0], yl[0]);
-    if (lane == 0) {
-      C.G[a * kMaxR + b] = make_double2(sx, sy);             // G[a][b] = sum conj(W_b) W_a ... (lower)
-      C.G[b * kMaxR + a] = make_double2(sx, -sy);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double* iL = reinterpret_cast<double*>(C.vec + 32);
-    // G here holds G[a][b] = sum_i conj(W_ib) W_ia = (W^H W)[b][a]; factor the
-    // Hermitian matrix M = W^H W with M[a][b] = conj(G[a][b]), column j by the
-    // lanes i >= j at once (lane j's entry is the pivot)
-    bool ok = true;
-    for (int j = 0; j < r; ++j) {
-      double2 t = make_double2(0.0, 0.0);
-      if (lane >= j && lane < r) {
-        t = make_double2(C.G[lane * kMaxR + j].x, -C.G[lane * kMaxR + j].y);
-        for (int p = 0; p < j; ++p) {
-          const double2 x = C.Lc[lane * kMaxR + p], y = C.Lc[j * kMaxR + p];
-          // t -= L[i][p] * conj(L[j][p])
-          t.x -= x.x * y.x + x.y * y.y;
-          t.y -= x.y * y.x - x.x * y.y;
-        }
-      }
-      const double sj = __shfl_sync(0xffffffffu, t.x, j);
-      if (!(sj > 1e-13 * C.G[j * kMaxR + j].x) || !(sj < 1e300)) {
-        ok = false;
-        break;
-      }
-      const double ij = rsqrt_newton(sj);
-      if (lane == j) {
-        C.Lc[j * kMaxR + j] = make_double2(sj * ij, 0.0);
-        iL[j] = ij;
-      } else if (lane > j && lane < r) {
-        C.Lc[lane * kMaxR + j] = make_double2(t.x * ij, t.y * ij);
-      }
-      __syncwarp();
-    }
-    if (!ok && lane == 0) {
-      report_error(C.err, kErrNotSPD, C.k);
-      for (int i = 0; i < r; ++i) {
-        for (int p = 0; p < r; ++p) C.Lc[i * kMaxR + p] = make_double2(i == p ? 1.0 : 0.0, 0.0);
-        iL[i] = 1.0;
-      }
-    }
-    __syncwarp();
-    if (lane < r) {  // column lane of L^{-1}
-      const int cc = lane;
-      for (int i = 0; i < r; ++i) {
-        double2 t = make_double2(i == cc ? 1.0 : 0.0, 0.0);
-        for (int p = cc; p < i; ++p) {
-          const double2 q = dcmul(C.Lc[i * kMaxR + p], C.Li[p * kMaxR + cc]);
-          t.x -= q.x;
-          t.y -= q.y;
-        }
-        C.Li[i * kMaxR + cc] = (i < cc) ? make_double2(0, 0) : make_double2(t.x * iL[i], t.y * iL[i]);
-      }
-    }
-    __syncwarp();
-    // G^{-1} = L^{-H} L^{-1}: Gi[a][b] = sum_p conj(Li[p][a]) Li[p][b]
-    for (int t = lane; t < r * r; t += 32) {
-      const int a = t / r, b = t - a * r;
-      double2 s = make_double2(0, 0);
-      for (int p = (a > b ? a : b); p < r; ++p) {
-        const double2 q = dccmul(C.Li[p * kMaxR + a], C.Li[p * kMaxR + b]);
-        s.x += q.x;
-        s.y += q.y;
-      }
-      C.Gi[a * kMaxR + b] = s;
-    }
-  }
-  __syncthreads();
-}
-
-// HardThreshold of the frame values X (modulus; ties to the lower pixel
-// index) -> the rho kept pixels and values (support order: by key).
-__device__ void fhard_threshold(const FCtx& C, bool keep_values) {
-  const int n = C.g.n, ld = C.g.ny + 1, rho = C.rho, lane = threadIdx.x & 31;
-  int* info = C.hist + 256;
-  int* sel = C.cand;            // rho entries
-  auto key_of = [&](int e) {
-    return __float_as_uint(cabs2(C.X[frow(C.g, e) * ld + fcol(C.g, e)]));
-  };
-  // Threshold filter (with a current support, after v = s - mu g): the rho
-  // entries of the support have keys >= T0, their smallest key, so the rho
-  // largest keys are all >= T0.  The entries at or above T0 are ranked by
-  // (key descending, pixel ascending), the order of the radix path below,
-  // unless there are more than kCandCap of them.
-  if (keep_values) {
-    if (threadIdx.x < 32) {
-      unsigned mn = 0xffffffffu;
-      for (int e = lane; e < rho; e += 32) mn = min(mn, key_of(C.sp[e]));
-      mn = __reduce_min_sync(0xffffffffu, mn);
-      if (lane == 0) {
-        info[4] = static_cast<int>(mn);
-        info[5] = 0;
-      }
-    }
-    __syncthreads();
-    const unsigned T0 = static_cast<unsigned>(info[4]);
-    for (int e0 = threadIdx.x - lane; e0 < n; e0 += blockDim.x) {
-      const int e = e0 + lane;
-      unsigned key = 0u;
-      bool c = false;
-      if (e < n) {
-        key = key_of(e);
-        c = key >= T0;
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, c);
-      int base = 0;
-      if (lane == 0 && bal) base = atomicAdd(&info[5], __popc(bal));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (c) {
-        const int pos = base + __popc(bal & ((1u << lane) - 1u));
-        if (pos < kCandCap) {
-          C.cl[pos] = e;
-          C.ck[pos] = key;
-        }
-      }
-    }
-    __syncthreads();
-    const int cnt = info[5];
-    if (cnt >= rho && cnt <= kCandCap) {
-      // bitonic sort of the candidates, descending by (key, ~pixel): the
-      // order (key descending, pixel ascending); the 64-bit sort keys take
-      // the place of cl and ck (adjacent, 2 kCandCap words)
-      int P = 1;
-      while (P < cnt) P <<= 1;
-      const int t = threadIdx.x;  // blockDim.x >= kCandCap >= P
-      unsigned long long mine = 0ull;
-      if (t < cnt)
-        mine = (static_cast<unsigned long long>(C.ck[t]) << 32) |
-               static_cast<unsigned long long>(0xffffffffu - static_cast<unsigned>(C.cl[t]));
-      __syncthreads();
-      unsigned long long* K = reinterpret_cast<unsigned long long*>(C.cl);
-      if (t < P) K[t] = mine;
-      __syncthreads();
-      for (int kk = 2; kk <= P; kk <<= 1) {
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-          const int o = t ^ j;
-          if (t < P && o > t) {
-            const unsigned long long x = K[t], y = K[o];
-            if (((t & kk) == 0) ? (x < y) : (x > y)) {
-              K[t] = y;
-              K[o] = x;
-            }
-          }
-          __syncthreads();
-        }
-      }
-      if (t < rho) sel[t] = static_cast<int>(0xffffffffu - static_cast<unsigned>(K[t] & 0xffffffffull));
-      __syncthreads();
-      for (int t = threadIdx.x; t < rho; t += blockDim.x) {  // ascending by pixel
-        const int e = sel[t];
-        int pos = 0;
-        for (int u = 0; u < rho; ++u) pos += sel[u] < e;
-        C.sp[pos] = e;
-        C.sv[pos] = C.X[frow(C.g, e) * ld + fcol(C.g, e)];
-      }
-      __syncthreads();
-      return;
-    }
-    __syncthreads();
-  }
-  unsigned prefix = 0, mask = 0;
-  if (threadIdx.x == 0) info[1] = rho;
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) C.hist[t] = 0;
-    __syncthreads();
-    for (int e0 = threadIdx.x - lane; e0 < n; e0 += blockDim.x) {
-      const int e = e0 + lane;
-      unsigned key = 0u;
-      if (e < n) {
-        const int row = frow(C.g, e), col = fcol(C.g, e);
-        key = __float_as_uint(cabs2(C.X[row * ld + col]));
-      }
-      const bool in = e < n && (key & mask) == prefix;
-      const unsigned digit = in ? ((key >> shift) & 255u) : 256u;
-      const unsigned peers = __match_any_sync(0xffffffffu, digit);
-      if (in && (__ffs(peers) - 1) == lane) atomicAdd(&C.hist[digit], __popc(peers));
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const int need = info[1];
-      int own[8], tot = 0;
-#pragma unroll
-      for (int z = 0; z < 8; ++z) { own[z] = C.hist[255 - 8 * lane - z]; tot += own[z]; }
-      int incl = tot;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const int excl = incl - tot;
-      if (excl < need && incl >= need) {
-        int acc = excl;
-        for (int z = 0; z < 8; ++z) {
-          if (acc + own[z] >= need) {
-            info[0] = 255 - 8 * lane - z;
-            info[1] = need - acc;
-            break;
-          }
-          acc += own[z];
-        }
-      }
-    }
-    __syncthreads();
-    prefix |= static_cast<unsigned>(info[0]) << shift;
-    mask |= 255u << shift;
-  }
-  const unsigned T = prefix;
-  const int need = info[1];
-  int* ties = C.cand + rho + 8; // tie candidates (bounded below)
-  const int tie_cap = 56;
-  if (threadIdx.x == 0) { info[2] = 0; info[3] = 0; }
-  __syncthreads();
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    const int row = frow(C.g, e), col = fcol(C.g, e);
-    const unsigned key = __float_as_uint(cabs2(C.X[row * ld + col]));
-    if (key > T) sel[atomicAdd(&info[3], 1)] = e;
-    else if (key == T) {
-      const int s = atomicAdd(&info[2], 1);
-      if (s < tie_cap) ties[s] = e;
-    }
-  }
-  __syncthreads();
-  const int nt = min(info[2], tie_cap), ngt = info[3];
-  if (info[2] > tie_cap && threadIdx.x == 0) report_error(C.err, kErrNaN, C.k);
-  for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-    const int e = ties[t];
-    int rank = 0;
-    for (int u = 0; u < nt; ++u) rank += ties[u] < e;
-    if (rank < need) sel[ngt + rank] = e;
-  }
-  __syncthreads();
-  // store ascending by pixel (fixed order for every later sum over the support)
-  for (int t = threadIdx.x; t < rho; t += blockDim.x) {
-    const int e = sel[t];
-    int pos = 0;
-    for (int u = 0; u < rho; ++u) pos += sel[u] < e;
-    const int row = frow(C.g, e), col = fcol(C.g, e);
-    C.sp[pos] = e;
-    C.sv[pos] = keep_values ? C.X[row * ld + col] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  const FCarve cv = fcarve(a.g, a.m, a.rho, a.vecs != nullptr);
-  FCtx C;
-  C.g = a.g;
-  C.m = a.m;
-  C.r = a.r;
-  C.rho = a.rho;
-  C.k = blockIdx.x;
-  C.X = reinterpret_cast<float2*>(sm + cv.X);
-  C.tx = reinterpret_cast<float2*>(sm + cv.tx);
-  C.ty = reinterpret_cast<float2*>(sm + cv.ty);
-  C.tl = reinterpret_cast<float2*>(sm + cv.tl);
-  C.pq = reinterpret_cast<int2*>(sm + cv.pq);
-  C.spo = reinterpret_cast<int*>(sm + cv.spo);
-  if (a.vecs) {
-    float2* v = a.vecs + static_cast<size_t>(blockIdx.x) * 3 * a.m;
-    C.yv = v;
-    C.dv = v + a.m;
-    C.ev = v + 2 * static_cast<size_t>(a.m);
-  } else {
-    C.yv = reinterpret_cast<float2*>(sm + cv.yv);
-    C.dv = reinterpret_cast<float2*>(sm + cv.dv);
-    C.ev = reinterpret_cast<float2*>(sm + cv.ev);
-  }
-  C.msk = reinterpret_cast<int*>(sm + cv.msk);
-  C.sp = reinterpret_cast<int*>(sm + cv.sp);
-  C.sv = reinterpret_cast<float2*>(sm + cv.sv);
-  C.gv = reinterpret_cast<float2*>(sm + cv.gv);
-  C.G = reinterpret_cast<double2*>(sm + cv.G);
-  C.Lc = C.G + kMaxR * kMaxR;
-  C.Li = C.G + 2 * kMaxR * kMaxR;
-  C.Gi = C.G + 3 * kMaxR * kMaxR;
-  C.vec = reinterpret_cast<double2*>(sm + cv.vec);
-  C.red = reinterpret_cast<float*>(sm + cv.red);
-  C.hist = reinterpret_cast<int*>(sm + cv.hist);
-  C.cand = reinterpret_cast<int*>(sm + cv.cand);
-  C.cl = reinterpret_cast<int*>(sm + cv.cl);
-  C.ck = reinterpret_cast<unsigned*>(sm + cv.ck);
-  C.FU = a.FU;
-  C.Wk = a.Wk + static_cast<size_t>(blockIdx.x) * a.r * a.m;
-  C.err = a.err;
-  const int k = C.k, m = C.m, r = C.r, rho = C.rho, n = C.g.n, ld = C.g.ny + 1;
-  for (int t = threadIdx.x; t < C.g.nx; t += blockDim.x) C.tx[t] = a.twx[t];
-  for (int t = threadIdx.x; t < C.g.ny; t += blockDim.x) C.ty[t] = a.twy[t];
-  for (int t = threadIdx.x; t < C.g.L; t += blockDim.x) C.tl[t] = a.twl[t];
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    C.yv[i] = a.y[static_cast<size_t>(k) * m + i];
-    C.msk[i] = a.mask[static_cast<size_t>(k) * m + i];
-  }
-  for (int e = threadIdx.x; e < rho; e += blockDim.x) {
-    if (a.mode != kModeInit) {
-      C.sp[e] = a.S_idx[static_cast<size_t>(k) * rho + e];
-      C.sv[e] = a.S_val[static_cast<size_t>(k) * rho + e];
-    } else {
-      C.sp[e] = 0;
-      C.sv[e] = make_float2(0.f, 0.f);
-    }
-  }
-  __syncthreads();
-  // phase cycle counters (profile): thread 0's clock between the CTA's phases
-  // (kept in shared memory: registers are scarce in this kernel)
-  __shared__ unsigned long long pc[kFProf];
-  __shared__ long long tl;
-  if (a.prof && threadIdx.x == 0) {
-    for (int slot = 0; slot < kFProf; ++slot) pc[slot] = 0ull;
-    tl = clock64();
-  }
-  auto mark = [&](int slot) {
-    if (a.prof && threadIdx.x == 0) {
-      const long long t = clock64();
-      pc[slot] += static_cast<unsigned long long>(t - tl);
-      tl = t;
-    }
-  };
-  // A_k s_k of this s_k from the previous sweep's final stage (the same
-  // sparse DFT of the same support, pixels and values in the same order)
-  const bool as_ok = a.asv[k] != 0;
-  const bool project = (a.mode != kModeInit);
-  if (project) {
-    // W_k = (F2 U)[Omega_k] into the frame's contiguous copy (read
-    // coalesced by the Gram, the solves and the projections)
-    constexpr int kG = 8;  // gathers issued together per thread
-    for (int t0 = threadIdx.x; t0 < r * m; t0 += kG * blockDim.x) {
-      float2 g[kG];
-#pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int t = t0 + u * blockDim.x;
-        if (t < r * m) {
-          const int l = t / m, i = t - l * m;
-          g[u] = __ldg(C.FU + static_cast<size_t>(l) * n + C.msk[i]);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kG; ++u) {
-        const int t = t0 + u * blockDim.x;
-        if (t < r * m) C.Wk[t] = g[u];
-      }
-    }
-    __syncthreads();
-    fgram_factor(C);
-  }
-  mark(0);
-  const int tau = (a.mode == kModeLS || rho == 0) ? 0 : a.tau;
-  // After a sweep whose HardThreshold kept the support, s_new = s - mu g_G on
-  // it, so the next u = P_perp(A s_new - y) is u - mu P_perp A g_G, both of
-  // which the sweep still holds (dv, ev): no sparse DFT or projection then.
-  bool kept = false;
-  float mu_prev = 0.f;
-  for (int it = 0; it < tau; ++it) {
-    const bool zero_start = (a.mode == kModeInit && it == 0);
-    // u = P_perp (A s - y)
-    if (zero_start) {
-      for (int i = threadIdx.x; i < m; i += blockDim.x) C.dv[i] = make_float2(-C.yv[i].x, -C.yv[i].y);
-      __syncthreads();
-    } else if (kept) {
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const float2 d = C.dv[i], e = C.ev[i];
-        C.dv[i] = make_float2(fmaf(-mu_prev, e.x, d.x), fmaf(-mu_prev, e.y, d.y));
-      }
-      __syncthreads();
-      mark(2);
-    } else {
-      if (it == 0 && as_ok) {
-        for (int i = threadIdx.x; i < m; i += blockDim.x) C.dv[i] = a.AS[static_cast<size_t>(k) * m + i];
-      } else {
-        sparse_dft(C, C.sp, C.sv, rho, C.dv);
-      }
-      __syncthreads();
-      for (int i = threadIdx.x; i < m; i += blockDim.x) C.dv[i] = csub(C.dv[i], C.yv[i]);
-      __syncthreads();
-      mark(1);
-      if (project) {
-        fls_solve(C, C.dv);
-        mark(6);
-        fapply_Wx(C, C.dv, -1.f);
-        mark(7);
-      }
-    }
-    // g = A^H u: zero-filled frame, inverse 2D FFT
-    for (int e = threadIdx.x; e < C.g.nx * ld; e += blockDim.x) C.X[e] = make_float2(0.f, 0.f);
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      const int om = C.msk[i];
-      C.X[(frow(C.g, om)) * ld + (fcol(C.g, om))] = C.dv[i];
-    }
-    __syncthreads();
-    fft2_smem(C.X, C.g.nx, C.g.ny, C.g.lnx, C.g.lny, C.tx, C.ty, true);
-    mark(3);
-    if (zero_start) {
-      fhard_threshold(C, false);  // support of the zero start: the rho largest |g|
-    }
-    // g on the support, ||g_G||^2, A g_G
-    __syncthreads();
-    mark(4);
-    for (int e = threadIdx.x; e < rho; e += blockDim.x) {
-      const int p = C.sp[e];
-      C.gv[e] = C.X[(frow(C.g, p)) * ld + (fcol(C.g, p))];
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {  // ||g_G||^2: lanes over the support, a fixed butterfly
-      float s = 0.f;
-      for (int e = threadIdx.x; e < rho; e += 32) s += cabs2(C.gv[e]);
-      s = warp_sumf(s);
-      if (threadIdx.x == 0) C.vec[48] = make_double2(s, 0.0);
-    }
-    __syncthreads();
-    mark(2);
-    sparse_dft(C, C.sp, C.gv, rho, C.ev);
-    __syncthreads();
-    mark(1);
-    if (project) {
-      fls_solve(C, C.ev);
-      mark(6);
-      fapply_Wx(C, C.ev, -1.f);
-      mark(7);
-    }
-    const double num = C.vec[48].x;
-    const double den = fnorm2(C, C.ev);
-    mark(2);
-    if (!(den > 0.0)) break;
-    double mu = num / den;
-    if (!isfinite(mu)) {
-      if (threadIdx.x == 0) report_error(a.err, kErrNaN, k);
-      mu = 0.0;
-    }
-    const float muf = static_cast<float>(mu);
-    // v = s - mu g in the frame
-    for (int e = threadIdx.x; e < C.g.nx * ld; e += blockDim.x) {
-      C.X[e].x *= -muf;
-      C.X[e].y *= -muf;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < rho; e += blockDim.x) {
-      const int p = C.sp[e];
-      float2& x = C.X[(frow(C.g, p)) * ld + (fcol(C.g, p))];
-      x = cadd(x, C.sv[e]);
-    }
-    __syncthreads();
-    mark(3);
-    for (int e = threadIdx.x; e < rho; e += blockDim.x) C.spo[e] = C.sp[e];
-    __syncthreads();
-    fhard_threshold(C, true);
-    int same = 1;
-    for (int e = threadIdx.x; e < rho; e += blockDim.x) same &= C.spo[e] == C.sp[e];
-    kept = __syncthreads_and(same) != 0;
-    mu_prev = muf;
-    mark(4);
-  }
-  // ---- final stage ----
-  const bool as_kept = (tau == 0 && as_ok);  // s unchanged by this sweep
-  if (as_kept) {
-    for (int i = threadIdx.x; i < m; i += blockDim.x) C.dv[i] = a.AS[static_cast<size_t>(k) * m + i];
-  } else {
-    sparse_dft(C, C.sp, C.sv, rho, C.dv);  // A s
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {  // y - A s; A s kept for the next sweep
-    const float2 as = C.dv[i];
-    if (!as_kept) a.AS[static_cast<size_t>(k) * m + i] = as;
-    C.dv[i] = csub(C.yv[i], as);
-  }
-  if (threadIdx.x == 0) a.asv[k] = 1;
-  __syncthreads();
-  if (a.mode == kModeInit) {
-    for (int e = threadIdx.x; e < C.g.nx * ld; e += blockDim.x) C.X[e] = make_float2(0.f, 0.f);
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      const int om = C.msk[i];
-      C.X[(frow(C.g, om)) * ld + (fcol(C.g, om))] = C.dv[i];
-    }
-    __syncthreads();
-    fft2_smem(C.X, C.g.nx, C.g.ny, C.g.lnx, C.g.lny, C.tx, C.ty, true);
-    float2* Hk = a.H + static_cast<size_t>(k) * n;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) Hk[e] = C.X[(frow(C.g, e)) * ld + (fcol(C.g, e))];
-  } else {
-    fls_solve(C, C.dv);  // b = G^{-1} W^H (y - A s)
-    if (threadIdx.x < r) {
-      const double2 b = C.vec[16 + threadIdx.x];
-      a.B[static_cast<size_t>(k) * r + threadIdx.x] = make_float2(static_cast<float>(b.x), static_cast<float>(b.y));
-    }
-    if (a.mode == kModeIter) {
-      // res = W b - (y - A s)
-      for (int i = threadIdx.x; i < m; i += blockDim.x) C.ev[i] = make_float2(-C.dv[i].x, -C.dv[i].y);
-      __syncthreads();
-      fapply_Wx(C, C.ev, 1.f);
-      for (int i = threadIdx.x; i < m; i += blockDim.x) a.RES[static_cast<size_t>(k) * m + i] = C.ev[i];
-    }
-  }
-  if (a.mode != kModeLS) {
-    // S_k ascending by pixel
-    for (int e = threadIdx.x; e < rho; e += blockDim.x) {
-      const int p = C.sp[e];
-      int pos = 0;
-      for (int f = 0; f < rho; ++f) pos += C.sp[f] < p;
-      a.S_idx[static_cast<size_t>(k) * rho + pos] = p;
-      a.S_val[static_cast<size_t>(k) * rho + pos] = C.sv[e];
-    }
-  }
-  mark(5);
-  if (a.prof && threadIdx.x == 0)
-    for (int slot = 0; slot < kFProf; ++slot) atomicAdd(a.prof + slot, pc[slot]);
 }
 
 // K[l][w] = sum over the (k, i) with mask_k[i] = w of res_k[i] conj(b_k[l]).
@@ -1819,10 +728,12 @@ struct FourierSolver {
   double* eta = nullptr;
   double* scal = nullptr;
   float2* vecs = nullptr;  // the sweep's m-vectors in global memory (large m)
-  float2* Wk = nullptr;    // q x r x m gathered W_k of the sweep
-  float2* AS = nullptr;    // q x m: A_k s_k from the last sweep's final stage
+  float2* Wk = nullptr;    // q x r x m: the sweep's W_k and Q_k (not when in shared memory)
+  float2* AS = nullptr;    // q x m: A_k s_k - y_k from the last sweep's final stage
   int* asv = nullptr;      // q flags: AS[k] matches the current s_k
   unsigned long long* prof = nullptr;  // kFProf sweep cycle counters (profiling)
+  void* sweep = nullptr;   // fsweep_kernel of the rank width
+  int tb = 0, qmode = 0;   // its table's columns and Q_k's place (FArgs)
   size_t smem = 0;
 };
 
@@ -1830,10 +741,12 @@ static size_t fft_smem(const Geo& g) {
   return al16(static_cast<size_t>(g.nx) * (g.ny + 1) * 8) + static_cast<size_t>(g.nx + g.ny) * 8;
 }
 
+// by_sample: out is n x nframes (frame f at out[e * nframes + f])
 static cudaError_t fft_frames(FourierSolver* F, const float2* in, float2* out, int nframes,
-                              bool inverse) {
-  fft_frames_kernel<<<nframes, kFT, fft_smem(F->g), F->s>>>(F->g, in, out, inverse ? 1 : 0, F->twx,
-                                                             F->twy);
+                              bool inverse, bool by_sample) {
+  const size_t es = by_sample ? nframes : 1, fs = by_sample ? 1 : F->g.n;
+  fft_frames_kernel<<<nframes, kFT, fft_smem(F->g), F->s>>>(F->g, in, out, es, fs, inverse ? 1 : 0,
+                                                             F->twx, F->twy);
   return cudaGetLastError();
 }
 
@@ -1864,6 +777,8 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     F->g.sxL = F->g.L / nx;
     F->g.syL = F->g.L / ny;
     F->g.lL = ilog2(F->g.L);
+    const double span = static_cast<double>(std::max(nx, ny)) * F->g.L * F->g.L;
+    F->g.magic = span < 4294967296.0 ? static_cast<unsigned>((0x100000000ull + F->g.L - 1) / F->g.L) : 0u;
   }
   F->m = m;
   F->q = q;
@@ -1878,7 +793,6 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
   F->s = s;
   const int n = F->g.n;
   F->nblk = std::max(1, std::min(152, (n + 63) / 64));
-  F->smem = fcarve(F->g, m, rho).total;
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   {  // the fused Cholesky-QR2 needs all its blocks resident at once
@@ -1890,17 +804,45 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     F->coop = coop != 0 && per_sm * nsm >= F->nblk;
   }
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // the m-vectors go to global memory when they do not fit beside the frame
-  // (the sweep also holds kFStaticSmem bytes of static shared memory)
+  // Shared memory of the sweep: what lets as many frames run at once as its
+  // threads and the frames there are allow, else one frame's limit.  First the
+  // sparse DFT's table (every column a support can have), then Q_k; the m-vectors
+  // go to global memory when less than four columns of it fit beside them.
+  // (The sweep also holds kFStaticSmem bytes of static shared memory.)
   const size_t room = static_cast<size_t>(optin) - kFStaticSmem;
-  const bool vglob = F->smem > room;
-  if (vglob) F->smem = fcarve(F->g, m, rho, true).total;
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int ctas = std::max(1, std::min(kFT / fsweep_threads(n), (q + nsm - 1) / std::max(1, nsm)));
+  const size_t share = ctas == 1 ? room : (room + 1024) / ctas - 1024 - kFStaticSmem;
+  const int want = m >= 2 * nx ? std::min(std::max(1, rho), ny) : 0;
+  bool vglob = false;
+  auto total = [&](bool vg, int tb, bool qs) { return fcarve(F->g, m, r, rho, vg, tb, qs).total; };
+  auto plan = [&](size_t limit, int least) {  // the most that fits, or false
+    for (int vg = 0; vg < 2; ++vg) {
+      int tb = want;
+      while (tb > least && total(vg, tb, false) > limit) --tb;
+      if (total(vg, tb, false) > limit) continue;
+      vglob = vg != 0;
+      F->tb = tb;
+      const size_t frame = static_cast<size_t>(nx) * (ny + 1);
+      F->qmode = tb == want && total(vg, tb, true) <= limit ? 1 : static_cast<size_t>(r) * m <= frame ? 2 : 0;
+      F->smem = total(vg, tb, F->qmode == 1);
+      return true;
+    }
+    return false;
+  };
+  if (!plan(share, std::min(want, 4)) && !plan(room, std::min(want, 4))) F->smem = room + 1;
   if (F->smem > room || fft_smem(F->g) > static_cast<size_t>(optin)) {
     *msg = "frame too large for one CTA's shared memory (n <= 16384 fits)";
     delete F;
     return nullptr;
   }
-  cudaFuncSetAttribute(fsweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  switch (r <= 2 ? 2 : r <= 4 ? 4 : r <= 6 ? 6 : r <= 8 ? 8 : r <= 12 ? 12 : 16) {
+#define LRS_CASE(R) case R: F->sweep = fsweep_kernel_r##R(F->g.lnx >= 0 && F->g.lny >= 0); break;
+    LRS_FSWEEP_R(LRS_CASE)
+#undef LRS_CASE
+  }
+  cudaFuncSetAttribute(F->sweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        smem_optin_limit() - static_cast<int>(kFStaticSmem));
   cudaFuncSetAttribute(fft_frames_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        smem_optin_limit());
@@ -1930,13 +872,13 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
             cudaMallocAsync(reinterpret_cast<void**>(&F->rfac), sizeof(double2) * 2 * rr, F->s) == cudaSuccess &&
             cudaMallocAsync(reinterpret_cast<void**>(&F->eta), sizeof(double), F->s) == cudaSuccess &&
             cudaMallocAsync(reinterpret_cast<void**>(&F->scal), sizeof(double) * 4, F->s) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&F->Wk),
-                            sizeof(float2) * static_cast<size_t>(r) * m * q, F->s) == cudaSuccess &&
+            (F->qmode == 1 || cudaMallocAsync(reinterpret_cast<void**>(&F->Wk),
+                                       sizeof(float2) * static_cast<size_t>(r) * m * q, F->s) == cudaSuccess) &&
             cudaMallocAsync(reinterpret_cast<void**>(&F->AS),
                             sizeof(float2) * static_cast<size_t>(m) * q, F->s) == cudaSuccess &&
             cudaMallocAsync(reinterpret_cast<void**>(&F->asv), sizeof(int) * q, F->s) == cudaSuccess &&
             (!vglob || cudaMallocAsync(reinterpret_cast<void**>(&F->vecs),
-                                       sizeof(float2) * 3 * static_cast<size_t>(m) * q, F->s) == cudaSuccess);
+                                       sizeof(float2) * 2 * static_cast<size_t>(m) * q, F->s) == cudaSuccess);
   if (!ok) {
     *msg = "device allocation failed";
     return F;  // caller frees
@@ -2051,8 +993,10 @@ static cudaError_t launch_fsweep(FourierSolver* F, int mode, int tau) {
   a.AS = F->AS;
   a.asv = F->asv;
   a.prof = F->prof;
-  fsweep_kernel<<<F->q, kFT, F->smem, F->s>>>(a);
-  return cudaGetLastError();
+  a.tb = F->tb;
+  a.qmode = F->qmode;
+  void* args[] = {&a};
+  return cudaLaunchKernel(F->sweep, dim3(F->q), dim3(fsweep_threads(F->g.n)), args, F->smem, F->s);
 }
 
 // complex Cholesky-QR2 of Zin (r x n column-major) into Uout
@@ -2174,7 +1118,7 @@ int fourier_init(FourierSolver* F, std::string* msg) {
                   static_cast<void*>(Pp), static_cast<void*>(rpart)})
     if (p) cudaFreeAsync(p, F->s);
   // b_k = (A_k U0)^+ (y_k - A_k s_k)
-  if (e == cudaSuccess) e = fft_frames(F, F->U, F->FU, r, false);
+  if (e == cudaSuccess) e = fft_frames(F, F->U, F->FU, r, false, true);
   if (e == cudaSuccess) e = launch_fsweep(F, kModeLS, 0);
   if (e != cudaSuccess) {
     *msg = cudaGetErrorString(e);
@@ -2192,11 +1136,11 @@ int fourier_iterate(FourierSolver* F, int iters, std::string* msg, cudaEvent_t* 
   for (int i = 0; i < iters; ++i) {
     cudaEvent_t* ev = evs ? evs + 4 * static_cast<size_t>(i) : nullptr;
     if (ev) cudaEventRecord(ev[0], F->s);
-    cudaError_t e = fft_frames(F, F->U, F->FU, r, false);            // FU = F2 U
+    cudaError_t e = fft_frames(F, F->U, F->FU, r, false, true);            // FU = F2 U
     if (e == cudaSuccess) e = launch_fsweep(F, kModeIter, F->tau);   // per-frame work
     if (ev) cudaEventRecord(ev[1], F->s);
     kspace_kernel<<<(n + 7) / 8, 256, 0, F->s>>>(n, F->m, r, F->iptr, F->ilist, F->RES, F->B, F->K);
-    if (e == cudaSuccess) e = fft_frames(F, F->K, F->grad, r, true);  // grad = F2^H K
+    if (e == cudaSuccess) e = fft_frames(F, F->K, F->grad, r, true, false);  // grad = F2^H K
     if (e == cudaSuccess && F->t == 0) {
       cgram_part_kernel<<<F->nblk, 256, 0, F->s>>>(n, r, F->grad, nullptr, nullptr, nullptr, F->part);
       ceta_kernel<<<1, 32, 0, F->s>>>(r, F->nblk, F->part, F->c_eta, F->eta);

@@ -1,0 +1,282 @@
+// Shared by the DFT operator's kernels: complex and double-float arithmetic,
+// the frame geometry and the 2D FFT of a frame in shared memory.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "lrs_dev.cuh"
+#include "lrs_internal.h"
+
+namespace lrs {
+namespace fourier {
+
+constexpr int kFT = 512;   // threads of the frame kernels (the sweep: fsweep_threads)
+// sweep profile slots: set-up and Gram, sparse DFTs, norms and vector
+// updates, 2D FFTs with the frame's fills, HardThreshold, final stage,
+// projections' Q^H v, projections' v - Q c
+constexpr int kFProf = 8;
+// static shared memory of the sweep (its profile counters), an upper bound
+constexpr size_t kFStaticSmem = 256;
+constexpr int kMaxR = 16;
+
+// ------------------------------------------------------------ complex --
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
+// acc += a * b
+__device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 acc) {
+  acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
+  acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
+  return acc;
+}
+// acc += conj(a) * b
+__device__ __forceinline__ float2 ccfma(float2 a, float2 b, float2 acc) {
+  acc.x = fmaf(a.x, b.x, fmaf(a.y, b.y, acc.x));
+  acc.y = fmaf(a.x, b.y, fmaf(-a.y, b.x, acc.y));
+  return acc;
+}
+__device__ __forceinline__ double2 dcmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 dccmul(double2 a, double2 b) {  // conj(a) * b
+  return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
+}
+__device__ __forceinline__ float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
+
+// Double-float accumulation (a value carried as hi + lo, two float32 words:
+// about 48 bits of significand on the FP32 units, whose dependent operations
+// are far cheaper than FP64's on this part).  df_fma: (hi, lo) += a * b with
+// the product's rounding error from an fma and the sum's from Knuth's
+// two-sum.  df_add: (hi, lo) += (bh, bl).
+__device__ __forceinline__ void df_fma(float& hi, float& lo, float a, float b) {
+  const float p = a * b;
+  const float pe = fmaf(a, b, -p);
+  const float s = hi + p;
+  const float bb = s - hi;
+  const float se = (hi - (s - bb)) + (p - bb);
+  hi = s;
+  lo += se + pe;
+}
+__device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl) {
+  const float s = hi + bh;
+  const float bb = s - hi;
+  const float se = (hi - (s - bb)) + (bh - bb);
+  hi = s;
+  lo += se + bl;
+}
+// warp sum of double-float values (xor butterfly: every lane ends with the
+// same value, the pairs added in a fixed order)
+__device__ __forceinline__ double warp_sum_df(float hi, float lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
+    const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
+    df_add(hi, lo, oh, ol);
+  }
+  return static_cast<double>(hi) + static_cast<double>(lo);
+}
+
+__device__ __forceinline__ float warp_sumf(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// ------------------------------------------------------------ 2D FFT --
+// Sides that are not powers of two take a direct DFT (frames of at most
+// kDirectPer * blockDim.x pixels): each thread keeps its outputs in
+// registers until every thread has read the frame.
+constexpr int kDirectPer = 8;
+
+__device__ inline void dft_direct_smem(float2* X, int nx, int ny, bool rows, const float2* tw,
+                                bool inverse) {
+  const int ld = ny + 1, n = nx * ny, len = rows ? ny : nx;
+  float2 acc[kDirectPer];
+#pragma unroll
+  for (int u = 0; u < kDirectPer; ++u) {
+    const int e = threadIdx.x + u * blockDim.x;
+    float2 s = make_float2(0.f, 0.f);
+    if (e < n) {
+      const int row = e / ny, col = e - row * ny;
+      const int j = rows ? col : row;  // output frequency along the transformed side
+      int idx = 0;                     // j * k mod len
+      for (int k = 0; k < len; ++k) {
+        float2 w = tw[idx];
+        if (inverse) w.y = -w.y;
+        s = cfma(rows ? X[row * ld + k] : X[k * ld + col], w, s);
+        idx += j;
+        if (idx >= len) idx -= len;
+      }
+    }
+    acc[u] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kDirectPer; ++u) {
+    const int e = threadIdx.x + u * blockDim.x;
+    if (e < n) {
+      const int row = e / ny, col = e - row * ny;
+      X[row * ld + col] = acc[u];
+    }
+  }
+  __syncthreads();
+}
+
+// Two radix-2 decimation-in-time stages s and s + 1 on the quad x0, x1, x2,
+// x3 at offsets 0, h, 2h, 3h (h = 2^s) of a block of 4h: stage s pairs
+// (x0, x1) and (x2, x3) with twiddle w1, stage s + 1 pairs (x0, x2) with w2a
+// and (x1, x3) with w2b.  Every element gets the operations of the two
+// stages run one after the other, in the same order, so the result is that
+// of two single-stage passes, with one shared-memory round trip instead of two.
+__device__ __forceinline__ void stage_pair(float2& x0, float2& x1, float2& x2, float2& x3,
+                                           float2 w1, float2 w2a, float2 w2b, bool inverse) {
+  if (inverse) {
+    w1.y = -w1.y;
+    w2a.y = -w2a.y;
+    w2b.y = -w2b.y;
+  }
+  const float2 a0 = x0, a2 = x2;
+  const float2 c1 = cmul(x1, w1), c3 = cmul(x3, w1);
+  const float2 b0 = cadd(a0, c1), b1 = csub(a0, c1), b2 = cadd(a2, c3), b3 = csub(a2, c3);
+  const float2 d2 = cmul(b2, w2a), d3 = cmul(b3, w2b);
+  x0 = cadd(b0, d2);
+  x2 = csub(b0, d2);
+  x1 = cadd(b1, d3);
+  x3 = csub(b1, d3);
+}
+
+struct Geo {
+  int nx, ny, lnx, lny, n;  // lnx / lny: log2 of a power-of-two side, else -1
+  int L, sxL, syL, lL;      // L = lcm(nx, ny), L / nx, L / ny, log2 L (or -1)
+  unsigned magic;           // ceil(2^32 / L) when v mod L may use it (below), else 0
+};
+
+// row, column of pixel e = row * ny + column, and an index modulo nx (ny)
+__device__ __forceinline__ int frow(const Geo& g, int e) { return g.lny >= 0 ? e >> g.lny : e / g.ny; }
+__device__ __forceinline__ int fcol(const Geo& g, int e) {
+  return g.lny >= 0 ? e & (g.ny - 1) : e - (e / g.ny) * g.ny;
+}
+__device__ __forceinline__ int fwrapx(const Geo& g, int v) { return g.lnx >= 0 ? v & (g.nx - 1) : v % g.nx; }
+__device__ __forceinline__ int fwrapy(const Geo& g, int v) { return g.lny >= 0 ? v & (g.ny - 1) : v % g.ny; }
+// v mod L, 0 <= v < max(nx, ny) L.  floor(v / L) = (v magic) >> 32 while
+// v (magic L - 2^32) < 2^32, which v L < 2^32 ensures; the host sets magic
+// only when max(nx, ny) L^2 < 2^32 (an integer division costs about 20
+// instructions, and the sparse DFTs take one per term).
+__device__ __forceinline__ int fwrapL(const Geo& g, int v) {
+  if (g.lL >= 0) return v & (g.L - 1);
+  if (g.magic) return v - static_cast<int>(__umulhi(static_cast<unsigned>(v), g.magic)) * g.L;
+  return v % g.L;
+}
+// where pixel or frequency e of a frame goes before fft2_smem
+__device__ __forceinline__ int frev(const Geo& g, int e) {
+  int x = frow(g, e), y = fcol(g, e);
+  if (g.lnx > 0) x = static_cast<int>(__brev(static_cast<unsigned>(x)) >> (32 - g.lnx));
+  if (g.lny > 0) y = static_cast<int>(__brev(static_cast<unsigned>(y)) >> (32 - g.lny));
+  return x * (g.ny + 1) + y;
+}
+
+// In-place unitary 2D FFT of the frame X (nx rows x ny columns, row stride
+// ny + 1 complex) in shared memory: along the rows, then along the columns,
+// each by radix-2 decimation in time (a power-of-two side, lny / lnx its
+// log2) or a direct DFT (lny / lnx = -1).  The input lies bit-reversed along
+// the power-of-two sides (frev: the sweep scatters its samples there, which
+// saves the two reversal passes); the output is in natural order.  tx[k] = exp(-2 pi i k / nx),
+// k < nx (same for ty); inverse uses the conjugate twiddles.  All threads of
+// the CTA call it.
+__device__ inline void fft2_smem(float2* X, int nx, int ny, int lnx, int lny, const float2* tx,
+                          const float2* ty, bool inverse) {
+  const int ld = ny + 1, n = nx * ny;
+  if (lny < 0) {
+    dft_direct_smem(X, nx, ny, true, ty, inverse);
+  } else {
+    // consecutive threads take the same position in consecutive rows: the row
+    // stride ny + 1 puts them in distinct banks, and they share the twiddle (a
+    // broadcast)
+    int s = 0;
+    for (; s + 1 < lny; s += 2) {  // stages s and s + 1 in one pass
+      const int h = 1 << s;
+      for (int b = threadIdx.x; b < n / 4; b += blockDim.x) {
+        const int t = lnx >= 0 ? b >> lnx : b / nx, row = b - t * nx;
+        const int j = t & (h - 1), i0 = ((t >> s) << (s + 2)) + j;
+        float2* x = X + row * ld;
+        stage_pair(x[i0], x[i0 + h], x[i0 + 2 * h], x[i0 + 3 * h], ty[j * (ny >> (s + 1))],
+                   ty[j * (ny >> (s + 2))], ty[(j + h) * (ny >> (s + 2))], inverse);
+      }
+      __syncthreads();
+    }
+    if (s < lny) {  // a last single stage
+      const int half = 1 << s, step = ny >> (s + 1);
+      for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
+        const int t = lnx >= 0 ? b >> lnx : b / nx, row = b - t * nx;
+        const int j = t & (half - 1), i1 = ((t >> s) << (s + 1)) + j, i2 = i1 + half;
+        float2 w = ty[j * step];
+        if (inverse) w.y = -w.y;
+        const float2 a = X[row * ld + i1], c = cmul(X[row * ld + i2], w);
+        X[row * ld + i1] = cadd(a, c);
+        X[row * ld + i2] = csub(a, c);
+      }
+      __syncthreads();
+    }
+  }
+  // the unitary scale 1/sqrt(n) is applied by the last column pass as it
+  // stores (the same multiply as a separate pass), else by a pass of its own
+  const float sc = rsqrtf(static_cast<float>(n));
+  bool scaled = false;
+  if (lnx < 0) {
+    dft_direct_smem(X, nx, ny, false, tx, inverse);
+  } else {
+    int s = 0;
+    for (; s + 1 < lnx; s += 2) {  // stages s and s + 1 in one pass
+      const int h = 1 << s;
+      const float f = (s + 2 == lnx) ? sc : 1.f;  // the last pass scales
+      for (int b = threadIdx.x; b < n / 4; b += blockDim.x) {
+        const int t = lny >= 0 ? b >> lny : b / ny, col = b - t * ny;
+        const int j = t & (h - 1), i0 = ((t >> s) << (s + 2)) + j;
+        float2* p0 = X + i0 * ld + col;
+        float2 x0 = p0[0], x1 = p0[h * ld], x2 = p0[2 * h * ld], x3 = p0[3 * h * ld];
+        stage_pair(x0, x1, x2, x3, tx[j * (nx >> (s + 1))], tx[j * (nx >> (s + 2))],
+                   tx[(j + h) * (nx >> (s + 2))], inverse);
+        if (s + 2 == lnx) {
+          x0 = make_float2(x0.x * f, x0.y * f);
+          x1 = make_float2(x1.x * f, x1.y * f);
+          x2 = make_float2(x2.x * f, x2.y * f);
+          x3 = make_float2(x3.x * f, x3.y * f);
+        }
+        p0[0] = x0;
+        p0[h * ld] = x1;
+        p0[2 * h * ld] = x2;
+        p0[3 * h * ld] = x3;
+      }
+      __syncthreads();
+    }
+    if (s < lnx) {  // a last single stage
+      const int half = 1 << s, step = nx >> (s + 1);
+      for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
+        const int t = lny >= 0 ? b >> lny : b / ny, col = b - t * ny;
+        const int j = t & (half - 1), i1 = ((t >> s) << (s + 1)) + j, i2 = i1 + half;
+        float2 w = tx[j * step];
+        if (inverse) w.y = -w.y;
+        const float2 a = X[i1 * ld + col], c = cmul(X[i2 * ld + col], w);
+        const float2 o1 = cadd(a, c), o2 = csub(a, c);
+        X[i1 * ld + col] = make_float2(o1.x * sc, o1.y * sc);
+        X[i2 * ld + col] = make_float2(o2.x * sc, o2.y * sc);
+      }
+      __syncthreads();
+    }
+    scaled = lnx > 0;
+  }
+  if (!scaled) {
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+      const int row = e / ny, j = e - row * ny;
+      X[row * ld + j].x *= sc;
+      X[row * ld + j].y *= sc;
+    }
+    __syncthreads();
+  }
+}
+
+}  // namespace fourier
+}  // namespace lrs

@@ -36,12 +36,6 @@ struct QrArgs {
   int* err;
 };
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float z = s - a;
-  e = (a - (s - z)) + (b - z);
-}
-
 // One warp: FP32 Cholesky of the r x r matrix G (dev: of G = I + E, in
 // deviations), lane i <-> row i, and its inverse, lane c <-> column c:
 // Rinv[c * 16 + i] = (L^{-1})(i, c), the entry (c, i) of R^{-1} = L^{-T}

@@ -385,67 +385,6 @@ __device__ __forceinline__ float stream_elem(const StreamProblem& pr, int k, int
 }
 
 // ------------------------------------------------------------- column steps --
-// double-float: a value carried as the unevaluated sum hi + lo of two floats
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float z = s - a;
-  e = (a - (s - z)) + (b - z);
-}
-struct df {
-  float h, l;
-};
-__device__ __forceinline__ df df_norm(float s, float e) {
-  df r;
-  r.h = s + e;
-  r.l = e - (r.h - s);
-  return r;
-}
-__device__ __forceinline__ df df_make(double x) {
-  df r;
-  r.h = static_cast<float>(x);
-  r.l = static_cast<float>(x - static_cast<double>(r.h));
-  return r;
-}
-__device__ __forceinline__ df df_mul(df a, df b) {
-  const float p = a.h * b.h;
-  return df_norm(p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h));
-}
-__device__ __forceinline__ df df_sub(df a, df b) {
-  float s, e;
-  two_sum(a.h, -b.h, s, e);
-  return df_norm(s, e + (a.l - b.l));
-}
-__device__ __forceinline__ df df_shfl(df a, int src) {
-  return df{__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src)};
-}
-// 1 / sqrt(a): float estimate and one Newton step y + y (1 - a y^2) / 2
-__device__ __forceinline__ df df_rsqrt(df a) {
-  const float y = rsqrtf(a.h);
-  const float y2 = y * y, y2l = fmaf(y, y, -y2);
-  const df t = df_mul(a, df_norm(y2, y2l));
-  const float d = (1.f - t.h) - t.l;  // exact difference near 1
-  return df_norm(y, 0.5f * y * d);
-}
-
-// Sums over the warp of N values at once (N a power of two <= 16): after
-// the halving exchanges lane i holds the total of value i / (32 / N).
-template <int N>
-__device__ __forceinline__ float reduce_multi(float (&v)[N]) {
-  const int lane = threadIdx.x & 31;
-  int off = 16;
-#pragma unroll
-  for (int n = N; n > 1; n >>= 1, off >>= 1) {
-    const bool up = lane & off;
-#pragma unroll
-    for (int k = 0; k < n / 2; ++k) {
-      const float send = up ? v[k] : v[k + n / 2], keep = up ? v[k + n / 2] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-  for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-  return v[0];
-}
-
 // Column steps come in three variants by the column's size (stream_plan):
 // 128 threads with the support's columns in shared memory, 256 threads with
 // them, 256 threads reading them from AG_k.

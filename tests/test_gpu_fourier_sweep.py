@@ -1,0 +1,76 @@
+"""The DFT sweep's branches against the FP64 oracle: supports by columns and term
+by term, projections with the basis in its own shared memory, in the frame's
+place or in global memory, every rank width, and given supports in any order.
+
+Bars are those of the other parity tests (one GDmin step from the oracle's
+iterates).  The order test compares two runs that differ in the order of
+float32 sums over the support alone: 1e-5 relative."""
+import numpy as np
+import pytest
+
+import oracle.altgdmin_lrs as O
+from lrsgen import FourierInstance
+from tests.gpu_helpers import Problem, check_records, gpu_available, new_fourier_solver, one_step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    if not gpu_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_03824_gb300 import build
+    build.build()
+
+
+# fewer samples than two per row; runs of more than four adjacent columns in a
+# 256-thread frame; a rank below its width; the basis in the frame's place; in
+# global memory (r m pixels do not fit the frame); the widest ranks
+@pytest.mark.parametrize("nx,ny,q,r,m,rho,T", [
+    (64, 4, 8, 2, 100, 3, 12), (32, 32, 10, 3, 400, 40, 12), (64, 64, 6, 5, 1300, 20, 12),
+    (128, 128, 9, 7, 2300, 60, 4), (128, 128, 10, 8, 3000, 60, 4), (16, 16, 16, 9, 160, 3, 6),
+    (20, 20, 24, 13, 260, 3, 6)])
+def test_sweep_one_step(nx, ny, q, r, m, rho, T):
+    inst = FourierInstance(nx=nx, ny=ny, q=q, r=r, m=m, rho=rho, seed=50 + nx + r,
+                           mask_law="uniform", b_law="gauss")
+    _, log = O.run_alg1(O.FourierOperator(inst.masks, nx, ny), inst.Y, r, rho, T,
+                        keep=tuple(range(T + 1)), Xstar=inst.Xstar)
+    s = new_fourier_solver(inst)
+    try:
+        recs = one_step(Problem.fourier(inst), s, log, range(T))
+    finally:
+        s.close()
+    check_records(recs, min_whole=T // 2)
+
+
+@pytest.mark.parametrize("repeat", [False, True])
+def test_support_in_any_order(repeat):
+    """A state's support may come unsorted, or with a pixel twice (value zero)."""
+    inst = FourierInstance(nx=32, ny=32, q=6, r=2, m=400, rho=8, seed=61)
+    rng = np.random.default_rng(3)
+    outs = []
+    for order in (False, True):
+        s = new_fourier_solver(inst)
+        try:
+            s.init()
+            s.iterate(3)
+            U, B, Si, Sv = s.get()
+            Si, Sv = Si.copy(), Sv.copy()
+            if repeat:
+                Si[:, 1], Sv[:, 1] = Si[:, 0], Sv[:, 0]
+            if order:
+                for k in range(len(Si)):
+                    p = rng.permutation(Si.shape[1])
+                    Si[k], Sv[k] = Si[k, p], Sv[k, p]
+            from paper_2311_03824_gb300 import lrs as L
+            L.lrs_set_state(s.h, np.ascontiguousarray(U.T), np.ascontiguousarray(B.T), Si, Sv, 3,
+                            s.progress()[0])
+            s.iterate(2)
+            outs.append(s.X())
+            got = s.get()[2]
+            assert (np.diff(got, axis=1) > 0).all()
+        finally:
+            s.close()
+    if not repeat:
+        rel = np.linalg.norm(outs[0] - outs[1]) / np.linalg.norm(outs[0])
+        assert rel <= 1e-5, rel
