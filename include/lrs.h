@@ -456,7 +456,7 @@ lrs_status lrs_sweep_trace(lrs_t h, uint64_t* out, int64_t len);
  * CTAs per column or frame, slab width, shared memory per CTA, resident
  * clusters, and "launches_per_iteration": the kernels one steady iteration
  * launches; DFT handles also give "fused_qr", 1 when the step and its
- * Cholesky-QR2 run as one cooperative launch) into buf (NUL-terminated,
+ * Cholesky-QR2 run as one launch) into buf (NUL-terminated,
  * truncated to len bytes).  Errors: LRS_ERR_ARG. */
 lrs_status lrs_describe(lrs_t h, char* buf, int32_t len);
 

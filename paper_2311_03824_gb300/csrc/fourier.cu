@@ -721,6 +721,7 @@ struct FourierSolver {
          *twy = nullptr;
   int *mask = nullptr, *S_idx = nullptr, *iptr = nullptr, *ilist = nullptr, *err = nullptr;
   double2* part = nullptr;
+  bool cluster = false;      // the matrix fits the cluster Cholesky-QR2
   double2* part2 = nullptr;  // second Gram partials of the fused Cholesky-QR2
   unsigned* qbar = nullptr;  // its grid-barrier counter
   bool coop = false;         // the fused Cholesky-QR2 fits one cooperative launch
@@ -795,7 +796,8 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
   F->nblk = std::max(1, std::min(152, (n + 63) / 64));
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
-  {  // the fused Cholesky-QR2 needs all its blocks resident at once
+  F->cluster = cqr_cluster_fits(n, r);
+  {  // the cooperative Cholesky-QR2 needs all its blocks resident at once
     int coop = 0, nsm = 0, per_sm = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1012,8 +1014,9 @@ static cudaError_t ccholqr2(FourierSolver* F, const float2* Zin, float2* Uout) {
   return cudaGetLastError();
 }
 
-// Z = X - eta G2 (G2 null: Z = X), then Uout = its Cholesky-QR2: one
-// cooperative launch when every block fits on the device at once, else the
+// Z = X - eta G2 (G2 null: Z = X), then Uout = its Cholesky-QR2: one cluster
+// launch when the matrix fits its shared memory (r up to 11 at n = 16384), else
+// one cooperative launch when every block fits on the device at once, else the
 // separate kernels.  Uout may be X.
 static cudaError_t cqr2(FourierSolver* F, const float2* X, const float2* G2, const double* eta,
                         float2* Uout) {
@@ -1026,6 +1029,7 @@ static cudaError_t cqr2(FourierSolver* F, const float2* X, const float2* G2, con
     unsigned long long wait_ns = 10ull * 1000 * 1000 * 1000;
     int nn = n, rr = r;
     void* args[] = {&nn, &rr, const_cast<float2**>(&X), const_cast<float2**>(&G2),
+  if (F->cluster) return cqr_cluster(n, r, X, G2, eta, Uout, F->err, F->s);
                     const_cast<double**>(&eta), &Z, &Z2, &Uout, &F->part, &F->part2, &F->qbar,
                     &F->err, &wait_ns};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(cqr2_fused_kernel),

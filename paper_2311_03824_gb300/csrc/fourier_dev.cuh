@@ -147,6 +147,232 @@ __device__ __forceinline__ void stage_pair(float2& x0, float2& x1, float2& x2, f
   x1 = cadd(b1, d3);
   x3 = csub(b1, d3);
 }
+// ------------------------------------------- Gram and Cholesky, complex --
+// Entries (a, b <= a), A0 <= a < A1, of the Gram conj(W_b) W_a over this warp's
+// rows, in double-float from exact products; the warp's sums to part.
+// Sixteen warps share the rows, not the entries (21 entries of r = 6 on 16
+// warps took two rounds), and a row of W is read once for several entries.
+template <int A0, int A1>
+__device__ __forceinline__ void cgram_part(const float2* W, size_t ld, int m, int r, int nw, float2* part) {
+  if (A0 >= r) return;
+  constexpr int NE = (A1 * (A1 + 1) - A0 * (A0 + 1)) / 2;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float xh[NE], xl[NE], yh[NE], yl[NE];
+#pragma unroll
+  for (int t = 0; t < NE; ++t) xh[t] = xl[t] = yh[t] = yl[t] = 0.f;
+  for (int i = 32 * w + lane; i < m; i += 32 * nw) {
+    float2 x[A1];
+#pragma unroll
+    for (int l = 0; l < A1; ++l) x[l] = l < r ? W[l * ld + i] : make_float2(0.f, 0.f);
+    int t = 0;
+#pragma unroll
+    for (int a = A0; a < A1; ++a)
+#pragma unroll
+      for (int b = 0; b <= a; ++b, ++t) {
+        df_fma(xh[t], xl[t], x[b].x, x[a].x);
+        df_fma(xh[t], xl[t], x[b].y, x[a].y);
+        if (b < a) {  // the diagonal is real
+          df_fma(yh[t], yl[t], x[b].x, x[a].y);
+          df_fma(yh[t], yl[t], -x[b].y, x[a].x);
+        }
+      }
+  }
+  // the real parts, then the imaginary parts of the entries off the diagonal,
+  // in blocks of sixteen values: halving exchanges leave one per lane pair
+  constexpr int NV = 2 * NE - (A1 - A0);
+#pragma unroll
+  for (int v0 = 0; v0 < NV; v0 += 16) {
+    float h[16], l[16];
+#pragma unroll
+    for (int z = 0; z < 16; ++z) {
+      h[z] = l[z] = 0.f;
+      int v = 0;
+#pragma unroll
+      for (int a = A0; a < A1; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {
+          const int t = (a * (a + 1) - A0 * (A0 + 1)) / 2 + b;
+          if (v == v0 + z) { h[z] = xh[t]; l[z] = xl[t]; }
+          ++v;
+          if (b < a) {
+            if (v == v0 + z) { h[z] = yh[t]; l[z] = yl[t]; }
+            ++v;
+          }
+        }
+    }
+#pragma unroll
+    for (int k = 8, off = 16; k >= 1; k >>= 1, off >>= 1) {
+      const bool up = lane & off;
+#pragma unroll
+      for (int z = 0; z < k; ++z) {
+        const float sh = up ? h[z] : h[z + k], sl = up ? l[z] : l[z + k];
+        const float kh = up ? h[z + k] : h[z], kl = up ? l[z + k] : l[z];
+        h[z] = kh;
+        l[z] = kl;
+        df_add(h[z], l[z], __shfl_xor_sync(0xffffffffu, sh, off), __shfl_xor_sync(0xffffffffu, sl, off));
+      }
+    }
+    df_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], 1), __shfl_xor_sync(0xffffffffu, l[0], 1));
+    // lane 2 z holds value v0 + z: row a's values start at a^2 (2 b and 2 b + 1,
+    // the diagonal's real part last)
+    if ((lane & 1) == 0 && v0 + (lane >> 1) < NV) part[A0 * A0 + v0 + (lane >> 1)] = make_float2(h[0], l[0]);
+  }
+}
+
+// double-float complex
+struct cdf {
+  df x, y;
+};
+__device__ __forceinline__ cdf cdf_shfl(const cdf& a, int src) { return cdf{df_shfl(a.x, src), df_shfl(a.y, src)}; }
+// c - a b, and c - a conj(b)
+__device__ __forceinline__ cdf cdf_sub_mul(const cdf& c, const cdf& a, const cdf& b) {
+  return cdf{df_sub(df_sub(c.x, df_mul(a.x, b.x)), df_mul(df{-a.y.h, -a.y.l}, b.y)),
+             df_sub(df_sub(c.y, df_mul(a.x, b.y)), df_mul(a.y, b.x))};
+}
+__device__ __forceinline__ cdf cdf_sub_mulc(const cdf& c, const cdf& a, const cdf& b) {
+  return cdf_sub_mul(c, a, cdf{b.x, df{-b.y.h, -b.y.l}});
+}
+
+// every entry of the lower triangle
+template <int R>
+__device__ __forceinline__ void cgram_warp(const float2* W, size_t ld, int m, int r, int nw, float2* part) {
+  cgram_part<0, (R < 4 ? R : 4)>(W, ld, m, r, nw, part);
+  if constexpr (R > 4) cgram_part<4, 6>(W, ld, m, r, nw, part);
+  if constexpr (R > 6) cgram_part<6, 8>(W, ld, m, r, nw, part);
+  if constexpr (R > 8) {
+    cgram_part<8, 9>(W, ld, m, r, nw, part);
+    cgram_part<9, 10>(W, ld, m, r, nw, part);
+    cgram_part<10, 11>(W, ld, m, r, nw, part);
+    cgram_part<11, 12>(W, ld, m, r, nw, part);
+  }
+  if constexpr (R > 12) {
+    cgram_part<12, 13>(W, ld, m, r, nw, part);
+    cgram_part<13, 14>(W, ld, m, r, nw, part);
+    cgram_part<14, 15>(W, ld, m, r, nw, part);
+    cgram_part<15, 16>(W, ld, m, r, nw, part);
+  }
+}
+
+// One warp: the complex Cholesky factor L of M (Gd: the sums of cgram_warp) and
+// L^{-1} in double-float in registers (lane = row, then lane = column; an FP64
+// factor through shared memory took 31 K cycles at r = 6); Lf is L^{-1} rounded,
+// or with dev its deviation from I.  A pivot below 1e-9 of its diagonal goes to
+// FP64 (scratch: 2 kMaxR^2 + kMaxR / 2 values).  False when M is not positive
+// definite; L is then I.
+template <int R>
+__device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, double2* Li, float2* Lf) {
+  const int lane = threadIdx.x & 31;
+  double2* G = scratch;
+  bool done = true;
+  // M[i][q] = conj(W_i) W_q, q <= i: the conjugate of the sums
+  cdf a[R];
+  df inv[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    a[q] = cdf{df{0.f, 0.f}, df{0.f, 0.f}};
+    if (q <= lane && lane < r) {
+      const float2 x = Gd[lane * lane + 2 * q];
+      a[q].x = df_norm(x.x, x.y);
+      if (q < lane) {
+        const float2 yv = Gd[lane * lane + 2 * q + 1];
+        a[q].y = df_norm(-yv.x, -yv.y);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    inv[j] = df{1.f, 0.f};
+    if (j >= r || !done) continue;
+    const df pv = df_shfl(a[j].x, j);
+    const float dj = Gd[j * j + 2 * j].x;
+    done = pv.h > 1e-9f * dj && pv.h > 1e-30f && pv.h < 1e30f;
+    inv[j] = df_rsqrt(pv);
+    a[j].x = df_mul(a[j].x, inv[j]);
+    a[j].y = df_mul(a[j].y, inv[j]);
+#pragma unroll
+    for (int q = j + 1; q < R; ++q) a[q] = cdf_sub_mulc(a[q], a[j], cdf_shfl(a[j], q));
+  }
+  if (done) {
+    cdf x[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {  // column lane of L^{-1}
+      cdf t = cdf{df{0.f, 0.f}, df{0.f, 0.f}};
+#pragma unroll
+      for (int q = 0; q < i; ++q) t = cdf_sub_mul(t, cdf_shfl(a[q], i), x[q]);
+      t.x = df_mul(t.x, inv[i]);
+      t.y = df_mul(t.y, inv[i]);
+      const df z = df{0.f, 0.f};
+      x[i] = i < lane ? cdf{z, z} : i == lane ? cdf{inv[i], z} : t;
+      if (lane < kMaxR && i < r) {
+        Li[i * kMaxR + lane] = make_double2(static_cast<double>(x[i].x.h) + static_cast<double>(x[i].x.l),
+                                              static_cast<double>(x[i].y.h) + static_cast<double>(x[i].y.l));
+        Lf[i * kMaxR + lane] = make_float2(dev && i == lane ? (x[i].x.h - 1.f) + x[i].x.l : x[i].x.h, x[i].y.h);
+      }
+    }
+  } else if (lane < r) {
+    for (int q = 0; q <= lane; ++q) {
+      const float2 x = Gd[lane * lane + 2 * q], yv = q < lane ? Gd[lane * lane + 2 * q + 1] : make_float2(0.f, 0.f);
+      G[lane * kMaxR + q] = make_double2(static_cast<double>(x.x) + static_cast<double>(x.y),
+                                         -(static_cast<double>(yv.x) + static_cast<double>(yv.y)));
+    }
+  }
+  __syncwarp();
+  if (done) return true;
+  double2* Lc = scratch + kMaxR * kMaxR;
+  double* iL = reinterpret_cast<double*>(scratch + 2 * kMaxR * kMaxR);
+  bool ok = true;
+  for (int j = 0; j < r; ++j) {
+    double2 t = make_double2(0.0, 0.0);
+    if (lane >= j && lane < r) {
+      t = G[lane * kMaxR + j];
+      for (int p = 0; p < j; ++p) {
+        const double2 x = Lc[lane * kMaxR + p], y = Lc[j * kMaxR + p];
+        // t -= L[i][p] * conj(L[j][p])
+        t.x -= x.x * y.x + x.y * y.y;
+        t.y -= x.y * y.x - x.x * y.y;
+      }
+    }
+    const double sj = __shfl_sync(0xffffffffu, t.x, j);
+    if (!(sj > 1e-13 * G[j * kMaxR + j].x) || !(sj < 1e300)) {
+      ok = false;
+      break;
+    }
+    const double ij = rsqrt_newton(sj);
+    if (lane == j) {
+      Lc[j * kMaxR + j] = make_double2(sj * ij, 0.0);
+      iL[j] = ij;
+    } else if (lane > j && lane < r) {
+      Lc[lane * kMaxR + j] = make_double2(t.x * ij, t.y * ij);
+    }
+    __syncwarp();
+  }
+  if (!ok && lane == 0) {
+    for (int i = 0; i < r; ++i) {
+      for (int p = 0; p < r; ++p) Lc[i * kMaxR + p] = make_double2(i == p ? 1.0 : 0.0, 0.0);
+      iL[i] = 1.0;
+    }
+  }
+  __syncwarp();
+  if (lane < kMaxR) {  // column lane of L^{-1}
+    const int cc = lane;
+    for (int i = 0; i < r; ++i) {
+      double2 t = make_double2(i == cc ? 1.0 : 0.0, 0.0);
+      for (int p = cc; p < i; ++p) {
+        const double2 q = dcmul(Lc[i * kMaxR + p], Li[p * kMaxR + cc]);
+        t.x -= q.x;
+        t.y -= q.y;
+      }
+      t = i < cc ? make_double2(0, 0) : make_double2(t.x * iL[i], t.y * iL[i]);
+      Li[i * kMaxR + cc] = t;
+      Lf[i * kMaxR + cc] =
+            make_float2(static_cast<float>(t.x - (dev && i == cc ? 1.0 : 0.0)), static_cast<float>(t.y));
+    }
+  }
+  __syncwarp();
+  return ok;
+}
+
+// ---------------------------------------------------------------- frames --
 
 struct Geo {
   int nx, ny, lnx, lny, n;  // lnx / lny: log2 of a power-of-two side, else -1

@@ -379,6 +379,10 @@ bool qr_cluster_fits(int n, int r);
 cudaError_t qr_cluster(int n, int r, const float* X, const float* Gparts, int nparts,
                        const double* eta, float* Q, float* Qpad, int rpad, int* err,
                        cudaStream_t s);
+// The same for the DFT operator's complex r x n matrices (cqr_cluster.cu).
+bool cqr_cluster_fits(int n, int r);
+cudaError_t cqr_cluster(int n, int r, const float2* X, const float2* G, const double* eta, float2* Q,
+                        int* err, cudaStream_t s);
 cudaError_t cholqr2(const GlobalWork& g, const float* Zin, float* Uout, int* err,
                     cudaStream_t s);
 cudaError_t project_cols(const GlobalWork& g, const float* H, const float* U, float* P,
