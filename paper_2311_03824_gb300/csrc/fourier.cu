@@ -721,9 +721,9 @@ struct FourierSolver {
          *twy = nullptr;
   int *mask = nullptr, *S_idx = nullptr, *iptr = nullptr, *ilist = nullptr, *err = nullptr;
   double2* part = nullptr;
-  bool cluster = false;      // the matrix fits the cluster Cholesky-QR2
   double2* part2 = nullptr;  // second Gram partials of the fused Cholesky-QR2
   unsigned* qbar = nullptr;  // its grid-barrier counter
+  bool cluster = false;      // the matrix fits the cluster Cholesky-QR2
   bool coop = false;         // the fused Cholesky-QR2 fits one cooperative launch
   double2* rfac = nullptr;
   double* eta = nullptr;
@@ -1021,6 +1021,7 @@ static cudaError_t ccholqr2(FourierSolver* F, const float2* Zin, float2* Uout) {
 static cudaError_t cqr2(FourierSolver* F, const float2* X, const float2* G2, const double* eta,
                         float2* Uout) {
   const int n = F->g.n, r = F->r;
+  if (F->cluster) return cqr_cluster(n, r, X, G2, eta, Uout, F->err, F->s);
   if (F->coop) {
     cudaError_t e = cudaMemsetAsync(F->qbar, 0, sizeof(unsigned), F->s);
     if (e != cudaSuccess) return e;
@@ -1029,7 +1030,6 @@ static cudaError_t cqr2(FourierSolver* F, const float2* X, const float2* G2, con
     unsigned long long wait_ns = 10ull * 1000 * 1000 * 1000;
     int nn = n, rr = r;
     void* args[] = {&nn, &rr, const_cast<float2**>(&X), const_cast<float2**>(&G2),
-  if (F->cluster) return cqr_cluster(n, r, X, G2, eta, Uout, F->err, F->s);
                     const_cast<double**>(&eta), &Z, &Z2, &Uout, &F->part, &F->part2, &F->qbar,
                     &F->err, &wait_ns};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(cqr2_fused_kernel),
