@@ -146,87 +146,137 @@ __device__ __forceinline__ void dit_side(float2* X, int nl, int ls, int es, int 
   }
 }
 
-// The unitary 2D FFT of the frame kernel: as fft2_smem, with every side in
-// register passes of up to three stages (the bit reversal read by the first).
-__device__ void fft2_dit(float2* X, int nx, int ny, int lnx, int lny, const float2* tx,
-                         const float2* ty, bool inverse) {
-  const int ld = ny + 1, n = nx * ny;
-  const float sc = rsqrtf(static_cast<float>(n));
-  if (lny < 0)
-    dft_direct_smem(X, nx, ny, true, ty, inverse);
-  else
-    dit_side<3>(X, nx, ld, 1, ny, lny, ty, inverse, 1.f);  // rows
-  bool scaled = false;
-  if (lnx < 0) {
-    dft_direct_smem(X, nx, ny, false, tx, inverse);
-  } else {
-    dit_side<3>(X, ny, 1, ld, nx, lnx, tx, inverse, sc);  // columns
-    scaled = lnx > 0;
-  }
-  if (!scaled) {
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int row = e / ny, j = e - row * ny;
-      X[row * ld + j].x *= sc;
-      X[row * ld + j].y *= sc;
-    }
-    __syncthreads();
-  }
-}
 // out[f] = F2(in[f]) (or F2^H) for frames f; frames are n-vectors in natural
 // row-major order (pixel kx*ny + ky), frame f at in + f*n; its pixel e goes to
-// out[e * es + f * fs] (F2 U is stored sample by sample, so that the sweep reads
-// the r values of a sampled frequency from one or two sectors, not from r).
-__global__ void __launch_bounds__(kFT) fft_frames_kernel(Geo g, const float2* __restrict__ in,
-                                                         float2* __restrict__ out, size_t es, size_t fs,
-                                                         int inverse,
-                                                         const float2* __restrict__ twx,
-                                                         const float2* __restrict__ twy) {
+// out[e * es + f * fs].  One cluster of eight CTAs per frame: a CTA transforms
+// its rows, then gathers its columns from the peers' shared memory and
+// transforms them.  A power-of-two side by register passes, any other by a
+// direct DFT.
+//
+// One CTA per frame kept r of the 152 SMs busy (26 us at 128 x 128, r = 6); a
+// launch per side was faster there and slower on frames up to 64 x 64.
+constexpr int kFC = 8;    // CTAs per frame
+constexpr int kFCT = 256;
+
+struct FftCarve {
+  size_t X1, X1b, X2, tx, ty, total;
+  int rl, cl;  // rows and columns of a CTA
+};
+__host__ __device__ inline FftCarve fft_carve(const Geo& g) {
+  FftCarve c;
+  size_t o = 0;
+  auto put = [&](size_t bytes) {
+    const size_t at = o;
+    o += al16(bytes);
+    return at;
+  };
+  c.rl = (g.nx + kFC - 1) / kFC;
+  c.cl = (g.ny + kFC - 1) / kFC;
+  const size_t rows = static_cast<size_t>(c.rl) * (g.ny + 1) * 8;
+  c.X1 = put(rows);
+  c.X1b = put(g.lny < 0 ? rows : 0);
+  c.X2 = put(static_cast<size_t>(c.cl) * (g.nx + 1) * 8);
+  c.tx = put(static_cast<size_t>(g.nx) * 8);
+  c.ty = put(static_cast<size_t>(g.ny) * 8);
+  c.total = o;
+  return c;
+}
+
+// entry p of the direct DFT of the line X (N elements)
+__device__ __forceinline__ float2 dft_entry(const float2* X, const float2* t, int N, int p, bool inverse) {
+  float2 v = make_float2(0.f, 0.f);
+  int idx = 0;  // p k mod N
+  for (int k = 0; k < N; ++k) {
+    float2 w = t[idx];
+    if (inverse) w.y = -w.y;
+    v = cfma(X[k], w, v);
+    idx += p;
+    if (idx >= N) idx -= N;
+  }
+  return v;
+}
+
+__global__ void __launch_bounds__(kFCT) __cluster_dims__(kFC, 1, 1)
+    fft_frames_kernel(Geo g, const float2* __restrict__ in, float2* __restrict__ out, size_t es, size_t fs,
+                      int inverse, const float2* __restrict__ twx, const float2* __restrict__ twy) {
   extern __shared__ __align__(16) unsigned char sm[];
-  float2* X = reinterpret_cast<float2*>(sm);
-  float2* tx = X + static_cast<size_t>(g.nx) * (g.ny + 1);
-  float2* ty = tx + g.nx;
-  const size_t f = blockIdx.x;
-  for (int k = threadIdx.x; k < g.nx; k += blockDim.x) tx[k] = twx[k];
-  for (int k = threadIdx.x; k < g.ny; k += blockDim.x) ty[k] = twy[k];
-  for (int e = threadIdx.x; e < g.n; e += blockDim.x) {
-    const int row = e / g.ny, j = e - row * g.ny;
-    X[row * (g.ny + 1) + j] = in[f * g.n + e];
+  const FftCarve c = fft_carve(g);
+  float2* X1 = reinterpret_cast<float2*>(sm + c.X1);
+  float2* X2 = reinterpret_cast<float2*>(sm + c.X2);
+  float2* tx = reinterpret_cast<float2*>(sm + c.tx);
+  float2* ty = reinterpret_cast<float2*>(sm + c.ty);
+  const int rank = static_cast<int>(cluster_rank()), nx = g.nx, ny = g.ny;
+  const size_t f = blockIdx.x / kFC;
+  const int r0 = min(nx, rank * c.rl), nr = min(nx, r0 + c.rl) - r0;
+  const int c0 = min(ny, rank * c.cl), nc = min(ny, c0 + c.cl) - c0;
+  for (int k = threadIdx.x; k < nx; k += kFCT) tx[k] = __ldg(twx + k);
+  for (int k = threadIdx.x; k < ny; k += kFCT) ty[k] = __ldg(twy + k);
+  const float2* src = in + f * g.n + static_cast<size_t>(r0) * ny;
+#pragma unroll 4
+  for (int u = threadIdx.x; u < nr * ny; u += kFCT) {
+    const int l = frow(g, u);
+    X1[l * (ny + 1) + (u - l * ny)] = src[u];
   }
   __syncthreads();
-  fft2_dit(X, g.nx, g.ny, g.lnx, g.lny, tx, ty, inverse != 0);
-  for (int e = threadIdx.x; e < g.n; e += blockDim.x) {
-    const int row = e / g.ny, j = e - row * g.ny;
-    out[e * es + f * fs] = X[row * (g.ny + 1) + j];
+  if (g.lny >= 0) {
+    if (nr > 0) dit_side<3>(X1, nr, ny + 1, 1, ny, g.lny, ty, inverse != 0, 1.f);
+  } else {
+    float2* Xb = reinterpret_cast<float2*>(sm + c.X1b);
+    for (int u = threadIdx.x; u < nr * ny; u += kFCT) {
+      const int l = u / ny, p = u - l * ny;
+      Xb[l * (ny + 1) + p] = dft_entry(X1 + l * (ny + 1), ty, ny, p, inverse != 0);
+    }
+    X1 = Xb;
+  }
+  cluster_sync_all();
+#pragma unroll 4
+  for (int u = threadIdx.x; u < nx * nc; u += kFCT) {
+    const int x = u / nc, l = u - x * nc, from = x / c.rl;
+    X2[l * (nx + 1) + x] = *peer_ptr(X1 + (x - from * c.rl) * (ny + 1) + c0 + l, from);
+  }
+  cluster_sync_all();  // also: no CTA leaves while a peer reads its rows
+  if (g.lnx >= 0 && nc > 0) dit_side<3>(X2, nc, nx + 1, 1, nx, g.lnx, tx, inverse != 0, 1.f);
+  const float sc = rsqrtf(static_cast<float>(g.n));
+  for (int u = threadIdx.x; u < nx * nc; u += kFCT) {
+    const int x = u / nc, l = u - x * nc;
+    const float2* L = X2 + l * (nx + 1);
+    const float2 v = g.lnx >= 0 ? L[x] : dft_entry(L, tx, nx, x, inverse != 0);
+    out[(static_cast<size_t>(x) * ny + c0 + l) * es + f * fs] = make_float2(v.x * sc, v.y * sc);
   }
 }
 
 // K[l][w] = sum over the (k, i) with mask_k[i] = w of res_k[i] conj(b_k[l]).
 // One warp per frequency w (a frequency every frame samples has q entries,
-// most have a few): lanes take entries lane, lane + 32, ... of its list, then
-// a butterfly per component (fixed order).
-__global__ void kspace_kernel(int n, int m, int r, const int* __restrict__ ptr,
-                              const int* __restrict__ list, const float2* __restrict__ RES,
-                              const float2* __restrict__ B, float2* __restrict__ K) {
+// most have a few): lanes take entries lane, lane + 32, ... of its list, then the
+// 2 R sums at once by halving exchanges (fixed order; a butterfly per sum was
+// 120 of the 200 instructions of a frequency with 32 entries at R = 6).
+template <int R>
+__global__ void __launch_bounds__(256) kspace_kernel(int n, int m, int r, const int* __restrict__ ptr,
+                                                     const int* __restrict__ list,
+                                                     const float2* __restrict__ RES,
+                                                     const float2* __restrict__ B, float2* __restrict__ K) {
+  constexpr int N = R <= 2 ? 4 : R <= 4 ? 8 : R <= 8 ? 16 : 32, G = 32 / N;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= n) return;  // uniform over the warp
-  float2 acc[kMaxR];
+  float v[N];
 #pragma unroll
-  for (int l = 0; l < kMaxR; ++l) acc[l] = make_float2(0.f, 0.f);
-  for (int t = ptr[w] + lane; t < ptr[w + 1]; t += 32) {
+  for (int j = 0; j < N; ++j) v[j] = 0.f;
+  const int t1 = ptr[w + 1];
+  for (int t = ptr[w] + lane; t < t1; t += 32) {
     const int ki = list[t];
-    const int k = ki / m;
+    const float2* b = B + static_cast<size_t>(ki / m) * r;
     const float2 rv = RES[ki];
 #pragma unroll
-    for (int l = 0; l < kMaxR; ++l)
-      if (l < r) acc[l] = cfma(rv, cconj(B[static_cast<size_t>(k) * r + l]), acc[l]);
+    for (int l = 0; l < R; ++l)
+      if (l < r) {
+        const float2 s = cfma(rv, cconj(b[l]), make_float2(v[2 * l], v[2 * l + 1]));
+        v[2 * l] = s.x;
+        v[2 * l + 1] = s.y;
+      }
   }
-#pragma unroll
-  for (int l = 0; l < kMaxR; ++l) {
-    if (l < r) {
-      const float x = warp_sum(acc[l].x), y = warp_sum(acc[l].y);
-      if (lane == 0) K[static_cast<size_t>(l) * n + w] = make_float2(x, y);
-    }
-  }
+  const float s = reduce_multi<N>(v);
+  const int j = lane / G;
+  if (lane % G == 0 && j < 2 * r) reinterpret_cast<float*>(K + static_cast<size_t>(j >> 1) * n + w)[j & 1] = s;
 }
 
 // ---- complex column-reduced ops on r x n column-major matrices (l-major) ----
@@ -738,16 +788,14 @@ struct FourierSolver {
   size_t smem = 0;
 };
 
-static size_t fft_smem(const Geo& g) {
-  return al16(static_cast<size_t>(g.nx) * (g.ny + 1) * 8) + static_cast<size_t>(g.nx + g.ny) * 8;
-}
-
-// by_sample: out is n x nframes (frame f at out[e * nframes + f])
+// by_sample: out is n x nframes (frame f at out[e * nframes + f]), so that the
+// sweep reads the values of a sampled frequency from one or two sectors, not
+// from nframes
 static cudaError_t fft_frames(FourierSolver* F, const float2* in, float2* out, int nframes,
                               bool inverse, bool by_sample) {
   const size_t es = by_sample ? nframes : 1, fs = by_sample ? 1 : F->g.n;
-  fft_frames_kernel<<<nframes, kFT, fft_smem(F->g), F->s>>>(F->g, in, out, es, fs, inverse ? 1 : 0,
-                                                             F->twx, F->twy);
+  fft_frames_kernel<<<kFC * nframes, kFCT, fft_carve(F->g).total, F->s>>>(F->g, in, out, es, fs, inverse ? 1 : 0,
+                                                                          F->twx, F->twy);
   return cudaGetLastError();
 }
 
@@ -834,7 +882,7 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     return false;
   };
   if (!plan(share, std::min(want, 4)) && !plan(room, std::min(want, 4))) F->smem = room + 1;
-  if (F->smem > room || fft_smem(F->g) > static_cast<size_t>(optin)) {
+  if (F->smem > room || fft_carve(F->g).total > static_cast<size_t>(optin)) {
     *msg = "frame too large for one CTA's shared memory (n <= 16384 fits)";
     delete F;
     return nullptr;
@@ -1143,7 +1191,15 @@ int fourier_iterate(FourierSolver* F, int iters, std::string* msg, cudaEvent_t* 
     cudaError_t e = fft_frames(F, F->U, F->FU, r, false, true);            // FU = F2 U
     if (e == cudaSuccess) e = launch_fsweep(F, kModeIter, F->tau);   // per-frame work
     if (ev) cudaEventRecord(ev[1], F->s);
-    kspace_kernel<<<(n + 7) / 8, 256, 0, F->s>>>(n, F->m, r, F->iptr, F->ilist, F->RES, F->B, F->K);
+    {
+      const dim3 nb((n + 7) / 8), nt(256);
+      switch (r <= 2 ? 2 : r <= 4 ? 4 : r <= 6 ? 6 : r <= 8 ? 8 : r <= 12 ? 12 : 16) {
+#define LRS_CASE(R) \
+  case R: kspace_kernel<R><<<nb, nt, 0, F->s>>>(n, F->m, r, F->iptr, F->ilist, F->RES, F->B, F->K); break;
+        LRS_FSWEEP_R(LRS_CASE)
+#undef LRS_CASE
+      }
+    }
     if (e == cudaSuccess) e = fft_frames(F, F->K, F->grad, r, true, false);  // grad = F2^H K
     if (e == cudaSuccess && F->t == 0) {
       cgram_part_kernel<<<F->nblk, 256, 0, F->s>>>(n, r, F->grad, nullptr, nullptr, nullptr, F->part);
@@ -1198,10 +1254,10 @@ double fourier_eta(FourierSolver* F) {
 int fourier_t(FourierSolver* F) { return F->t; }
 
 // Kernels one steady iteration launches: F2 U, the sweep, the k-space
-// reduction, F2^H K, and the step with its Cholesky-QR2 (one cooperative
-// launch, else the Gram partials and two factorisations and applications).
-int fourier_launches_per_iteration(FourierSolver* F) { return 4 + (F->coop ? 1 : 6); }
-int fourier_fused_qr(FourierSolver* F) { return F->coop ? 1 : 0; }
+// reduction, F2^H K, and the step with its Cholesky-QR2 (one launch, else the
+// Gram partials and two factorisations and applications).
+int fourier_launches_per_iteration(FourierSolver* F) { return 4 + (F->cluster || F->coop ? 1 : 6); }
+int fourier_fused_qr(FourierSolver* F) { return F->cluster || F->coop ? 1 : 0; }
 
 // Sweep cycle counters: enable (allocate, zero) and read-and-zero.
 int fourier_prof_enable(FourierSolver* F) {
