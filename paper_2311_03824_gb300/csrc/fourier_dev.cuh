@@ -10,7 +10,6 @@
 namespace lrs {
 namespace fourier {
 
-constexpr int kFT = 512;   // threads of the frame kernels (the sweep: fsweep_threads)
 // sweep profile slots: set-up and Gram, sparse DFTs, norms and vector
 // updates, 2D FFTs with the frame's fills, HardThreshold, final stage,
 // projections' Q^H v, projections' v - Q c
@@ -147,6 +146,7 @@ __device__ __forceinline__ void stage_pair(float2& x0, float2& x1, float2& x2, f
   x1 = cadd(b1, d3);
   x3 = csub(b1, d3);
 }
+
 // ------------------------------------------- Gram and Cholesky, complex --
 // Entries (a, b <= a), A0 <= a < A1, of the Gram conj(W_b) W_a over this warp's
 // rows, in double-float from exact products; the warp's sums to part.
@@ -373,7 +373,6 @@ __device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, 
 }
 
 // ---------------------------------------------------------------- frames --
-
 struct Geo {
   int nx, ny, lnx, lny, n;  // lnx / lny: log2 of a power-of-two side, else -1
   int L, sxL, syL, lL;      // L = lcm(nx, ny), L / nx, L / ny, log2 L (or -1)

@@ -60,11 +60,15 @@ struct FArgs {
 
 // Threads per frame, by its size: a 20 x 20 frame has 400 pixels and a few
 // hundred samples, and four 128-thread CTAs per SM (128 registers) take the
-// place of one of 512 threads that mostly waits at barriers.
-__host__ __device__ constexpr int fsweep_threads(int n) { return n <= 512 ? 128 : n < 2048 ? 256 : 512; }
+// place of one of 512 threads that mostly waits at barriers (a 20 x 20 solve of
+// 400 frames: 215 -> 62 us per sweep).  On the largest frames 768 and 1024
+// threads were slower (128 x 128: 353 us per sweep with 512, 382 with 768, 449
+// with 1024: spills and more redundant work per warp).
+constexpr int kFT = 512;  // at most
+__host__ __device__ constexpr int fsweep_threads(int n) { return n <= 512 ? 128 : n < 2048 ? 256 : kFT; }
 
 struct FCarve {
-  size_t X, tx, ty, tl, dv, ev, msk, rptr, sp, sv, gv, vn, ord, prow, cof, cs, ccol, pcs, Li, Lf, red,
+  size_t X, tx, ty, tl, dv, ev, msk, rptr, sp, sv, gv, vn, ord, ent, cs, ccol, pcs, Li, Lf, red,
       scal, hist, cand, cl, T, Q, total;
 };
 
@@ -102,8 +106,7 @@ __host__ __device__ inline FCarve fcarve(const Geo& g, int m, int r, int rho, bo
   c.gv = put(rh * 8);
   c.vn = put(rh * 8);
   c.ord = put(rh * 2);
-  c.prow = put(rh * 2);
-  c.cof = put(rh * 2);
+  c.ent = put(rh * 4);
   c.cs = put((rh + 1) * 2);
   c.ccol = put(rh * 2);
   c.pcs = put((rh + 1) * 2);
@@ -139,10 +142,12 @@ struct FCtx {
   int* spo;        // the support before the last HardThreshold, in the place
                    // of gv (read before it)
   float2* vn;      // s - mu g on the support
-  // the support by (column, row): entry, row and column index of each; the
-  // distinct columns' first positions (and the end), and the columns; the first
-  // column of each piece (at most four adjacent columns; and the end)
-  unsigned short *ord, *prow, *cof, *cs, *ccol, *pcs;
+  // the support by (column, row): entry of each position, its row and (above 16
+  // bits) column index; the distinct columns' first positions (and the end), and
+  // the columns; the first column of each piece (at most four adjacent columns;
+  // and the end)
+  unsigned short *ord, *cs, *ccol, *pcs;
+  int* ent;
   double2* Li;     // L^{-1} (ld kMaxR)
   float2* Lf;
   float* red;
@@ -223,11 +228,13 @@ __device__ inline void sparse_direct(const FCtx& C, const float2* v, int nnz, fl
 }
 
 // out = A x by support columns (head of the file); T holds cap columns (four
-// or all of them at least).  Ends with a barrier.
+// or all of them at least).  Scratch: vn.  Ends with a barrier.
 __device__ inline void sparse_cols(const FCtx& C, int np, const float2* v, float2* out, int cap) {
   float2* T = C.T;
   const float sc = rsqrtf(static_cast<float>(C.g.n));
   const int bd = blockDim.x, nx = C.g.nx, ng = max(1, bd / nx);
+  for (int e = threadIdx.x; e < C.rho; e += bd) C.vn[e] = v[C.ord[e]];  // in column order
+  __syncthreads();
   int j0 = 0;
   do {
     int j1 = j0;
@@ -241,7 +248,7 @@ __device__ inline void sparse_cols(const FCtx& C, int np, const float2* v, float
       if (c0 == c1) continue;
       float2* Tk = T + kx * ldc - cA;
       const int p1 = C.cs[cA + c1];
-      int p = C.cs[cA + c0], c = C.cof[p];
+      int p = C.cs[cA + c0], c = cA + c0;
       float2 acc = make_float2(0.f, 0.f);
       for (; p < p1; p += 4) {
         int cc[4];
@@ -249,9 +256,10 @@ __device__ inline void sparse_cols(const FCtx& C, int np, const float2* v, float
 #pragma unroll
         for (int z = 0; z < 4; ++z) {
           const int at = min(p + z, p1 - 1);
-          cc[z] = C.cof[at];
-          x[z] = v[C.ord[at]];
-          w[z] = C.tl[fwrapL(C.g, kxL * C.prow[at])];
+          cc[z] = C.ent[at];
+          x[z] = C.vn[at];
+          w[z] = C.tl[fwrapL(C.g, kxL * (cc[z] & 0xffff))];
+          cc[z] >>= 16;
         }
 #pragma unroll
         for (int z = 0; z < 4; ++z)
@@ -367,8 +375,8 @@ __device__ inline void sparse_adjoint(const FCtx& C, int np, const float2* u, in
 #pragma unroll
       for (int z = 0; z < 4; ++z) {
         const int e = min(e0 + z, pB - 1);
-        p[z] = C.prow[e] * C.g.sxL;
-        c[z] = C.cof[e];
+        p[z] = (C.ent[e] & 0xffff) * C.g.sxL;
+        c[z] = C.ent[e] >> 16;
         v[2 * z] = v[2 * z + 1] = 0.f;
       }
       for (int kx = lane; kx < nx; kx += 32)
@@ -402,15 +410,14 @@ __device__ inline int support_cols(const FCtx& C, int* np_s) {
 #pragma unroll 8
     for (int f = 0; f < rho; ++f) pos += key[f] < mine;
     C.ord[pos] = static_cast<unsigned short>(e);
-    C.prow[pos] = static_cast<unsigned short>(mine & 0xffff);
-    C.cof[pos] = static_cast<unsigned short>(mine >> 16);  // the column, its index below
+    C.ent[pos] = mine;  // the column's index in its place below
   }
   __syncthreads();
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     int nc = 0, np = 0, run = 0, before = -2;  // run: index of the last run's first column
     for (int e0 = 0; e0 < rho; e0 += 32) {
-      const int e = e0 + lane, col = e < rho ? C.cof[e] : -1;
+      const int e = e0 + lane, col = e < rho ? C.ent[e] >> 16 : -1;
       int prev = __shfl_up_sync(0xffffffffu, col, 1);
       if (lane == 0) prev = before;
       before = __shfl_sync(0xffffffffu, col, 31);
@@ -425,7 +432,7 @@ __device__ inline int support_cols(const FCtx& C, int* np_s) {
       const bool ps = st && ((c - r0) & 3) == 0;
       const unsigned pb = __ballot_sync(0xffffffffu, ps);
       __syncwarp();
-      if (e < rho) C.cof[e] = static_cast<unsigned short>(c);
+      if (e < rho) C.ent[e] = (c << 16) | (C.ent[e] & 0xffff);
       if (st) {
         C.cs[c] = static_cast<unsigned short>(e);
         C.ccol[c] = static_cast<unsigned short>(col);
@@ -477,21 +484,13 @@ __device__ void fcoefs(const FCtx& C, const float2* v, float2 (&cf)[R]) {
   constexpr int G = 32 / N;
   if (lane % G == 0) C.red[w * 2 * kMaxR + lane / G] = t;
   __syncthreads();
+  // every warp adds the partials, lane = value, and hands them round
+  float s = 0.f;
+#pragma unroll 8
+  for (int ww = 0; ww < C.nw; ++ww) s += C.red[ww * 2 * kMaxR + lane];
 #pragma unroll
-  for (int l = 0; l < R; ++l) cf[l] = make_float2(0.f, 0.f);
-  for (int ww = 0; ww < C.nw; ++ww) {
-    const float4* from = reinterpret_cast<const float4*>(C.red + ww * 2 * kMaxR);
-#pragma unroll
-    for (int l = 0; l < R; l += 2) {
-      const float4 f = from[l / 2];
-      cf[l].x += f.x;
-      cf[l].y += f.y;
-      if (l + 1 < R) {
-        cf[l + 1 < R ? l + 1 : 0].x += f.z;
-        cf[l + 1 < R ? l + 1 : 0].y += f.w;
-      }
-    }
-  }
+  for (int l = 0; l < R; ++l)
+    cf[l] = make_float2(__shfl_sync(0xffffffffu, s, 2 * l), __shfl_sync(0xffffffffu, s, 2 * l + 1));
 }
 
 // v <- v + sign Q cf; returns this thread's part of ||v||^2
@@ -798,8 +797,7 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
   C.spo = reinterpret_cast<int*>(sm + cv.gv);
   C.vn = reinterpret_cast<float2*>(sm + cv.vn);
   C.ord = reinterpret_cast<unsigned short*>(sm + cv.ord);
-  C.prow = reinterpret_cast<unsigned short*>(sm + cv.prow);
-  C.cof = reinterpret_cast<unsigned short*>(sm + cv.cof);
+  C.ent = reinterpret_cast<int*>(sm + cv.ent);
   C.cs = reinterpret_cast<unsigned short*>(sm + cv.cs);
   C.ccol = reinterpret_cast<unsigned short*>(sm + cv.ccol);
   C.pcs = reinterpret_cast<unsigned short*>(sm + cv.pcs);
