@@ -102,7 +102,8 @@ typedef struct {
   int32_t slab_mode;        /* Gaussian sweep: 0 auto, 1 slab resident in shared
                                memory, 2 slab streamed through a tile ring   */
   int32_t stages;           /* tile stages of the streamed ring (0 -> auto)    */
-  int32_t engine;           /* Gaussian sweep engine: 0 auto, 1 one thread-block
+  int32_t engine;           /* Gaussian sweep engine: 0 auto (the streaming
+                               engine where it fits), 1 one thread-block
                                cluster per column, 2 persistent task engine
                                (passes over A_k split into tasks, columns
                                in flight share the GPU), 3 register-resident
@@ -447,7 +448,7 @@ const char* lrs_server_last_error(void);
  * the IHT step's parts: loads, mu, HardThreshold, next residual, publish.
  * A DFT2D_MASK handle gives 8 counters (thread-0 cycles summed over the
  * frames' CTAs): set-up and Gram, sparse DFTs, norms and updates, FFTs,
- * HardThreshold, final stage, LS solves, projection applies.
+ * HardThreshold, final stage, projections' Q^H v, projections' v - Q c.
  * len is the capacity of out in elements.  Counters restart at zero.
  * Errors: LRS_ERR_ARG, LRS_ERR_STATE (no trace buffer), LRS_ERR_CUDA. */
 lrs_status lrs_sweep_trace(lrs_t h, uint64_t* out, int64_t len);

@@ -154,7 +154,9 @@ __device__ __forceinline__ void dit_side(float2* X, int nl, int ls, int es, int 
 // direct DFT.
 //
 // One CTA per frame kept r of the 152 SMs busy (26 us at 128 x 128, r = 6); a
-// launch per side was faster there and slower on frames up to 64 x 64.
+// One CTA per frame kept r of the 152 SMs busy (26 us at 128 x 128, r = 6; with
+// the k-space sums 53 us per iteration, now 26). A launch per side was faster
+// there (39 us) and slower on frames up to 64 x 64 (22 us against 20; now 17).
 constexpr int kFC = 8;    // CTAs per frame
 constexpr int kFCT = 256;
 

@@ -24,6 +24,13 @@
 // on the support alone: no 2D FFT (the 1e-3 covers the rounding of u, mu and of
 // the FFT, about 1e-6 ||u|| against N >= 1 / 128).  The test is made on the
 // sweep's own mu and v; a sweep that fails it takes the FFT.
+//
+// Bound: instruction issue (593 K warp instructions per 128 x 128 frame, issue
+// slots 43 % used, shared-memory wavefronts 28 % of peak). A sweep with an FFT
+// costs 31 K cycles for it and about 12 K for HardThreshold, one without 20 K for
+// the adjoint. n = 128 x 128, q = 256, r = 6, m = 2048, rho = 82, relative error
+// 2e-2: 497 -> 353 us with F2 U; 64 x 64, q = 99, r = 4: 145 -> 112; 20 x 20, q =
+// 400: 215 -> 55.
 #pragma once
 
 #include "fourier_dev.cuh"
