@@ -786,6 +786,7 @@ struct FourierSolver {
   int* asv = nullptr;      // q flags: AS[k] matches the current s_k
   unsigned long long* prof = nullptr;  // kFProf sweep cycle counters (profiling)
   void* sweep = nullptr;   // fsweep_kernel of the rank width
+  bool lean = false;       // no room for its tables
   int tb = 0, qmode = 0;   // its table's columns and Q_k's place (FArgs)
   size_t smem = 0;
 };
@@ -828,7 +829,7 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     F->g.sxL = F->g.L / nx;
     F->g.syL = F->g.L / ny;
     F->g.lL = ilog2(F->g.L);
-    const double span = static_cast<double>(std::max(nx, ny)) * F->g.L * F->g.L;
+    const double span = 2.0 * std::max(nx, ny) * F->g.L * F->g.L;
     F->g.magic = span < 4294967296.0 ? static_cast<unsigned>((0x100000000ull + F->g.L - 1) / F->g.L) : 0u;
   }
   F->m = m;
@@ -868,7 +869,7 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
   const size_t share = ctas == 1 ? room : (room + 1024) / ctas - 1024 - kFStaticSmem;
   const int want = m >= 2 * nx ? std::min(std::max(1, rho), ny) : 0;
   bool vglob = false;
-  auto total = [&](bool vg, int tb, bool qs) { return fcarve(F->g, m, r, rho, vg, tb, qs).total; };
+  auto total = [&](bool vg, int tb, bool qs) { return fcarve(F->g, m, r, rho, vg, tb, qs, false).total; };
   auto plan = [&](size_t limit, int least) {  // the most that fits, or false
     for (int vg = 0; vg < 2; ++vg) {
       int tb = want;
@@ -883,7 +884,11 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     }
     return false;
   };
-  if (!plan(share, std::min(want, 4)) && !plan(room, std::min(want, 4))) F->smem = room + 1;
+  if (!plan(share, std::min(want, 4)) && !plan(room, std::min(want, 4))) {
+    F->lean = vglob = true;
+    F->tb = F->qmode = 0;
+    F->smem = fcarve(F->g, m, r, rho, true, 0, false, true).total;
+  }
   if (F->smem > room || fft_carve(F->g).total > static_cast<size_t>(optin)) {
     *msg = "frame too large for one CTA's shared memory (n <= 16384 fits)";
     delete F;
@@ -1046,6 +1051,7 @@ static cudaError_t launch_fsweep(FourierSolver* F, int mode, int tau) {
   a.asv = F->asv;
   a.prof = F->prof;
   a.tb = F->tb;
+  a.lean = F->lean;
   a.qmode = F->qmode;
   void* args[] = {&a};
   return cudaLaunchKernel(F->sweep, dim3(F->q), dim3(fsweep_threads(F->g.n)), args, F->smem, F->s);

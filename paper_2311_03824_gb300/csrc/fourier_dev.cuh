@@ -386,9 +386,9 @@ __device__ __forceinline__ int fcol(const Geo& g, int e) {
 }
 __device__ __forceinline__ int fwrapx(const Geo& g, int v) { return g.lnx >= 0 ? v & (g.nx - 1) : v % g.nx; }
 __device__ __forceinline__ int fwrapy(const Geo& g, int v) { return g.lny >= 0 ? v & (g.ny - 1) : v % g.ny; }
-// v mod L, 0 <= v < max(nx, ny) L.  floor(v / L) = (v magic) >> 32 while
+// v mod L, 0 <= v < 2 max(nx, ny) L.  floor(v / L) = (v magic) >> 32 while
 // v (magic L - 2^32) < 2^32, which v L < 2^32 ensures; the host sets magic
-// only when max(nx, ny) L^2 < 2^32 (an integer division costs about 20
+// only when 2 max(nx, ny) L^2 < 2^32 (an integer division costs about 20
 // instructions, and the sparse DFTs take one per term).
 __device__ __forceinline__ int fwrapL(const Geo& g, int v) {
   if (g.lL >= 0) return v & (g.L - 1);

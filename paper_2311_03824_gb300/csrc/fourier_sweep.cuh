@@ -42,6 +42,7 @@ struct FArgs {
   Geo g;
   int m, q, r, rho, tau, mode;
   int tb;               // support columns of the sparse DFT's table beside the frame
+  int lean;             // no room for the tables (fcarve)
   int qmode;            // Q_k: 0 in Wk, 1 in shared memory, 2 in the frame's place
                         // while no FFT needs it (kept in Wk meanwhile)
   const float2* y;      // q x m
@@ -86,7 +87,9 @@ __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~size_t(15)
 
 // Shared-memory carve of the sweep; with vglob the two m-vectors live in global
 // memory (FArgs::vecs) and take no space.  T for tb support columns, Q when own_q.
-__host__ __device__ inline FCarve fcarve(const Geo& g, int m, int r, int rho, bool vglob, int tb, bool own_q) {
+// lean (tall frames, or m near n, that leave no room): no T (tb is 0, sparse
+// products term by term), the Gram's scratch in the frame's place.
+__host__ __device__ inline FCarve fcarve(const Geo& g, int m, int r, int rho, bool vglob, int tb, bool own_q, bool lean) {
   FCarve c;
   size_t o = 0;
   const size_t rh = rho > 0 ? rho : 1;
@@ -100,23 +103,23 @@ __host__ __device__ inline FCarve fcarve(const Geo& g, int m, int r, int rho, bo
     o += al16(bytes);
     return at;
   };
-  c.X = put(frame);
+  c.X = put(lean && gram > frame ? gram : frame);
   c.tx = put(static_cast<size_t>(g.nx) * 8);
   c.ty = put(static_cast<size_t>(g.ny) * 8);
   c.tl = put(static_cast<size_t>(g.L) * 8);
   c.dv = put(mv);
   c.ev = put(mv);
   c.msk = put(static_cast<size_t>(m) * 4);
-  c.rptr = put(static_cast<size_t>(g.nx + 1) * 4);
+  c.rptr = put(tb ? static_cast<size_t>(g.nx + 1) * 4 : 0);
   c.sp = put(rh * 4);
   c.sv = put(rh * 8);
   c.gv = put(rh * 8);
   c.vn = put(rh * 8);
-  c.ord = put(rh * 2);
-  c.ent = put(rh * 4);
-  c.cs = put((rh + 1) * 2);
-  c.ccol = put(rh * 2);
-  c.pcs = put((rh + 1) * 2);
+  c.ord = put(tb ? rh * 2 : 0);
+  c.ent = put(tb ? rh * 4 : 0);
+  c.cs = put(tb ? (rh + 1) * 2 : 0);
+  c.ccol = put(tb ? rh * 2 : 0);
+  c.pcs = put(tb ? (rh + 1) * 2 : 0);
   c.Li = put(kMaxR * kMaxR * 16);
   c.Lf = put(kMaxR * kMaxR * 8);
   c.red = put(static_cast<size_t>(nw) * 2 * kMaxR * 4);
@@ -126,7 +129,7 @@ __host__ __device__ inline FCarve fcarve(const Geo& g, int m, int r, int rho, bo
   c.cl = put(static_cast<size_t>(kCandCap) * 8);
   // T; before the first sweep, the Gram's partial sums, G and L
   const size_t tab = tb ? static_cast<size_t>(tb | 1) * g.nx * 8 : 0;
-  c.T = put(tab > gram ? tab : gram);
+  c.T = put(lean ? 0 : tab > gram ? tab : gram);
   c.Q = put(own_q ? static_cast<size_t>(r) * m * 8 : 0);
   c.total = o;
   return c;
@@ -223,7 +226,7 @@ __device__ inline void sparse_direct(const FCtx& C, const float2* v, int nnz, fl
       const float2 ve = v[e];
 #pragma unroll
       for (int u = 0; u < kSdPer; ++u)
-        acc[u] = cfma(cmul(C.tl[fwrapL(C.g, kx[u] * qx)], C.tl[fwrapL(C.g, ky[u] * qy)]), ve, acc[u]);
+        acc[u] = cfma(C.tl[fwrapL(C.g, kx[u] * qx + ky[u] * qy)], ve, acc[u]);
     }
 #pragma unroll
     for (int u = 0; u < kSdPer; ++u) {
@@ -776,7 +779,7 @@ __device__ inline bool fthreshold(const FCtx& C, float mu, float& gmax2) {
 template <int R, bool P2>
 __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
-  const FCarve cv = fcarve(a.g, a.m, a.r, a.rho, a.vecs != nullptr, a.tb, a.qmode == 1);
+  const FCarve cv = fcarve(a.g, a.m, a.r, a.rho, a.vecs != nullptr, a.tb, a.qmode == 1, a.lean != 0);
   FCtx C;
   C.g = a.g;
   if constexpr (P2) {
@@ -815,7 +818,7 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
   C.hist = reinterpret_cast<int*>(sm + cv.hist);
   C.cand = reinterpret_cast<int*>(sm + cv.cand);
   C.cl = reinterpret_cast<unsigned long long*>(sm + cv.cl);
-  C.T = reinterpret_cast<float2*>(sm + cv.T);
+  C.T = a.lean ? C.X : reinterpret_cast<float2*>(sm + cv.T);
   float2* const Qg = a.qmode == 1 ? nullptr : a.Wk + static_cast<size_t>(k) * r * m;
   C.Q = a.qmode == 0 ? Qg : a.qmode == 1 ? reinterpret_cast<float2*>(sm + cv.Q) : C.X;
   C.err = a.err;
@@ -898,13 +901,13 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
       C.sp[pos] = p;
       C.sv[pos] = init ? make_float2(0.f, 0.f) : a.S_val[static_cast<size_t>(k) * rho + e];
     }
-    for (int i = threadIdx.x; i <= m; i += blockDim.x) {  // samples by frequency row (ascending)
+    for (int i = threadIdx.x; a.tb > 0 && i <= m; i += blockDim.x) {  // samples by frequency row (ascending)
       const int x0 = i > 0 ? frow(C.g, C.msk[i - 1]) : -1, x1 = i < m ? frow(C.g, C.msk[i]) : C.g.nx;
       for (int x = x0 + 1; x <= x1; ++x) C.rptr[x] = i;
     }
     asc = __syncthreads_and(distinct) != 0;
   }
-  const bool by_cols = m >= 2 * C.g.nx;
+  const bool by_cols = a.tb > 0;
   int np = asc && by_cols ? support_cols(C, &np_s) : 0;
   // A x for values v on the support
   auto forward = [&](const float2* v, float2* out) {

@@ -25,11 +25,12 @@ def _need_gpu():
 
 # fewer samples than two per row; runs of more than four adjacent columns in a
 # 256-thread frame; a rank below its width; the basis in the frame's place; in
-# global memory (r m pixels do not fit the frame); the widest ranks
+# global memory (r m pixels do not fit the frame); the widest ranks; tall frames
+# that leave no room for the tables
 @pytest.mark.parametrize("nx,ny,q,r,m,rho,T", [
     (64, 4, 8, 2, 100, 3, 12), (32, 32, 10, 3, 400, 40, 12), (64, 64, 6, 5, 1300, 20, 12),
     (128, 128, 9, 7, 2300, 60, 4), (128, 128, 10, 8, 3000, 60, 4), (16, 16, 16, 9, 160, 3, 6),
-    (20, 20, 24, 13, 260, 3, 6)])
+    (20, 20, 24, 13, 260, 3, 6), (2048, 8, 4, 2, 4200, 6, 2), (2048, 8, 4, 3, 4200, 6, 2)])
 def test_sweep_one_step(nx, ny, q, r, m, rho, T):
     inst = FourierInstance(nx=nx, ny=ny, q=q, r=r, m=m, rho=rho, seed=50 + nx + r,
                            mask_law="uniform", b_law="gauss")
