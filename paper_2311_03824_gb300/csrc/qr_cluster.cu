@@ -189,10 +189,12 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
 
 template <int R>
 cudaError_t launch(const QrArgs& q, size_t smem, cudaStream_t s) {
-  // the limit is set for the largest request once per process and device
-  // (the attribute call is idempotent)
+  // A block has 48 KB without asking for more, and the kernel's static arrays
+  // (9.3 KB at R = 16) count: the limit of the largest request (idempotent) is
+  // set from 32 KB on, every time, since nothing says that this process and
+  // device had a larger call before.
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
+  if (smem > 32 * 1024)
     e = cudaFuncSetAttribute(qr_cluster_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kQrSmem);
   if (e != cudaSuccess) return e;
