@@ -122,8 +122,8 @@ typedef struct {
                                all that fit; fewer let concurrent handles on
                                other streams share the GPU); resident engine:
                                at most grid / cluster clusters             */
-  int32_t wait_ms;          /* bound of every device-side wait of the task and
-                               resident engines (0 -> 10000 ms); a wait that
+  int32_t wait_ms;          /* bound of every device-side wait of the task,
+                               streaming and resident engines (0 -> 10000 ms); a wait that
                                expires makes the call return LRS_ERR_TIMEOUT */
   int32_t grad_block;       /* columns per partial sum of the column reductions
                                (0 -> chosen for the grid; fixed when a
@@ -135,11 +135,13 @@ typedef struct {
   void* reduce_ctx;         /* first argument of reduce                        */
   int32_t reduce_cap;       /* partial blocks of all shards together (the `cap`
                                of reduce)                                    */
-  int32_t test_withhold;    /* test aid for the failure path (0 in use): the
+  int32_t test_withhold;    /* test aid for the failure path (0 in use): 1: the
                                task engine's queue holds one ticket that is
-                               never published, so the wait for it runs out
-                               after wait_ms and the call returns
-                               LRS_ERR_TIMEOUT with the device still usable  */
+                               never published; 2, 3: a copy of the streaming
+                               engine's W pass, of its column steps, is waited
+                               for longer than it is.  The wait runs out after
+                               wait_ms and the call returns LRS_ERR_TIMEOUT
+                               with the device still usable                  */
 } lrs_options;
 
 /* Create a solver for one problem (Section I-A sizes).

@@ -302,6 +302,7 @@ lrs_status launch_sweep(lrs_ctx* h, int mode, int tau) {
     T.cnt = h->s_cnt;
     T.list = h->s_list;
     T.ncnt = h->sshape[mode].te + 1;
+    T.withhold = h->opt.test_withhold;
     T.wait_ns = wait_bound_ns(h);
     CUDA_TRY(stream_sweep(T, h->sshape[mode], mode, h->sasg, h->n_sasg, h->stream));
     return LRS_OK;
@@ -1098,7 +1099,7 @@ lrs_status lrs_create(int64_t n, int64_t m, int64_t q, int32_t r, int32_t rho, l
     // The library's own choice is the streaming engine (a third of the task
     // engine's time at n = q = 1000 near convergence); options that only the
     // task engine has ask for that one.
-    const bool task_only = o.inflight || o.task_kib || o.ctas_per_sm || o.test_withhold || o.profile == 2;
+    const bool task_only = o.inflight || o.task_kib || o.ctas_per_sm || o.test_withhold == 1 || o.profile == 2;
     if (o.engine == 0 && !task_only && plan_stream(h, nsm)) h->engine = 4;
   }
   if (h->engine == 2) {

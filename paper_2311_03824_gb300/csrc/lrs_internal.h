@@ -257,6 +257,7 @@ struct StreamTable {
   int* cnt;                    // [ncnt] columns in the list of each round
   int* list;                   // [2][ncols] columns waiting for a pass (round & 1)
   int ncnt;
+  int withhold;                // test aid (lrs_options::test_withhold): 2 W pass, 3 column steps
   unsigned long long wait_ns;
 };
 constexpr int kStreamMaxRounds = 126;  // IHT sweeps of a problem (counters: one per round)

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   P.init(static_cast<unsigned>(wid * S) * stage,
          reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(kSW) * S * stage) + wid * kMaxStage,
          stage, S, T.wait_ns);
-  P.err = T.probs[0].err;
   const int wk = blockIdx.x * kSW + wid, nw = gridDim.x * kSW;
   auto column = [&](int i) { return list ? list[i] : (final ? ncol - 1 - i : i); };
   // units (entry i of the list, tile b) in steps of all warps
@@ -120,6 +119,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
     const StreamProblem& pr = T.probs[prob_of(T, c)];
     if (b >= pr.L.ns / kTW) continue;
     const int k = c - pr.col0, m = pr.L.m;
+    P.err = pr.err;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i0 = 0; i0 < m; i0 += rp) {
       const unsigned char* st = smem + P.take();

@@ -36,8 +36,9 @@
 // CTAs or on the other problems of the launch, so results are the same alone,
 // in a batch, under any grid and in a column-sharded solve.
 //
-// Every wait is bounded by wait_ns; on expiry the warp records kErrTimeout,
-// drains its own copies (bounded) and leaves.
+// Every wait is bounded by wait_ns; on expiry the warp (of a column step: the
+// CTA) records kErrTimeout, drains its own copies (bounded) and leaves, with no
+// barrier armed again.
 #pragma once
 
 #include "sweep_gauss_impl.cuh"
@@ -58,6 +59,14 @@ __device__ __forceinline__ unsigned long long gtimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+__device__ __forceinline__ bool wait_phase(uint64_t* bar, unsigned parity, unsigned long long wait_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const unsigned long long t0 = gtimer();
+  while (!mbar_try_wait(bar, parity))
+    if (gtimer() - t0 > wait_ns) return false;
+  return true;
 }
 
 // ------------------------------------------------------------- warp pipeline --
@@ -99,14 +108,7 @@ struct Pipe {
     ++flying;
     si = si + 1 == S ? 0 : si + 1;
   }
-  __device__ bool wait() const {
-    uint64_t* bar = full + st;
-    if (mbar_try_wait(bar, ph)) return true;
-    const unsigned long long t0 = gtimer();
-    while (!mbar_try_wait(bar, ph))
-      if (gtimer() - t0 > wait_ns) return false;
-    return true;
-  }
+  __device__ bool wait() const { return wait_phase(full + st, ph, wait_ns); }
   // the oldest piece in flight (every lane waits); taken() when it has been read
   __device__ unsigned take() {
     if (!__all_sync(0xffffffffu, wait())) {
@@ -186,6 +188,8 @@ __global__ void __launch_bounds__(kStreamNT, 2)
              wid * kMaxStage,
          stage, S, T.wait_ns);
   if (blockIdx.x == 0 && threadIdx.x < T.ncnt) T.cnt[threadIdx.x] = 0;
+  // test aid: the first piece waits for 16 bytes that no copy brings
+  unsigned extra = T.withhold == 2 && blockIdx.x == 0 && wid == 0 ? 16u : 0u;
   for (int a = blockIdx.x; a < nasg; a += gridDim.x) {
     const StreamAssign as = asg[a];
     const StreamProblem& pr = T.probs[as.prob];
@@ -219,7 +223,8 @@ __global__ void __launch_bounds__(kStreamNT, 2)
       const int nt = min(tpp, b1 - pbt);
       const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
       unsigned char* dst = smem + P.issue_at();
-      if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt);
+      if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt + extra);
+      extra = 0u;
       __syncwarp();
       if (lane < nt * planes) {
         const int t = lane / planes, pl = lane - t * planes;
@@ -481,24 +486,29 @@ struct Step {
       if (threadIdx.x == 0 && rho > 0) {
         asm volatile("fence.proxy.async;" ::: "memory");  // earlier reads of the buffer first
         const unsigned bytes = static_cast<unsigned>(rho * as * 4);
-        mbar_arrive_expect_tx(bar, bytes);
+        mbar_arrive_expect_tx(bar, bytes + (T.withhold == 3 ? 16u : 0u));  // (test aid)
         bulk_copy_g2s(ag, ag_global(), bytes, bar);
       }
     }
   }
-  __device__ void stage_end(uint64_t* bar, unsigned& phase) const {
+  // Every thread waits for the copy; false when the wait ran out: the CTA then
+  // leaves by stage_abandon.
+  __device__ bool stage_end(uint64_t* bar, unsigned& phase) const {
+    bool ok = true;
     if constexpr (step_staged(V)) {
       if (rho > 0) {
-        if (!mbar_try_wait(bar, phase)) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(bar, phase))
-            if (gtimer() - t0 > T.wait_ns) {
-              report_error(pr.err, kErrTimeout, -1);
-              break;
-            }
-        }
+        ok = wait_phase(bar, phase, T.wait_ns);
         phase ^= 1u;
       }
+    }
+    return ok;
+  }
+  // the copy may still be under way: one more bounded wait, after which the CTA
+  // goes without touching the barrier or the buffer again
+  __device__ void stage_abandon(uint64_t* bar, unsigned phase) const {
+    if (threadIdx.x == 0) {
+      report_error(pr.err, kErrTimeout, -1);
+      wait_phase(bar, phase ^ 1u, T.wait_ns);
     }
   }
 
@@ -971,11 +981,13 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 8 : 3)
     __syncthreads();
     s.nl = snl;
     s.factor();
-    s.stage_end(&abar, phase);
+    if (!__syncthreads_and(s.stage_end(&abar, phase))) {
+      s.stage_abandon(&abar, phase);
+      break;
+    }
     if (s.nl != rho) {
       // entries of the given support were dropped: the columns of the others
       // move down to their slots (in AG_k too, where the next step finds them)
-      __syncthreads();
       for (int i = threadIdx.x; i < m; i += NT) {
         int at = 0;
         for (int e = 0; e < rho; ++e) {
@@ -987,8 +999,8 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 8 : 3)
           ++at;
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
     if (spr.mode == kModeLS || s.te == 0) {
       s.finish(spr.mode == kModeIter);
       continue;
@@ -1128,8 +1140,10 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
       for (int t = threadIdx.x; t < 256; t += NT) s.G[512 + t] = spr.Li[static_cast<size_t>(k) * 256 + t];
     }
     for (int j = threadIdx.x; j < n; j += NT) vv[j] = __ldcg(g + j);
-    if (!zero) s.stage_end(&abar, phase);
-    __syncthreads();
+    if (!__syncthreads_and(zero || s.stage_end(&abar, phase))) {
+      s.stage_abandon(&abar, phase);
+      break;
+    }
     if (zero) {
       // support of the zero start
       const int K = topk_radix<NT>(vv, n, rho, hist, ties, sel);

@@ -133,3 +133,25 @@ def test_autotune_call_keeps_the_iterate():
             assert np.array_equal(a, b)
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("withhold", [2, 3])
+def test_expired_wait_returns_timeout_and_the_device_stays_usable(withhold):
+    """Failure detection without a fault: one copy of the W pass (2), or those of
+    the column steps (3), are waited for 16 bytes beyond what they bring.  The
+    waits run out after 100 ms, the warp (the CTA, which has other columns to
+    come: two CTAs of the streaming grid) leaves, and the call reports
+    LRS_ERR_TIMEOUT.  A solver created afterwards runs normally."""
+    from paper_2311_03824_gb300 import lrs as L
+    inst = GaussianInstance(n=64, q=40, r=2, m=32, rho=2, seed=7)
+    good = run(inst, 4, grid=2)
+    s = new_solver(inst, grid=2, wait_ms=100, test_withhold=withhold)
+    try:
+        assert L.lrs_describe(s.h)["engine"] == "stream"
+        with pytest.raises(L.LrsError) as e:
+            s.init()
+        assert e.value.status == L.LRS_ERR_TIMEOUT, str(e.value)
+    finally:
+        s.close()
+    for x, y in zip(good, run(inst, 4, grid=2)):
+        assert np.array_equal(x, y)
