@@ -257,8 +257,11 @@ lrs_status lrs_get_x(lrs_t h, void* X, int32_t mem_kind);
 
 /* Restore a state written by lrs_get (same layouts, host or device), so that
  * a run can be resumed: t is the number of iterations already done and eta
- * the frozen step size (ignored when t == 0).  State: MEASURED or later ->
- * INITIALISED (t == 0) or ITERATING.  Errors: LRS_ERR_ARG, LRS_ERR_STATE,
+ * the frozen step size (ignored when t == 0).  S_k is taken as the vector
+ * that its entries add up to: those outside [0, n) are dropped, the values of
+ * a repeated index are added, and the support is completed to rho_max distinct
+ * indices as HardThreshold would (lowest other indices, value zero).  State:
+ * MEASURED or later -> INITIALISED (t == 0) or ITERATING.  Errors: LRS_ERR_ARG, LRS_ERR_STATE,
  * LRS_ERR_CUDA. */
 lrs_status lrs_set_state(lrs_t h, const void* U, const void* B,
                          const int32_t* S_idx, const void* S_val, int32_t t,

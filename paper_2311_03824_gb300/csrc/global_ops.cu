@@ -351,7 +351,70 @@ __global__ void sum_fin_kernel(int nblk, const double* __restrict__ part, double
   }
 }
 
+// set_support (lrs_internal.h), a warp per column: one pass over a support that
+// is strictly ascending and in range (every support that the library has
+// written), else the warp compares each entry with the ones before it.
+__global__ void __launch_bounds__(128) support_kernel(int n, int q, int rho, int w, const int* src_idx,
+                                                      const float* src_val, int* dst_idx, float* dst_val) {
+  const int lane = threadIdx.x & 31, k = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (k >= q) return;
+  const size_t at = static_cast<size_t>(k) * rho;
+  int* idx = dst_idx + at;
+  float* val = dst_val + at * w;
+  bool ok = true;
+  for (int e = lane; e < rho; e += 32) {
+    const int j = src_idx[at + e];
+    ok = ok && j >= 0 && j < n && (e == 0 || src_idx[at + e - 1] < j);
+    if (src_idx != dst_idx) {
+      idx[e] = j;
+      for (int c = 0; c < w; ++c) val[e * w + c] = src_val[(at + e) * w + c];
+    }
+  }
+  if (__all_sync(0xffffffffu, ok)) return;
+  __syncwarp();
+  // first entry before e (of rho: anywhere) that holds j, or -1
+  auto find = [&](int j, int e) {
+    for (int f0 = 0; f0 < e; f0 += 32) {
+      const unsigned hit = __ballot_sync(0xffffffffu, f0 + lane < e && idx[f0 + lane] == j);
+      if (hit) return f0 + __ffs(hit) - 1;
+    }
+    return -1;
+  };
+  int free = 0;
+  for (int e = 0; e < rho; ++e) {
+    const int j = idx[e];
+    const bool in = j >= 0 && j < n;
+    const int f = in ? find(j, e) : -1;
+    if (in && f < 0) continue;
+    ++free;
+    __syncwarp();
+    if (lane == 0) {
+      idx[e] = -1;
+      for (int c = 0; c < w; ++c) {
+        if (f >= 0) val[f * w + c] += val[e * w + c];
+        val[e * w + c] = 0.f;
+      }
+    }
+    __syncwarp();
+  }
+  int e = 0;
+  for (int j = 0; free > 0; ++j) {
+    if (find(j, rho) >= 0) continue;
+    while (idx[e] >= 0) ++e;
+    --free;
+    __syncwarp();
+    if (lane == 0) idx[e] = j;
+    __syncwarp();
+  }
+}
+
 }  // namespace
+
+cudaError_t set_support(int n, int q, int rho, int w, const int* src_idx, const float* src_val, int* idx,
+                        float* val, cudaStream_t s) {
+  support_kernel<<<(q + 3) / 4, 128, 0, s>>>(n, q, rho, w, src_idx, src_val, idx, val);
+  return cudaGetLastError();
+}
 
 cudaError_t subspace_change(const GlobalWork& g, const float* Uold, const float* Unew,
                             double* D_rr, double* out, cudaStream_t s) {

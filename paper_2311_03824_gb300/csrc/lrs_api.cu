@@ -1750,8 +1750,16 @@ lrs_status lrs_set_state(lrs_t h, const void* U, const void* B, const int32_t* S
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemcpyAsync(h->Bk, B, sizeof(float) * h->q * h->r, kin, h->stream));
   if (h->rho) {
-    CUDA_TRY(cudaMemcpyAsync(h->S_idx, S_idx, sizeof(int) * h->q * h->rho, kin, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(h->S_val, S_val, sizeof(float) * h->q * h->rho, kin, h->stream));
+    const int* si = S_idx;
+    const float* sv = static_cast<const float*>(S_val);
+    if (!mem_kind) {
+      CUDA_TRY(cudaMemcpyAsync(h->S_idx, S_idx, sizeof(int) * h->q * h->rho, kin, h->stream));
+      CUDA_TRY(cudaMemcpyAsync(h->S_val, S_val, sizeof(float) * h->q * h->rho, kin, h->stream));
+      si = h->S_idx;
+      sv = h->S_val;
+    }
+    CUDA_TRY(set_support(static_cast<int>(h->n), static_cast<int>(h->q), h->rho, 1, si, sv, h->S_idx,
+                         h->S_val, h->stream));
   }
   CUDA_TRY(cudaMemcpyAsync(h->eta, &eta, sizeof(double), cudaMemcpyHostToDevice, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));

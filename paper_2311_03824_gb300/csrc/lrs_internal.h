@@ -374,6 +374,13 @@ cudaError_t eta_from_grad(const GlobalWork& g, double c_eta, double* eta_dev, cu
 // parts == g.grad).
 cudaError_t qr_step(const GlobalWork& g, float* U, const float* parts, int nparts,
                     const double* eta_dev, int* err, cudaStream_t s);
+// The supports of a caller's state (q x rho indices, values of w floats) as
+// HardThreshold of the dense s_k keeps them: rho distinct indices in [0, n).
+// Entries outside the column are dropped, the values of a repeated index are
+// added, and what that leaves free goes to the lowest other indices with value
+// zero (ties at zero go to the lower index).  Order as given.  (src may be dst.)
+cudaError_t set_support(int n, int q, int rho, int w, const int* src_idx, const float* src_val, int* idx,
+                        float* val, cudaStream_t s);
 // Cholesky-QR2 of X - eta sum of the blocks on one cluster (qr_cluster.cu).
 constexpr int kQrSmem = 200 * 1024;  // shared memory of the matrix rows of a CTA
 bool qr_cluster_fits(int n, int r);

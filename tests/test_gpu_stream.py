@@ -155,3 +155,82 @@ def test_expired_wait_returns_timeout_and_the_device_stays_usable(withhold):
         s.close()
     for x, y in zip(good, run(inst, 4, grid=2)):
         assert np.array_equal(x, y)
+
+
+def given_support_steps(P, s, log, ts, outside):
+    """One step from the oracle's iterates with the support of every odd column
+    cut to its first half, in the ways a caller may write that: an index again
+    with value zero, a value in two parts, entries outside the column.  Each is
+    the step from the dense s_k and the support that HardThreshold gives it."""
+    import oracle.altgdmin_lrs as O
+    from paper_2311_03824_gb300 import lrs as L
+    from tests.gpu_helpers import compare_step, probe_step, state_of
+    ct = np.complex64 if P.cplx else np.float32
+    recs = []
+    for t in ts:
+        st = state_of(log, t, P.n)
+        Si, rho = st.S_idx.astype(np.int32), st.S_idx.shape[1]
+        keep = rho // 2
+        for k in range(1, P.q, 2):
+            st.S[k, st.S_idx[k, keep:]] = 0
+        vals = np.take_along_axis(st.S, st.S_idx, 1).astype(ct)
+        st.S = st.S.astype(ct).astype(P.dt)
+        for k in range(1, P.q, 2):
+            st.S_idx[k] = O.hard_threshold(st.S[k:k + 1], rho)[0][0]
+        st64, _, dec, dev = probe_step(P, st)
+        for form in ("zero", "split", "outside"):
+            I, V = Si.copy(), vals.copy()
+            I[1::2, keep:] = outside if form == "outside" else I[1::2, :1]
+            V[1::2, keep:] = 7 if form == "outside" else 0
+            if form == "split":
+                V[1::2, 0] *= 0.5
+                V[1::2, -1] = V[1::2, 0]
+            L.lrs_set_state(s.h, np.ascontiguousarray(st.U.T, ct), np.ascontiguousarray(st.B.T, ct), I, V,
+                            st.t, float(st.eta or 0.0))
+            got = s.get()[2]
+            assert np.array_equal(np.sort(got, 1), np.sort(st.S_idx, 1)), form
+            s.iterate(1)
+            recs.append(compare_step(st64, dec, s.get(), dev=dev))
+    return recs
+
+
+@pytest.mark.parametrize("engine", [0, 1, 2, 3])
+def test_given_support_with_repeats_and_entries_outside(engine):
+    from tests.gpu_helpers import Problem, check_records, oracle_run
+    inst = GaussianInstance(n=200, q=40, r=3, m=80, rho=6, seed=71)
+    P, (_, log) = Problem.gaussian(inst), oracle_run(inst, 4)
+    s = new_solver(inst, engine=engine)
+    try:
+        recs = given_support_steps(P, s, log, range(1, 4), [-1, 200, 2 ** 31 - 1])
+    finally:
+        s.close()
+    check_records(recs, min_whole=4, max_excluded=0.03)
+
+
+def test_state_on_the_device_and_unsorted():
+    """Device arrays take the same way; entries in another order are the same
+    support, and the output is ascending."""
+    import torch
+    from paper_2311_03824_gb300 import lrs as L
+    inst = GaussianInstance(n=1100, q=9, r=2, m=90, rho=40, seed=72)
+    outs = []
+    for how in ("host", "device", "unsorted"):
+        s = new_solver(inst)
+        try:
+            s.init()
+            U, B, Si, Sv = s.get()
+            a = [np.ascontiguousarray(U.T), np.ascontiguousarray(B.T), Si.copy(), Sv.copy()]
+            if how == "unsorted":
+                p = np.random.default_rng(1).permutation(40)
+                a[2], a[3] = np.ascontiguousarray(a[2][:, p]), np.ascontiguousarray(a[3][:, p])
+            if how == "device":
+                a = [torch.from_numpy(x).cuda() for x in a]
+            L.lrs_set_state(s.h, *a, 1, 1e-3)
+            s.iterate(2)
+            outs.append(s.get())
+        finally:
+            s.close()
+    for x, y, z in zip(*outs):
+        assert np.array_equal(x, y)
+        assert np.allclose(x, z, rtol=1e-4, atol=1e-5 * np.abs(x).max())
+    assert (np.diff(outs[2][2], axis=1) > 0).all()
