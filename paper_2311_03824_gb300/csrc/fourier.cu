@@ -1244,8 +1244,17 @@ int fourier_set_state(FourierSolver* F, const void* U, const void* B, const int*
   cudaMemcpyAsync(F->U, U, sizeof(float2) * n * F->r, k, F->s);
   cudaMemcpyAsync(F->B, B, sizeof(float2) * F->q * F->r, k, F->s);
   if (F->rho) {
-    cudaMemcpyAsync(F->S_idx, S_idx, sizeof(int) * F->q * F->rho, k, F->s);
-    cudaMemcpyAsync(F->S_val, S_val, sizeof(float2) * F->q * F->rho, k, F->s);
+    const int* si = S_idx;
+    const float* sv = static_cast<const float*>(S_val);
+    if (!mem_kind) {
+      cudaMemcpyAsync(F->S_idx, S_idx, sizeof(int) * F->q * F->rho, k, F->s);
+      cudaMemcpyAsync(F->S_val, S_val, sizeof(float2) * F->q * F->rho, k, F->s);
+      si = F->S_idx;
+      sv = reinterpret_cast<const float*>(F->S_val);
+    }
+    if (set_support(F->g.n, F->q, F->rho, 2, si, sv, F->S_idx, reinterpret_cast<float*>(F->S_val), F->s) !=
+        cudaSuccess)
+      return 4;
   }
   cudaMemsetAsync(F->asv, 0, sizeof(int) * F->q, F->s);  // a new s_k
   cudaMemcpyAsync(F->eta, &eta, sizeof(double), cudaMemcpyHostToDevice, F->s);

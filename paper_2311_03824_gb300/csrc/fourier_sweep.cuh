@@ -204,10 +204,9 @@ __device__ __forceinline__ float fget_max(const FCtx& C, int slot) {
 // ------------------------------------------------------------ sparse DFTs --
 constexpr int kSdPer = 4;  // frequencies a thread takes at once
 
-// out = A x for the pixels sp[e] in any order, values v[e], term by term: the
-// path of a support with repeated pixels (a caller's state may hold anything),
-// and of frames with fewer samples than two per row, where a table over kx is
-// no saving.  Ends with a barrier.
+// out = A x for the pixels sp[e], values v[e], term by term: frames with fewer
+// samples than two per row, where a table over kx is no saving, and those that
+// leave no room for it.  Ends with a barrier.
 __device__ inline void sparse_direct(const FCtx& C, const float2* v, int nnz, float2* out) {
   const float sc = rsqrtf(static_cast<float>(C.g.n));
   const int bd = blockDim.x;
@@ -882,21 +881,16 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
   // the support, sorted by pixel
   for (int e = threadIdx.x; e < rho; e += blockDim.x) C.spo[e] = init ? e : a.S_idx[static_cast<size_t>(k) * rho + e];
   __syncthreads();
-  bool asc = true;  // strictly ascending: distinct pixels
   {
     int inorder = 1;
     for (int e = threadIdx.x; e + 1 < rho; e += blockDim.x) inorder &= C.spo[e] < C.spo[e + 1];
     inorder = __syncthreads_and(inorder);
-    int distinct = 1;
     for (int e = threadIdx.x; e < rho; e += blockDim.x) {
       const int p = C.spo[e];
       int pos = e;
       if (!inorder) {
         pos = 0;
-        for (int f = 0; f < rho; ++f) {
-          pos += C.spo[f] < p || (C.spo[f] == p && f < e);
-          distinct &= f == e || C.spo[f] != p;
-        }
+        for (int f = 0; f < rho; ++f) pos += C.spo[f] < p;  // (distinct: lrs_set_state)
       }
       C.sp[pos] = p;
       C.sv[pos] = init ? make_float2(0.f, 0.f) : a.S_val[static_cast<size_t>(k) * rho + e];
@@ -905,13 +899,13 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
       const int x0 = i > 0 ? frow(C.g, C.msk[i - 1]) : -1, x1 = i < m ? frow(C.g, C.msk[i]) : C.g.nx;
       for (int x = x0 + 1; x <= x1; ++x) C.rptr[x] = i;
     }
-    asc = __syncthreads_and(distinct) != 0;
+    __syncthreads();
   }
   const bool by_cols = a.tb > 0;
-  int np = asc && by_cols ? support_cols(C, &np_s) : 0;
+  int np = by_cols ? support_cols(C, &np_s) : 0;
   // A x for values v on the support
   auto forward = [&](const float2* v, float2* out) {
-    if (!asc || !by_cols) sparse_direct(C, v, rho, out);
+    if (!by_cols) sparse_direct(C, v, rho, out);
     else sparse_cols(C, np, v, out, a.tb);
   };
   if (project) ffactor<R>(C);
@@ -985,7 +979,7 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
     if (have_ref) bound = fminf(bound, fmaf(N, dist, gmax));
     mark(2);
     // worth trying without the FFT: the bound with the last mu and the present s
-    bool cert = !zero_start && asc && by_cols && bound * mu_prev < sqrtf(smin);
+    bool cert = !zero_start && by_cols && bound * mu_prev < sqrtf(smin);
     bool stop = false;
     float mu = 0.f, den = 0.f;
     for (;;) {
@@ -1061,7 +1055,7 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
     if (cert) {
       for (int e = threadIdx.x; e < rho; e += blockDim.x) C.sv[e] = C.vn[e];
       dist = fmaf(mu, sqrtf(den), dist);
-    } else if (asc) {
+    } else {
       float g2 = 0.f;
       valid = fthreshold(C, mu, g2);
       have_ref = valid;
@@ -1071,20 +1065,6 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
         gmax = sqrtf(fget_max(C, 3));
         dist = mu * sqrtf(den);
       }
-    } else {  // v in the frame (repeated pixels of the given support: any one of them)
-      for (int e = threadIdx.x; e < C.g.nx * ld; e += blockDim.x) {
-        C.X[e].x *= -mu;
-        C.X[e].y *= -mu;
-      }
-      __syncthreads();
-      for (int e = threadIdx.x; e < rho; e += blockDim.x) {
-        const int p = C.sp[e];
-        C.X[frow(C.g, p) * ld + fcol(C.g, p)] = C.vn[e];
-      }
-      __syncthreads();
-      fhard_threshold(C, true);
-      valid = have_ref = false;
-      asc = true;
     }
     if (valid) {  // s_new = s - mu g_G on the same support
       nn = 0.f;

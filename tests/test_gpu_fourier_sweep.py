@@ -75,3 +75,16 @@ def test_support_in_any_order(repeat):
     if not repeat:
         rel = np.linalg.norm(outs[0] - outs[1]) / np.linalg.norm(outs[0])
         assert rel <= 1e-5, rel
+
+
+@pytest.mark.parametrize("nx,ny,m", [(32, 32, 400), (20, 12, 140), (64, 4, 100)])
+def test_given_support_with_repeats_and_entries_outside(nx, ny, m):
+    from tests.test_gpu_stream import given_support_steps
+    inst = FourierInstance(nx=nx, ny=ny, q=6, r=2, m=m, rho=8, seed=61, mask_law="uniform", b_law="gauss")
+    _, log = O.run_alg1(O.FourierOperator(inst.masks, nx, ny), inst.Y, 2, 8, 4, keep=tuple(range(5)), Xstar=inst.Xstar)
+    s = new_fourier_solver(inst)
+    try:
+        recs = given_support_steps(Problem.fourier(inst), s, log, range(1, 4), [-1, nx * ny, 2 ** 31 - 1, -2 ** 31])
+    finally:
+        s.close()
+    check_records(recs, min_whole=2, max_excluded=0.1)
