@@ -7,13 +7,16 @@
 // keeps n / 8 rows; the two Grams are exchanged through distributed shared
 // memory (two cluster barriers) and every CTA factors them redundantly.
 //   Pass 1: Gram in double-float from exact products, summed over the CTAs in
-//     FP64; Cholesky in FP32 when every pivot is above 1e-3 of its diagonal,
-//     else in FP64 (R1 needs to be good enough only for the second pass to
-//     start from a Gram near I: any upper triangular R1 leaves Q unchanged).
+//     FP64; Cholesky in FP32 when every pivot is above 1e-3 of its diagonal
+//     (R1 needs to be good enough only for the second pass to start from a Gram
+//     near I: any upper triangular R1 leaves Q unchanged).
 //   Pass 2: the Gram is I + E; Cholesky and inverse are carried as deviations
 //     from I in FP32 (relative to E), so that Q = Q1 + Q1 H adds a correction
 //     known to about 1e-7 |E|, where a rounded R2^{-1} would put 6e-8 on every
-//     entry.  FP64 when E is not small.
+//     entry.
+//   When a factor fails (small pivots, E not small, a Gram outside float32's
+//   range: entries of Z beyond about 1e-15 .. 1e15) Gram and factor are done
+//   again in FP64, in every CTA alike, since all hold the same sums.
 #include "lrs_dev.cuh"
 #include "lrs_internal.h"
 
@@ -63,7 +66,7 @@ __device__ bool chol_f32(const double* G, float* Rinv, int r, bool dev) {
       inv[j] = 1.f / (1.f + l1);
       dinv[j] = -l1 * inv[j];
     } else {
-      ok = p > 1e-3f * static_cast<float>(G[j * kMaxR + j]) && p < 1e30f;
+      ok = p > 1e-3f * static_cast<float>(G[j * kMaxR + j]) && p > 1e-30f && p < 1e30f;
       inv[j] = rsqrtf(p);
     }
     a[j] *= inv[j];
@@ -94,9 +97,10 @@ template <int R>
 __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_kernel(QrArgs q) {
   extern __shared__ __align__(16) float Zt[];  // [R][ldz], column l of this CTA's rows
   constexpr int NE = R * (R + 1) / 2;
-  __shared__ double part[2][NE];
+  __shared__ double part[2][NE], part64[NE];
   __shared__ double G[kMaxR * kMaxR], Ld[kMaxR * kMaxR], Li[kMaxR * kMaxR], iL[kMaxR];
   __shared__ float Rinv[kMaxR * kMaxR];
+  __shared__ int factored;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, r = q.r;
   const unsigned rank = cluster_rank();
   const int lo = min(q.n, static_cast<int>(rank) * q.rows), cnt = min(q.n, lo + q.rows) - lo;
@@ -140,27 +144,47 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
       }
       if (lane == 0) part[pass][t] = static_cast<double>(hi) + static_cast<double>(lw);
     }
-    cluster_sync_all();
-    if (tid < r * (r + 1) / 2) {  // every CTA sums the parts in rank order
-      double s = 0.0;
+    auto sum_parts = [&](const double* p) {  // every CTA sums the parts in rank order
+      cluster_sync_all();
+      if (tid < r * (r + 1) / 2) {
+        double s = 0.0;
 #pragma unroll
-      for (int c = 0; c < kQC; ++c) s += *peer_ptr(&part[pass][tid], c);
-      int a = 0;
-      while ((a + 1) * (a + 2) / 2 <= tid) ++a;
-      const int b = tid - a * (a + 1) / 2;
-      G[a * kMaxR + b] = s;
-      G[b * kMaxR + a] = s;
-    }
-    __syncthreads();
-    if (w == 0 && !chol_f32<R>(G, Rinv, r, pass == 1)) {
-      if (!chol_inverse_warp(G, Ld, Li, iL, r, kMaxR) && lane == 0 && rank == 0)
-        report_error(q.err, kErrNotSPD, -1);
-      for (int t = lane; t < r * r; t += 32) {
-        const int a = t / r, b = t - a * r;
-        Rinv[a * kMaxR + b] = static_cast<float>(Li[b * kMaxR + a] - (pass == 1 && a == b ? 1.0 : 0.0));
+        for (int c = 0; c < kQC; ++c) s += *peer_ptr(p + tid, c);
+        int a = 0;
+        while ((a + 1) * (a + 2) / 2 <= tid) ++a;
+        const int b = tid - a * (a + 1) / 2;
+        G[a * kMaxR + b] = s;
+        G[b * kMaxR + a] = s;
       }
+      __syncthreads();
+    };
+    sum_parts(part[pass]);
+    if (w == 0) {
+      const bool ok = chol_f32<R>(G, Rinv, r, pass == 1);
+      if (lane == 0) factored = ok;
     }
     __syncthreads();
+    if (!factored) {
+      for (int t = w; t < r * (r + 1) / 2; t += kQT / 32) {
+        int a = 0;
+        while ((a + 1) * (a + 2) / 2 <= t) ++a;
+        const float *za = Zt + a * q.ldz, *zb = Zt + (t - a * (a + 1) / 2) * q.ldz;
+        double s = 0.0;
+        for (int i = lane; i < cnt; i += 32) s = __fma_rn(static_cast<double>(za[i]), static_cast<double>(zb[i]), s);
+        s = warp_sum(s);
+        if (lane == 0) part64[t] = s;
+      }
+      sum_parts(part64);
+      if (w == 0) {
+        if (!chol_inverse_warp(G, Ld, Li, iL, r, kMaxR) && lane == 0 && rank == 0)
+          report_error(q.err, kErrNotSPD, -1);
+        for (int t = lane; t < r * r; t += 32) {
+          const int a = t / r, b = t - a * r;
+          Rinv[a * kMaxR + b] = static_cast<float>(Li[b * kMaxR + a] - (pass == 1 && a == b ? 1.0 : 0.0));
+        }
+      }
+      __syncthreads();
+    }
     // rows times R^{-1} (pass 1) or I + H (pass 2), a thread per row
     for (int i = tid; i < cnt; i += kQT) {
       float z[R];
@@ -190,7 +214,7 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
 template <int R>
 cudaError_t launch(const QrArgs& q, size_t smem, cudaStream_t s) {
   // A block has 48 KB without asking for more, and the kernel's static arrays
-  // (9.3 KB at R = 16) count: the limit of the largest request (idempotent) is
+  // (10.6 KB at R = 16) count: the limit of the largest request (idempotent) is
   // set from 32 KB on, every time, since nothing says that this process and
   // device had a larger call before.
   cudaError_t e = cudaSuccess;

@@ -51,3 +51,45 @@ def test_shared_memory_limit_in_a_fresh_process():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+def _qr(Z):
+    import torch
+    from paper_2311_03824_gb300 import lrs as L
+    Zd = torch.from_numpy(np.ascontiguousarray(Z, np.float32)).cuda()
+    Qd = torch.empty_like(Zd)
+    L.lrs_orthonormalize(Zd, Qd)
+    return Qd.cpu().numpy().astype(np.float64)
+
+
+# n below, at and above the cluster kernel's rows and its size (n r = 409600),
+# beyond which the separate kernels run; n < 8 r
+@pytest.mark.parametrize("cond", [1.0, 20.0, 1e3, 1e5])
+@pytest.mark.parametrize("n,r", [(17, 16), (40, 6), (1000, 5), (25600, 16), (25700, 16), (70000, 7)], ids=str)
+def test_kernels_and_factors_of_any_condition(n, r, cond):
+    """The rows take r float32 products with entries of R^-1 in each pass:
+    ||Q - Q_exact||_F <= (r + 2) 2^-24 cond ||Q_exact||_F; Q^T Q - I, which the
+    second pass mends, is that of cond = 1."""
+    if not gpu_available():
+        pytest.skip("no CUDA device")
+    rng = np.random.default_rng(n + r)
+    Q0, _ = np.linalg.qr(rng.standard_normal((n, r)))
+    V, _ = np.linalg.qr(rng.standard_normal((r, r)))
+    Z = ((Q0 * np.geomspace(1.0, 1.0 / cond, r)) @ V.T).astype(np.float32)
+    Q = _qr(Z)
+    Qo, _ = O.qr_positive(Z.astype(np.float64))
+    assert np.linalg.norm(Q - Qo) <= (r + 2) * 2.0 ** -24 * cond * np.sqrt(r)
+    assert np.abs(Q.T @ Q - np.eye(r)).max() <= (r + 2) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("e", [-70, 62])
+@pytest.mark.parametrize("n,r", [(1000, 5), (300, 16), (70000, 7)], ids=str)
+def test_matrices_of_any_scale(n, r, e):
+    """Z times 2^e (the Gram's entries leave float32's range) and columns of
+    different scales: the same Q."""
+    if not gpu_available():
+        pytest.skip("no CUDA device")
+    Z = np.random.default_rng(n + r).standard_normal((n, r)).astype(np.float32)
+    Qo, _ = O.qr_positive(Z.astype(np.float64))
+    for Zs in (np.ldexp(Z, e), Z * np.exp2(np.linspace(0, e, r).round()).astype(np.float32)):
+        assert np.linalg.norm(_qr(Zs) - Qo) <= 3 * 2.0 ** -24 * np.linalg.norm(Qo)
