@@ -255,14 +255,12 @@ __device__ __forceinline__ void cgram_warp(const float2* W, size_t ld, int m, in
 
 // One warp: the complex Cholesky factor L of M (Gd: the sums of cgram_warp) and
 // L^{-1} in double-float in registers (lane = row, then lane = column; an FP64
-// factor through shared memory took 31 K cycles at r = 6); Lf is L^{-1} rounded,
-// or with dev its deviation from I.  A pivot below 1e-9 of its diagonal goes to
-// FP64 (scratch: 2 kMaxR^2 + kMaxR / 2 values).  False when M is not positive
-// definite; L is then I.
+// factor through shared memory took 31 K cycles at r = 6); Lf is L^{-1} rounded.
+// False, and nothing written, when a pivot is below 1e-9 of its diagonal or
+// outside float32's range (a NaN is).
 template <int R>
-__device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, double2* Li, float2* Lf) {
+__device__ bool cchol_df(const float2* Gd, int r, double2* Li, float2* Lf) {
   const int lane = threadIdx.x & 31;
-  double2* G = scratch;
   bool done = true;
   // M[i][q] = conj(W_i) W_q, q <= i: the conjugate of the sums
   cdf a[R];
@@ -292,7 +290,8 @@ __device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, 
 #pragma unroll
     for (int q = j + 1; q < R; ++q) a[q] = cdf_sub_mulc(a[q], a[j], cdf_shfl(a[j], q));
   }
-  if (done) {
+  if (!done) return false;
+  {
     cdf x[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) {  // column lane of L^{-1}
@@ -306,18 +305,20 @@ __device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, 
       if (lane < kMaxR && i < r) {
         Li[i * kMaxR + lane] = make_double2(static_cast<double>(x[i].x.h) + static_cast<double>(x[i].x.l),
                                               static_cast<double>(x[i].y.h) + static_cast<double>(x[i].y.l));
-        Lf[i * kMaxR + lane] = make_float2(dev && i == lane ? (x[i].x.h - 1.f) + x[i].x.l : x[i].x.h, x[i].y.h);
+        Lf[i * kMaxR + lane] = make_float2(x[i].x.h, x[i].y.h);
       }
-    }
-  } else if (lane < r) {
-    for (int q = 0; q <= lane; ++q) {
-      const float2 x = Gd[lane * lane + 2 * q], yv = q < lane ? Gd[lane * lane + 2 * q + 1] : make_float2(0.f, 0.f);
-      G[lane * kMaxR + q] = make_double2(static_cast<double>(x.x) + static_cast<double>(x.y),
-                                         -(static_cast<double>(yv.x) + static_cast<double>(yv.y)));
     }
   }
   __syncwarp();
-  if (done) return true;
+  return true;
+}
+
+// The same in FP64 from the lower triangle G of M (ld kMaxR), the first part of
+// scratch (2 kMaxR^2 + kMaxR / 2 values).  False when M is not positive
+// definite; L is then I.
+__device__ inline bool cchol_f64(int r, double2* scratch, double2* Li, float2* Lf) {
+  const int lane = threadIdx.x & 31;
+  const double2* G = scratch;
   double2* Lc = scratch + kMaxR * kMaxR;
   double* iL = reinterpret_cast<double*>(scratch + 2 * kMaxR * kMaxR);
   bool ok = true;
@@ -364,8 +365,7 @@ __device__ bool cchol_warp(const float2* Gd, int r, bool dev, double2* scratch, 
       }
       t = i < cc ? make_double2(0, 0) : make_double2(t.x * iL[i], t.y * iL[i]);
       Li[i * kMaxR + cc] = t;
-      Lf[i * kMaxR + cc] =
-            make_float2(static_cast<float>(t.x - (dev && i == cc ? 1.0 : 0.0)), static_cast<float>(t.y));
+      Lf[i * kMaxR + cc] = make_float2(static_cast<float>(t.x), static_cast<float>(t.y));
     }
   }
   __syncwarp();

@@ -547,8 +547,16 @@ __device__ void ffactor(const FCtx& C) {
     Gd[t] = make_float2(h, l);
   }
   __syncthreads();
-  if (threadIdx.x < 32 && !cchol_warp<R>(Gd, r, false, G, C.Li, C.Lf) && lane == 0)
-    report_error(C.err, kErrNotSPD, C.k);
+  if (threadIdx.x < 32 && !cchol_df<R>(Gd, r, C.Li, C.Lf)) {
+    if (lane < r)
+      for (int q = 0; q <= lane; ++q) {
+        const float2 x = Gd[lane * lane + 2 * q], y = q < lane ? Gd[lane * lane + 2 * q + 1] : make_float2(0.f, 0.f);
+        G[lane * kMaxR + q] = make_double2(static_cast<double>(x.x) + static_cast<double>(x.y),
+                                           -(static_cast<double>(y.x) + static_cast<double>(y.y)));
+      }
+    __syncwarp();
+    if (!cchol_f64(r, G, C.Li, C.Lf) && lane == 0) report_error(C.err, kErrNotSPD, C.k);
+  }
   __syncthreads();
   // Q_l = sum_{p <= l} W_p conj(L^{-1}[l][p])
   for (int i = threadIdx.x; i < C.m; i += blockDim.x) {

@@ -88,3 +88,60 @@ def test_given_support_with_repeats_and_entries_outside(nx, ny, m):
     finally:
         s.close()
     check_records(recs, min_whole=2, max_excluded=0.1)
+
+@pytest.mark.parametrize("e", [-40, 40])
+def test_measurements_of_any_scale(e):
+    """y scaled by a power of two scales B and S and leaves U, whether or not the
+    Grams of the initialisation (fourth powers of y) leave float32's range."""
+    inst = FourierInstance(nx=16, ny=16, q=24, r=2, m=140, rho=3, seed=63)
+    X = []
+    for k in (0, e):
+        s = new_fourier_solver(inst)
+        try:
+            f = np.float32(2.0 ** k)
+            s.set_measurements(np.ascontiguousarray(inst.Y, np.complex64) * f, np.ascontiguousarray(inst.masks, np.int32))
+            s.init()
+            s.iterate(10)
+            X.append(s.X() / f)
+        finally:
+            s.close()
+    assert np.linalg.norm(X[1] - X[0]) <= 1e-5 * np.linalg.norm(X[0])
+
+
+def test_cooperative_qr():
+    """128 x 128 frames at r = 12: the matrix does not fit one cluster."""
+    inst = FourierInstance(nx=128, ny=128, q=14, r=12, m=2500, rho=8, seed=64, mask_law="uniform", b_law="gauss")
+    _, log = O.run_alg1(O.FourierOperator(inst.masks, 128, 128), inst.Y, 12, 8, 2, keep=(0, 1, 2), Xstar=inst.Xstar)
+    s = new_fourier_solver(inst)
+    try:
+        recs = one_step(Problem.fourier(inst), s, log, range(2))
+    finally:
+        s.close()
+    check_records(recs, min_whole=1)
+
+
+@pytest.mark.parametrize("cond", [1.0, 30.0, 1e3, 1e4])
+@pytest.mark.parametrize("nx,ny,r", [(20, 20, 4), (64, 64, 6), (64, 64, 16), (4, 4, 7)], ids=str)
+def test_rows_of_the_step_are_rounded_once_a_pass(nx, ny, r, cond):
+    """A step of length zero is the QR of the state's own U.  One or two passes,
+    exact products and at least 45-bit factors leave a rounding to float32 each
+    (2^-24 relative per entry, the first one doubled at most by the second
+    factor): ||U1 - Q||_F <= 3 * 2^-24 ||Q||_F at any condition whose square the
+    factors resolve."""
+    from paper_2311_03824_gb300 import lrs as L
+    n = nx * ny
+    inst = FourierInstance(nx=nx, ny=ny, q=3, r=r, m=n - n // 4, rho=2, seed=65, mask_law="uniform", b_law="gauss")
+    rng = np.random.default_rng(r)
+    Q0, _ = np.linalg.qr(rng.standard_normal((n, r)) + 1j * rng.standard_normal((n, r)))
+    V, _ = np.linalg.qr(rng.standard_normal((r, r)) + 1j * rng.standard_normal((r, r)))
+    U = ((Q0 * np.geomspace(1.0, 1.0 / cond, r)) @ V.conj().T).astype(np.complex64)
+    s = new_fourier_solver(inst)
+    try:
+        L.lrs_set_state(s.h, np.ascontiguousarray(U.T), np.zeros((3, r), np.complex64),
+                        np.tile(np.arange(2, dtype=np.int32), (3, 1)), np.zeros((3, 2), np.complex64), 1, 1e-30)
+        s.iterate(1)
+        U1 = s.get()[0].astype(np.complex128)
+    finally:
+        s.close()
+    Q, _ = O.qr_positive(U.astype(np.complex128))
+    assert np.linalg.norm(U1 - Q) <= 3 * 2.0 ** -24 * np.sqrt(r), np.linalg.norm(U1 - Q) / np.sqrt(r)
