@@ -137,11 +137,11 @@ typedef struct {
                                of reduce)                                    */
   int32_t test_withhold;    /* test aid for the failure path (0 in use): 1: the
                                task engine's queue holds one ticket that is
-                               never published; 2, 3: a copy of the streaming
-                               engine's W pass, of its column steps, is waited
-                               for longer than it is.  The wait runs out after
-                               wait_ms and the call returns LRS_ERR_TIMEOUT
-                               with the device still usable                  */
+                               never published; 2, 3: a barrier of the
+                               streaming engine's W pass, those of its column
+                               steps, wait for one arrival too many.  The wait
+                               runs out after wait_ms and the call returns
+                               LRS_ERR_TIMEOUT with the device still usable  */
 } lrs_options;
 
 /* Create a solver for one problem (Section I-A sizes).

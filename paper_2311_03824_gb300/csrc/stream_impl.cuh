@@ -87,7 +87,8 @@ struct Pipe {
   int* err;
   unsigned long long wait_ns;
 
-  __device__ void init(unsigned b, uint64_t* f, unsigned stg, int s, unsigned long long w) {
+  // withhold (test aid): the first stage expects an arrival that never comes
+  __device__ void init(unsigned b, uint64_t* f, unsigned stg, int s, unsigned long long w, bool withhold = false) {
     base = b;
     full = f;
     stage = stg;
@@ -99,7 +100,7 @@ struct Pipe {
     err = nullptr;
     wait_ns = w;
     if ((threadIdx.x & 31) == 0)
-      for (int i = 0; i < S; ++i) mbar_init(&full[i], 1);
+      for (int i = 0; i < S; ++i) mbar_init(&full[i], withhold && i == 0 ? 2 : 1);
     __syncwarp();
   }
   __device__ uint64_t* issue_bar() const { return full + si; }
@@ -186,10 +187,8 @@ __global__ void __launch_bounds__(kStreamNT, 2)
   P.init(us_bytes + static_cast<unsigned>(wid * S) * stage,
          reinterpret_cast<uint64_t*>(smem + us_bytes + static_cast<size_t>(kSW) * S * stage) +
              wid * kMaxStage,
-         stage, S, T.wait_ns);
+         stage, S, T.wait_ns, T.withhold == 2 && blockIdx.x == 0 && wid == 0);
   if (blockIdx.x == 0 && threadIdx.x < T.ncnt) T.cnt[threadIdx.x] = 0;
-  // test aid: the first piece waits for 16 bytes that no copy brings
-  unsigned extra = T.withhold == 2 && blockIdx.x == 0 && wid == 0 ? 16u : 0u;
   for (int a = blockIdx.x; a < nasg; a += gridDim.x) {
     const StreamAssign as = asg[a];
     const StreamProblem& pr = T.probs[as.prob];
@@ -223,8 +222,7 @@ __global__ void __launch_bounds__(kStreamNT, 2)
       const int nt = min(tpp, b1 - pbt);
       const unsigned hb = static_cast<unsigned>(nr * kTW * pb);
       unsigned char* dst = smem + P.issue_at();
-      if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt + extra);
-      extra = 0u;
+      if (lane == 0) mbar_arrive_expect_tx(P.issue_bar(), hb * planes * nt);
       __syncwarp();
       if (lane < nt * planes) {
         const int t = lane / planes, pl = lane - t * planes;
@@ -486,7 +484,7 @@ struct Step {
       if (threadIdx.x == 0 && rho > 0) {
         asm volatile("fence.proxy.async;" ::: "memory");  // earlier reads of the buffer first
         const unsigned bytes = static_cast<unsigned>(rho * as * 4);
-        mbar_arrive_expect_tx(bar, bytes + (T.withhold == 3 ? 16u : 0u));  // (test aid)
+        mbar_arrive_expect_tx(bar, bytes);
         bulk_copy_g2s(ag, ag_global(), bytes, bar);
       }
     }
@@ -935,7 +933,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 8 : 3)
   __shared__ uint64_t abar;
   constexpr int NT = step_threads(V);
   const int lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) mbar_init(&abar, 1);
+  if (threadIdx.x == 0) mbar_init(&abar, T.withhold == 3 ? 2 : 1);  // (2: test aid)
   unsigned phase = 0;
   int cur = -1;
   for (int c = blockIdx.x; c < T.ncols; c += gridDim.x) {
@@ -1106,7 +1104,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
   const int lane = threadIdx.x & 31;
   const int count = zero ? T.ncols : T.cnt[round];
   if (count == 0) return;
-  if (threadIdx.x == 0) mbar_init(&abar, 1);
+  if (threadIdx.x == 0) mbar_init(&abar, T.withhold == 3 ? 2 : 1);  // (2: test aid)
   unsigned phase = 0;
   int cur = -1;
   for (int at = blockIdx.x; at < count; at += gridDim.x) {

@@ -137,11 +137,10 @@ def test_autotune_call_keeps_the_iterate():
 
 @pytest.mark.parametrize("withhold", [2, 3])
 def test_expired_wait_returns_timeout_and_the_device_stays_usable(withhold):
-    """Failure detection without a fault: one copy of the W pass (2), or those of
-    the column steps (3), are waited for 16 bytes beyond what they bring.  The
-    waits run out after 100 ms, the warp (the CTA, which has other columns to
-    come: two CTAs of the streaming grid) leaves, and the call reports
-    LRS_ERR_TIMEOUT.  A solver created afterwards runs normally."""
+    """Failure detection without a fault: a barrier of the W pass (2), or those of
+    the column steps (3), wait for one arrival more than there is.  The waits
+    run out after 100 ms, the warp (the CTA, which has other columns to come: two
+    CTAs of the streaming grid) leaves, and the call reports LRS_ERR_TIMEOUT.  A solver created afterwards runs normally."""
     from paper_2311_03824_gb300 import lrs as L
     inst = GaussianInstance(n=64, q=40, r=2, m=32, rho=2, seed=7)
     good = run(inst, 4, grid=2)
