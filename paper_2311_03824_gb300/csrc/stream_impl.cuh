@@ -430,6 +430,35 @@ __host__ __device__ inline StepCarve step_carve(int R, int m, int n, int rho, in
   return c;
 }
 
+// Gram of W (columns at Q + l ms) and its factor in FP64, one warp: L^{-1} at
+// G + 512, rounded in Lf, its diagonal's remainder at G + 256.  Out of line: the
+// column steps are short and run on cold instruction caches.
+static __device__ __noinline__ void factor_f64(const float* Q, int ms, int m, int r, int k, double* G, float* Lf, int* err) {
+  __shared__ double iL[16];
+  const int lane = threadIdx.x & 31, ne = r * (r + 1) / 2;
+  double *L = G + 256, *Li = G + 512;
+  float* dlo = reinterpret_cast<float*>(L);
+  for (int t = 0; t < ne; ++t) {
+    int a = 0;
+    while ((a + 1) * (a + 2) / 2 <= t) ++a;
+    const int b = t - a * (a + 1) / 2;
+    double g = 0.0;
+    for (int i = lane; i < m; i += 32)
+      g = __fma_rn(static_cast<double>(Q[a * ms + i]), static_cast<double>(Q[b * ms + i]), g);
+    g = warp_sum(g);
+    if (lane == 0) G[a * 16 + b] = G[b * 16 + a] = g;
+  }
+  __syncwarp();
+  if (!chol_inverse_warp(G, L, Li, iL, r, 16) && lane == 0) report_error(err, kErrNotSPD, k);
+  __syncwarp();
+  for (int t = lane; t < 256; t += 32) {
+    const int i = t >> 4, q = t & 15;
+    if (q > i || i >= r) Li[t] = 0.0;
+    Lf[t] = static_cast<float>(Li[t]);
+    if (q == i) dlo[i] = static_cast<float>(Li[t] - static_cast<double>(Lf[t]));
+  }
+}
+
 // One column on one CTA.  P_perp is applied through an orthonormal basis Q of
 // range(W_k): Q = W L^{-T} with G = W^T W = L L^T, so P v = v - Q (Q^T v), the
 // residual of the LS step is e = Q Q^T r - r and b = L^{-T} (Q^T r): one matrix
@@ -542,27 +571,53 @@ struct Step {
     for (int w = 0; w < NW; ++w) x += scal(s)[w];
     return x;
   }
-  // sum_e AG(i, e) x_e over the support
+  // sum_e AG(i, e) x_e over the support in two interleaved sums; where the
+  // columns come from memory, in one such pair per sixteen entries (one sum of
+  // 400 put half as much again into U's error), whose loads are in flight
+  // together: 3.54 -> 2.65 ms for 4 iterations of n = 2000, q = 100, m = 600,
+  // rho = 400.  Staged columns have fewer entries and pay for the longer code
+  // (per iteration 47 -> 49 us at n = q = 200, 315 -> 320 at n = 1537, q = 301).
   __device__ float support_row(int i, const float* x) const {
-    float t = 0.f;
+    constexpr int B = 16;
     const float* a = ag + i;
+    float t = 0.f, t0 = 0.f, t1 = 0.f;
     int e = 0;
+    for (; !step_staged(V) && e + B <= nl; e += B, a += B * as) {
+      float v[B];
+#pragma unroll
+      for (int z = 0; z < B; ++z) v[z] = a[z * as];
+      t0 = t1 = 0.f;
+#pragma unroll
+      for (int z = 0; z < B; z += 4) {
+        const float4 xe = *reinterpret_cast<const float4*>(x + e + z);
+        t0 = fmaf(v[z], xe.x, t0);
+        t1 = fmaf(v[z + 1], xe.y, t1);
+        t0 = fmaf(v[z + 2], xe.z, t0);
+        t1 = fmaf(v[z + 3], xe.w, t1);
+      }
+      t += t0 + t1;
+    }
+    t0 = t1 = 0.f;
     for (; e + 4 <= nl; e += 4, a += 4 * as) {
       const float4 xe = *reinterpret_cast<const float4*>(x + e);
-      t = fmaf(a[0], xe.x, t);
-      t = fmaf(a[as], xe.y, t);
-      t = fmaf(a[2 * as], xe.z, t);
-      t = fmaf(a[3 * as], xe.w, t);
+      t0 = fmaf(a[0], xe.x, t0);
+      t1 = fmaf(a[as], xe.y, t1);
+      t0 = fmaf(a[2 * as], xe.z, t0);
+      t1 = fmaf(a[3 * as], xe.w, t1);
     }
-    for (; e < nl; ++e, a += as) t = fmaf(a[0], x[e], t);
-    return t;
+    for (; e < nl; ++e, a += as) t0 = fmaf(a[0], x[e], t0);
+    return t + (t0 + t1);
   }
 
   // ---- Gram of W (in Q's buffer), its inverse factor, Q = W L^{-T} in place ----
   // The Gram is summed in double-float from exact products; the factor and
   // its inverse are double-float in one warp's registers (lane = row, then
-  // lane = column).  A pivot below 1e-9 of its diagonal goes to the FP64
-  // routine, which also reports a Gram that is not positive.
+  // lane = column).  A pivot below 1e-9 of its diagonal or outside float32's
+  // range sends Gram and factor to FP64, which also reports a Gram that is not
+  // positive.
+  // Q's rows take L^{-1} rounded, but the diagonal with what its rounding left
+  // (dlo): a column of Q that is off by a common factor of 1 + 3e-8 puts the
+  // error into b and e whole, where the rounding of its entries averages out.
   __device__ void factor() const {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int ne = r * (r + 1) / 2;
@@ -620,6 +675,7 @@ struct Step {
     }
     __syncthreads();
     double* Li = G + 512;
+    float* dlo = reinterpret_cast<float*>(G + 256);
     if (w == 0) {
       bool ok = true;
       df a[R], inv[R];
@@ -649,18 +705,11 @@ struct Step {
             const bool in = i < r && lane < r;
             Li[i * 16 + lane] = in ? static_cast<double>(x[i].h) + static_cast<double>(x[i].l) : 0.0;
             Lf[i * 16 + lane] = in ? x[i].h : 0.f;
+            if (i == lane) dlo[i] = in ? x[i].l : 0.f;
           }
         }
       } else {
-        double* L = G + 256;
-        __shared__ double iL[16];
-        if (!chol_inverse_warp(G, L, Li, iL, r, 16) && lane == 0) report_error(pr.err, kErrNotSPD, k);
-        __syncwarp();
-        for (int t = lane; t < 256; t += 32) {
-          const int i = t >> 4, q = t & 15;
-          if (q > i || i >= r) Li[t] = 0.0;
-          Lf[t] = static_cast<float>(Li[t]);
-        }
+        factor_f64(Q, ms, m, r, k, G, Lf, pr.err);
       }
     }
     __syncthreads();
@@ -670,7 +719,7 @@ struct Step {
       for (int l = 0; l < R; ++l) x[l] = Q[l * ms + i];
 #pragma unroll
       for (int l = 0; l < R; ++l) {
-        float s = 0.f;
+        float s = x[l] * dlo[l];
 #pragma unroll
         for (int q = 0; q <= l; ++q) s = fmaf(x[q], Lf[l * 16 + q], s);
         Q[l * ms + i] = s;
