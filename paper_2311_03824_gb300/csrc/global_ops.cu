@@ -351,18 +351,17 @@ __global__ void sum_fin_kernel(int nblk, const double* __restrict__ part, double
   }
 }
 
-// set_support (lrs_internal.h), a warp per column: one pass over a support that
+// set_support (lrs_internal.h), a block per column: one pass over a support that
 // is strictly ascending and in range (every support that the library has
-// written), else the warp compares each entry with the ones before it.
-__global__ void __launch_bounds__(128) support_kernel(int n, int q, int rho, int w, const int* src_idx,
+// written), else a warp compares each entry with the ones before it.
+__global__ void __launch_bounds__(128) support_kernel(int n, int rho, int w, const int* src_idx,
                                                       const float* src_val, int* dst_idx, float* dst_val) {
-  const int lane = threadIdx.x & 31, k = blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (k >= q) return;
+  const int lane = threadIdx.x & 31, k = blockIdx.x;
   const size_t at = static_cast<size_t>(k) * rho;
   int* idx = dst_idx + at;
   float* val = dst_val + at * w;
   bool ok = true;
-  for (int e = lane; e < rho; e += 32) {
+  for (int e = threadIdx.x; e < rho; e += blockDim.x) {
     const int j = src_idx[at + e];
     ok = ok && j >= 0 && j < n && (e == 0 || src_idx[at + e - 1] < j);
     if (src_idx != dst_idx) {
@@ -370,8 +369,7 @@ __global__ void __launch_bounds__(128) support_kernel(int n, int q, int rho, int
       for (int c = 0; c < w; ++c) val[e * w + c] = src_val[(at + e) * w + c];
     }
   }
-  if (__all_sync(0xffffffffu, ok)) return;
-  __syncwarp();
+  if (__syncthreads_and(ok) || threadIdx.x >= 32) return;
   // first entry before e (of rho: anywhere) that holds j, or -1
   auto find = [&](int j, int e) {
     for (int f0 = 0; f0 < e; f0 += 32) {
@@ -412,7 +410,7 @@ __global__ void __launch_bounds__(128) support_kernel(int n, int q, int rho, int
 
 cudaError_t set_support(int n, int q, int rho, int w, const int* src_idx, const float* src_val, int* idx,
                         float* val, cudaStream_t s) {
-  support_kernel<<<(q + 3) / 4, 128, 0, s>>>(n, q, rho, w, src_idx, src_val, idx, val);
+  support_kernel<<<q, 128, 0, s>>>(n, rho, w, src_idx, src_val, idx, val);
   return cudaGetLastError();
 }
 
