@@ -45,39 +45,6 @@ __device__ __forceinline__ double2 dccmul(double2 a, double2 b) {  // conj(a) * 
 }
 __device__ __forceinline__ float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 
-// Double-float accumulation (a value carried as hi + lo, two float32 words:
-// about 48 bits of significand on the FP32 units, whose dependent operations
-// are far cheaper than FP64's on this part).  df_fma: (hi, lo) += a * b with
-// the product's rounding error from an fma and the sum's from Knuth's
-// two-sum.  df_add: (hi, lo) += (bh, bl).
-__device__ __forceinline__ void df_fma(float& hi, float& lo, float a, float b) {
-  const float p = a * b;
-  const float pe = fmaf(a, b, -p);
-  const float s = hi + p;
-  const float bb = s - hi;
-  const float se = (hi - (s - bb)) + (p - bb);
-  hi = s;
-  lo += se + pe;
-}
-__device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl) {
-  const float s = hi + bh;
-  const float bb = s - hi;
-  const float se = (hi - (s - bb)) + (bh - bb);
-  hi = s;
-  lo += se + bl;
-}
-// warp sum of double-float values (xor butterfly: every lane ends with the
-// same value, the pairs added in a fixed order)
-__device__ __forceinline__ double warp_sum_df(float hi, float lo) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-    df_add(hi, lo, oh, ol);
-  }
-  return static_cast<double>(hi) + static_cast<double>(lo);
-}
-
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

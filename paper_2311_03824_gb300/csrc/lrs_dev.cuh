@@ -157,6 +157,22 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   const float z = s - a;
   e = (a - (s - z)) + (b - z);
 }
+// (hi, lo) += a * b, the product's rounding error from an fma; about 48 bits
+// on the FP32 units, whose dependent operations are far cheaper than FP64's
+__device__ __forceinline__ void df_fma(float& hi, float& lo, float a, float b) {
+  const float p = a * b, pe = fmaf(a, b, -p);
+  float s, e;
+  two_sum(hi, p, s, e);
+  hi = s;
+  lo += e + pe;
+}
+// (hi, lo) += (bh, bl)
+__device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl) {
+  float s, e;
+  two_sum(hi, bh, s, e);
+  hi = s;
+  lo += e + bl;
+}
 struct df {
   float h, l;
 };
@@ -191,6 +207,43 @@ __device__ __forceinline__ df df_rsqrt(df a) {
   const df t = df_mul(a, df_norm(y2, y2l));
   const float d = (1.f - t.h) - t.l;  // exact difference near 1
   return df_norm(y, 0.5f * y * d);
+}
+
+// One warp: the Cholesky factor L of the r x r Gram G (ld 16) and L^{-1} in
+// double-float in registers (lane = row, then lane = column); put(i, x) gets the
+// entry (i, lane) of L^{-1}, i < R, lane < 16 (zero beyond r).  False, and
+// nothing put, when a pivot is below 1e-9 of its diagonal or outside float32's
+// range (a NaN is).
+template <int R, class Put>
+__device__ __forceinline__ bool chol_df(const double* G, int r, Put put) {
+  const int lane = threadIdx.x & 31;
+  bool ok = true;
+  df a[R], inv[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) a[q] = lane < r && q < r ? df_make(G[lane * 16 + q]) : df{0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    inv[j] = df{1.f, 0.f};
+    if (j >= r || !ok) continue;
+    const df pv = df_shfl(a[j], j);
+    ok = pv.h > 1e-9f * static_cast<float>(G[j * 16 + j]) && pv.h > 1e-30f && pv.h < 1e30f;
+    inv[j] = df_rsqrt(pv);
+    a[j] = df_mul(a[j], inv[j]);
+#pragma unroll
+    for (int q = j + 1; q < R; ++q) a[q] = df_sub(a[q], df_mul(a[j], df_shfl(a[j], q)));
+  }
+  if (!ok) return false;
+  df x[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {  // column `lane` of L^{-1}
+    df t = df{0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < i; ++q) t = df_sub(t, df_mul(df_shfl(a[q], i), x[q]));
+    t = df_mul(t, inv[i]);
+    x[i] = i < lane ? df{0.f, 0.f} : i == lane ? inv[i] : t;
+    if (lane < 16) put(i, i < r && lane < r ? x[i] : df{0.f, 0.f});
+  }
+  return true;
 }
 
 // Sums over the warp of N values at once (N a power of two <= 32): after

@@ -1,22 +1,26 @@
-// Cholesky-QR2 in one launch: one cluster of eight CTAs holds the n x r matrix
-// in shared memory through both passes (Algorithm 1, "Set U <- U+": the sum of
-// the gradient's partial blocks, Z = U - eta grad and Q(Z)).
+// Cholesky-QR in one launch: one cluster of eight CTAs holds the n x r matrix in
+// shared memory (Algorithm 1, "Set U <- U+": the sum of the gradient's partial
+// blocks, Z = U - eta grad and Q(Z)).
 //
 // The five launches of the separate kernels took 46 us at n = 1000, r = 5
 // (FP64 Gram loops and FP64 Cholesky chains, each on a cold SM).  Here a CTA
-// keeps n / 8 rows; the two Grams are exchanged through distributed shared
-// memory (two cluster barriers) and every CTA factors them redundantly.
-//   Pass 1: Gram in double-float from exact products, summed over the CTAs in
-//     FP64; Cholesky in FP32 when every pivot is above 1e-3 of its diagonal
-//     (R1 needs to be good enough only for the second pass to start from a Gram
-//     near I: any upper triangular R1 leaves Q unchanged).
-//   Pass 2: the Gram is I + E; Cholesky and inverse are carried as deviations
-//     from I in FP32 (relative to E), so that Q = Q1 + Q1 H adds a correction
-//     known to about 1e-7 |E|, where a rounded R2^{-1} would put 6e-8 on every
-//     entry.
-//   When a factor fails (small pivots, E not small, a Gram outside float32's
-//   range: entries of Z beyond about 1e-15 .. 1e15) Gram and factor are done
-//   again in FP64, in every CTA alike, since all hold the same sums.
+// keeps n / 8 rows; the Gram is a double-float sum of exact products, exchanged
+// through distributed shared memory and added over the CTAs in FP64, and every
+// CTA factors it redundantly, in double-float in one warp's registers.  The rows
+// times R^{-1} = L^{-T} are sums of exact products with its 48 bits: each entry
+// of Q is rounded once.
+//
+// With cond(Z)^2 <= K^2 = sum over p, l of L^{-1}(l, p)^2 G(p, p) (columns of norm
+// one), Q^T Q - I is at most r 2^-45 K^2: one pass is enough up to kOnePass = 4096
+// (2^-29 at r = 16, below the rounding of Q), which every step of a solve meets;
+// beyond, a second pass takes the rounded rows, whose Gram is near I.  (Two
+// passes with FP32 factors left two roundings, 3.5e-8 to 4.9e-8 of Q against
+// 2.5e-8; U after two iterations at n = 200, q = 2000, r = 2: 6.1e-8, now 4.9e-8.
+// They took 2 us more at r = 3, and 30 us less at r = 16, where the double-float
+// factor is a long chain in one warp.)  A Gram that this factor cannot take (a
+// pivot below 1e-9 of its diagonal, or outside float32's range: entries of Z
+// beyond about 1e-15 .. 1e15) is summed and factored again in FP64, in every CTA
+// alike, since all hold the same sums.
 #include "lrs_dev.cuh"
 #include "lrs_internal.h"
 
@@ -26,6 +30,7 @@ namespace {
 constexpr int kQT = 512;   // threads per CTA
 constexpr int kQC = 8;     // CTAs (portable cluster size)
 constexpr int kMaxR = 16;
+constexpr float kOnePass = 4096.f;
 
 struct QrArgs {
   int n, r, rows, ldz;
@@ -39,68 +44,14 @@ struct QrArgs {
   int* err;
 };
 
-// One warp: FP32 Cholesky of the r x r matrix G (dev: of G = I + E, in
-// deviations), lane i <-> row i, and its inverse, lane c <-> column c:
-// Rinv[c * 16 + i] = (L^{-1})(i, c), the entry (c, i) of R^{-1} = L^{-T}
-// (dev: minus the identity).  False when a pivot asks for FP64.
-template <int R>
-__device__ bool chol_f32(const double* G, float* Rinv, int r, bool dev) {
-  const int lane = threadIdx.x & 31;
-  float a[R], inv[R], dinv[R];
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    double g = lane < r && k < r ? G[lane * kMaxR + k] : 0.0;
-    if (dev && k == lane) g -= 1.0;
-    a[k] = static_cast<float>(g);
-  }
-  bool ok = true;
-#pragma unroll
-  for (int j = 0; j < R; ++j) {
-    inv[j] = 1.f;
-    dinv[j] = 0.f;
-    if (j >= r || !ok) continue;
-    const float p = __shfl_sync(0xffffffffu, a[j], j);
-    if (dev) {
-      ok = fabsf(p) < 0.25f;
-      const float l1 = p / (1.f + sqrtf(1.f + p));  // L_jj - 1
-      inv[j] = 1.f / (1.f + l1);
-      dinv[j] = -l1 * inv[j];
-    } else {
-      ok = p > 1e-3f * static_cast<float>(G[j * kMaxR + j]) && p > 1e-30f && p < 1e30f;
-      inv[j] = rsqrtf(p);
-    }
-    a[j] *= inv[j];
-#pragma unroll
-    for (int k = j + 1; k < R; ++k) {
-      const float lk = __shfl_sync(0xffffffffu, a[j], k);
-      a[k] = fmaf(-a[j], lk, a[k]);  // used for rows >= k only
-    }
-  }
-  if (!ok) return false;
-  float x[R];
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    float t = 0.f;
-#pragma unroll
-    for (int p = 0; p < i; ++p) t = fmaf(-__shfl_sync(0xffffffffu, a[p], i), x[p], t);
-    x[i] = i < lane ? 0.f : i == lane ? inv[i] : t * inv[i];
-  }
-  if (lane < r)
-#pragma unroll
-    for (int i = 0; i < R; ++i)
-      if (i >= lane && i < r) Rinv[lane * kMaxR + i] = dev && i == lane ? dinv[i] : x[i];
-  __syncwarp();
-  return true;
-}
-
 template <int R>
 __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_kernel(QrArgs q) {
   extern __shared__ __align__(16) float Zt[];  // [R][ldz], column l of this CTA's rows
   constexpr int NE = R * (R + 1) / 2;
   __shared__ double part[2][NE], part64[NE];
   __shared__ double G[kMaxR * kMaxR], Ld[kMaxR * kMaxR], Li[kMaxR * kMaxR], iL[kMaxR];
-  __shared__ float Rinv[kMaxR * kMaxR];
-  __shared__ int factored;
+  __shared__ float2 LL[kMaxR * kMaxR];  // L^{-1} and what its rounding left
+  __shared__ int factored, one;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, r = q.r;
   const unsigned rank = cluster_rank();
   const int lo = min(q.n, static_cast<int>(rank) * q.rows), cnt = min(q.n, lo + q.rows) - lo;
@@ -119,7 +70,7 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
     Zt[l * q.ldz + i] = v;
   }
   __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
+  for (int pass = 0;; ++pass) {
     // this CTA's part of the Gram: a warp per entry, lanes over the rows
     for (int t = w; t < r * (r + 1) / 2; t += kQT / 32) {
       int a = 0;
@@ -127,21 +78,10 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
       const int b = t - a * (a + 1) / 2;
       const float *za = Zt + a * q.ldz, *zb = Zt + b * q.ldz;
       float hi = 0.f, lw = 0.f;
-      for (int i = lane; i < cnt; i += 32) {
-        const float x = za[i], y = zb[i], p = x * y;
-        float s, d;
-        two_sum(hi, p, s, d);
-        hi = s;
-        lw += d + fmaf(x, y, -p);
-      }
+      for (int i = lane; i < cnt; i += 32) df_fma(hi, lw, za[i], zb[i]);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lw, o);
-        float s, d;
-        two_sum(hi, bh, s, d);
-        hi = s;
-        lw += bl + d;
-      }
+      for (int o = 16; o > 0; o >>= 1)
+        df_add(hi, lw, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lw, o));
       if (lane == 0) part[pass][t] = static_cast<double>(hi) + static_cast<double>(lw);
     }
     auto sum_parts = [&](const double* p) {  // every CTA sums the parts in rank order
@@ -160,8 +100,17 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
     };
     sum_parts(part[pass]);
     if (w == 0) {
-      const bool ok = chol_f32<R>(G, Rinv, r, pass == 1);
-      if (lane == 0) factored = ok;
+      float k2 = 0.f;
+      const float g = lane < r ? static_cast<float>(G[lane * kMaxR + lane]) : 0.f;
+      const bool ok = chol_df<R>(G, r, [&](int i, df x) {
+        LL[i * kMaxR + lane] = make_float2(x.h, x.l);
+        k2 = fmaf(x.h * x.h, g, k2);
+      });
+      k2 = warp_sum(k2);
+      if (lane == 0) {
+        factored = ok;
+        one = ok && k2 <= kOnePass;
+      }
     }
     __syncthreads();
     if (!factored) {
@@ -178,29 +127,35 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
       if (w == 0) {
         if (!chol_inverse_warp(G, Ld, Li, iL, r, kMaxR) && lane == 0 && rank == 0)
           report_error(q.err, kErrNotSPD, -1);
-        for (int t = lane; t < r * r; t += 32) {
-          const int a = t / r, b = t - a * r;
-          Rinv[a * kMaxR + b] = static_cast<float>(Li[b * kMaxR + a] - (pass == 1 && a == b ? 1.0 : 0.0));
+        __syncwarp();
+        for (int t = lane; t < r * kMaxR; t += 32) {
+          const float h = static_cast<float>(Li[t]);
+          LL[t] = make_float2(h, static_cast<float>(Li[t] - static_cast<double>(h)));
         }
       }
       __syncthreads();
     }
-    // rows times R^{-1} (pass 1) or I + H (pass 2), a thread per row
+    const bool last = pass == 1 || one;
+    // rows times R^{-1}, a thread per row
     for (int i = tid; i < cnt; i += kQT) {
       float z[R];
 #pragma unroll
       for (int l = 0; l < R; ++l) z[l] = l < r ? Zt[l * q.ldz + i] : 0.f;
 #pragma unroll
-      for (int l = R - 1; l >= 0; --l) {
-        if (l >= r) continue;
-        float s = 0.f;
+      for (int l = 0; l < R; ++l) {
+        if (l >= r) break;
+        float h = 0.f, lw = 0.f;
 #pragma unroll
-        for (int p = 0; p <= l; ++p) s = fmaf(z[p], Rinv[p * kMaxR + l], s);
-        if (pass == 1) s += z[l];
-        Zt[l * q.ldz + i] = s;
+        for (int p = 0; p <= l; ++p) {
+          const float2 f = LL[l * kMaxR + p];
+          df_fma(h, lw, f.x, z[p]);
+          lw = fmaf(f.y, z[p], lw);
+        }
+        Zt[l * q.ldz + i] = h + lw;
       }
     }
     __syncthreads();
+    if (last) break;  // (the same in every CTA)
   }
   for (int u = tid; u < cnt * r; u += kQT) {
     const int i = u / r, l = u - i * r;
@@ -214,7 +169,7 @@ __global__ void __launch_bounds__(kQT) __cluster_dims__(kQC, 1, 1) qr_cluster_ke
 template <int R>
 cudaError_t launch(const QrArgs& q, size_t smem, cudaStream_t s) {
   // A block has 48 KB without asking for more, and the kernel's static arrays
-  // (10.6 KB at R = 16) count: the limit of the largest request (idempotent) is
+  // (11.6 KB at R = 16) count: the limit of the largest request (idempotent) is
   // set from 32 KB on, every time, since nothing says that this process and
   // device had a larger call before.
   cudaError_t e = cudaSuccess;

@@ -677,38 +677,12 @@ struct Step {
     double* Li = G + 512;
     float* dlo = reinterpret_cast<float*>(G + 256);
     if (w == 0) {
-      bool ok = true;
-      df a[R], inv[R];
-#pragma unroll
-      for (int q = 0; q < R; ++q) a[q] = lane < r && q < r ? df_make(G[lane * 16 + q]) : df{0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        inv[j] = df{1.f, 0.f};
-        if (j >= r || !ok) continue;
-        const df pv = df_shfl(a[j], j);
-        ok = pv.h > 1e-9f * static_cast<float>(G[j * 16 + j]) && pv.h > 1e-30f && pv.h < 1e30f;
-        inv[j] = df_rsqrt(pv);
-        a[j] = df_mul(a[j], inv[j]);
-#pragma unroll
-        for (int q = j + 1; q < R; ++q) a[q] = df_sub(a[q], df_mul(a[j], df_shfl(a[j], q)));
-      }
-      if (ok) {
-        df x[R];
-#pragma unroll
-        for (int i = 0; i < R; ++i) {  // column `lane` of L^{-1}
-          df t = df{0.f, 0.f};
-#pragma unroll
-          for (int q = 0; q < i; ++q) t = df_sub(t, df_mul(df_shfl(a[q], i), x[q]));
-          t = df_mul(t, inv[i]);
-          x[i] = i < lane ? df{0.f, 0.f} : i == lane ? inv[i] : t;
-          if (lane < 16) {
-            const bool in = i < r && lane < r;
-            Li[i * 16 + lane] = in ? static_cast<double>(x[i].h) + static_cast<double>(x[i].l) : 0.0;
-            Lf[i * 16 + lane] = in ? x[i].h : 0.f;
-            if (i == lane) dlo[i] = in ? x[i].l : 0.f;
-          }
-        }
-      } else {
+      const bool ok = chol_df<R>(G, r, [&](int i, df x) {
+        Li[i * 16 + lane] = static_cast<double>(x.h) + static_cast<double>(x.l);
+        Lf[i * 16 + lane] = x.h;
+        if (i == lane) dlo[i] = x.l;
+      });
+      if (!ok) {
         factor_f64(Q, ms, m, r, k, G, Lf, pr.err);
       }
     }
