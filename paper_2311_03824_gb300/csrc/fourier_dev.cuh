@@ -222,7 +222,8 @@ __device__ __forceinline__ void cgram_warp(const float2* W, size_t ld, int m, in
 
 // One warp: the complex Cholesky factor L of M (Gd: the sums of cgram_warp) and
 // L^{-1} in double-float in registers (lane = row, then lane = column; an FP64
-// factor through shared memory took 31 K cycles at r = 6); Lf is L^{-1} rounded.
+// factor through shared memory took 31 K cycles at r = 6); Lf is L^{-1} rounded,
+// with what the rounding of its (real) diagonal left in the imaginary part.
 // False, and nothing written, when a pivot is below 1e-9 of its diagonal or
 // outside float32's range (a NaN is).
 template <int R>
@@ -272,7 +273,7 @@ __device__ bool cchol_df(const float2* Gd, int r, double2* Li, float2* Lf) {
       if (lane < kMaxR && i < r) {
         Li[i * kMaxR + lane] = make_double2(static_cast<double>(x[i].x.h) + static_cast<double>(x[i].x.l),
                                               static_cast<double>(x[i].y.h) + static_cast<double>(x[i].y.l));
-        Lf[i * kMaxR + lane] = make_float2(x[i].x.h, x[i].y.h);
+        Lf[i * kMaxR + lane] = make_float2(x[i].x.h, i == lane ? x[i].x.l : x[i].y.h);
       }
     }
   }
@@ -332,7 +333,9 @@ __device__ inline bool cchol_f64(int r, double2* scratch, double2* Li, float2* L
       }
       t = i < cc ? make_double2(0, 0) : make_double2(t.x * iL[i], t.y * iL[i]);
       Li[i * kMaxR + cc] = t;
-      Lf[i * kMaxR + cc] = make_float2(static_cast<float>(t.x), static_cast<float>(t.y));
+      const float h = static_cast<float>(t.x);
+      Lf[i * kMaxR + cc] =
+          make_float2(h, static_cast<float>(i == cc ? t.x - static_cast<double>(h) : t.y));
     }
   }
   __syncwarp();

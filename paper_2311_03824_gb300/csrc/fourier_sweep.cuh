@@ -536,7 +536,7 @@ __device__ void ffactor(const FCtx& C) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = C.r;
   double2* G = reinterpret_cast<double2*>(C.T);
   float2* part = reinterpret_cast<float2*>(G + 2 * kMaxR * kMaxR + kMaxR);
-  float2* Gd = part + C.nw * R * R;  // value layout of fgram_part, summed over the warps
+  float2* Gd = part + C.nw * R * R;  // value layout of cgram_part, summed over the warps
   float2* mine = part + w * R * R;
   cgram_warp<R>(C.Q, C.m, C.m, r, C.nw, mine);
   __syncthreads();
@@ -558,7 +558,9 @@ __device__ void ffactor(const FCtx& C) {
     if (!cchol_f64(r, G, C.Li, C.Lf) && lane == 0) report_error(C.err, kErrNotSPD, C.k);
   }
   __syncthreads();
-  // Q_l = sum_{p <= l} W_p conj(L^{-1}[l][p])
+  // Q_l = sum_{p <= l} W_p conj(L^{-1}[l][p]), the diagonal with its remainder: a
+  // column that is off by a common factor of 1 + 3e-8 puts the error into b and the
+  // residual whole, where the rounding of its entries averages out
   for (int i = threadIdx.x; i < C.m; i += blockDim.x) {
     float2 x[R];
 #pragma unroll
@@ -568,7 +570,10 @@ __device__ void ffactor(const FCtx& C) {
       if (l >= r) break;
       float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int p = 0; p <= l; ++p) s = ccfma(C.Lf[l * kMaxR + p], x[p], s);
+      for (int p = 0; p < l; ++p) s = ccfma(C.Lf[l * kMaxR + p], x[p], s);
+      const float2 d = C.Lf[l * kMaxR + l];
+      s.x = fmaf(d.x, x[l].x, fmaf(d.y, x[l].x, s.x));
+      s.y = fmaf(d.x, x[l].y, fmaf(d.y, x[l].y, s.y));
       C.Q[static_cast<size_t>(l) * C.m + i] = s;
     }
   }

@@ -145,3 +145,44 @@ def test_rows_of_the_step_are_rounded_once_a_pass(nx, ny, r, cond):
         s.close()
     Q, _ = O.qr_positive(U.astype(np.complex128))
     assert np.linalg.norm(U1 - Q) <= 3 * 2.0 ** -24 * np.sqrt(r), np.linalg.norm(U1 - Q) / np.sqrt(r)
+
+
+# Errors of B and U after two steps against the FP64 oracle, root mean square over
+# three instances, of FP64 r x r solves and the FP64 Cholesky-QR2.  (B where the
+# support has two pixels: a larger one's A s takes two rounded twiddles a term.)
+FP64_FACTORS = {(64, 64, 24, 4, 1229, 20): (None, 6.28e-8), (32, 32, 60, 6, 400, 8): (None, 5.63e-8),
+                (20, 20, 100, 4, 250, 2): (7.08e-8, 6.42e-8)}
+
+
+@pytest.mark.parametrize("shape", FP64_FACTORS, ids=str)
+def test_no_less_precise_than_fp64_factors(shape):
+    """At most 1.02 of those errors: the sums of tens of thousands of roundings
+    differ by less from one order of the float32 sums to another."""
+    from tests.gpu_helpers import cast_state, rel, set_gpu_state
+    nx, ny, q, r, m, rho = shape
+    n, tot = nx * ny, np.zeros(2)
+    for seed in range(3):
+        inst = FourierInstance(nx=nx, ny=ny, q=q, r=r, m=m, rho=rho, seed=500 + seed, mask_law="uniform", b_law="gauss")
+        P = Problem.fourier(inst)
+        rng = np.random.default_rng(seed)
+        g = lambda *sh: rng.standard_normal(sh) + 1j * rng.standard_normal(sh)
+        U, _ = np.linalg.qr(inst.Ustar + 0.01 * g(n, r) / np.sqrt(n))
+        U = U.astype(np.complex64).astype(np.complex128)
+        val = (inst.S_val + 0.01 * inst.rms_L * g(q, rho)).astype(np.complex64).astype(np.complex128)
+        eta = 0.3 / (m / n * np.linalg.norm(inst.Bstar, 2) ** 2)
+        st = O.OracleState(U=U, B=U.conj().T @ inst.Ustar @ inst.Bstar, S=O.densify(inst.S_idx, val, n),
+                           S_idx=inst.S_idx.copy(), eta=eta, t=5)
+        s = new_fourier_solver(inst)
+        try:
+            set_gpu_state(s, st, True)
+            s.iterate(2)
+            U1, B1, Si, Sv = s.get()
+        finally:
+            s.close()
+        ref = cast_state(st, np.complex128)
+        for _ in range(2):
+            O.iterate_alg1(P.op64, P.Y, ref, rho)
+        assert np.array_equal(Si, ref.S_idx)
+        tot += np.array([rel(B1, ref.B), rel(U1, ref.U)]) ** 2 / 3
+    for err, bar in zip(np.sqrt(tot), FP64_FACTORS[shape]):
+        assert bar is None or err <= 1.02 * bar, (err, bar)
