@@ -787,6 +787,7 @@ struct FourierSolver {
   unsigned long long* prof = nullptr;  // kFProf sweep cycle counters (profiling)
   void* sweep = nullptr;   // fsweep_kernel of the rank width
   bool lean = false;       // no room for its tables
+  float fft_err = 0.f;     // FArgs
   int tb = 0, qmode = 0;   // its table's columns and Q_k's place (FArgs)
   size_t smem = 0;
 };
@@ -831,6 +832,10 @@ FourierSolver* fourier_create(int nx, int ny, int m, int q, int r, int rho, int 
     F->g.lL = ilog2(F->g.L);
     const double span = 2.0 * std::max(nx, ny) * F->g.L * F->g.L;
     F->g.magic = span < 4294967296.0 ? static_cast<unsigned>((0x100000000ull + F->g.L - 1) / F->g.L) : 0u;
+  }
+  {  // 7 roundings a radix-2 stage; a direct DFT of N terms: (N + 4) |F| |x|, || |F| || = sqrt(N)
+    auto side = [](int len, int l) { return l >= 0 ? 7.0 * l : (len + 4) * std::sqrt(static_cast<double>(len)); };
+    F->fft_err = static_cast<float>(0x1p-24 * (side(nx, F->g.lnx) + side(ny, F->g.lny)));
   }
   F->m = m;
   F->q = q;
@@ -1052,6 +1057,7 @@ static cudaError_t launch_fsweep(FourierSolver* F, int mode, int tau) {
   a.prof = F->prof;
   a.tb = F->tb;
   a.lean = F->lean;
+  a.fft_err = F->fft_err;
   a.qmode = F->qmode;
   void* args[] = {&a};
   return cudaLaunchKernel(F->sweep, dim3(F->q), dim3(fsweep_threads(F->g.n)), args, F->smem, F->s);

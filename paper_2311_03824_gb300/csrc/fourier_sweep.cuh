@@ -21,8 +21,9 @@
 // ||u - u_ref|| <= sum of mu ||P A g_G|| over the sweeps since.  When mu times
 // that bound (1 + 1e-3) is below the smallest new |v_i| on the support,
 // HardThreshold keeps the support whatever g is off it, and the sweep needs g
-// on the support alone: no 2D FFT (the 1e-3 covers the rounding of u, mu and of
-// the FFT, about 1e-6 ||u|| against N >= 1 / 128).  The test is made on the
+// on the support alone: no 2D FFT (the 1e-3 covers the rounding of mu and the
+// norms; the FFT's own, at most fft_err ||u_ref||, is added to the max |g_j|,
+// however small).  The test is made on the
 // sweep's own mu and v; a sweep that fails it takes the FFT.
 //
 // Bound: instruction issue (593 K warp instructions per 128 x 128 frame, issue
@@ -43,6 +44,7 @@ struct FArgs {
   int m, q, r, rho, tau, mode;
   int tb;               // support columns of the sparse DFT's table beside the frame
   int lean;             // no room for the tables (fcarve)
+  float fft_err;        // bound of the 2D FFT's rounding error in the 2-norm
   int qmode;            // Q_k: 0 in Wk, 1 in shared memory, 2 in the frame's place
                         // while no FFT needs it (kept in Wk meanwhile)
   const float2* y;      // q x m
@@ -82,6 +84,8 @@ struct FCarve {
 
 // HardThreshold candidates of the threshold filter
 constexpr int kCandCap = 512;
+// what the squares of a norm lose below float32's range
+constexpr float kTinySq = 4e-41f;
 
 __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -988,7 +992,8 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) smin = fminf(smin, __shfl_xor_sync(0xffffffffu, smin, o));
     __syncthreads();
-    float bound = N * sqrtf(fget(C, 0));
+    const float un = sqrtf(fget(C, 0) + kTinySq);
+    float bound = N * un;
     if (have_ref) bound = fminf(bound, fmaf(N, dist, gmax));
     mark(2);
     // worth trying without the FFT: the bound with the last mu and the present s
@@ -1075,7 +1080,7 @@ __global__ void __launch_bounds__(kFT, 1) fsweep_kernel(const FArgs a) {
       if (valid) {
         fput_max(C, 3, g2);
         __syncthreads();
-        gmax = sqrtf(fget_max(C, 3));
+        gmax = fmaf(a.fft_err, un, sqrtf(fget_max(C, 3) + kTinySq));
         dist = mu * sqrtf(den);
       }
     }

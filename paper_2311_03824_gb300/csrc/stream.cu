@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(256) norms_kernel(GaussLayout L, const unsigne
 }
 __global__ void norms_fin_kernel(int k0, int kc, float* nmax) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < kc) nmax[k0 + t] = sqrtf(nmax[k0 + t]);
+  if (t < kc) nmax[k0 + t] = sqrtf(nmax[k0 + t] + kTinySq);
 }
 
 }  // namespace

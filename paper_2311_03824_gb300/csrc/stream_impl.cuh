@@ -17,10 +17,12 @@
 // (kept per column, set with the operator).  So when
 //     mu N_k ||u|| (1 + 1e-3) < min_{i in G} |v_i|
 // HardThreshold returns G whatever g is, and the sweep is done without it
-// (the 1e-3 covers the rounding of u, mu and of the pass's own float32 sums,
-// m 2^-24 N ||u|| at most).  After a pass at u_ref has given g, the same
-// holds with max_{j not in G} |g_j| + N_k ||u - u_ref|| in the place of
-// N_k ||u||.  Every other sweep goes through g_kernel and the full
+// (the 1e-3 covers the rounding of mu and of the norms, m / 4 2^-24 with m at
+// most 11000; kTinySq what the squares lose below float32's range).  After a pass
+// at u_ref has given g, the same holds with max_{j not in G} |g_j| + N_k (||u -
+// u_ref|| + (m + 4) 2^-24 ||u_ref||) in the place of N_k ||u||: the last term
+// bounds the rounding of the pass's sums, which a small max |g_j| says nothing
+// about.  Every other sweep goes through g_kernel and the full
 // HardThreshold.  A solve's error e_k enters the test as about ||e_k|| <
 // min |s_i|: it holds from a relative error of about 1/sqrt(n) on, after which
 // an iteration streams A_k twice (W, h) and not 2 + tau times.
@@ -54,6 +56,8 @@ using sweep::kTW;
 constexpr int kSW = 8;            // warps per streaming CTA
 constexpr int kStreamNT = 32 * kSW;
 constexpr int kMaxStage = 4;
+// half the spacing below float32's normal range, for 2^15 squares of a sum
+constexpr float kTinySq = 4e-41f;
 
 __device__ __forceinline__ unsigned long long gtimer() {
   unsigned long long t;
@@ -811,7 +815,7 @@ struct Step {
     const float N = pr.nmax[k];
     __syncthreads();
     for (; sw < te; ++sw) {
-      const float nu = sqrtf(get_scal(1 + (sw & 1)));
+      const float nu = sqrtf(get_scal(1 + (sw & 1)) + kTinySq);
       support_gradient();
       __syncthreads();
       float num, den;
@@ -819,7 +823,7 @@ struct Step {
       if (!(den > 0.f)) return te;  // s is stationary: the remaining sweeps keep it
       const float mu = num / den;
       float bound = N * nu;
-      if (have_ref) bound = fminf(bound, fmaf(N, sqrtf(get_scal(3)), gmax));
+      if (have_ref) bound = fminf(bound, fmaf(N, sqrtf(get_scal(3) + kTinySq), gmax));
       bound = bound * mu * 1.001f;
       // all comparisons are false for NaN: such a column takes the full path
       bool ok = nl == rho && isfinite(mu) && (bound >= 0.f || rho >= n);
@@ -1191,6 +1195,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
     }
     s.put_scal(0, sq);
     __syncthreads();
+    const float nref = sqrtf(s.get_scal(1));
     for (int i = threadIdx.x; i < m; i += NT) s.uref[i] = s.u[i];
     float num, den, gmax = 0.f;
     s.curvature(num, den, false);
@@ -1306,6 +1311,7 @@ __global__ void __launch_bounds__(step_threads(V), V == 0 ? 6 : 3)
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NT / 32; ++w) gmax = fmaxf(gmax, s.scal(0)[w]);
+    gmax = fmaf(spr.nmax[k] * nref, (m + 4) * 0x1p-24f, gmax);  // rounding of the pass's sums
     const int slot = 1 + ((sw + 1) & 1);
     if (kept) {
       float nn = 0.f;
