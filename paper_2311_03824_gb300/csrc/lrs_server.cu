@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "../../include/lrs.h"
+#include "lrs_internal.h"
 
 namespace {
 
@@ -283,7 +284,20 @@ size_t lrs_request_footprint(const lrs_request* rq) {
     const int64_t stored = q * m * ns * eb;
     const int64_t exact = rq->opt.a_dtype != LRS_A_FP32 ? q * m * n * 4 : 0;
     const int64_t staging = rq->mem_kind == 0 ? std::min<int64_t>(q * m * n * 4, int64_t(256) << 20) : 0;
-    const int64_t scratch = q * (n + ns + 2 * m + 16 * 16 * 2 + 4 * 16 * m) * 4;
+    // the task engine's partial sums, or what the streaming engine (the library's
+    // choice) keeps per column: W by column chunks, Q, the support's columns
+    int64_t per_col = 4 * 16 * m;
+    if (rq->opt.engine == 0 && n > 0 && m > 0 && r > 0 && r <= 16 && std::max(n, m) < (int64_t(1) << 24)) {
+      lrs::StreamProblem p{};
+      p.L.n = static_cast<int>(n);
+      p.L.ns = static_cast<int>(ns);
+      p.L.m = static_cast<int>(m);
+      p.L.r = static_cast<int>(r);
+      p.L.rho = static_cast<int>(rho);
+      lrs::stream_plan(p, lrs::sweep_rpad(static_cast<int>(r)));
+      per_col = std::max<int64_t>(per_col, int64_t(p.ncw + 1) * p.wstride + (rho + 2) * p.astride + 2 * rho);
+    }
+    const int64_t scratch = q * (n + ns + 2 * m + 16 * 16 * 2 + per_col) * 4;
     b = stored + exact + staging + scratch + q * m * 8 + q * rho * 8 + 4 * n * 16;
   }
   return static_cast<size_t>(b + b / 10) + (size_t(64) << 20);

@@ -144,3 +144,14 @@ def test_compatible_gaussian_requests_are_admitted_together():
     assert all(r.error is None for r in res)
     for i in (2, 3):                   # one worker, one start and end per batch
         assert abs(by[i].start - by[1].start) < 1e-3 and abs(by[i].end - by[1].end) < 1e-3
+
+
+@pytest.mark.parametrize("n,m,r,rho", [(256, 200, 16, 10), (1000, 300, 5, 500), (4096, 512, 10, 800)])
+def test_footprint_covers_the_streaming_engine(n, m, r, rho):
+    """Per column: A_k, y_k, h_k, eight (from 96 tiles of 32 columns on, four) partial
+    W and Q of r ranks, and the support's columns in float32."""
+    q = 10000
+    rq = L.lrs_request(n=n, m=m, q=q, r=r, rho=rho, kind=L.LRS_OP_GAUSSIAN, mem_kind=1)
+    chunks = 4 if n >= 96 * 32 else 8
+    per_col = m * n + m + n + (chunks + 1) * r * m + rho * m
+    assert L.lrs_request_footprint(rq) >= q * per_col * 4
