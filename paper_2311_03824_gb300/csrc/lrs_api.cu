@@ -839,6 +839,28 @@ lrs_status alloc_task_engine(lrs_ctx* h) {
   return plan_tables(h, kib, h->tF);
 }
 
+// The streaming engine's scratch did not fit memory (it keeps the support's
+// columns: with wide supports as much again as A_k): the task engine, over the
+// same layout of A_k.
+lrs_status stream_to_task(lrs_ctx* h, int nsm) {
+  void** ps[] = {reinterpret_cast<void**>(&h->dsp),     reinterpret_cast<void**>(&h->sasg),
+                 reinterpret_cast<void**>(&h->s_cnt),   reinterpret_cast<void**>(&h->s_list),
+                 reinterpret_cast<void**>(&h->s_supj),  reinterpret_cast<void**>(&h->s_nsup),
+                 reinterpret_cast<void**>(&h->s_sweep), reinterpret_cast<void**>(&h->s_nmax),
+                 reinterpret_cast<void**>(&h->s_Wp),    reinterpret_cast<void**>(&h->s_Wk),
+                 reinterpret_cast<void**>(&h->s_AG),    reinterpret_cast<void**>(&h->s_u),
+                 reinterpret_cast<void**>(&h->s_g),     reinterpret_cast<void**>(&h->s_supv),
+                 reinterpret_cast<void**>(&h->s_Li)};
+  for (void** p : ps) {
+    if (*p) cudaFreeAsync(*p, h->stream);
+    *p = nullptr;
+  }
+  cudaGetLastError();
+  h->engine = 2;
+  if (!plan_task_engine(h, nsm)) return fail(LRS_ERR_OOM, "the sweep's scratch does not fit memory");
+  return alloc_task_engine(h);
+}
+
 // The shared sweep of a batch: its device tables (freed by release, stream-
 // ordered) and its launch.
 struct BatchLaunch {
@@ -1143,7 +1165,9 @@ lrs_status lrs_create(int64_t n, int64_t m, int64_t q, int32_t r, int32_t rho, l
       (st = dalloc(&h->P, size_t(q) * r, h->stream)) || (st = dalloc(&h->part, size_t(h->nblk) * r * r, h->stream)) ||
       (st = dalloc(&h->small, 4 * 16 * 16 + 64, h->stream)) || (st = dalloc(&h->eta, 1, h->stream)) ||
       (st = dalloc(&h->err, 2, h->stream)) || (st = dalloc(&h->errpart, 2 * size_t(q), h->stream)) ||
-      (h->engine == 2 && (st = alloc_task_engine(h))) || (h->engine == 4 && (st = alloc_stream(h))) || (st = alloc_split(h, nsm))) {
+      (h->engine == 2 && (st = alloc_task_engine(h))) || (h->engine == 4 && (st = alloc_stream(h)) &&
+       (st != LRS_ERR_OOM || (st = stream_to_task(h, nsm)))) ||
+      (st = alloc_split(h, nsm))) {
     std::string msg = g_last_error;
     free_all(h);
     delete h;

@@ -332,3 +332,25 @@ def test_no_less_precise_than_the_task_engine(n, q, r, m, rho, err):
             tot[eng] += np.array([rel(g[1], ref.B), rel(g[3], Rv), rel(g[0], ref.U)]) ** 2
     print("B S U", np.sqrt(tot[0] / 3), np.sqrt(tot[2] / 3))
     assert (np.sqrt(tot[0]) <= 1.15 * np.sqrt(tot[2])).all(), (np.sqrt(tot[0] / 3), np.sqrt(tot[2] / 3))
+
+
+def test_task_engine_where_the_streaming_scratch_does_not_fit():
+    """rho = n: the support's columns are as large as A_k (1.07 GB).  With 1.9 GB
+    free the task engine takes the problem; with memory to spare, streaming."""
+    import torch
+    from paper_2311_03824_gb300 import Solver
+    from paper_2311_03824_gb300 import lrs as L
+    engines, keep = [], None
+    for room in (None, 1900 << 20):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        if room:
+            keep = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        s = Solver(2048, 512, 256, 4, 2048)
+        try:
+            engines.append(L.lrs_describe(s.h)["engine"])
+        finally:
+            s.close()
+    del keep
+    torch.cuda.empty_cache()
+    assert engines == ["stream", "task"]
