@@ -186,3 +186,36 @@ def test_no_less_precise_than_fp64_factors(shape):
         tot += np.array([rel(B1, ref.B), rel(U1, ref.U)]) ** 2 / 3
     for err, bar in zip(np.sqrt(tot), FP64_FACTORS[shape]):
         assert bar is None or err <= 1.02 * bar, (err, bar)
+
+
+def test_ill_conditioned_least_squares():
+    """m = r + 1 samples per frame, as for the Gaussian operator: b_k of the frames of
+    cond(G_k) > 1e3 within max(1e-5, 10 x the float32 probe's deviation, 2 cond(G_k)
+    2^-24) of the FP64 step (the normal equations' float32 bound)."""
+    from tests.gpu_helpers import cast_state, probe_step, set_gpu_state, state_of
+    inst = FourierInstance(nx=8, ny=8, q=150, r=6, m=7, rho=1, seed=66, mask_law="uniform", b_law="gauss")
+    T, P = 4, Problem.fourier(inst)
+    _, log = O.run_alg1(O.FourierOperator(inst.masks, 8, 8), inst.Y, 6, 1, T, keep=tuple(range(T + 1)), Xstar=inst.Xstar)
+    s = new_fourier_solver(inst)
+    checked, worst = 0, 0.0
+    try:
+        for t in range(1, T):
+            st = state_of(log, t, P.n)
+            st64, _, dec, _ = probe_step(P, st)
+            st32 = cast_state(st, np.complex64)
+            O.iterate_alg1(P.op32, P.y32(P.Y), st32, P.rho)
+            set_gpu_state(s, st, True)
+            s.iterate(1)
+            B1 = s.get()[1]
+            W = P.op64.AU(st.U)
+            cond = np.array([np.linalg.cond(w.conj().T @ w) for w in W])
+            for k in np.where((cond > 1e3) & dec)[0]:
+                b64 = st64.B[:, k]
+                d32 = np.linalg.norm(st32.B[:, k] - b64) / np.linalg.norm(b64)
+                dg = np.linalg.norm(B1[:, k] - b64) / np.linalg.norm(b64)
+                assert dg <= max(1e-5, 10 * d32, 2 * cond[k] * 2.0 ** -24), (t, k, cond[k], dg, d32)
+                checked += 1
+                worst = max(worst, cond[k])
+    finally:
+        s.close()
+    assert checked >= 20 and worst > 3e3, (checked, worst)
