@@ -311,13 +311,16 @@ def run_ours(args):
             "config": {"workload": "gaussian n=1000 q=1000 r=5 m=150 rho=10 (float32 A_k, 600 MB)",
                        "l2": "inputs larger than L2 (A 600 MB)", "iterations_per_step": 1,
                        "engine": desc.get("engine"), "cuda_graph": True,
-                       "task_shape": {k: desc.get(k) for k in ("grid", "inflight", "w_tasks", "g_tasks", "rows_per_piece")},
+                       "engine_shape": {k: desc[k] for k in ("grid", "inflight", "w_tasks", "g_tasks", "rows_per_piece",
+                                                             "w_chunks", "w_row_blocks", "w_stages", "g_stages",
+                                                             "step_grid") if k in desc},
                        "rel_err_after": {"iterations": args.warmup + args.steps, "rel_err": rel_err}},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
                          "traffic": TASK_KERNEL_DRAM_BYTES if desc.get("engine") == "task" else None,
                          "peak_kind": peak_kind,
-                         "kernel": "task_kernel" if desc.get("engine") == "task" else "sweep_kernel",
+                         "kernel": {"task": "task_kernel", "stream": "w_kernel + step kernels + g_kernel"}.get(
+                             desc.get("engine"), "sweep_kernel"),
                          "kernel_ms": sweep_ms, "bytes_per_launch": bytes_launch},
             "phases_ms_per_step": {k: ph[k] / max(1, ph["iters"]) for k in ("sweep_ms", "grad_ms", "qr_ms")},
             "e2e": {"value": e2e_value, "unit": "column-iters/s", "h2d_bytes_per_step": h2d,

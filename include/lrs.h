@@ -117,8 +117,11 @@ typedef struct {
                                when two do not fit; 3 allowed for r <= 6)    */
   int32_t autotune;         /* task engine: 1 = run lrs_autotune (2 trial
                                iterations per shape) before the first
-                               iteration unless this shape is cached         */
-  int32_t grid;             /* task engine: CTAs of the persistent launch (0 ->
+                               iteration unless this shape is cached (the
+                               streaming engine has one shape: no effect)    */
+  int32_t grid;             /* task engine: CTAs of the persistent launch,
+                               streaming engine: CTAs of its passes over A_k,
+                               with the column steps in proportion (0 ->
                                all that fit; fewer let concurrent handles on
                                other streams share the GPU); resident engine:
                                at most grid / cluster clusters             */
@@ -177,8 +180,8 @@ lrs_status lrs_set_measurements(lrs_t h, const void* y, const void* A_or_mask,
 
 /* Initialisation of Algorithm 1: s_k = IHT(y_k, A_k, rho, tau0, 0),
  * L0 = [A_k^T (y_k - A_k s_k)], U0 = top-r left singular subspace of L0
- * (subspace iteration: float32 products L0^T U and L0 P, Cholesky-QR2 with
- * FP64 r x r factors, to power_tol), b_k = (A_k U0)^+ (y_k - A_k s_k).  State: MEASURED or later -> INITIALISED.
+ * (subspace iteration: float32 products L0^T U and L0 P, Cholesky-QR with
+ * FP64 or double-float r x r factors, to power_tol), b_k = (A_k U0)^+ (y_k - A_k s_k).  State: MEASURED or later -> INITIALISED.
  * Errors: LRS_ERR_STATE, LRS_ERR_NUMERICAL (non-SPD Gram, NaN), LRS_ERR_CUDA. */
 lrs_status lrs_init(lrs_t h);
 
@@ -221,14 +224,15 @@ lrs_status lrs_estimate_rank(lrs_t h, double energy, int32_t* r_out, double* sv,
  * LRS_ERR_NUMERICAL (column id in lrs_last_error), LRS_ERR_CUDA. */
 lrs_status lrs_iterate(lrs_t h, int32_t iters, double* err_log);
 
-/* `iters` GDmin iterations of several problems at once: every sweep is one
- * persistent launch of the task engine whose work table holds the columns of
+/* `iters` GDmin iterations of several problems at once: every launch of a sweep
+ * (of the streaming engine, or the task engine's one) holds the columns of
  * all nh handles (Section II-E: the per-column work is independent, so
  * uneven problems share the GPU's SMs in one launch); each handle then runs
  * its own gradient, step size and QR on its own stream.  Every handle ends
  * exactly as lrs_iterate(h, iters, NULL) would leave it alone, bit for bit.
  * hs: nh distinct handles (1 <= nh <= 64), INITIALISED or later, Gaussian,
- * task engine (engine 2), one rank width class and one A_k form, no reducer.
+ * streaming or task engine (handles of both run one after another), one rank
+ * width class and one A_k form, no reducer.
  * The call returns when every handle's work is done.  State -> ITERATING.
  * Errors: LRS_ERR_ARG, LRS_ERR_STATE, LRS_ERR_UNSUPPORTED (handles that
  * cannot share a launch), LRS_ERR_NUMERICAL, LRS_ERR_TIMEOUT, LRS_ERR_CUDA. */
@@ -287,7 +291,8 @@ lrs_status lrs_set_reference(lrs_t h, const void* Xref, int32_t mem_kind);
  * LRS_ERR_CUDA. */
 lrs_status lrs_phase_times(lrs_t h, double* out4);
 
-/* Autotuner of the task engine (the paper has no counterpart): from the
+/* Autotuner of the task engine (the paper has no counterpart; on a streaming
+ * handle it times the one shape and changes nothing): from the
  * current iterate, run trial_iters GDmin iterations
  * with each candidate task shape (128 / 256 / 512 KiB of A_k per task x
  * q, q/2 or 2 x grid columns in flight), restoring the iterate (U, B, S,
@@ -303,8 +308,9 @@ lrs_status lrs_autotune(lrs_t h, int32_t trial_iters, char* report, int32_t len)
 /* Orthonormalise the columns of Z by Cholesky-QR2 (the QR step of
  * Algorithm 1, U+ = QR(U - eta grad)): Q = Z R^{-1} with R the upper
  * triangular factor with positive diagonal, i.e. the Q factor of the QR
- * decomposition with diag(R) > 0.  Gram matrices and Cholesky factors are
- * FP64 (r x r), products FP32, two passes.
+ * decomposition with diag(R) > 0.  Up to n r = 409600 in one launch: Gram and
+ * factor in double-float (FP64 where that ends), Q rounded once, a second pass
+ * for ill-conditioned Z; beyond, FP64 factors, FP32 products, two passes.
  *  Z, Q:   device pointers, n x r row-major float (row i at offset i*r);
  *          Q may equal Z.  1 <= r <= 16, n >= r.
  *  stream: cudaStream_t (NULL = legacy default stream); the call allocates
@@ -393,7 +399,7 @@ typedef struct {
   void* runner_ctx;
   int32_t batch;            /* up to this many Gaussian requests admitted
                                together run their iterations in one
-                               persistent launch per sweep (lrs_iterate_batch;
+                               launch per phase of a sweep (lrs_iterate_batch;
                                0 or 1: every request alone)                 */
 } lrs_server_options;
 

@@ -3,7 +3,7 @@
 //
 // The cooperative launch of 152 blocks that it replaces where the matrix fits
 // took 82 us at n = 16384, r = 6 and 44 us at n = 400, r = 4: FP64 Gram loops,
-// two FP64 factors and two grid barriers; this one takes 30 and 14 us (44 and 17
+// two FP64 factors and two grid barriers; this one takes 35 and 14 us (44 and 17
 // with two passes always).  The
 // Gram is a double-float sum of exact products, exchanged through distributed
 // shared memory, and every CTA factors it redundantly in one warp's registers,

@@ -13,7 +13,8 @@
 //   K = sum_k zero-fill_k(res_k) b_k^H   k-space accumulation through the
 //                                  inverse index of the masks (fixed order)
 //   grad = F2^H K                  r inverse 2D FFTs (linearity of F2)
-//   eta at t = 1, U <- Q(U - eta grad) by complex Cholesky-QR2 (FP64 r x r).
+//   eta at t = 1, U <- Q(U - eta grad) by complex Cholesky-QR (cqr_cluster.cu;
+//                                  cqr2 below for what one cluster does not hold).
 // The initialisation forms L0 = [A_k^H (y_k - A_k s_k)] and its top-r left
 // singular subspace by FP64 complex subspace iteration.
 #include <cuda_runtime.h>
@@ -153,7 +154,6 @@ __device__ __forceinline__ void dit_side(float2* X, int nl, int ls, int es, int 
 // transforms them.  A power-of-two side by register passes, any other by a
 // direct DFT.
 //
-// One CTA per frame kept r of the 152 SMs busy (26 us at 128 x 128, r = 6); a
 // One CTA per frame kept r of the 152 SMs busy (26 us at 128 x 128, r = 6; with
 // the k-space sums 53 us per iteration, now 26). A launch per side was faster
 // there (39 us) and slower on frames up to 64 x 64 (22 us against 20; now 17).

@@ -71,7 +71,7 @@ struct FArgs {
 // Threads per frame, by its size: a 20 x 20 frame has 400 pixels and a few
 // hundred samples, and four 128-thread CTAs per SM (128 registers) take the
 // place of one of 512 threads that mostly waits at barriers (a 20 x 20 solve of
-// 400 frames: 215 -> 62 us per sweep).  On the largest frames 768 and 1024
+// 400 frames: with the rest of this sweep 215 -> 55 us).  On the largest frames 768 and 1024
 // threads were slower (128 x 128: 353 us per sweep with 512, 382 with 768, 449
 // with 1024: spills and more redundant work per warp).
 constexpr int kFT = 512;  // at most

@@ -3,10 +3,11 @@
 //   grad = sum_k h_k b_k^T                         (Section II-A, U-gradient)
 //   eta  = c_eta / ||grad||_2  at t = 1            (Algorithm 1, step size)
 //   U+   = Q(U - eta grad)                         (Algorithm 1, projected GD)
-// The Q factor comes from Cholesky-QR2: Gram matrices and Cholesky factors
+// The Q factor comes from one cluster (qr_cluster.cu) up to n r = 409600;
+// beyond, from the Cholesky-QR2 below: Gram matrices and Cholesky factors
 // in FP64 (r x r), the n x r products in FP32, two passes so that the
-// result is orthonormal to float32 precision.  R = R2 R1 has a positive
-// diagonal, so Q is the unique QR factor with positive diag(R).
+// result is orthonormal to float32 precision.  R has a positive diagonal, so Q
+// is the unique QR factor with positive diag(R).
 // Every reduction runs in a fixed order: results are bit-reproducible.
 #include "lrs_dev.cuh"
 #include "lrs_internal.h"

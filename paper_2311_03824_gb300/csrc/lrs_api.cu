@@ -264,7 +264,7 @@ lrs_status check_device_error(lrs_ctx* h, const char* where) {
   return fail(e[0] == kErrTimeout ? LRS_ERR_TIMEOUT : LRS_ERR_NUMERICAL, msg);
 }
 
-// Bound of every device-side wait of the task and resident engines.
+// Bound of every device-side wait of the task, streaming and resident engines.
 unsigned long long wait_bound_ns(const lrs_ctx* h) {
   return static_cast<unsigned long long>(h->opt.wait_ms > 0 ? h->opt.wait_ms : 10000) * 1000000ull;
 }
